@@ -16,10 +16,11 @@
 // Three kernels.  bwd_point_kernel does what belongs to the query pixel: a, dl (kept in a workspace for
 // the other two), dq and the bias gradient.  bwd_gather_kernel computes dk and dv per key / value pixel by
 // gathering from the k x k query pixels whose windows hold it (out-of-map queries contribute nothing:
-// their q, g tiles read as zero).  bwd_weight_kernel (persistent CTAs, one head each) sums the weight
-// gradients over the pixels with lane = channel, so that a lane's 2 k^4 accumulators live in registers
-// over all its tiles and no reduction across lanes is needed; one addition per weight and CTA goes to
-// global memory at its end.
+// their q, g tiles read as zero).  The weight gradients: for k = 3 on the tensor cores (bwd_weight_kernel.cu); for
+// k = 1, where there is nothing to contract, bwd_weight_kernel here (persistent CTAs, one head each) sums them over
+// the pixels with lane = channel, so that a lane's 2 k^4 accumulators live in registers over all its tiles; one
+// addition per weight and CTA goes to global memory at its end.
+#include "bwd_common.cuh"
 #include "tile_common.cuh"
 
 namespace slide_attn {
@@ -27,23 +28,6 @@ namespace slide_attn {
 namespace {
 
 using namespace tile;
-
-struct BwdParams {
-    const float* wt;                 // transposed weights wk^T then wv^T, [slot][tap][C]
-    const float* bias;
-    void* dq;
-    void* dk;
-    void* dv;
-    float* dwk;
-    float* dwv;
-    float* dbias;
-    float* ws_a;                     // [pixel][head][k*k]
-    float* ws_dl;
-    int* status;
-    int B, H, W, heads;
-    int tiles_x, tiles_y;
-    float scale;                     // 1 / sqrt(head_dim)
-};
 
 // the lane's eight weights of one (slot, tap) vector of 32 floats, and the same addressing for adds
 template <typename T> struct WVec;
@@ -571,10 +555,9 @@ template <typename T, int K>
 cudaError_t launch_t(const Problem& p, const BackwardArgs& ga, const float* wt, float* ws_a, float* ws_dl,
                      int* d_status, int num_sms, cudaStream_t stream) {
     using C_ = Cfg<T, K>;
-    static bool done_a[64] = {}, done_b[64] = {}, done_c[64] = {};
+    static bool done_a[64] = {}, done_b[64] = {};
     cudaError_t e = ensure_smem(bwd_point_kernel<T, K>, PointCfg<T, K>::total, done_a);
     if (e == cudaSuccess) e = ensure_smem(bwd_gather_kernel<T, K>, GatherCfg<T, K>::total, done_b);
-    if (e == cudaSuccess) e = ensure_smem(bwd_weight_kernel<T, K>, WeightCfg<T, K>::total, done_c);
     if (e != cudaSuccess) return e;
     BwdParams P;
     P.wt = wt; P.bias = p.bias;
@@ -604,11 +587,18 @@ cudaError_t launch_t(const Problem& p, const BackwardArgs& ga, const float* wt, 
     bwd_gather_kernel<T, K><<<(unsigned)ctas, C_::threads, GatherCfg<T, K>::total, stream>>>(mqh, mgh, P);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    long long per_head = (2LL * num_sms + p.heads - 1) / p.heads;            // persistent CTAs of the weight kernel
-    if (per_head > tiles_per_head) per_head = tiles_per_head;
-    if (per_head < 1) per_head = 1;
-    bwd_weight_kernel<T, K><<<(unsigned)(per_head * p.heads), C_::threads, WeightCfg<T, K>::total, stream>>>(mq, mk, mv, mg, P);
-    return cudaGetLastError();
+    if constexpr (K == 3) {
+        return launch_bwd_weight_mma(p, ga, P, num_sms, stream);
+    } else {
+        static bool done_c[64] = {};
+        e = ensure_smem(bwd_weight_kernel<T, K>, WeightCfg<T, K>::total, done_c);
+        if (e != cudaSuccess) return e;
+        long long per_head = (2LL * num_sms + p.heads - 1) / p.heads;        // persistent CTAs of the weight kernel
+        if (per_head > tiles_per_head) per_head = tiles_per_head;
+        if (per_head < 1) per_head = 1;
+        bwd_weight_kernel<T, K><<<(unsigned)(per_head * p.heads), C_::threads, WeightCfg<T, K>::total, stream>>>(mq, mk, mv, mg, P);
+        return cudaGetLastError();
+    }
 }
 
 template <typename T>

@@ -1,0 +1,364 @@
+// Weight gradients of the backward pass for k = 3 (head_dim 32, fp32 or bf16 storage) on tensor cores:
+//
+//   dwk[c,s,t] = scale * sum over pixels of dl[s] (q[c] k_t[c])        dwv[c,s,t] = sum of a[s] (g[c] v_t[c])
+//
+// For one tap t and one side this is a matrix product over the pixels: [channels x pixels] . [pixels x slots],
+// with the elementwise products as the left operand.  mma.sync.m16n8k16, M = 16 channels, K = 16 pixels (2 rows
+// x 8 columns), N = 32 columns that hold the nine slots three times: the upper, middle and lower 8 bits of the
+// fp32 dl (a), so that a bf16 tensor-core product loses none of them.  The left operand is split too: bf16
+// inputs multiply exactly into hi + lo, fp32 products into hi + mid + lo; the pairs below 2^-24 are left out
+// (hi meets all four 8-column tiles, the next part the first three, the last part the first two).
+//
+// Persistent, one CTA per SM and one head per CTA.  Twelve compute warps = side x 16-channel half x tap row,
+// three per scheduler; a warp keeps the sums of its three taps in registers over all its tiles.  The tensor core
+// truncates when it accumulates, so the columns that hold upper parts move to a second set of fp32 registers
+// after every kFlush pixel groups (eight to twelve tensor-core steps).  Tiles (4 rows x up to 56 columns + halo)
+// come by TMA into two stages, in channel planes that give a conflict-free fragment load: bf16 eight channels
+// (16 bytes a pixel), so that one transposing ldmatrix is a whole left operand at any tap's offset; fp32, which
+// ldmatrix cannot transpose, 16 channels (four pixels x eight channel pairs = 256 contiguous bytes).  Four more
+// warps turn the attention weights and logit gradients into the split columns (64 bytes per pixel, 16-byte chunks
+// swizzled so that ldmatrix meets no bank conflict).
+//
+// Bound by the mma.sync pipe and the CUDA-core work beside it, which hardly overlap (measured: 8 cycles per MMA and
+// scheduler, and each packed bf16 multiply or fp32 add next to it adds 0.75 - 1.5): 252 MMAs (bf16; 324 for fp32) per
+// 16 pixels of a head.  64 x 56 x 56, 3 heads, bf16: 410 us with fp32 FMAs (lane = channel, 2 x 81 sums in registers),
+// 145 us here; 2 x 128 x 128, 3 heads, fp32: 76 and 49 us.
+#include "bwd_common.cuh"
+#include "split.cuh"
+
+namespace slide_attn {
+
+namespace {
+
+using namespace split;
+
+constexpr int kHeadDim = 32;
+constexpr int kK2 = 9;
+constexpr int kTH = 4;                         // tile rows
+constexpr int kComputeWarps = 12, kConvertWarps = 4;
+constexpr int kThreads = (kComputeWarps + kConvertWarps) * 32;
+constexpr int kFlush = 4;
+constexpr uint32_t kSumBytes = 2u * kK2 * kHeadDim * 32u * 4u;        // the CTA's sums at its end, [side][tap][channel][32 columns]
+
+template <typename T> struct WTile;
+template <> struct WTile<__nv_bfloat16> { static constexpr int max_w = 56, planes = 4; };
+template <> struct WTile<float> { static constexpr int max_w = 32, planes = 2; };
+
+// Stage layout for tiles of tw columns (bytes); the channel planes of a tensor follow each other.
+struct WLayout {
+    uint32_t halo_plane, tile_plane;           // one plane with halo (k, v), without (q, g)
+    uint32_t k_off, v_off, q_off, g_off;
+    uint32_t split_off, split_side;            // dl columns, then a columns: [pixel][32] bf16
+    uint32_t stage;                            // bytes of a stage
+    uint32_t tx_bytes;
+};
+template <typename T>
+__host__ __device__ inline WLayout w_layout(int tw) {
+    constexpr uint32_t np = (uint32_t)WTile<T>::planes, pb = 32u / np * (uint32_t)sizeof(T);
+    auto up = [](uint32_t x) { return (x + 127u) & ~127u; };
+    WLayout L;
+    const uint32_t halo = (uint32_t)((kTH + 2) * (tw + 2)) * pb, tile = (uint32_t)(kTH * tw) * pb;
+    L.halo_plane = up(halo); L.tile_plane = up(tile);
+    L.k_off = 0; L.v_off = np * L.halo_plane; L.q_off = 2 * np * L.halo_plane; L.g_off = L.q_off + np * L.tile_plane;
+    L.split_off = L.g_off + np * L.tile_plane;
+    L.split_side = (uint32_t)(kTH * tw) * 64u;
+    L.stage = L.split_off + 2 * L.split_side;
+    L.tx_bytes = 2 * np * (halo + tile);
+    return L;
+}
+
+template <typename T>
+uint32_t w_smem_bytes(int tw) {
+    const uint32_t stages = 2 * w_layout<T>(tw).stage;
+    return (stages > kSumBytes ? stages : kSumBytes) + 64 + 128;      // + barriers + alignment slack
+}
+
+struct WParams {
+    const float* ws_a;
+    const float* ws_dl;
+    float* dwk;
+    float* dwv;
+    int* status;
+    int B, H, W, heads;
+    int tw, tiles_x, tiles_y;
+    float scale;
+};
+
+// One 16-pixel (2 rows x 8 columns), 16-channel operand tile in registers: for bf16 the A fragment of the raw
+// values, for fp32 the values of channels 2g, 2g + 1 of the lane's four pixels.  `offset` and `col` say where a lane
+// reads, in a tile whose planes are `plane` bytes and whose rows are `pitch` bytes apart, and which column of the
+// group the K index k (of its row's eight) is.
+template <typename T> struct Frag;
+template <> struct Frag<__nv_bfloat16> {
+    static constexpr uint32_t pixel_bytes = 16;
+    uint32_t a[4];
+    // lane i: row i % 8 of matrix i / 8 = (channels 0-7 row 0, channels 8-15 row 0, channels 0-7 row 1, ..)
+    static __device__ __forceinline__ uint32_t offset(int lane, int half, uint32_t plane, uint32_t pitch) {
+        return (uint32_t)(2 * half + ((lane >> 3) & 1)) * plane + (uint32_t)(lane >> 4) * pitch + (uint32_t)(lane & 7) * pixel_bytes;
+    }
+    static __device__ __forceinline__ int col(int k) { return k; }
+    static __device__ __forceinline__ int channel(int row) { return row; }
+    __device__ __forceinline__ void load(uint32_t p, uint32_t) { ldmatrix_x4_trans(p, a[0], a[1], a[2], a[3]); }
+};
+template <> struct Frag<float> {
+    static constexpr uint32_t pixel_bytes = 64;
+    float2 a[4];
+    static __device__ __forceinline__ uint32_t offset(int lane, int half, uint32_t plane, uint32_t) {
+        return (uint32_t)half * plane + (uint32_t)(lane & 3) * pixel_bytes + (uint32_t)(lane >> 2) * 8u;
+    }
+    static __device__ __forceinline__ int col(int k) { return (k & 1) * 4 + (k >> 1); }
+    static __device__ __forceinline__ int channel(int row) { return 2 * (row & 7) + (row >> 3); }
+    __device__ __forceinline__ void load(uint32_t p, uint32_t pitch) {
+        a[0] = lds_f2(p); a[1] = lds_f2(p + 4 * pixel_bytes);
+        a[2] = lds_f2(p + pitch); a[3] = lds_f2(p + pitch + 4 * pixel_bytes);
+    }
+};
+
+// acc += (x . y) times the split columns b[tile][2]
+__device__ __forceinline__ void accumulate(float (&acc)[4][4], const Frag<__nv_bfloat16>& x, const Frag<__nv_bfloat16>& y,
+                                           const uint32_t (&b)[4][2]) {
+    uint32_t hi[4], lo[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) product2(x.a[i], y.a[i], hi[i], lo[i]);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) mma_bf16(acc[j], hi, b[j][0], b[j][1]);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) mma_bf16(acc[j], lo, b[j][0], b[j][1]);
+}
+__device__ __forceinline__ void accumulate(float (&acc)[4][4], const Frag<float>& x, const Frag<float>& y, const uint32_t (&b)[4][2]) {
+    float2 p[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) p[i] = mul2(x.a[i], y.a[i]);
+#pragma unroll
+    for (int part = 0; part < 3; ++part) {
+        const uint32_t a[4] = {pack_upper(p[0].x, p[1].x), pack_upper(p[0].y, p[1].y), pack_upper(p[2].x, p[3].x), pack_upper(p[2].y, p[3].y)};
+#pragma unroll
+        for (int j = 0; j < 4 - part; ++j) mma_bf16(acc[j], a, b[j][0], b[j][1]);
+        if (part < 2)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) p[i] = rest2(p[i]);
+    }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kThreads, 1)
+bwd_weight_mma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
+                      const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_g, const WParams P)
+{
+    constexpr uint32_t PB = Frag<T>::pixel_bytes;                    // of one plane
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char* smem = smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u);
+    const WLayout L = w_layout<T>(P.tw);
+    const uint32_t stages = 2 * L.stage;
+    const uint32_t bar0 = smem_u32(smem) + (stages > kSumBytes ? stages : kSumBytes);
+    auto bar_full = [&](int s) { return bar0 + 8u * (uint32_t)s; };
+    auto bar_empty = [&](int s) { return bar0 + 16u + 8u * (uint32_t)s; };
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int g = lane >> 2, tig = lane & 3;
+    const int h = blockIdx.x % P.heads, rank = blockIdx.x / P.heads;
+    const int nrank = (int)gridDim.x / P.heads;                      // the grid is a multiple of the heads
+    const int tiles = P.B * P.tiles_y * P.tiles_x;
+    const int HW = P.tw + 2;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < 2; ++s) { mbar_init_only(bar_full(s), 1 + kConvertWarps); mbar_init_only(bar_empty(s), kComputeWarps); }
+        mbar_init_fence();
+    }
+    __syncthreads();
+
+    float acc[3][4][4], sum[3][2][4];
+    bool ok = true;
+    const int side = warp / 6, half = (warp / 3) & 1, ty = warp % 3;  // of a compute warp
+
+    if (warp >= kComputeWarps) {
+        // ---- loads and split columns ----------------------------------------------------------------
+        const int ct = threadIdx.x - kComputeWarps * 32;
+        const int npix = kTH * P.tw;
+        int it = 0;
+        for (int tile = rank; tile < tiles && ok; tile += nrank, ++it) {
+            const int st = it & 1;
+            int rest_ = tile;
+            const int tx = rest_ % P.tiles_x; rest_ /= P.tiles_x;
+            const int tyy = rest_ % P.tiles_y;
+            const int b = rest_ / P.tiles_y;
+            const int x0 = tx * P.tw, y0 = tyy * kTH;
+            unsigned char* stage = smem + (uint32_t)st * L.stage;
+            if (it >= 2 && !__all_sync(0xffffffffu, mbar_wait(bar_empty(st), (uint32_t)(it / 2 - 1) & 1u) ? 1 : 0)) { ok = false; break; }
+            if (ct == 0) {
+                mbar_expect_tx(bar_full(st), L.tx_bytes);
+#pragma unroll
+                for (int pl = 0; pl < WTile<T>::planes; ++pl) {
+                    const int c0 = h * kHeadDim + pl * (32 / WTile<T>::planes);
+                    tma_load_4d(smem_u32(stage + L.k_off + pl * L.halo_plane), &map_k, bar_full(st), c0, x0 - 1, y0 - 1, b);
+                    tma_load_4d(smem_u32(stage + L.v_off + pl * L.halo_plane), &map_v, bar_full(st), c0, x0 - 1, y0 - 1, b);
+                    tma_load_4d(smem_u32(stage + L.q_off + pl * L.tile_plane), &map_q, bar_full(st), c0, x0, y0, b);
+                    tma_load_4d(smem_u32(stage + L.g_off + pl * L.tile_plane), &map_g, bar_full(st), c0, x0, y0, b);
+                }
+            }
+            for (int i = ct; i < 2 * npix; i += kConvertWarps * 32) {
+                const int sd = i >= npix, px = sd ? i - npix : i;
+                const int py = px / P.tw, pxx = px - py * P.tw;
+                const int y = y0 + py, x = x0 + pxx;
+                float f[kK2];
+                if (y < P.H && x < P.W) {
+                    const float* src = (sd ? P.ws_a : P.ws_dl) + (((size_t)(b * P.H + y) * P.W + x) * P.heads + h) * kK2;
+#pragma unroll
+                    for (int s = 0; s < kK2; ++s) f[s] = __ldg(src + s);
+                } else {
+#pragma unroll
+                    for (int s = 0; s < kK2; ++s) f[s] = 0.f;
+                }
+                // columns: 9 upper parts, 9 middle parts, 9 lower parts, zeros
+                float v[28];
+#pragma unroll
+                for (int s = 0; s < kK2; ++s) {
+                    v[s] = f[s];
+                    v[9 + s] = rest(v[s]);
+                    v[18 + s] = rest(v[9 + s]);
+                }
+                v[27] = 0.f;
+                unsigned char* dst = stage + L.split_off + (uint32_t)sd * L.split_side + (uint32_t)px * 64u;
+                const uint32_t swz = (uint32_t)(px >> 1) & 3u;
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    uint4 o;
+                    o.x = pack_upper(v[8 * c], v[8 * c + 1]); o.y = pack_upper(v[8 * c + 2], v[8 * c + 3]);
+                    o.z = c < 3 ? pack_upper(v[8 * c + 4], v[8 * c + 5]) : 0u;
+                    o.w = c < 3 ? pack_upper(v[8 * c + 6], v[8 * c + 7]) : 0u;
+                    *reinterpret_cast<uint4*>(dst + (((uint32_t)c ^ swz) << 4)) = o;
+                }
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar_full(st));
+        }
+    } else {
+        // ---- products and sums ----------------------------------------------------------------------
+#pragma unroll
+        for (int t = 0; t < 3; ++t) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+#pragma unroll
+                for (int x = 0; x < 4; ++x) acc[t][j][x] = 0.f;
+#pragma unroll
+            for (int j = 0; j < 2; ++j)
+#pragma unroll
+                for (int x = 0; x < 4; ++x) sum[t][j][x] = 0.f;
+        }
+        auto flush = [&]() {
+#pragma unroll
+            for (int t = 0; t < 3; ++t)
+#pragma unroll
+                for (int j = 0; j < 2; ++j)
+#pragma unroll
+                    for (int x = 0; x < 4; ++x) { sum[t][j][x] += acc[t][j][x]; acc[t][j][x] = 0.f; }
+        };
+        // lane i of the ldmatrix of the split columns: K index i % 8 of row (i / 8) % 2, 16-byte chunk i / 16 (+ 2)
+        const int kcol = Frag<T>::col(lane & 7);
+        const uint32_t b_off = L.split_off + (uint32_t)side * L.split_side + (uint32_t)(((lane >> 3) & 1) * P.tw + kcol) * 64u;
+        const uint32_t b_chunk0 = (((uint32_t)lane >> 4) ^ ((uint32_t)kcol >> 1)) << 4;
+        const uint32_t b_chunk1 = ((2u + ((uint32_t)lane >> 4)) ^ ((uint32_t)kcol >> 1)) << 4;
+        const uint32_t x_pitch = (uint32_t)P.tw * PB, y_pitch = (uint32_t)HW * PB;
+        const uint32_t x_off = (side ? L.g_off : L.q_off) + Frag<T>::offset(lane, half, L.tile_plane, x_pitch);
+        const uint32_t y_off = (side ? L.v_off : L.k_off) + (uint32_t)ty * y_pitch + Frag<T>::offset(lane, half, L.halo_plane, y_pitch);
+        int it = 0, pending = 0;
+        for (int tile = rank; tile < tiles; tile += nrank, ++it) {
+            const int st = it & 1;
+            int rest_ = tile;
+            const int tx = rest_ % P.tiles_x; rest_ /= P.tiles_x;
+            const int tyy = rest_ % P.tiles_y;
+            const int gx = min(P.tw, P.W - tx * P.tw), gy = min(kTH, P.H - tyy * kTH);   // part of the tile inside the map
+            const uint32_t stage = smem_u32(smem) + (uint32_t)st * L.stage;
+            if (!__all_sync(0xffffffffu, mbar_wait(bar_full(st), (uint32_t)(it / 2) & 1u) ? 1 : 0)) { ok = false; break; }
+            for (int r = 0; r < gy; r += 2) {
+                uint32_t ba = stage + b_off + (uint32_t)(r * P.tw) * 64u;
+                uint32_t xa = stage + x_off + (uint32_t)r * x_pitch, ya = stage + y_off + (uint32_t)r * y_pitch;
+                for (int c = 0; c < gx; c += 8, ba += 8 * 64, xa += 8 * PB, ya += 8 * PB) {
+                    uint32_t b[4][2];
+                    ldmatrix_x4_trans(ba + b_chunk0, b[0][0], b[0][1], b[1][0], b[1][1]);
+                    ldmatrix_x4_trans(ba + b_chunk1, b[2][0], b[2][1], b[3][0], b[3][1]);
+                    Frag<T> x, y[3];
+                    x.load(xa, x_pitch);
+#pragma unroll
+                    for (int t = 0; t < 3; ++t) y[t].load(ya + t * PB, y_pitch);
+#pragma unroll
+                    for (int t = 0; t < 3; ++t) accumulate(acc[t], x, y[t], b);
+                    if (++pending == kFlush) { pending = 0; flush(); }
+                }
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar_empty(st));
+        }
+        flush();
+    }
+    if (!ok && lane == 0) atomicExch(P.status, 1);
+    __syncthreads();                                                 // every load has been waited for: the stages are free
+    float* s_sum = reinterpret_cast<float*>(smem);
+    if (warp < kComputeWarps) {
+#pragma unroll
+        for (int t = 0; t < 3; ++t)
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+#pragma unroll
+                for (int x = 0; x < 4; ++x) {
+                    const int ch = half * 16 + Frag<T>::channel(g + 8 * (x >> 1));
+                    const float v = j < 2 ? sum[t][j & 1][x] : acc[t][j][x];
+                    s_sum[((side * kK2 + ty * 3 + t) * kHeadDim + ch) * 32 + 8 * j + 2 * tig + (x & 1)] = v;
+                }
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < 2 * kHeadDim * kK2 * kK2; i += kThreads) {
+        const int sd = i >= kHeadDim * kK2 * kK2, rem = sd ? i - kHeadDim * kK2 * kK2 : i;
+        const int ch = rem / (kK2 * kK2), st = rem - ch * kK2 * kK2;
+        const int s = st / kK2, t = st - s * kK2;
+        const float* p = s_sum + ((sd * kK2 + t) * kHeadDim + ch) * 32 + s;
+        const float v = p[0] + (p[9] + p[18]);
+        atomicAdd((sd ? P.dwv : P.dwk) + (size_t)(h * kHeadDim) * kK2 * kK2 + rem, sd ? v : v * P.scale);
+    }
+}
+
+template <typename T>
+cudaError_t launch_t(const Problem& p, const BackwardArgs& ga, const BwdParams& BP, int num_sms, cudaStream_t stream) {
+    static bool done[64] = {};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev >= 64 || !done[dev]) {
+        e = cudaFuncSetAttribute(bwd_weight_mma_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)w_smem_bytes<T>(WTile<T>::max_w));
+        if (e != cudaSuccess) return e;
+        if (dev < 64) done[dev] = true;
+    }
+    // the tile width (a multiple of 8) that covers the map with the fewest columns, the widest of those
+    int tw = 8, cover = 1 << 30;
+    for (int t = 8; t <= WTile<T>::max_w; t += 8) {
+        const int c = (p.W + t - 1) / t * t;
+        if (c <= cover) { cover = c; tw = t; }
+    }
+    WParams P;
+    P.ws_a = BP.ws_a; P.ws_dl = BP.ws_dl; P.dwk = BP.dwk; P.dwv = BP.dwv; P.status = BP.status;
+    P.B = p.B; P.H = p.H; P.W = p.W; P.heads = p.heads;
+    P.tw = tw; P.tiles_x = (p.W + tw - 1) / tw; P.tiles_y = (p.H + kTH - 1) / kTH;
+    P.scale = BP.scale;
+    const int Ctot = p.heads * kHeadDim, es = (int)sizeof(T), bc = kHeadDim / WTile<T>::planes;
+    CUtensorMap mq, mk, mv, mg;
+    if (!make_tile_map(&mq, p.q, es, p.B, p.H, p.W, Ctot, bc, tw, kTH) ||
+        !make_tile_map(&mg, ga.dout, es, p.B, p.H, p.W, Ctot, bc, tw, kTH) ||
+        !make_tile_map(&mk, p.k, es, p.B, p.H, p.W, Ctot, bc, tw + 2, kTH + 2) ||
+        !make_tile_map(&mv, p.v, es, p.B, p.H, p.W, Ctot, bc, tw + 2, kTH + 2))
+        return cudaErrorInvalidValue;
+    const long long tiles = (long long)P.tiles_x * P.tiles_y * p.B;
+    if (tiles > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+    long long per_head = num_sms / p.heads;                          // one CTA per SM, all heads alike
+    if (per_head > tiles) per_head = tiles;
+    if (per_head < 1) per_head = 1;
+    bwd_weight_mma_kernel<T><<<(unsigned)(per_head * p.heads), kThreads, w_smem_bytes<T>(tw), stream>>>(mq, mk, mv, mg, P);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_bwd_weight_mma(const Problem& p, const BackwardArgs& ga, const BwdParams& P, int num_sms, cudaStream_t stream) {
+    return p.dtype == SLIDE_ATTN_BF16 ? launch_t<__nv_bfloat16>(p, ga, P, num_sms, stream) : launch_t<float>(p, ga, P, num_sms, stream);
+}
+
+}  // namespace slide_attn

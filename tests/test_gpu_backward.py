@@ -89,6 +89,20 @@ def test_backward_no_bias_dense_weights_and_repeat(dtype):
         assert np.array_equal(a[n], b[n])           # no atomics on these: bit-identical
 
 
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("shape", [(4, 21, 60, 8, 3), (2, 19, 57, 5, 3), (3, 6, 120, 4, 3)], ids=lambda s: "x".join(map(str, s)))
+def test_backward_several_tiles_per_cta(shape, dtype):
+    """More tiles than CTAs per head (both stages of the weight kernel used again), widths at the edges of its
+    tile widths, odd heights.  dq, dk, dv as elsewhere; the weight gradients are fp32 sums of about 5000 exact
+    products in two levels of accumulation: 1e-5 of the largest entry."""
+    x, dout = inputs(shape, dtype)
+    ref = ob.backward(x["q"], x["k"], x["v"], x["wk"], x["wv"], x["bias"], 3, dout)
+    got = gpu_backward(x, dout, 3, dtype)[0]
+    check(got, ref, dtype, f"{shape} {dtype}")
+    for n in ("dwk", "dwv", "dbias"):
+        assert np.abs(got[n] - ref[n]).max() <= 1e-5 * np.abs(ref[n]).max(), n
+
+
 def test_backward_stage_shape_sample():
     """Four images of the bench shape (56 x 56, 2 heads), bf16."""
     x, dout = inputs((4, 56, 56, 2, 3), "bf16", sigma_w=0.02)
