@@ -67,6 +67,12 @@ size_t umma_ts_workspace_bytes(int heads);
 cudaError_t launch_umma_ts_prep(const Problem& p, void* workspace, cudaStream_t stream);
 cudaError_t launch_umma_ts(const Problem& p, const void* workspace, int* d_status, int num_sms, cudaStream_t stream);
 
+// UMMA_SPLIT variant: fp32 arithmetic on tcgen05 through exact splits (k = 3, head_dim 32 or 64, both dtypes); a prep
+// launch writes the weight images of every head to `workspace`.
+bool umma_split_supports(int head_dim, int ksize);
+size_t umma_split_workspace_bytes(int heads, int head_dim);
+cudaError_t launch_umma_split(const Problem& p, void* workspace, int* d_status, int num_sms, cudaStream_t stream);
+
 // Fixed-shift fast path: plain k x k local attention for weights that are exactly the one-hot shift
 // kernels (head_dim 32, k <= 9, fp32 or bf16).  launch_shift_check sets the status word to 2 when a
 // weight differs from the one-hot kernel.

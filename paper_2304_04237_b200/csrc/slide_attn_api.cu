@@ -14,10 +14,11 @@ struct slide_attn_ctx {
     int device;
     int num_sms;
     int* d_status;                   // device status word (0 = ok)
-    void* workspace;                 // re-laid-out weights for the variants that need them
-    size_t workspace_bytes;
+    void* arena;                     // one allocation: the status word and the five workspaces that follow
+    void* workspace;                 // weight fragments of the MMA variant
     void* strip_ws;                  // transposed weights of the STRIP variant
     void* umma_ws;                   // bf16 B images of the UMMA_TS variant
+    void* split_ws;                  // weight images of the UMMA_SPLIT variant
     void* wide_ws;                   // bf16 B fragments of the MMA_WIDE variant
     void* bwd_ws;                    // attention weights and logit gradients between the two backward kernels (first backward)
     void* block_ws;                  // q, k, v, z of slide_attn_block_forward (first use)
@@ -59,13 +60,14 @@ bool variant_supported(const slide_attn_ctx* c, slide_attn_variant v) {
         case SLIDE_ATTN_VARIANT_UMMA_TS: return c->umma_ws && umma_ts_supports(c->dtype, c->head_dim, c->ksize);
         case SLIDE_ATTN_VARIANT_TILE: return c->strip_ws && tile_supports(c->head_dim, c->ksize);
         case SLIDE_ATTN_VARIANT_MMA_WIDE: return c->wide_ws && mma_wide_supports(c->dtype, c->head_dim, c->ksize);
+        case SLIDE_ATTN_VARIANT_UMMA_SPLIT: return c->split_ws && umma_split_supports(c->head_dim, c->ksize);
         default: return false;
     }
 }
 
 slide_attn_variant pick_variant(const slide_attn_ctx* c) {
-    const slide_attn_variant order[] = {SLIDE_ATTN_VARIANT_UMMA_TS, SLIDE_ATTN_VARIANT_MMA, SLIDE_ATTN_VARIANT_MMA_WIDE, SLIDE_ATTN_VARIANT_TILE,
-                                        SLIDE_ATTN_VARIANT_STRIP, SLIDE_ATTN_VARIANT_DIRECT};
+    const slide_attn_variant order[] = {SLIDE_ATTN_VARIANT_UMMA_TS, SLIDE_ATTN_VARIANT_MMA, SLIDE_ATTN_VARIANT_MMA_WIDE, SLIDE_ATTN_VARIANT_UMMA_SPLIT,
+                                        SLIDE_ATTN_VARIANT_TILE, SLIDE_ATTN_VARIANT_STRIP, SLIDE_ATTN_VARIANT_DIRECT};
     for (slide_attn_variant v : order)
         if (variant_supported(c, v)) return v;
     return SLIDE_ATTN_VARIANT_DIRECT;
@@ -124,6 +126,10 @@ slide_attn_status launch_problem(slide_attn_ctx* c, const Problem& p, cudaStream
             if (ev) cudaEventRecord(ev[1], stream);          // the prep launch is issued inside launch_mma_wide
             err = launch_mma_wide(p, c->wide_ws, c->d_status, stream);
             break;
+        case SLIDE_ATTN_VARIANT_UMMA_SPLIT:
+            if (ev) cudaEventRecord(ev[1], stream);          // the prep launch is issued inside launch_umma_split
+            err = launch_umma_split(p, c->split_ws, c->d_status, c->num_sms, stream);
+            break;
         case SLIDE_ATTN_VARIANT_TILE:
             err = launch_strip_prep(p, c->strip_ws, stream);
             if (ev) cudaEventRecord(ev[1], stream);
@@ -170,46 +176,32 @@ slide_attn_status slide_attn_create(slide_attn_ctx** ctx, int B, int H, int W, i
     c->dtype = dtype;
     c->device = dev;
     c->num_sms = num_sms;
-    c->d_status = nullptr; c->workspace = nullptr; c->workspace_bytes = 0;
     c->stage = nullptr; c->stage_bytes = 0;
     c->profiling = false; c->prof_count = 0; c->prof_events = nullptr;
-    if (cudaMalloc(&c->d_status, sizeof(int)) != cudaSuccess ||
-        cudaMemset(c->d_status, 0, sizeof(int)) != cudaSuccess) {
+    if (mma_supports(dtype, head_dim, ksize) && (mma_setup() != cudaSuccess || umma_ts_setup() != cudaSuccess)) {
         cudaGetLastError();
+        slide_attn_destroy(c);
+        return SLIDE_ATTN_ERR_CUDA;
+    }
+    // the status word and every variant's workspace in one allocation: each cudaMalloc is tens of microseconds of a create
+    auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
+    const size_t b_mma = mma_supports(dtype, head_dim, ksize) ? up(mma_workspace_bytes(heads)) : 0;
+    const size_t b_umma = mma_supports(dtype, head_dim, ksize) ? up(umma_ts_workspace_bytes(heads)) : 0;
+    const size_t b_split = umma_split_supports(head_dim, ksize) ? up(umma_split_workspace_bytes(heads, head_dim)) : 0;
+    const size_t b_wide = mma_wide_supports(dtype, head_dim, ksize) ? up(mma_wide_workspace_bytes(heads, ksize)) : 0;
+    const size_t b_strip = strip_supports(head_dim, ksize) ? up(strip_workspace_bytes(heads, head_dim, ksize)) : 0;
+    if (cudaMalloc(&c->arena, 256 + b_mma + b_umma + b_split + b_wide + b_strip) != cudaSuccess) {
+        cudaGetLastError();
+        c->arena = nullptr;
         slide_attn_destroy(c);
         return SLIDE_ATTN_ERR_ALLOC;
     }
-    if (mma_supports(dtype, head_dim, ksize)) {
-        if (mma_setup() != cudaSuccess || umma_ts_setup() != cudaSuccess) {
-            cudaGetLastError();
-            slide_attn_destroy(c);
-            return SLIDE_ATTN_ERR_CUDA;
-        }
-        c->workspace_bytes = mma_workspace_bytes(heads);
-        if (cudaMalloc(&c->workspace, c->workspace_bytes) != cudaSuccess) {
-            cudaGetLastError();
-            c->workspace = nullptr;
-            slide_attn_destroy(c);
-            return SLIDE_ATTN_ERR_ALLOC;
-        }
-        if (cudaMalloc(&c->umma_ws, umma_ts_workspace_bytes(heads)) != cudaSuccess) {
-            cudaGetLastError();
-            c->umma_ws = nullptr;
-            slide_attn_destroy(c);
-            return SLIDE_ATTN_ERR_ALLOC;
-        }
-    }
-    if (mma_wide_supports(dtype, head_dim, ksize) &&
-        cudaMalloc(&c->wide_ws, mma_wide_workspace_bytes(heads, ksize)) != cudaSuccess) {
+    unsigned char* at = static_cast<unsigned char*>(c->arena);
+    c->d_status = reinterpret_cast<int*>(at); at += 256;
+    auto take = [&](size_t bytes) { void* w = bytes ? at : nullptr; at += bytes; return w; };
+    c->workspace = take(b_mma); c->umma_ws = take(b_umma); c->split_ws = take(b_split); c->wide_ws = take(b_wide); c->strip_ws = take(b_strip);
+    if (cudaMemset(c->d_status, 0, sizeof(int)) != cudaSuccess) {
         cudaGetLastError();
-        c->wide_ws = nullptr;
-        slide_attn_destroy(c);
-        return SLIDE_ATTN_ERR_ALLOC;
-    }
-    if (strip_supports(head_dim, ksize) &&
-        cudaMalloc(&c->strip_ws, strip_workspace_bytes(heads, head_dim, ksize)) != cudaSuccess) {
-        cudaGetLastError();
-        c->strip_ws = nullptr;
         slide_attn_destroy(c);
         return SLIDE_ATTN_ERR_ALLOC;
     }
@@ -461,7 +453,8 @@ slide_attn_status slide_attn_set_variant(slide_attn_ctx* c, slide_attn_variant v
     if (!c) return SLIDE_ATTN_ERR_INVALID_ARG;
     if (variant == SLIDE_ATTN_VARIANT_AUTO) { c->variant = pick_variant(c); return SLIDE_ATTN_OK; }
     if (variant != SLIDE_ATTN_VARIANT_DIRECT && variant != SLIDE_ATTN_VARIANT_MMA && variant != SLIDE_ATTN_VARIANT_UMMA_TS &&
-        variant != SLIDE_ATTN_VARIANT_STRIP && variant != SLIDE_ATTN_VARIANT_TILE && variant != SLIDE_ATTN_VARIANT_MMA_WIDE)
+        variant != SLIDE_ATTN_VARIANT_STRIP && variant != SLIDE_ATTN_VARIANT_TILE && variant != SLIDE_ATTN_VARIANT_MMA_WIDE &&
+        variant != SLIDE_ATTN_VARIANT_UMMA_SPLIT)
         return SLIDE_ATTN_ERR_INVALID_ARG;
     if (!variant_supported(c, variant)) return SLIDE_ATTN_ERR_UNSUPPORTED;
     c->variant = variant;
@@ -517,6 +510,7 @@ slide_attn_status slide_attn_launches_per_forward(const slide_attn_ctx* c, int* 
         case SLIDE_ATTN_VARIANT_UMMA_TS: *n = 2; break;  // B-image prep + fused kernel
         case SLIDE_ATTN_VARIANT_TILE: *n = 2; break;     // weight transpose + fused kernel
         case SLIDE_ATTN_VARIANT_MMA_WIDE: *n = 2; break; // weight fragments + fused kernel
+        case SLIDE_ATTN_VARIANT_UMMA_SPLIT: *n = 2; break; // weight images + fused kernel
         default: *n = 1; break;
     }
     return SLIDE_ATTN_OK;
@@ -585,12 +579,8 @@ slide_attn_status slide_attn_destroy(slide_attn_ctx* c)
 {
     if (!c) return SLIDE_ATTN_OK;
     bool ok = true;
-    if (c->d_status) ok &= cudaFree(c->d_status) == cudaSuccess;
-    if (c->workspace) ok &= cudaFree(c->workspace) == cudaSuccess;
-    if (c->strip_ws) ok &= cudaFree(c->strip_ws) == cudaSuccess;
-    if (c->umma_ws) ok &= cudaFree(c->umma_ws) == cudaSuccess;
+    if (c->arena) ok &= cudaFree(c->arena) == cudaSuccess;
     if (c->bwd_ws) ok &= cudaFree(c->bwd_ws) == cudaSuccess;
-    if (c->wide_ws) ok &= cudaFree(c->wide_ws) == cudaSuccess;
     if (c->block_ws) ok &= cudaFree(c->block_ws) == cudaSuccess;
     if (c->stage) ok &= cudaFree(c->stage) == cudaSuccess;
     if (c->host_pipe) {

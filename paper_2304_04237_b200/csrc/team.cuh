@@ -1,0 +1,339 @@
+// Shared by the kernels that run the split contractions on tcgen05 (exact products, fp32 accumulation; see
+// split.cuh): geometry, the shared-memory images of the weights and the hand-offs of a team.
+//
+// A TEAM is eight warps with one block of 128 pixels (the 128 lanes of tensor memory) at a time; two teams share an SM
+// and its weight images and run independently of each other, so that one team's hand-offs (180 - 220 cycles from an
+// MMA's issue to the wake-up of its readers) are covered by the other's arithmetic.  (Four teams of four warps with
+// one tap per hand-off, which leaves each team 128 columns, were 13 % slower with 64 channels a head.)
+// A block is four STRIPS of 4 rows x 8 columns of the map; warps q and q + 4 of a team have quadrant q of tensor memory
+// = strip q, the first its rows 0 and 1, the second rows 2 and 3: lane (g, tig) works on column g and piece tig of the
+// channels of two rows, TMEM lane 32 q + 16 half + 8 row + g.  A strip is loaded by TMA with its halo (6 x 10 pixels,
+// 64-byte channel planes, zero fill = the padding).  Four more warps: an MMA thread and a TMA thread per team.
+//
+//   products    x . y per (plane, tap column dx), split into parts, to tensor memory (a chunk; two buffers)
+//   contraction L[p][n] += parts . Bk.  The columns of Bk are three groups of 16, nine used: the upper, middle and
+//               lower 8 bits of the weight of each slot.  Upper x upper accumulates in tiles H of its own - the tensor
+//               core truncates at every step, and two or three tiles mean half or a third of the steps for each (one
+//               tile for everything: relative error 8.4e-7 of the forward, so: 2.1e-7) -, everything that is 2^-8
+//               smaller in the first half of a tile R, 2^-16 smaller in the second; they meet in registers.
+//   softmax     one thread has a pixel's nine slots
+//   expansion   D[p][(tap, channel)] = A'[p][32] . Bv[32][(tap, channel)], fp16 operands: upper and middle part of the
+//               slot value against upper and middle part of the weight (middle . middle is below 2^-22 and left out)
+//   sum         sum_t D[p][t][c] y_t[p][c] with packed fp32 FMAs
+//
+// Tensor-memory columns of a team: product chunks, H tiles, R tile (32 columns at the end); later D in 0 - 191 and A' in
+// the last 16.
+#pragma once
+#include <cuda_fp16.h>
+
+#include "common.cuh"
+#include "ptx.cuh"
+#include "split.cuh"
+
+namespace slide_attn {
+namespace team {
+
+constexpr int kTeams = 2, kTeamWarps = 8;
+constexpr int kComputeWarps = kTeams * kTeamWarps;
+constexpr int kMmaWarp = kComputeWarps, kTmaWarp = kMmaWarp + kTeams;          // one of each per team
+constexpr int kThreads = (kTmaWarp + kTeams) * 32;
+constexpr int kK2 = 9;
+constexpr int kHaloPlane = 60 * 64;                     // bytes of one plane of a strip with its halo
+constexpr int kSlot = 4 * kHaloPlane;                   // of a block: a slot of the team's ring
+constexpr float kLog2e = 1.4426950408889634f;
+constexpr uint32_t kCols = 256, kColP = 0, kColR = 224, kColA = 240, kColD = 0;
+constexpr float kScaleA = 8192.f;                       // softmax weights (at most 1) enter fp16 times 2^13
+
+// How the channels of a storage type are cut: planes of 64 bytes, chunks of one plane and one tap column.
+template <typename T> struct Cut;
+template <> struct Cut<__nv_bfloat16> {
+    static constexpr int channels = 32;                 // of a plane
+    static constexpr int per_lane = 8;
+    static constexpr int d_buffers = 2;                 // N = 96 columns per tap column of a plane
+    static constexpr int tap_cols = 32, h_tiles = 2;    // products are hi + lo: 2 x 3 x 32 + 2 x 16 + 32 = 256 columns
+};
+template <> struct Cut<float> {
+    static constexpr int channels = 16;
+    static constexpr int per_lane = 4;
+    static constexpr int d_buffers = 3;                 // N = 48
+    static constexpr int tap_cols = 24, h_tiles = 3;    // hi + mid + lo: 2 x 3 x 24 + 3 x 16 + 32 = 224
+};
+template <typename T> constexpr uint32_t kColH = 6 * Cut<T>::tap_cols;
+
+// Channel of K index kappa within a plane (the order in which tcgen05.st lays the pieces out); the channel of column n of
+// a tap of D (the order in which tcgen05.ld hands them to the lanes) is (CH / 4) ((n & 7) >> 1) + 2 (n >> 3) + (n & 1).
+template <typename T> __host__ __device__ constexpr int channel_of_k(int kappa) {
+    return Cut<T>::channels == 32 ? 8 * ((kappa & 15) >> 2) + (kappa & 3) + (kappa >= 16 ? 4 : 0) : kappa;
+}
+
+// Weight images of one head (bytes).  Contraction: [plane][tap][K / 8][48 n][8 k] bf16.  Expansion: [plane][tap
+// column dx][dy][n][32 k] fp16 in core matrices, then one float per channel that undoes the channel's scale.
+__host__ __device__ constexpr uint32_t contract_bytes(int head_dim) { return (uint32_t)head_dim * 9u * 96u; }
+__host__ __device__ constexpr uint32_t expand_image_bytes(int head_dim) { return (uint32_t)head_dim * 9u * 64u; }
+__host__ __device__ constexpr uint32_t expand_bytes(int head_dim) { return expand_image_bytes(head_dim) + (uint32_t)head_dim * 4u; }
+
+// Contraction image item: 16 bytes = 8 k of column n.  w: fp32 [head_dim][slot][tap] of the head.
+template <typename T>
+__device__ __forceinline__ void build_contract_item(const float* __restrict__ w, unsigned char* img, int item) {
+    constexpr int KG = Cut<T>::channels / 8;             // k groups of a (plane, tap)
+    const int n = item % 48, kg = item / 48;
+    const int j = kg % KG, pt = kg / KG, tap = pt % kK2, plane = pt / kK2;
+    const int s = n & 15, part = n >> 4;
+    float v[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+        float x = 0.f;
+        if (s < kK2) {
+            x = w[((plane * Cut<T>::channels + channel_of_k<T>(8 * j + e)) * kK2 + s) * kK2 + tap];
+            if (part >= 1) x = split::rest(x);
+            if (part >= 2) x = split::rest(x);
+        }
+        v[e] = x;
+    }
+    *reinterpret_cast<uint4*>(img + (size_t)kg * 768 + (n >> 3) * 128 + (n & 7) * 16) =
+        make_uint4(split::pack_upper(v[0], v[1]), split::pack_upper(v[2], v[3]), split::pack_upper(v[4], v[5]), split::pack_upper(v[6], v[7]));
+}
+
+// A power of two that brings `most` (the largest magnitude of what it will multiply) to [2^13, 2^14), and its inverse.
+__device__ __forceinline__ void fp16_scale(float most, float& scale, float& inverse) {
+    int e = (int)(__float_as_uint(most) >> 23) & 0xff;
+    e = e < 14 ? 14 : e;
+    scale = __uint_as_float((uint32_t)(267 - e) << 23);
+    inverse = __uint_as_float((uint32_t)(e - 13) << 23);
+}
+// x = hi + mid to 2^-22 of x (as far as 2^-24 allows)
+__device__ __forceinline__ void split_fp16(float x, __half& hi, __half& mid) {
+    hi = __float2half_rn(x);
+    mid = __float2half_rn(x - __half2float(hi));
+}
+__device__ __forceinline__ uint32_t pack_half(__half a, __half b) {
+    return (uint32_t)__half_as_ushort(a) | ((uint32_t)__half_as_ushort(b) << 16);
+}
+
+// Expansion image of one channel by one warp (w: the channel's fp32 [slot][tap]).  Column ((plane 3 + dx) 3 + dy)
+// channels + n; its K rows: 0 - 7 upper parts of slots 0 - 7, 8 - 15 their middle parts, 16 - 23 the upper parts again,
+// 24 - 26 slot 8: upper, middle, upper.
+template <typename T>
+__device__ __forceinline__ void build_expand_channel(const float* __restrict__ w, unsigned char* img, int head_dim, int c, int lane) {
+    constexpr int CH = Cut<T>::channels;
+    float most = 0.f, v[kK2];
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+        if (lane + 32 * i < kK2 * kK2) most = fmaxf(most, fabsf(w[lane + 32 * i]));
+#pragma unroll
+    for (int s = 0; s < kK2; ++s) v[s] = lane < kK2 ? w[s * kK2 + lane] : 0.f;      // lane = tap
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) most = fmaxf(most, __shfl_xor_sync(0xffffffffu, most, o));
+    float scale, inverse;
+    fp16_scale(most, scale, inverse);
+    if (lane == 0) reinterpret_cast<float*>(img + expand_image_bytes(head_dim))[c] = inverse;
+    if (lane >= kK2) return;
+    const int plane = c / CH, ch = c % CH, dy = lane / 3, dx = lane % 3;
+    const int q4 = CH / 4, n = 8 * ((ch % q4) >> 1) + 2 * (ch / q4) + (ch & 1);      // the column of this channel
+    const int item = ((plane * 3 + dx) * 3 + dy) * CH + n;
+    __half hi[kK2], mid[kK2];
+#pragma unroll
+    for (int s = 0; s < kK2; ++s) split_fp16(v[s] * scale, hi[s], mid[s]);
+    unsigned char* col = img + (size_t)(item >> 3) * 512 + (item & 7) * 16;
+    const uint4 h = make_uint4(pack_half(hi[0], hi[1]), pack_half(hi[2], hi[3]), pack_half(hi[4], hi[5]), pack_half(hi[6], hi[7]));
+    *reinterpret_cast<uint4*>(col) = h;
+    *reinterpret_cast<uint4*>(col + 128) = make_uint4(pack_half(mid[0], mid[1]), pack_half(mid[2], mid[3]), pack_half(mid[4], mid[5]), pack_half(mid[6], mid[7]));
+    *reinterpret_cast<uint4*>(col + 256) = h;
+    const __half zero = __float2half_rn(0.f);
+    *reinterpret_cast<uint4*>(col + 384) = make_uint4(pack_half(hi[8], mid[8]), pack_half(hi[8], zero), 0u, 0u);
+}
+// The A' row that meets it, from nine slot values already scaled: 16 registers of two halves.
+__device__ __forceinline__ void expand_row(const float (&a)[kK2], uint32_t (&row)[16]) {
+    __half hi[kK2], mid[kK2];
+#pragma unroll
+    for (int s = 0; s < kK2; ++s) split_fp16(a[s], hi[s], mid[s]);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        row[i] = pack_half(hi[2 * i], hi[2 * i + 1]);
+        row[4 + i] = row[i];
+        row[8 + i] = pack_half(mid[2 * i], mid[2 * i + 1]);
+    }
+    row[12] = pack_half(hi[8], hi[8]);
+    row[13] = pack_half(mid[8], __float2half_rn(0.f));
+    row[14] = 0u; row[15] = 0u;
+}
+
+// The images of one head by prep_parts(head_dim) blocks of 256 threads, of which this one is `part`: a warp per channel of
+// the expansion image, then a thread per item of the contraction image.  (Four blocks a head, each looking for the
+// channels' largest weights by itself, took 12 us, most of what a small map needs.)
+__host__ __device__ constexpr int prep_parts(int head_dim) { return head_dim / 8 + (head_dim / 8 * 9 * 48 + 255) / 256; }
+template <typename T>
+__device__ __forceinline__ void build_images(const float* wc, unsigned char* cimg, const float* we, unsigned char* eimg, int head_dim, int part) {
+    if (part < head_dim / 8) {
+        const int c = part * 8 + (threadIdx.x >> 5);
+        build_expand_channel<T>(we + c * kK2 * kK2, eimg, head_dim, c, threadIdx.x & 31);
+    } else {
+        const int i = (part - head_dim / 8) * 256 + threadIdx.x;
+        if (i < head_dim / 8 * 9 * 48) build_contract_item<T>(wc, cimg, i);
+    }
+}
+
+__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity) {
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity) ? 1 : 0) != 0;
+}
+
+// Barriers of a team; kFull, kEmpty: its ring of planes.
+constexpr int kMaxRing = 5;
+enum : int { kPFull = 0, kPFree = 2, kLFull = 4, kAFull = 5, kDFull = 6, kDFree = 9, kFull = 12, kEmpty = kFull + kMaxRing,
+             kTeamBars = kEmpty + kMaxRing };
+
+__device__ __forceinline__ void init_team_bars(uint32_t base) {
+    auto init = [&](int i, uint32_t count) { mbar_init_only(base + 8u * (uint32_t)i, count); };
+    for (int i = 0; i < 2; ++i) { init(kPFull + i, kTeamWarps); init(kPFree + i, 1); }
+    init(kLFull, 1);
+    init(kAFull, 4);
+    for (int i = 0; i < 3; ++i) { init(kDFull + i, 1); init(kDFree + i, kTeamWarps); }
+    for (int i = 0; i < kMaxRing; ++i) { init(kFull + i, 1); init(kEmpty + i, kTeamWarps); }
+}
+
+// Which strip of 4 rows x 8 columns.
+struct Strip { int b, y0, x0; bool inside; };          // the first pixel
+struct Strips {
+    int sx, bands;
+    long long total;                                     // B * bands * sx
+    __device__ __forceinline__ Strip at(long long i) const {
+        Strip s;
+        s.inside = i < total;
+        int j = (int)(s.inside ? i : total - 1);         // past the end: the last one again, its results dropped
+        s.x0 = (j % sx) * 8; j /= sx;
+        s.y0 = (j % bands) * 4; s.b = j / bands;
+        return s;
+    }
+};
+
+// The 16 bytes of piece tig at pixel (row, column) of a halo plane.
+__device__ __forceinline__ uint4 halo_piece(const unsigned char* plane, int row, int col, int tig) {
+    return *reinterpret_cast<const uint4*>(plane + (uint32_t)(row * 10 + col) * 64u + (uint32_t)tig * 16u);
+}
+__device__ __forceinline__ float f4(const uint4& v, int i) {
+    return __uint_as_float(i == 0 ? v.x : i == 1 ? v.y : i == 2 ? v.z : v.w);
+}
+
+// Products of one tap of a plane for the lane's two pixels, split, into tensor memory at column `t`.
+__device__ __forceinline__ void store_products(__nv_bfloat16, uint32_t t, const uint4 (&x)[2], const uint4& y0, const uint4& y1) {
+    uint32_t r[16];
+    split::product2(x[0].x, y0.x, r[0], r[8]); split::product2(x[0].y, y0.y, r[1], r[9]);
+    split::product2(x[1].x, y1.x, r[2], r[10]); split::product2(x[1].y, y1.y, r[3], r[11]);
+    split::product2(x[0].z, y0.z, r[4], r[12]); split::product2(x[0].w, y0.w, r[5], r[13]);
+    split::product2(x[1].z, y1.z, r[6], r[14]); split::product2(x[1].w, y1.w, r[7], r[15]);
+    tmem_st_16x256b_x4(t, r);
+}
+__device__ __forceinline__ void store_products(float, uint32_t t, const uint4 (&x)[2], const uint4& y0, const uint4& y1) {
+    float2 p[4];                                         // first row: channels 0 1, 2 3; second row
+    p[0] = split::mul2(make_float2(f4(x[0], 0), f4(x[0], 1)), make_float2(f4(y0, 0), f4(y0, 1)));
+    p[1] = split::mul2(make_float2(f4(x[0], 2), f4(x[0], 3)), make_float2(f4(y0, 2), f4(y0, 3)));
+    p[2] = split::mul2(make_float2(f4(x[1], 0), f4(x[1], 1)), make_float2(f4(y1, 0), f4(y1, 1)));
+    p[3] = split::mul2(make_float2(f4(x[1], 2), f4(x[1], 3)), make_float2(f4(y1, 2), f4(y1, 3)));
+    uint32_t r[8], s[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) { r[i] = split::pack_upper(p[i].x, p[i].y); p[i] = split::rest2(p[i]); }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) { r[4 + i] = split::pack_upper(p[i].x, p[i].y); p[i] = split::rest2(p[i]); }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) s[i] = split::pack_upper(p[i].x, p[i].y);
+    tmem_st_16x256b_x2(t, r);
+    tmem_st_16x256b_x1(t + 16, s);
+}
+
+// Descriptor of a contraction image; a (plane, tap) further is contract_step.
+__device__ __forceinline__ uint64_t contract_desc(uint32_t img) { return umma_smem_desc(img, 768, 128); }
+template <typename T> __host__ __device__ constexpr uint32_t contract_step(int plane, int tap) {
+    return (uint32_t)((plane * kK2 + tap) * (Cut<T>::channels / 8) * 48);          // in 16-byte units
+}
+// The MMAs of one tap, issued by one thread.  `fresh`: the first tap of a block for its H tile (f32: tile dx; bf16: both
+// tiles, one per k-step); `first`: the first tap of the block.
+template <typename T>
+__device__ __forceinline__ void issue_contract(uint32_t tmem, uint32_t p_col, uint64_t b, int dx, bool fresh, bool first) {
+    constexpr uint32_t id32 = umma_idesc_bf16(128, 32), id16 = umma_idesc_bf16(128, 16);
+    constexpr uint32_t mid = 16;                                             // 256 bytes on: the columns of the middle parts
+    const uint32_t r = tmem + kColR, h = tmem + kColH<T>;
+    if constexpr (sizeof(T) == 2) {
+        constexpr uint32_t k1 = 96;                                          // 1536 bytes on: the next 16 k
+        umma_bf16_ts(h, p_col, b, id16, fresh ? 0u : 1u);
+        umma_bf16_ts(r, p_col, b + mid, id32, first ? 0u : 1u);              // upper . middle | upper . lower
+        umma_bf16_ts(h + 16, p_col + 8, b + k1, id16, fresh ? 0u : 1u);
+        umma_bf16_ts(r, p_col + 8, b + k1 + mid, id32, 1);
+        umma_bf16_ts(r, p_col + 16, b, id32, 1);                             // lower . upper | lower . middle
+        umma_bf16_ts(r, p_col + 24, b + k1, id32, 1);
+    } else {
+        umma_bf16_ts(h + 16 * dx, p_col, b, id16, fresh ? 0u : 1u);
+        umma_bf16_ts(r, p_col, b + mid, id32, first ? 0u : 1u);
+        umma_bf16_ts(r, p_col + 8, b, id32, 1);                              // middle . upper | middle . middle
+        umma_bf16_ts(r + 16, p_col + 16, b, id16, 1);                        // lower . upper
+    }
+}
+// The contraction of the lane's pixel (thread = TMEM lane).
+template <typename T>
+__device__ __forceinline__ void load_contraction(uint32_t quad, float (&l)[kK2]) {
+    float h[32], r[32];
+    tmem_ld_32x32b_x32(quad + kColR, r);
+    tmem_ld_32x32b_x32(quad + kColH<T>, h);                                  // two H tiles
+#pragma unroll
+    for (int s = 0; s < kK2; ++s) l[s] = h[s] + h[16 + s];
+    if constexpr (Cut<T>::h_tiles == 3) {
+        tmem_ld_32x32b_x32(quad + kColH<T> + 16, h);                         // the second and the third
+#pragma unroll
+        for (int s = 0; s < kK2; ++s) l[s] += h[16 + s];
+    }
+#pragma unroll
+    for (int s = 0; s < kK2; ++s) l[s] += r[s] + r[16 + s];
+}
+// The MMAs of one D chunk (plane, dx): [128 x 32] . [32 x 3 channels].
+template <typename T>
+__device__ __forceinline__ void issue_expand(uint32_t d_col, uint32_t a_col, uint32_t b_smem) {
+    constexpr uint32_t idesc = umma_idesc_f16(128, 3 * Cut<T>::channels);
+    umma_bf16_ts(d_col, a_col, umma_smem_desc(b_smem, 128, 512), idesc, 0);
+    umma_bf16_ts(d_col, a_col + 8, umma_smem_desc(b_smem + 256, 128, 512), idesc, 1);
+}
+
+// acc[row][channel of the lane] += D chunk (three taps of column dx) at `t` times the halo rows of that column, which are
+// loaded while the chunk is on its way.
+__device__ __forceinline__ void sum_chunk(__nv_bfloat16, uint32_t t, const unsigned char* plane, int row, int col, int tig, float (&acc)[2][8]) {
+    uint32_t d[48];
+    tmem_ld3_16x256b_x4_nowait(t, t + 32, t + 64, d);
+    uint4 y[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) y[r] = halo_piece(plane, row + r, col, tig);
+    float f[4][8];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        f[r][0] = bf16_lo(y[r].x); f[r][1] = bf16_hi(y[r].x); f[r][2] = bf16_lo(y[r].y); f[r][3] = bf16_hi(y[r].y);
+        f[r][4] = bf16_lo(y[r].z); f[r][5] = bf16_hi(y[r].z); f[r][6] = bf16_lo(y[r].w); f[r][7] = bf16_hi(y[r].w);
+    }
+    tmem_wait_ld48(d);
+#pragma unroll
+    for (int dy = 0; dy < 3; ++dy)
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                ffma2(acc[r][2 * j], acc[r][2 * j + 1], __uint_as_float(d[16 * dy + 4 * j + 2 * r]), __uint_as_float(d[16 * dy + 4 * j + 2 * r + 1]),
+                      f[r + dy][2 * j], f[r + dy][2 * j + 1]);
+}
+__device__ __forceinline__ void sum_chunk(float, uint32_t t, const unsigned char* plane, int row, int col, int tig, float (&acc)[2][4]) {
+    uint32_t d[3][8];
+#pragma unroll
+    for (int dy = 0; dy < 3; ++dy) tmem_ld_16x256b_x2_nowait(t + 16 * dy, d[dy]);
+    uint4 y[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) y[r] = halo_piece(plane, row + r, col, tig);
+    tmem_wait_ld();
+#pragma unroll
+    for (int dy = 0; dy < 3; ++dy) {
+        tmem_pass(d[dy]);
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+#pragma unroll
+            for (int j = 0; j < 2; ++j)
+                ffma2(acc[r][2 * j], acc[r][2 * j + 1], __uint_as_float(d[dy][4 * j + 2 * r]), __uint_as_float(d[dy][4 * j + 2 * r + 1]),
+                      f4(y[r + dy], 2 * j), f4(y[r + dy], 2 * j + 1));
+    }
+}
+
+}  // namespace team
+}  // namespace slide_attn

@@ -1,0 +1,359 @@
+// UMMA_SPLIT variant (k = 3; fp32 storage or bf16; head_dim 32 or 64): the fused forward (Eq. 2 with Eq. 12 inside)
+// with fp32 arithmetic, both k^4 contractions on tcgen05.  Where UMMA_TS rounds the q.k products and the softmax
+// weights to bf16, this kernel splits them, and the weights, into parts whose tensor-core products are exact
+// (split.cuh), so fp32 storage keeps its 1e-4 - in fact 1e-6 - and wide heads the accuracy of an fp32 kernel.
+//
+//   logits   l[s] = scale * sum_{t,c} (q[c] k_t[c]) wk[c,s,t] + bias[s]     a = softmax(l)
+//   values   out[c] = sum_t v_t[c] (sum_s a[s] wv[c,s,t])
+//
+// Persistent, one CTA per SM, CTA c -> head c mod heads; two teams (team.cuh), each with a block of four strips at a time,
+// blocks dealt over teams round-robin, neighbouring CTAs on neighbouring blocks.  A block's K planes, then its V planes
+// come through the team's ring.
+//
+// Bound by instruction issue and the hand-offs between the warps and the tensor core (issue slots 51 % busy, tensor pipe
+// 15 - 24 %, DRAM 13 - 16 %).  A call: 2 x 128 x 128, 3 heads, fp32: 45.3 us in tile_kernel, 30.7 here; 32 x 28 x 28,
+// 3 heads of 64, bf16: 232 us in strip_kernel, 28.3 here; 1 x 14 x 14, 1 head, fp32: 14.7 and 11.2 us.
+#include "team.cuh"
+
+namespace slide_attn {
+
+namespace {
+
+using namespace team;
+
+template <typename T, int D>
+struct Fwd {
+    static constexpr int planes = D / Cut<T>::channels;
+    static constexpr int chunks = 3 * planes;                                    // product chunks, and D chunks, of a block
+    static constexpr uint32_t image = contract_bytes(D) + expand_bytes(D);      // of a head, in shared memory and in the workspace
+    static constexpr uint32_t misc = 8u * (kTeams * kTeamBars + 1) + 16;
+    static constexpr int fit = (int)((227u * 1024u - image - misc - 128) / (kTeams * kSlot));
+    static constexpr int ring = fit < kMaxRing ? fit : kMaxRing;                 // slots of a team
+    static_assert(ring >= 2, "the ring does not fit");
+    static constexpr uint32_t w_off = (uint32_t)(kTeams * ring * kSlot);
+    static constexpr uint32_t bar_off = w_off + ((image + 15u) & ~15u);
+    static constexpr uint32_t total = bar_off + misc + 128;
+};
+
+struct SplitParams {
+    const unsigned char* img;        // [head] contraction image of wk, expansion image of wv
+    const void* q;
+    const float* bias;
+    void* out;
+    int* status;
+    int H, W, heads;
+    Strips strips;
+    float scale_log2e;
+};
+
+template <typename T, int D>
+__global__ void __launch_bounds__(256)
+umma_split_prep_kernel(const float* __restrict__ wk, const float* __restrict__ wv, unsigned char* __restrict__ img)
+{
+    grid_launch_dependents();        // the main kernel may start its own prologue now
+    const size_t w = (size_t)blockIdx.x * D * kK2 * kK2;
+    unsigned char* dst = img + (size_t)blockIdx.x * Fwd<T, D>::image;
+    build_images<T>(wk + w, dst, wv + w, dst + contract_bytes(D), D, blockIdx.y);
+}
+
+template <typename T, int D>
+__global__ void __launch_bounds__(kThreads, 1)
+umma_split_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v, const SplitParams P)
+{
+    using F = Fwd<T, D>;
+    constexpr int NPL = F::planes, CH = Cut<T>::channels, PL = Cut<T>::per_lane, DB = Cut<T>::d_buffers, R = F::ring;
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char* smem = smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u);
+    const uint32_t bars = smem_u32(smem + F::bar_off);
+    const uint32_t bar_weights = bars + 8u * (kTeams * kTeamBars);
+    unsigned char* tmem_slot = smem + F::bar_off + 8u * (kTeams * kTeamBars + 1);
+
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
+    const int h = blockIdx.x % P.heads, rank = blockIdx.x / P.heads, nrank = (int)gridDim.x / P.heads;
+    const int team_id = warp < kComputeWarps ? warp / kTeamWarps : (warp - kComputeWarps) % kTeams;
+    const int blocks = (int)((P.strips.total + 3) >> 2);
+    const int first = team_id * nrank + rank, step = kTeams * nrank;
+    const int my_blocks = first < blocks ? (blocks - first + step - 1) / step : 0;
+    const uint32_t tb = bars + 8u * (uint32_t)(team_id * kTeamBars);
+    auto bar = [&](int i) { return tb + 8u * (uint32_t)i; };
+
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < kTeams; ++i) init_team_bars(bars + 8u * (uint32_t)(i * kTeamBars));
+        mbar_init_only(bar_weights, 1);
+        mbar_init_fence();
+    }
+    if (warp == kMmaWarp) tmem_alloc(smem_u32(tmem_slot), 512);
+    tc_fence_before_sync();
+    __syncthreads();
+    tc_fence_after_sync();
+    const uint32_t tmem = *reinterpret_cast<const volatile uint32_t*>(tmem_slot) + kCols * (uint32_t)team_id;
+    unsigned char* ring = smem + (uint32_t)(team_id * R * kSlot);
+    bool ok = true;
+
+    if (warp >= kTmaWarp) {
+        // ---- TMA thread of a team: the K planes, then the V planes of every block -------------------------
+        uint32_t leader;
+        if (elect_one(leader)) {
+            int slot = 0;
+            uint32_t phase = 1;                                      // a fresh barrier is free
+            for (int bi = 0; ok && bi < my_blocks; ++bi) {
+                const long long s0 = 4LL * (first + (long long)bi * step);
+                Strip st[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) st[i] = P.strips.at(s0 + i);
+                for (int v = 0; v < 2 * NPL; ++v) {
+                    if (!mbar_wait(bar(kEmpty + slot), phase)) { ok = false; break; }
+                    mbar_expect_tx(bar(kFull + slot), kSlot);
+                    const CUtensorMap* map = v < NPL ? &map_k : &map_v;
+                    const int c0 = h * D + (v < NPL ? v : v - NPL) * CH;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        tma_load_4d(smem_u32(ring) + (uint32_t)(slot * kSlot + i * kHaloPlane), map, bar(kFull + slot), c0, st[i].x0 - 1, st[i].y0 - 1, st[i].b);
+                    if (++slot == R) { slot = 0; phase ^= 1u; }
+                }
+            }
+            if (!ok) atomicExch(P.status, 1);
+        }
+        __syncwarp();
+    } else if (warp >= kMmaWarp) {
+        // ---- MMA thread of a team -------------------------------------------------------------------
+        uint32_t leader;
+        if (elect_one(leader)) {
+            if (warp == kMmaWarp) {                                  // the prep kernel's images, once per CTA
+                grid_dependency_wait();
+                mbar_expect_tx(bar_weights, F::image);
+                bulk_load_1d(smem_u32(smem + F::w_off), P.img + (size_t)h * F::image, F::image, bar_weights);
+            }
+            if (my_blocks > 0) ok = mbar_wait(bar_weights, 0);
+            const uint64_t kdesc = contract_desc(smem_u32(smem + F::w_off));
+            const uint32_t dsrc = smem_u32(smem + F::w_off) + contract_bytes(D);
+            int pn = 0, dn = 0;                                      // chunks issued so far
+            for (int bi = 0; ok && bi < my_blocks; ++bi) {
+                for (int i = 0; i < F::chunks; ++i, ++pn) {          // plane, tap column
+                    const int pb = pn & 1, plane = i / 3, dx = i % 3;
+                    if (!mbar_wait(bar(kPFull + pb), (uint32_t)(pn >> 1) & 1u)) { ok = false; break; }
+                    tc_fence_after_sync();
+                    const uint32_t p_col = tmem + kColP + (uint32_t)(pb * 3 * Cut<T>::tap_cols);
+#pragma unroll
+                    for (int dy = 0; dy < 3; ++dy)
+                        issue_contract<T>(tmem, p_col + dy * Cut<T>::tap_cols, kdesc + contract_step<T>(plane, dy * 3 + dx), dx,
+                                          dy == 0 && (sizeof(T) == 2 ? i == 0 : plane == 0), dy == 0 && i == 0);
+                    umma_commit(bar(kPFree + pb));
+                }
+                if (!ok) break;
+                umma_commit(bar(kLFull));
+                if (!mbar_wait(bar(kAFull), (uint32_t)bi & 1u)) { ok = false; break; }
+                for (int i = 0; i < F::chunks; ++i, ++dn) {
+                    const int db = dn % DB;
+                    if (!mbar_wait(bar(kDFree + db), ((uint32_t)(dn / DB) & 1u) ^ 1u)) { ok = false; break; }
+                    tc_fence_after_sync();
+                    issue_expand<T>(tmem + kColD + (uint32_t)(db * 3 * CH), tmem + kColA, dsrc + (uint32_t)(i * 3 * CH * 64));
+                    umma_commit(bar(kDFull + db));
+                }
+            }
+            if (!ok) atomicExch(P.status, 1);
+        }
+        __syncwarp();
+    } else {
+        const int w = warp % kTeamWarps, wq = w & 3, half = w >> 2, g = lane >> 2, tig = lane & 3;
+        const uint32_t quad = tmem + ((uint32_t)(32 * wq) << 16), mine = quad + ((uint32_t)(16 * half) << 16);
+        const int C = P.heads * D;
+        float bias[kK2];
+#pragma unroll
+        for (int s = 0; s < kK2; ++s) bias[s] = P.bias ? P.bias[h * kK2 + s] * kLog2e : 0.f;
+        auto strip_of = [&](int bi) { return P.strips.at(4LL * (first + (long long)bi * step) + wq); };
+
+        int slot = 0, pn = 0, dn = 0;
+        uint32_t phase = 0;
+        auto release = [&]() {                                       // the plane at `slot` has been read
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar(kEmpty + slot));
+            if (++slot == R) { slot = 0; phase ^= 1u; }
+        };
+        auto load_q = [&](const Strip& s, int plane, uint4 (&x)[2]) {
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                const int y = s.y0 + 2 * half + r;
+                x[r] = make_uint4(0u, 0u, 0u, 0u);
+                if (y < P.H && s.x0 + g < P.W)
+                    x[r] = __ldg(reinterpret_cast<const uint4*>(static_cast<const T*>(P.q) + (((size_t)s.b * P.H + y) * P.W + s.x0 + g) * C +
+                                                                h * D + plane * CH + tig * PL));
+            }
+        };
+        Strip st = strip_of(0);
+        uint4 qn[2];
+        if (my_blocks > 0) load_q(st, 0, qn);
+        for (int bi = 0; bi < my_blocks; ++bi) {
+            // ---- products -------------------------------------------------------------------------
+            for (int pl = 0; pl < NPL; ++pl) {
+                const uint4 x[2] = {qn[0], qn[1]};
+                if (pl + 1 < NPL) load_q(st, pl + 1, qn);
+                if (!warp_wait(bar(kFull + slot), phase)) { ok = false; break; }
+                const unsigned char* plane = ring + (uint32_t)(slot * kSlot + wq * kHaloPlane);
+#pragma unroll
+                for (int dx = 0; dx < 3; ++dx, ++pn) {
+                    const int pb = pn & 1;
+                    uint4 y[4];
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) y[r] = halo_piece(plane, 2 * half + r, g + dx, tig);
+                    if (!warp_wait(bar(kPFree + pb), ((uint32_t)(pn >> 1) & 1u) ^ 1u)) { ok = false; break; }
+                    tc_fence_after_sync();
+                    const uint32_t t = mine + kColP + (uint32_t)(pb * 3 * Cut<T>::tap_cols);
+#pragma unroll
+                    for (int dy = 0; dy < 3; ++dy) store_products(T(), t + dy * Cut<T>::tap_cols, x, y[dy], y[dy + 1]);
+                    tmem_wait_st();
+                    tc_fence_before_sync();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar(kPFull + pb));
+                }
+                if (!ok) break;
+                release();
+            }
+            if (!ok) break;
+            const Strip cur = st;
+            if (bi + 1 < my_blocks) { st = strip_of(bi + 1); load_q(st, 0, qn); }
+
+            // ---- softmax: thread = pixel of the quadrant; the two warps of a quadrant take turns -------------
+            if (half == (bi & 1)) {
+                if (!warp_wait(bar(kLFull), (uint32_t)bi & 1u)) { ok = false; break; }
+                tc_fence_after_sync();
+                float a[kK2], m = -INFINITY, z = 0.f;
+                load_contraction<T>(quad, a);
+#pragma unroll
+                for (int s = 0; s < kK2; ++s) { a[s] = fmaf(a[s], P.scale_log2e, bias[s]); m = fmaxf(m, a[s]); }
+#pragma unroll
+                for (int s = 0; s < kK2; ++s) { a[s] = fast_exp2(a[s] - m); z += a[s]; }
+                const float iz = kScaleA / z;
+#pragma unroll
+                for (int s = 0; s < kK2; ++s) a[s] *= iz;
+                uint32_t row[16];
+                expand_row(a, row);
+                tmem_st_32x32b_x16(quad + kColA, row);
+                tmem_wait_st();
+                tc_fence_before_sync();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar(kAFull));
+            }
+
+            // ---- values ----------------------------------------------------------------------------
+            if (bi == 0 && !warp_wait(bar_weights, 0)) { ok = false; break; }     // for the channel scales
+            for (int pl = 0; pl < NPL; ++pl) {
+                float acc[2][PL];
+#pragma unroll
+                for (int r = 0; r < 2; ++r)
+#pragma unroll
+                    for (int c = 0; c < PL; ++c) acc[r][c] = 0.f;
+                if (!warp_wait(bar(kFull + slot), phase)) { ok = false; break; }
+                const unsigned char* plane = ring + (uint32_t)(slot * kSlot + wq * kHaloPlane);
+#pragma unroll
+                for (int dx = 0; dx < 3; ++dx, ++dn) {
+                    const int db = dn % DB;
+                    if (!warp_wait(bar(kDFull + db), (uint32_t)(dn / DB) & 1u)) { ok = false; break; }
+                    tc_fence_after_sync();
+                    sum_chunk(T(), mine + kColD + (uint32_t)(db * 3 * CH), plane, 2 * half, g + dx, tig, acc);
+                    tc_fence_before_sync();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar(kDFree + db));
+                }
+                if (!ok) break;
+                release();
+                const float* inv = reinterpret_cast<const float*>(smem + F::w_off + contract_bytes(D) + expand_image_bytes(D)) + pl * CH + tig * PL;
+                float sc[PL];
+#pragma unroll
+                for (int c = 0; c < PL; ++c) sc[c] = inv[c] * (1.f / kScaleA);
+                if (cur.inside && cur.x0 + g < P.W) {
+#pragma unroll
+                    for (int r = 0; r < 2; ++r) {
+                        const int y = cur.y0 + 2 * half + r;
+                        if (y < P.H) {
+                            T* op = static_cast<T*>(P.out) + (((size_t)cur.b * P.H + y) * P.W + cur.x0 + g) * C + h * D + pl * CH + tig * PL;
+                            uint4 o;
+                            if constexpr (sizeof(T) == 2) {
+                                o.x = pack_bf16(acc[r][0] * sc[0], acc[r][1] * sc[1]); o.y = pack_bf16(acc[r][2] * sc[2], acc[r][3] * sc[3]);
+                                o.z = pack_bf16(acc[r][4] * sc[4], acc[r][5] * sc[5]); o.w = pack_bf16(acc[r][6] * sc[6], acc[r][7] * sc[7]);
+                            } else {
+                                o.x = __float_as_uint(acc[r][0] * sc[0]); o.y = __float_as_uint(acc[r][1] * sc[1]);
+                                o.z = __float_as_uint(acc[r][2] * sc[2]); o.w = __float_as_uint(acc[r][3] * sc[3]);
+                            }
+                            *reinterpret_cast<uint4*>(op) = o;
+                        }
+                    }
+                }
+            }
+            if (!ok) break;
+        }
+        if (!ok && lane == 0) atomicExch(P.status, 1);
+    }
+    tc_fence_before_sync();
+    __syncthreads();
+    if (warp == kMmaWarp) {
+        tc_fence_after_sync();
+        tmem_dealloc(*reinterpret_cast<const volatile uint32_t*>(tmem_slot), 512);
+    }
+}
+
+template <typename T, int D>
+cudaError_t launch_t(const Problem& p, void* workspace, int* d_status, int num_sms, cudaStream_t stream) {
+    using F = Fwd<T, D>;
+    static bool configured[64] = {};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev >= 64 || !configured[dev]) {
+        e = cudaFuncSetAttribute(umma_split_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F::total);
+        if (e != cudaSuccess) return e;
+        if (dev < 64) configured[dev] = true;
+    }
+    SplitParams P;
+    P.img = static_cast<const unsigned char*>(workspace); P.q = p.q; P.bias = p.bias; P.out = p.out; P.status = d_status;
+    P.H = p.H; P.W = p.W; P.heads = p.heads;
+    P.strips.sx = (p.W + 7) / 8; P.strips.bands = (p.H + 3) / 4;
+    P.strips.total = (long long)p.B * P.strips.bands * P.strips.sx;
+    if (P.strips.total > 0x7fffffffLL - 4) return cudaErrorInvalidConfiguration;
+    P.scale_log2e = kLog2e / sqrtf((float)D);
+    CUtensorMap mk, mv;
+    const int C = p.heads * D;
+    if (!make_tile_map(&mk, p.k, (int)sizeof(T), p.B, p.H, p.W, C, Cut<T>::channels, 10, 6) ||
+        !make_tile_map(&mv, p.v, (int)sizeof(T), p.B, p.H, p.W, C, Cut<T>::channels, 10, 6))
+        return cudaErrorInvalidValue;
+    umma_split_prep_kernel<T, D><<<dim3((unsigned)p.heads, prep_parts(D)), 256, 0, stream>>>(p.wk, p.wv, static_cast<unsigned char*>(workspace));
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+
+    const long long blocks = (P.strips.total + 3) / 4;
+    long long per_head = num_sms / p.heads;
+    if (per_head > blocks) per_head = blocks;
+    if (per_head < 1) per_head = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(per_head * p.heads));
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = F::total;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, umma_split_kernel<T, D>, mk, mv, P);
+}
+
+}  // namespace
+
+bool umma_split_supports(int head_dim, int ksize) {
+    return (head_dim == 32 || head_dim == 64) && ksize == 3 && tensor_map_available();
+}
+
+size_t umma_split_workspace_bytes(int heads, int head_dim) {
+    return (size_t)heads * (contract_bytes(head_dim) + expand_bytes(head_dim));
+}
+
+// Prep launch (weights -> images in `workspace`) followed by the fused kernel.
+cudaError_t launch_umma_split(const Problem& p, void* workspace, int* d_status, int num_sms, cudaStream_t stream) {
+    if (p.dtype == SLIDE_ATTN_BF16)
+        return p.head_dim == 32 ? launch_t<__nv_bfloat16, 32>(p, workspace, d_status, num_sms, stream)
+                                : launch_t<__nv_bfloat16, 64>(p, workspace, d_status, num_sms, stream);
+    return p.head_dim == 32 ? launch_t<float, 32>(p, workspace, d_status, num_sms, stream)
+                            : launch_t<float, 64>(p, workspace, d_status, num_sms, stream);
+}
+
+}  // namespace slide_attn

@@ -1,0 +1,58 @@
+"""GPU parity of the UMMA_SPLIT variant (fp32 arithmetic on tcgen05 through exact splits) against the oracle.
+
+Tolerances.  fp32: a logit is 36 - 108 tensor-core accumulations, each truncated to 2^-23 of the running sum, and the
+softmax and the value sums add a few 2^-23 more: 1e-5 of max(1, |ref|) leaves a factor of about three.  bf16: the same
+before one rounding to 8 significant bits (half an ulp: at most 2^-8 of the value)."""
+import zlib
+
+import numpy as np
+import pytest
+
+import oracle
+import paper_2304_04237_b200 as sa
+from paper_2304_04237_b200 import synth
+
+from util import gpu_forward
+
+pytestmark = pytest.mark.gpu
+
+TIGHT = {"f32": 1e-5, "bf16": 2.0 ** -8 + 1e-5}
+# one strip of 4 x 8 pixels, its edges, part of a block, several blocks per team, every head count of a grid
+SHAPES = [(1, 1, 1, 1), (1, 4, 8, 1), (2, 5, 9, 2), (1, 2, 2, 3), (1, 14, 14, 1), (2, 17, 13, 3), (1, 33, 47, 2), (3, 28, 42, 6), (19, 28, 28, 8)]
+
+
+def inputs(shape, d, dtype, sigma_w, bias=True):
+    B, H, W, heads = shape
+    return synth.make_inputs(B, H, W, heads, d, 3, dtype, sigma_w, 0.3, bias, seed=zlib.crc32(repr((shape, d)).encode()) & 0xFFFFFF)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("d", [32, 64])
+@pytest.mark.parametrize("shape", SHAPES, ids=lambda s: "x".join(map(str, s)))
+def test_split_variant_matches_oracle(shape, d, dtype):
+    for sigma_w, bias in ((0.05, True), (0.4, False)):
+        x = inputs(shape, d, dtype, sigma_w, bias)
+        ref = oracle.forward(x["q"], x["k"], x["v"], x["wk"], x["wv"], x["bias"], 3)
+        got = gpu_forward(x, 3, dtype, sa.VARIANT_UMMA_SPLIT)
+        err = np.abs(got - ref) / np.maximum(1.0, np.abs(ref))
+        assert np.isfinite(got).all() and err.max() <= TIGHT[dtype], (sigma_w, float(err.max()))
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_split_variant_weights_of_any_scale(dtype):
+    """Channels whose value weights differ by 2^40 (each is scaled by its own power of two for the fp16 split)."""
+    x = inputs((1, 9, 10, 2), 32, dtype, 0.4)
+    scale = np.exp2(np.arange(64) % 41 - 20).astype(np.float32)
+    x["wv"] = x["wv"] * scale[:, None, None]
+    ref = oracle.forward(x["q"], x["k"], x["v"], x["wk"], x["wv"], x["bias"], 3)
+    got = gpu_forward(x, 3, dtype, sa.VARIANT_UMMA_SPLIT)
+    s = scale.reshape(2, 32)
+    err = np.abs(got - ref) / s / np.maximum(1.0, np.abs(ref) / s)
+    assert err.max() <= TIGHT[dtype], float(err.max())
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_split_variant_is_repeatable(dtype):
+    x = inputs((5, 30, 33, 3), 64, dtype, 0.05)
+    a, b = (gpu_forward(x, 3, dtype, sa.VARIANT_UMMA_SPLIT) for _ in range(2))
+    assert np.array_equal(a, b)
