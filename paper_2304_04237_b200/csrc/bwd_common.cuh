@@ -1,27 +1,22 @@
-// Shared by the backward kernels: what they are launched with.
+// Shared by the backward kernels for k = 3: what they are launched with.
 #pragma once
 #include "common.cuh"
 
 namespace slide_attn {
 
-struct BwdParams {
-    const float* wt;                 // transposed weights wk^T then wv^T, [slot][tap][C]
-    const float* bias;
-    void* dq;
-    void* dk;
-    void* dv;
-    float* dwk;
-    float* dwv;
-    float* dbias;
-    float* ws_a;                     // [pixel][head][k*k]
-    float* ws_dl;
-    int* status;
-    int B, H, W, heads;
-    int tiles_x, tiles_y;
-    float scale;                     // 1 / sqrt(head_dim)
+// Scratch of a backward pass with k = 3: the split rows (64 bytes, team.cuh) of the logit gradients and of the attention
+// weights, [pixel][head], then the weight images of every head.
+struct BwdScratch {
+    unsigned char* rows_dl;
+    unsigned char* rows_a;
+    unsigned char* images;
 };
+BwdScratch bwd_scratch(void* ws, int B, int H, int W, int heads);
+size_t bwd_team_workspace_bytes(int B, int H, int W, int heads);
 
-// dwk, dwv for k = 3 on the tensor cores; P as the point kernel was given it, a and dl already in its workspace.
-cudaError_t launch_bwd_weight_mma(const Problem& p, const BackwardArgs& ga, const BwdParams& P, int num_sms, cudaStream_t stream);
+// Clears the weight and bias gradients and builds the images, then dq, dbias and the split rows, then dk and dv.
+cudaError_t launch_bwd_team(const Problem& p, const BackwardArgs& ga, const BwdScratch& ws, int* d_status, int num_sms, cudaStream_t stream);
+// dwk, dwv from the split rows.
+cudaError_t launch_bwd_weight_mma(const Problem& p, const BackwardArgs& ga, const BwdScratch& ws, int* d_status, int num_sms, cudaStream_t stream);
 
 }  // namespace slide_attn

@@ -29,6 +29,23 @@ namespace {
 
 using namespace tile;
 
+struct BwdParams {
+    const float* wt;                 // transposed weights wk^T then wv^T, [slot][tap][C]
+    const float* bias;
+    void* dq;
+    void* dk;
+    void* dv;
+    float* dwk;
+    float* dwv;
+    float* dbias;
+    float* ws_a;                     // [pixel][head][k*k]
+    float* ws_dl;
+    int* status;
+    int B, H, W, heads;
+    int tiles_x, tiles_y;
+    float scale;                     // 1 / sqrt(head_dim)
+};
+
 // the lane's eight weights of one (slot, tap) vector of 32 floats, and the same addressing for adds
 template <typename T> struct WVec;
 template <> struct WVec<__nv_bfloat16> {
@@ -587,28 +604,14 @@ cudaError_t launch_t(const Problem& p, const BackwardArgs& ga, const float* wt, 
     bwd_gather_kernel<T, K><<<(unsigned)ctas, C_::threads, GatherCfg<T, K>::total, stream>>>(mqh, mgh, P);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    if constexpr (K == 3) {
-        return launch_bwd_weight_mma(p, ga, P, num_sms, stream);
-    } else {
-        static bool done_c[64] = {};
-        e = ensure_smem(bwd_weight_kernel<T, K>, WeightCfg<T, K>::total, done_c);
-        if (e != cudaSuccess) return e;
-        long long per_head = (2LL * num_sms + p.heads - 1) / p.heads;        // persistent CTAs of the weight kernel
-        if (per_head > tiles_per_head) per_head = tiles_per_head;
-        if (per_head < 1) per_head = 1;
-        bwd_weight_kernel<T, K><<<(unsigned)(per_head * p.heads), C_::threads, WeightCfg<T, K>::total, stream>>>(mq, mk, mv, mg, P);
-        return cudaGetLastError();
-    }
-}
-
-template <typename T>
-cudaError_t launch_k(const Problem& p, const BackwardArgs& ga, const float* wt, float* ws_a, float* ws_dl,
-                     int* d_status, int num_sms, cudaStream_t stream) {
-    switch (p.ksize) {
-        case 1: return launch_t<T, 1>(p, ga, wt, ws_a, ws_dl, d_status, num_sms, stream);
-        case 3: return launch_t<T, 3>(p, ga, wt, ws_a, ws_dl, d_status, num_sms, stream);
-        default: return cudaErrorInvalidConfiguration;
-    }
+    static bool done_c[64] = {};
+    e = ensure_smem(bwd_weight_kernel<T, K>, WeightCfg<T, K>::total, done_c);
+    if (e != cudaSuccess) return e;
+    long long per_head = (2LL * num_sms + p.heads - 1) / p.heads;            // persistent CTAs of the weight kernel
+    if (per_head > tiles_per_head) per_head = tiles_per_head;
+    if (per_head < 1) per_head = 1;
+    bwd_weight_kernel<T, K><<<(unsigned)(per_head * p.heads), C_::threads, WeightCfg<T, K>::total, stream>>>(mq, mk, mv, mg, P);
+    return cudaGetLastError();
 }
 
 }  // namespace
@@ -618,19 +621,28 @@ bool backward_supports(int head_dim, int ksize) {
 }
 
 size_t backward_workspace_bytes(int B, int H, int W, int heads, int ksize) {
-    return 2 * (size_t)B * H * W * heads * ksize * ksize * sizeof(float);
+    return ksize == 3 ? bwd_team_workspace_bytes(B, H, W, heads) : 2 * (size_t)B * H * W * heads * ksize * ksize * sizeof(float);
 }
 
-// `wt`: transposed weights as launch_strip_prep writes them; `ws`: backward_workspace_bytes of scratch.
-// The weight and bias gradients must be zero when the first kernel starts (the caller of this function
-// clears them on the same stream).
-cudaError_t launch_backward(const Problem& p, const BackwardArgs& ga, const void* wt, void* ws, int* d_status,
-                            int num_sms, cudaStream_t stream) {
+// `ws`: backward_workspace_bytes of scratch; `wt`: strip_workspace_bytes, used for k = 1.
+cudaError_t launch_backward(const Problem& p, const BackwardArgs& ga, void* wt, void* ws, int* d_status, int num_sms, cudaStream_t stream) {
+    cudaError_t e;
+    if (p.ksize == 3) {
+        const BwdScratch s = bwd_scratch(ws, p.B, p.H, p.W, p.heads);
+        e = launch_bwd_team(p, ga, s, d_status, num_sms, stream);
+        return e == cudaSuccess ? launch_bwd_weight_mma(p, ga, s, d_status, num_sms, stream) : e;
+    }
+    const size_t k2 = (size_t)p.ksize * p.ksize, wbytes = (size_t)p.heads * kHeadDim * k2 * k2 * sizeof(float);
+    e = cudaMemsetAsync(ga.dwk, 0, wbytes, stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(ga.dwv, 0, wbytes, stream);
+    if (e == cudaSuccess && ga.dbias) e = cudaMemsetAsync(ga.dbias, 0, (size_t)p.heads * k2 * sizeof(float), stream);
+    if (e == cudaSuccess) e = launch_strip_prep(p, wt, stream);
+    if (e != cudaSuccess) return e;
     float* ws_a = static_cast<float*>(ws);
-    float* ws_dl = ws_a + (size_t)p.B * p.H * p.W * p.heads * p.ksize * p.ksize;
+    float* ws_dl = ws_a + (size_t)p.B * p.H * p.W * p.heads * k2;
     const float* w = static_cast<const float*>(wt);
-    return p.dtype == SLIDE_ATTN_BF16 ? launch_k<__nv_bfloat16>(p, ga, w, ws_a, ws_dl, d_status, num_sms, stream)
-                                      : launch_k<float>(p, ga, w, ws_a, ws_dl, d_status, num_sms, stream);
+    return p.dtype == SLIDE_ATTN_BF16 ? launch_t<__nv_bfloat16, 1>(p, ga, w, ws_a, ws_dl, d_status, num_sms, stream)
+                                      : launch_t<float, 1>(p, ga, w, ws_a, ws_dl, d_status, num_sms, stream);
 }
 
 }  // namespace slide_attn

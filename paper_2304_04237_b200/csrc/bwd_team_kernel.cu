@@ -1,0 +1,612 @@
+// Backward pass for k = 3 (head_dim 32, fp32 or bf16 storage) on tcgen05 with fp32 arithmetic (split.cuh, team.cuh):
+//
+//   forward again   a = softmax_s( scale * sum_{t,c} q[c] k_t[c] wk[c,s,t] + bias[s] )
+//   da[s]    = sum_{t,c} g[c] v_t[c] wv[c,s,t]                 (the logit contraction with g, v, wv)
+//   dl[s]    = a[s] (da[s] - sum_s' a[s'] da[s'])              dbias[s] = sum over pixels of dl[s]
+//   dq[c]    = scale * sum_t k_t[c] (sum_s dl[s] wk[c,s,t])    (the value expansion with dl, wk, k)
+//   dk[p'][c] = scale * sum_t q[p' - off(t)][c] (sum_s dl[p' - off(t)][s] wk[c,s,t])
+//   dv[p'][c] =         sum_t g[p' - off(t)][c] (sum_s  a[p' - off(t)][s] wv[c,s,t])
+//
+// bwd_point_kernel: two contractions, then one expansion, per query pixel; leaves dl and a as split rows.
+// bwd_gather_kernel: dk and dv per key / value pixel, a gather over the nine query pixels whose window holds it.  The left
+// operand of tap t is the split rows of the block's pixels moved by -off(t): every tap has rows of its own, copied from a halo
+// in shared memory to tensor memory (out-of-map queries read as zero and contribute nothing), N = the channels of a plane.
+// Both persistent, one CTA per SM and one head per CTA, two teams; geometry and hand-offs as in umma_split_kernel.
+#include "bwd_common.cuh"
+#include "team.cuh"
+
+namespace slide_attn {
+
+namespace {
+
+using namespace team;
+
+constexpr int kHeadDim = 32;
+constexpr uint32_t kContract = contract_bytes(kHeadDim), kExpand = expand3_bytes(kHeadDim);
+// per head: contraction images of wk and wv, expansion images of wk and wv
+constexpr uint32_t kImages = 2 * kContract + 2 * kExpand;
+constexpr uint32_t kPointImages = 2 * kContract + kExpand, kGatherImages = 2 * kExpand, kGatherFrom = 2 * kContract;
+constexpr uint32_t kMisc = 8u * (kTeams * kTeamBars + 1) + 16 + 2 * kK2 * 4 + 8;      // barriers, tensor-memory slot, bias, dbias
+
+__host__ __device__ constexpr int ring_for(uint32_t images) {
+    const int fit = (int)((227u * 1024u - images - kMisc - 128) / (kTeams * kSlot));
+    return fit < kMaxRing ? fit : kMaxRing;
+}
+template <uint32_t Images> struct Plan {
+    static constexpr int ring = ring_for(Images);
+    static_assert(ring >= 4, "the ring does not fit");
+    static constexpr uint32_t w_off = (uint32_t)(kTeams * ring * kSlot);
+    static constexpr uint32_t bar_off = w_off + Images;
+    static constexpr uint32_t total = bar_off + kMisc + 128;
+};
+
+struct TeamParams {
+    const unsigned char* images;
+    const void* q;
+    const void* g;
+    const float* bias;
+    unsigned char* rows_dl;
+    unsigned char* rows_a;
+    void* dq;
+    void* dk;
+    void* dv;
+    float* dbias;
+    int* status;
+    int H, W, heads;
+    Strips strips;
+    float scale;
+};
+
+// Images of a head (blockIdx.x) and, spread over all blocks, zeros for what later kernels add to.
+template <typename T>
+__global__ void __launch_bounds__(256)
+bwd_prep_kernel(const float* __restrict__ wk, const float* __restrict__ wv, unsigned char* __restrict__ images, float* dwk, float* dwv, float* dbias)
+{
+    grid_launch_dependents();
+    const size_t w = (size_t)blockIdx.x * kHeadDim * kK2 * kK2;
+    unsigned char* img = images + (size_t)blockIdx.x * kImages;
+    constexpr int contract_items = kHeadDim / 8 * kK2 * 48, expand_items = kHeadDim * kK2;
+    const int step = gridDim.y * 256, at = blockIdx.y * 256 + threadIdx.x;
+    for (int i = at; i < 2 * (contract_items + expand_items); i += step) {
+        const int side = i >= contract_items + expand_items, j = side ? i - contract_items - expand_items : i;
+        const float* src = (side ? wv : wk) + w;
+        if (j < contract_items) build_contract_item<T>(src, img + side * kContract, j);
+        else build_expand3_item<T>(src, img + 2 * kContract + side * kExpand, j - contract_items);
+    }
+    for (int i = at; i < kHeadDim * kK2 * kK2; i += step) { dwk[w + i] = 0.f; dwv[w + i] = 0.f; }
+    if (dbias && at < kK2) dbias[blockIdx.x * kK2 + at] = 0.f;
+}
+
+// Eight (bf16) or four (fp32) channels of a pixel to memory.
+__device__ __forceinline__ void store_piece(__nv_bfloat16* p, const float (&f)[8], float s) {
+    *reinterpret_cast<uint4*>(p) = make_uint4(pack_bf16(f[0] * s, f[1] * s), pack_bf16(f[2] * s, f[3] * s), pack_bf16(f[4] * s, f[5] * s),
+                                              pack_bf16(f[6] * s, f[7] * s));
+}
+__device__ __forceinline__ void store_piece(float* p, const float (&f)[4], float s) {
+    *reinterpret_cast<float4*>(p) = make_float4(f[0] * s, f[1] * s, f[2] * s, f[3] * s);
+}
+
+// What both kernels share: the CTA's set-up and its geometry.
+struct Seat {
+    int warp, lane, h, team_id, first, step, my_blocks;
+    uint32_t bars, bar_weights, tmem;
+    unsigned char* ring;
+    __device__ __forceinline__ uint32_t bar(int i) const { return bars + 8u * (uint32_t)(team_id * kTeamBars + i); }
+    __device__ __forceinline__ long long strip0(int bi) const { return 4LL * (first + (long long)bi * step); }
+};
+template <uint32_t Images>
+__device__ __forceinline__ Seat take_seat(unsigned char* smem, const TeamParams& P) {
+    using L = Plan<Images>;
+    Seat s;
+    s.warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); s.lane = threadIdx.x & 31;
+    s.h = blockIdx.x % P.heads;
+    const int rank = blockIdx.x / P.heads, nrank = (int)gridDim.x / P.heads;
+    s.team_id = s.warp < kComputeWarps ? s.warp / kTeamWarps : (s.warp - kComputeWarps) % kTeams;
+    const int blocks = (int)((P.strips.total + 3) >> 2);
+    s.first = s.team_id * nrank + rank; s.step = kTeams * nrank;
+    s.my_blocks = s.first < blocks ? (blocks - s.first + s.step - 1) / s.step : 0;
+    s.bars = smem_u32(smem + L::bar_off);
+    s.bar_weights = s.bars + 8u * (kTeams * kTeamBars);
+    s.ring = smem + (uint32_t)(s.team_id * L::ring * kSlot);
+    unsigned char* tmem_slot = smem + L::bar_off + 8u * (kTeams * kTeamBars + 1);
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < kTeams; ++i) init_team_bars(s.bars + 8u * (uint32_t)(i * kTeamBars));
+        mbar_init_only(s.bar_weights, 1);
+        mbar_init_fence();
+    }
+    if (s.warp == kMmaWarp) tmem_alloc(smem_u32(tmem_slot), 512);
+    tc_fence_before_sync();
+    __syncthreads();
+    tc_fence_after_sync();
+    s.tmem = *reinterpret_cast<const volatile uint32_t*>(tmem_slot) + kCols * (uint32_t)s.team_id;
+    return s;
+}
+template <uint32_t Images>
+__device__ __forceinline__ void leave_seat(unsigned char* smem, const Seat& s) {
+    tc_fence_before_sync();
+    __syncthreads();
+    if (s.warp == kMmaWarp) {
+        tc_fence_after_sync();
+        tmem_dealloc(*reinterpret_cast<const volatile uint32_t*>(smem + Plan<Images>::bar_off + 8u * (kTeams * kTeamBars + 1)), 512);
+    }
+}
+// One slot of the ring: a plane of the block's four strips.
+__device__ __forceinline__ void load_slot(const Seat& s, const CUtensorMap* map, int slot, int c0, const Strip (&st)[4]) {
+    const uint32_t full = s.bar(kFull + slot);
+    mbar_expect_tx(full, kSlot);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) tma_load_4d(smem_u32(s.ring) + (uint32_t)(slot * kSlot + i * kHaloPlane), map, full, c0, st[i].x0 - 1, st[i].y0 - 1, st[i].b);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kThreads, 1)
+bwd_point_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v, const TeamParams P)
+{
+    using L = Plan<kPointImages>;
+    constexpr int CH = Cut<T>::channels, NPL = kHeadDim / CH, PL = Cut<T>::per_lane, DB = Cut<T>::d_buffers, R = L::ring, CHUNKS = 3 * NPL;
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char* smem = smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u);
+    float* s_bias = reinterpret_cast<float*>(smem + L::bar_off + 8u * (kTeams * kTeamBars + 1) + 16);
+    float* s_dbias = s_bias + kK2;
+    if (threadIdx.x < kK2) {
+        s_bias[threadIdx.x] = P.bias ? P.bias[(blockIdx.x % P.heads) * kK2 + threadIdx.x] * kLog2e : 0.f;
+        s_dbias[threadIdx.x] = 0.f;
+    }
+    const Seat seat = take_seat<kPointImages>(smem, P);
+    auto bar = [&](int i) { return seat.bar(i); };
+    const int warp = seat.warp, lane = seat.lane, h = seat.h, my_blocks = seat.my_blocks;
+    const uint32_t tmem = seat.tmem;
+    bool ok = true;
+
+    if (warp >= kTmaWarp) {
+        // ---- TMA thread of a team: K, V and K again ------------------------------------------------------
+        uint32_t leader;
+        if (elect_one(leader)) {
+            int slot = 0;
+            uint32_t phase = 1;
+            for (int bi = 0; ok && bi < my_blocks; ++bi) {
+                Strip st[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) st[i] = P.strips.at(seat.strip0(bi) + i);
+                for (int v = 0; v < 3 * NPL; ++v) {
+                    if (!mbar_wait(bar(kEmpty + slot), phase)) { ok = false; break; }
+                    load_slot(seat, v / NPL == 1 ? &map_v : &map_k, slot, h * kHeadDim + (v % NPL) * CH, st);
+                    if (++slot == R) { slot = 0; phase ^= 1u; }
+                }
+            }
+            if (!ok) atomicExch(P.status, 1);
+        }
+        __syncwarp();
+    } else if (warp >= kMmaWarp) {
+        // ---- MMA thread of a team ------------------------------------------------------------------------
+        uint32_t leader;
+        if (elect_one(leader)) {
+            const uint32_t w = smem_u32(smem + L::w_off);
+            if (warp == kMmaWarp) {
+                grid_dependency_wait();
+                mbar_expect_tx(seat.bar_weights, kPointImages);
+                bulk_load_1d(w, P.images + (size_t)h * kImages, kPointImages, seat.bar_weights);
+            }
+            if (my_blocks > 0) ok = mbar_wait(seat.bar_weights, 0);
+            const uint32_t dsrc = w + 2 * kContract;
+            int pn = 0, dn = 0;
+            for (int bi = 0; ok && bi < my_blocks; ++bi) {
+                for (int side = 0; ok && side < 2; ++side) {
+                    const uint64_t desc = contract_desc(w + side * kContract);
+                    for (int i = 0; i < CHUNKS; ++i, ++pn) {             // plane, tap column
+                        const int pb = pn & 1, plane = i / 3, dx = i % 3;
+                        if (!mbar_wait(bar(kPFull + pb), (uint32_t)(pn >> 1) & 1u)) { ok = false; break; }
+                        if (side == 1 && i == 0 && !mbar_wait(bar(kLFree), (uint32_t)bi & 1u)) { ok = false; break; }
+                        tc_fence_after_sync();
+                        const uint32_t p_col = tmem + kColP + (uint32_t)(pb * 3 * Cut<T>::tap_cols);
+#pragma unroll
+                        for (int dy = 0; dy < 3; ++dy)
+                            issue_contract<T>(tmem, p_col + dy * Cut<T>::tap_cols, desc + contract_step<T>(plane, dy * 3 + dx), dx,
+                                              dy == 0 && (sizeof(T) == 2 ? i == 0 : plane == 0), dy == 0 && i == 0);
+                        umma_commit(bar(kPFree + pb));
+                    }
+                    if (ok) umma_commit(bar(kLFull));
+                }
+                if (!ok || !mbar_wait(bar(kAFull), (uint32_t)bi & 1u)) { ok = false; break; }
+                for (int i = 0; i < CHUNKS; ++i, ++dn) {
+                    const int db = dn % DB;
+                    if (!mbar_wait(bar(kDFree + db), ((uint32_t)(dn / DB) & 1u) ^ 1u)) { ok = false; break; }
+                    tc_fence_after_sync();
+                    issue_expand3<3 * CH>(tmem + kColD + (uint32_t)(db * 3 * CH), tmem + kColA, dsrc + (uint32_t)(i * 3 * CH * 128));
+                    umma_commit(bar(kDFull + db));
+                }
+            }
+            if (!ok) atomicExch(P.status, 1);
+        }
+        __syncwarp();
+    } else {
+        const int w = warp % kTeamWarps, wq = w & 3, half = w >> 2, g = lane >> 2, tig = lane & 3;
+        const uint32_t quad = tmem + ((uint32_t)(32 * wq) << 16), mine = quad + ((uint32_t)(16 * half) << 16);
+        const int C = P.heads * kHeadDim;
+        auto strip_of = [&](int bi) { return P.strips.at(seat.strip0(bi) + wq); };
+        float dbias[kK2];
+#pragma unroll
+        for (int s = 0; s < kK2; ++s) dbias[s] = 0.f;
+        int slot = 0, pn = 0, dn = 0;
+        uint32_t phase = 0;
+        auto release = [&]() {
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar(kEmpty + slot));
+            if (++slot == R) { slot = 0; phase ^= 1u; }
+        };
+        auto load_x = [&](const Strip& s, int side, int plane, uint4 (&x)[2]) {
+            const T* src = static_cast<const T*>(side ? P.g : P.q);
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                const int y = s.y0 + 2 * half + r;
+                x[r] = make_uint4(0u, 0u, 0u, 0u);
+                if (y < P.H && s.x0 + g < P.W)
+                    x[r] = __ldg(reinterpret_cast<const uint4*>(src + (((size_t)s.b * P.H + y) * P.W + s.x0 + g) * C + h * kHeadDim + plane * CH + tig * PL));
+            }
+        };
+        Strip st = strip_of(0);
+        uint4 xn[2];
+        if (my_blocks > 0) load_x(st, 0, 0, xn);
+        for (int bi = 0; ok && bi < my_blocks; ++bi) {
+            const bool turn = half == (bi & 1);                      // the warps that do the softmax of this block
+            float a[kK2];
+            // ---- products of both sides ----------------------------------------------------------------
+            for (int v = 0; v < 2 * NPL; ++v) {
+                const uint4 x[2] = {xn[0], xn[1]};
+                if (v + 1 < 2 * NPL) load_x(st, (v + 1) / NPL, (v + 1) % NPL, xn);
+                if (!warp_wait(bar(kFull + slot), phase)) { ok = false; break; }
+                const unsigned char* plane = seat.ring + (uint32_t)(slot * kSlot + wq * kHaloPlane);
+#pragma unroll
+                for (int dx = 0; dx < 3; ++dx, ++pn) {
+                    const int pb = pn & 1;
+                    uint4 y[4];
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) y[r] = halo_piece(plane, 2 * half + r, g + dx, tig);
+                    if (!warp_wait(bar(kPFree + pb), ((uint32_t)(pn >> 1) & 1u) ^ 1u)) { ok = false; break; }
+                    tc_fence_after_sync();
+                    const uint32_t t = mine + kColP + (uint32_t)(pb * 3 * Cut<T>::tap_cols);
+#pragma unroll
+                    for (int dy = 0; dy < 3; ++dy) store_products(T(), t + dy * Cut<T>::tap_cols, x, y[dy], y[dy + 1]);
+                    tmem_wait_st();
+                    tc_fence_before_sync();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar(kPFull + pb));
+                    // the logits: complete while the first chunk of the other side was made
+                    if (dx == 0 && v == NPL && turn) {
+                        if (!warp_wait(bar(kLFull), 0)) { ok = false; break; }
+                        tc_fence_after_sync();
+                        load_contraction<T>(quad, a);
+                        tc_fence_before_sync();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(bar(kLFree));
+                    }
+                }
+                if (!ok) break;
+                release();
+            }
+            if (!ok) break;
+            const Strip cur = st;
+            if (bi + 1 < my_blocks) { st = strip_of(bi + 1); load_x(st, 0, 0, xn); }
+
+            // ---- a and dl: thread = pixel of the quadrant ------------------------------------------------
+            if (turn) {
+                float m = -INFINITY, z = 0.f;
+#pragma unroll
+                for (int s = 0; s < kK2; ++s) { a[s] = fmaf(a[s], P.scale * kLog2e, s_bias[s]); m = fmaxf(m, a[s]); }
+#pragma unroll
+                for (int s = 0; s < kK2; ++s) { a[s] = fast_exp2(a[s] - m); z += a[s]; }
+                const float iz = 1.f / z;
+#pragma unroll
+                for (int s = 0; s < kK2; ++s) a[s] *= iz;
+                if (!warp_wait(bar(kLFull), 1)) { ok = false; break; }
+                tc_fence_after_sync();
+                float dl[kK2], mean = 0.f;
+                load_contraction<T>(quad, dl);                       // da
+#pragma unroll
+                for (int s = 0; s < kK2; ++s) mean = fmaf(a[s], dl[s], mean);
+#pragma unroll
+                for (int s = 0; s < kK2; ++s) dl[s] = a[s] * (dl[s] - mean);
+                uint32_t row[16];
+                split_row(dl, row);
+                tmem_st_32x32b_x16(quad + kColA, row);
+                tmem_wait_st();
+                tc_fence_before_sync();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar(kAFull));
+                // lane = 8 row + column of the strip
+                const int y = cur.y0 + (lane >> 3), x = cur.x0 + (lane & 7);
+                if (cur.inside && y < P.H && x < P.W) {
+                    const size_t at = ((((size_t)cur.b * P.H + y) * P.W + x) * P.heads + h) * 64;
+                    const uint32_t swz = (uint32_t)(lane >> 1) & 3u;             // x0 is a multiple of 8
+#pragma unroll
+                    for (uint32_t c = 0; c < 4; ++c)
+                        *reinterpret_cast<uint4*>(P.rows_dl + at + ((c ^ swz) << 4)) = make_uint4(row[4 * c], row[4 * c + 1], row[4 * c + 2], row[4 * c + 3]);
+                    split_row(a, row);
+#pragma unroll
+                    for (uint32_t c = 0; c < 4; ++c)
+                        *reinterpret_cast<uint4*>(P.rows_a + at + ((c ^ swz) << 4)) = make_uint4(row[4 * c], row[4 * c + 1], row[4 * c + 2], row[4 * c + 3]);
+#pragma unroll
+                    for (int s = 0; s < kK2; ++s) dbias[s] += dl[s];
+                }
+            }
+
+            // ---- dq ----------------------------------------------------------------------------------
+            for (int pl = 0; pl < NPL; ++pl) {
+                float acc[2][PL];
+#pragma unroll
+                for (int r = 0; r < 2; ++r)
+#pragma unroll
+                    for (int c = 0; c < PL; ++c) acc[r][c] = 0.f;
+                if (!warp_wait(bar(kFull + slot), phase)) { ok = false; break; }
+                const unsigned char* plane = seat.ring + (uint32_t)(slot * kSlot + wq * kHaloPlane);
+#pragma unroll
+                for (int dx = 0; dx < 3; ++dx, ++dn) {
+                    const int db = dn % DB;
+                    if (!warp_wait(bar(kDFull + db), (uint32_t)(dn / DB) & 1u)) { ok = false; break; }
+                    tc_fence_after_sync();
+                    sum_chunk(T(), mine + kColD + (uint32_t)(db * 3 * CH), plane, 2 * half, g + dx, tig, acc);
+                    tc_fence_before_sync();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar(kDFree + db));
+                }
+                if (!ok) break;
+                release();
+                if (cur.inside && cur.x0 + g < P.W) {
+#pragma unroll
+                    for (int r = 0; r < 2; ++r) {
+                        const int y = cur.y0 + 2 * half + r;
+                        if (y < P.H)
+                            store_piece(static_cast<T*>(P.dq) + (((size_t)cur.b * P.H + y) * P.W + cur.x0 + g) * C + h * kHeadDim + pl * CH + tig * PL, acc[r], P.scale);
+                    }
+                }
+            }
+        }
+        if (!ok && lane == 0) atomicExch(P.status, 1);
+        if (P.dbias) {
+#pragma unroll
+            for (int s = 0; s < kK2; ++s) {
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) dbias[s] += __shfl_xor_sync(0xffffffffu, dbias[s], o);
+                if (lane == 0) atomicAdd(&s_dbias[s], dbias[s]);
+            }
+        }
+    }
+    leave_seat<kPointImages>(smem, seat);
+    if (P.dbias && threadIdx.x < kK2) atomicAdd(&P.dbias[h * kK2 + threadIdx.x], s_dbias[threadIdx.x]);
+}
+
+// Tensor memory of a team here: D chunks in 0 - 191, the left operands of a tap column's three taps in 192 - 239.
+template <typename T>
+__global__ void __launch_bounds__(kThreads, 1)
+bwd_gather_kernel(const __grid_constant__ CUtensorMap map_dl, const __grid_constant__ CUtensorMap map_a,
+                  const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_g, const TeamParams P)
+{
+    using L = Plan<kGatherImages>;
+    constexpr int CH = Cut<T>::channels, NPL = kHeadDim / CH, PL = Cut<T>::per_lane, DB = Cut<T>::d_buffers, R = L::ring;
+    constexpr uint32_t kColRows = 192;
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char* smem = smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u);
+    const Seat seat = take_seat<kGatherImages>(smem, P);
+    auto bar = [&](int i) { return seat.bar(i); };
+    const int warp = seat.warp, lane = seat.lane, h = seat.h, my_blocks = seat.my_blocks;
+    const uint32_t tmem = seat.tmem;
+    const int steps = my_blocks * 6;                                 // side, tap column
+    bool ok = true;
+
+    if (warp >= kTmaWarp) {
+        // ---- TMA thread of a team: per side the rows, then the planes ---------------------------------------
+        uint32_t leader;
+        if (elect_one(leader)) {
+            grid_dependency_wait();                                  // the rows come from the kernel before
+            int slot = 0;
+            uint32_t phase = 1;
+            for (int bi = 0; ok && bi < my_blocks; ++bi) {
+                Strip st[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) st[i] = P.strips.at(seat.strip0(bi) + i);
+                for (int v = 0; v < 2 * (NPL + 1); ++v) {
+                    const int side = v / (NPL + 1), pl = v % (NPL + 1) - 1;
+                    if (!mbar_wait(bar(kEmpty + slot), phase)) { ok = false; break; }
+                    load_slot(seat, pl < 0 ? (side ? &map_a : &map_dl) : (side ? &map_g : &map_q), slot, h * kHeadDim + (pl < 0 ? 0 : pl * CH), st);
+                    if (++slot == R) { slot = 0; phase ^= 1u; }
+                }
+            }
+            if (!ok) atomicExch(P.status, 1);
+        }
+        __syncwarp();
+    } else if (warp >= kMmaWarp) {
+        // ---- MMA thread of a team ------------------------------------------------------------------------
+        uint32_t leader;
+        if (elect_one(leader)) {
+            const uint32_t w = smem_u32(smem + L::w_off);
+            if (warp == kMmaWarp) {
+                grid_dependency_wait();
+                mbar_expect_tx(seat.bar_weights, kGatherImages);
+                bulk_load_1d(w, P.images + (size_t)h * kImages + kGatherFrom, kGatherImages, seat.bar_weights);
+            }
+            if (my_blocks > 0) ok = mbar_wait(seat.bar_weights, 0);
+            int dn = 0;
+            for (int s = 0; ok && s < steps; ++s) {
+                const int side = s / 3 & 1, dx = s % 3;
+                if (!mbar_wait(bar(kAFull), (uint32_t)s & 1u)) { ok = false; break; }
+                for (int pl = 0; pl < NPL; ++pl, ++dn) {
+                    const int db = dn % DB;
+                    if (!mbar_wait(bar(kDFree + db), ((uint32_t)(dn / DB) & 1u) ^ 1u)) { ok = false; break; }
+                    tc_fence_after_sync();
+#pragma unroll
+                    for (int dy = 0; dy < 3; ++dy)
+                        issue_expand3<CH>(tmem + kColD + (uint32_t)(db * 3 * CH + dy * CH), tmem + kColRows + 16 * dy,
+                                          w + side * kExpand + (uint32_t)(((pl * 3 + dx) * 3 + dy) * CH * 128));
+                    umma_commit(bar(kDFull + db));
+                }
+            }
+            if (!ok) atomicExch(P.status, 1);
+        }
+        __syncwarp();
+    } else {
+        const int w = warp % kTeamWarps, wq = w & 3, half = w >> 2, g = lane >> 2, tig = lane & 3;
+        const uint32_t quad = tmem + ((uint32_t)(32 * wq) << 16), mine = quad + ((uint32_t)(16 * half) << 16);
+        const int C = P.heads * kHeadDim;
+        // visit v of the stream of planes (NPL + 1 per side): slot v % R, phase v / R
+        int rows_slot = 0;
+        uint32_t rows_phase = 0;
+        auto ahead = [](int& slot, uint32_t& phase, int by) { slot += by; if (slot >= R) { slot -= R; phase ^= 1u; } };
+        // the left operands of step s: pixel (row, column) of the strip reads halo pixel (row + 2 - dy, column + 2 - dx)
+        auto store_rows = [&](int s) -> bool {
+            const int dx = s % 3;
+            if (dx == 0 && !warp_wait(bar(kFull + rows_slot), rows_phase)) return false;
+            if (half == (s & 1)) {
+                const int pr = lane >> 3, pc = lane & 7;
+                const uint32_t swz = (uint32_t)((pc + 1 - dx) >> 1) & 3u;
+                const unsigned char* src = seat.ring + (uint32_t)(rows_slot * kSlot + wq * kHaloPlane) + (uint32_t)((pr + 2) * 10 + pc + 2 - dx) * 64u;
+#pragma unroll
+                for (int dy = 0; dy < 3; ++dy) {
+                    uint32_t row[16];
+#pragma unroll
+                    for (uint32_t c = 0; c < 4; ++c) {
+                        const uint4 v = *reinterpret_cast<const uint4*>(src - dy * 640 + ((c ^ swz) << 4));
+                        row[4 * c] = v.x; row[4 * c + 1] = v.y; row[4 * c + 2] = v.z; row[4 * c + 3] = v.w;
+                    }
+                    tmem_st_32x32b_x16(quad + kColRows + 16 * dy, row);
+                }
+                tmem_wait_st();
+                tc_fence_before_sync();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar(kAFull));
+            }
+            if (dx == 2) {
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar(kEmpty + rows_slot));
+                ahead(rows_slot, rows_phase, NPL + 1);
+            }
+            return true;
+        };
+        int slot = 1, dn = 0;                                        // of the side's first plane
+        uint32_t phase = 0;
+        if (steps > 0) ok = store_rows(0);
+        float acc[NPL][2][PL];
+        for (int s = 0; ok && s < steps; ++s) {
+            const int bi = s / 6, side = s / 3 & 1, dx = s % 3;
+            if (dx == 0) {
+#pragma unroll
+                for (int pl = 0; pl < NPL; ++pl)
+#pragma unroll
+                    for (int r = 0; r < 2; ++r)
+#pragma unroll
+                        for (int c = 0; c < PL; ++c) acc[pl][r][c] = 0.f;
+            }
+            int ps = slot;
+            uint32_t pp = phase;
+#pragma unroll
+            for (int pl = 0; pl < NPL; ++pl, ++dn) {
+                const int db = dn % DB;
+                if (dx == 0 && !warp_wait(bar(kFull + ps), pp)) { ok = false; break; }
+                if (!warp_wait(bar(kDFull + db), (uint32_t)(dn / DB) & 1u)) { ok = false; break; }
+                tc_fence_after_sync();
+                // the last MMAs of this step are complete: its operands make room for the next ones
+                if (pl == NPL - 1 && s + 1 < steps && !store_rows(s + 1)) { ok = false; break; }
+                sum_chunk<true>(T(), mine + kColD + (uint32_t)(db * 3 * CH), seat.ring + (uint32_t)(ps * kSlot + wq * kHaloPlane), 2 * half, g + 2 - dx, tig, acc[pl]);
+                tc_fence_before_sync();
+                __syncwarp();
+                if (lane == 0) {
+                    mbar_arrive(bar(kDFree + db));
+                    if (dx == 2) mbar_arrive(bar(kEmpty + ps));
+                }
+                ahead(ps, pp, 1);
+            }
+            if (!ok) break;
+            if (dx == 2) {
+                ahead(slot, phase, NPL + 1);
+                const Strip st = P.strips.at(seat.strip0(bi) + wq);
+                if (st.inside && st.x0 + g < P.W) {
+                    T* out = static_cast<T*>(side ? P.dv : P.dk);
+#pragma unroll
+                    for (int r = 0; r < 2; ++r) {
+                        const int y = st.y0 + 2 * half + r;
+                        if (y < P.H)
+#pragma unroll
+                            for (int pl = 0; pl < NPL; ++pl)
+                                store_piece(out + (((size_t)st.b * P.H + y) * P.W + st.x0 + g) * C + h * kHeadDim + pl * CH + tig * PL, acc[pl][r], side ? 1.f : P.scale);
+                    }
+                }
+            }
+        }
+        if (!ok && lane == 0) atomicExch(P.status, 1);
+    }
+    leave_seat<kGatherImages>(smem, seat);
+}
+
+template <typename... Params, typename... Args>
+cudaError_t launch_chained(void (*kernel)(Params...), int grid, int threads, uint32_t smem, cudaStream_t stream, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+template <typename T>
+cudaError_t launch_t(const Problem& p, const BackwardArgs& ga, const BwdScratch& ws, int* d_status, int num_sms, cudaStream_t stream) {
+    static bool configured[64] = {};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev >= 64 || !configured[dev]) {
+        e = cudaFuncSetAttribute(bwd_point_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Plan<kPointImages>::total);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(bwd_gather_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Plan<kGatherImages>::total);
+        if (e != cudaSuccess) return e;
+        if (dev < 64) configured[dev] = true;
+    }
+    TeamParams P;
+    P.images = ws.images; P.q = p.q; P.g = ga.dout; P.bias = p.bias; P.rows_dl = ws.rows_dl; P.rows_a = ws.rows_a;
+    P.dq = ga.dq; P.dk = ga.dk; P.dv = ga.dv; P.dbias = ga.dbias; P.status = d_status;
+    P.H = p.H; P.W = p.W; P.heads = p.heads;
+    P.strips.sx = (p.W + 7) / 8; P.strips.bands = (p.H + 3) / 4;
+    P.strips.total = (long long)p.B * P.strips.bands * P.strips.sx;
+    if (P.strips.total > 0x7fffffffLL - 4) return cudaErrorInvalidConfiguration;
+    P.scale = 1.f / sqrtf((float)kHeadDim);
+    const int C = p.heads * kHeadDim, es = (int)sizeof(T), ch = Cut<T>::channels;
+    CUtensorMap mq, mk, mv, mg, mdl, ma;
+    if (!make_tile_map(&mq, p.q, es, p.B, p.H, p.W, C, ch, 10, 6) || !make_tile_map(&mk, p.k, es, p.B, p.H, p.W, C, ch, 10, 6) ||
+        !make_tile_map(&mv, p.v, es, p.B, p.H, p.W, C, ch, 10, 6) || !make_tile_map(&mg, ga.dout, es, p.B, p.H, p.W, C, ch, 10, 6) ||
+        !make_tile_map(&mdl, ws.rows_dl, 2, p.B, p.H, p.W, C, 32, 10, 6) || !make_tile_map(&ma, ws.rows_a, 2, p.B, p.H, p.W, C, 32, 10, 6))
+        return cudaErrorInvalidValue;
+    bwd_prep_kernel<T><<<dim3((unsigned)p.heads, 9), 256, 0, stream>>>(p.wk, p.wv, ws.images, ga.dwk, ga.dwv, ga.dbias);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    const long long blocks = (P.strips.total + 3) / 4;
+    long long per_head = num_sms / p.heads;
+    if (per_head > blocks) per_head = blocks;
+    if (per_head < 1) per_head = 1;
+    const int grid = (int)(per_head * p.heads);
+    e = launch_chained(bwd_point_kernel<T>, grid, kThreads, Plan<kPointImages>::total, stream, mk, mv, P);
+    if (e != cudaSuccess) return e;
+    return launch_chained(bwd_gather_kernel<T>, grid, kThreads, Plan<kGatherImages>::total, stream, mdl, ma, mq, mg, P);
+}
+
+size_t rows_bytes(int B, int H, int W, int heads) { return (size_t)B * H * W * heads * 64; }
+
+}  // namespace
+
+size_t bwd_team_workspace_bytes(int B, int H, int W, int heads) { return 2 * rows_bytes(B, H, W, heads) + (size_t)heads * kImages + 512; }
+
+BwdScratch bwd_scratch(void* ws, int B, int H, int W, int heads) {
+    auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
+    BwdScratch s;
+    s.rows_dl = static_cast<unsigned char*>(ws);
+    s.rows_a = s.rows_dl + up(rows_bytes(B, H, W, heads));
+    s.images = s.rows_a + up(rows_bytes(B, H, W, heads));
+    return s;
+}
+
+cudaError_t launch_bwd_team(const Problem& p, const BackwardArgs& ga, const BwdScratch& ws, int* d_status, int num_sms, cudaStream_t stream) {
+    return p.dtype == SLIDE_ATTN_BF16 ? launch_t<__nv_bfloat16>(p, ga, ws, d_status, num_sms, stream) : launch_t<float>(p, ga, ws, d_status, num_sms, stream);
+}
+
+}  // namespace slide_attn

@@ -35,8 +35,8 @@ using namespace split;
 constexpr int kHeadDim = 32;
 constexpr int kK2 = 9;
 constexpr int kTH = 4;                         // tile rows
-constexpr int kComputeWarps = 12, kConvertWarps = 4;
-constexpr int kThreads = (kComputeWarps + kConvertWarps) * 32;
+constexpr int kComputeWarps = 12;
+constexpr int kThreads = (kComputeWarps + 1) * 32;
 constexpr int kFlush = 4;
 constexpr uint32_t kSumBytes = 2u * kK2 * kHeadDim * 32u * 4u;        // the CTA's sums at its end, [side][tap][channel][32 columns]
 
@@ -63,7 +63,7 @@ __host__ __device__ inline WLayout w_layout(int tw) {
     L.split_off = L.g_off + np * L.tile_plane;
     L.split_side = (uint32_t)(kTH * tw) * 64u;
     L.stage = L.split_off + 2 * L.split_side;
-    L.tx_bytes = 2 * np * (halo + tile);
+    L.tx_bytes = 2 * np * (halo + tile) + 2 * L.split_side;
     return L;
 }
 
@@ -74,8 +74,6 @@ uint32_t w_smem_bytes(int tw) {
 }
 
 struct WParams {
-    const float* ws_a;
-    const float* ws_dl;
     float* dwk;
     float* dwv;
     int* status;
@@ -143,7 +141,8 @@ __device__ __forceinline__ void accumulate(float (&acc)[4][4], const Frag<float>
 template <typename T>
 __global__ void __launch_bounds__(kThreads, 1)
 bwd_weight_mma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
-                      const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_g, const WParams P)
+                      const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_g,
+                      const __grid_constant__ CUtensorMap map_dl, const __grid_constant__ CUtensorMap map_a, const WParams P)
 {
     constexpr uint32_t PB = Frag<T>::pixel_bytes;                    // of one plane
     extern __shared__ unsigned char smem_raw[];
@@ -162,7 +161,7 @@ bwd_weight_mma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
     const int HW = P.tw + 2;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < 2; ++s) { mbar_init_only(bar_full(s), 1 + kConvertWarps); mbar_init_only(bar_empty(s), kComputeWarps); }
+        for (int s = 0; s < 2; ++s) { mbar_init_only(bar_full(s), 1); mbar_init_only(bar_empty(s), kComputeWarps); }
         mbar_init_fence();
     }
     __syncthreads();
@@ -172,66 +171,35 @@ bwd_weight_mma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
     const int side = warp / 6, half = (warp / 3) & 1, ty = warp % 3;  // of a compute warp
 
     if (warp >= kComputeWarps) {
-        // ---- loads and split columns ----------------------------------------------------------------
-        const int ct = threadIdx.x - kComputeWarps * 32;
-        const int npix = kTH * P.tw;
-        int it = 0;
-        for (int tile = rank; tile < tiles && ok; tile += nrank, ++it) {
-            const int st = it & 1;
-            int rest_ = tile;
-            const int tx = rest_ % P.tiles_x; rest_ /= P.tiles_x;
-            const int tyy = rest_ % P.tiles_y;
-            const int b = rest_ / P.tiles_y;
-            const int x0 = tx * P.tw, y0 = tyy * kTH;
-            unsigned char* stage = smem + (uint32_t)st * L.stage;
-            if (it >= 2 && !__all_sync(0xffffffffu, mbar_wait(bar_empty(st), (uint32_t)(it / 2 - 1) & 1u) ? 1 : 0)) { ok = false; break; }
-            if (ct == 0) {
+        // ---- TMA thread --------------------------------------------------------------------------------
+        uint32_t leader;
+        if (elect_one(leader)) {
+            grid_dependency_wait();                                  // the split rows come from an earlier kernel
+            int it = 0;
+            for (int tile = rank; tile < tiles; tile += nrank, ++it) {
+                const int st = it & 1;
+                int rest_ = tile;
+                const int tx = rest_ % P.tiles_x; rest_ /= P.tiles_x;
+                const int tyy = rest_ % P.tiles_y;
+                const int b = rest_ / P.tiles_y;
+                const int x0 = tx * P.tw, y0 = tyy * kTH;
+                const uint32_t stage = smem_u32(smem) + (uint32_t)st * L.stage;
+                if (it >= 2 && !mbar_wait(bar_empty(st), (uint32_t)(it / 2 - 1) & 1u)) { ok = false; break; }
                 mbar_expect_tx(bar_full(st), L.tx_bytes);
+                tma_load_4d(stage + L.split_off, &map_dl, bar_full(st), h * 32, x0, y0, b);
+                tma_load_4d(stage + L.split_off + L.split_side, &map_a, bar_full(st), h * 32, x0, y0, b);
 #pragma unroll
                 for (int pl = 0; pl < WTile<T>::planes; ++pl) {
                     const int c0 = h * kHeadDim + pl * (32 / WTile<T>::planes);
-                    tma_load_4d(smem_u32(stage + L.k_off + pl * L.halo_plane), &map_k, bar_full(st), c0, x0 - 1, y0 - 1, b);
-                    tma_load_4d(smem_u32(stage + L.v_off + pl * L.halo_plane), &map_v, bar_full(st), c0, x0 - 1, y0 - 1, b);
-                    tma_load_4d(smem_u32(stage + L.q_off + pl * L.tile_plane), &map_q, bar_full(st), c0, x0, y0, b);
-                    tma_load_4d(smem_u32(stage + L.g_off + pl * L.tile_plane), &map_g, bar_full(st), c0, x0, y0, b);
+                    tma_load_4d(stage + L.k_off + pl * L.halo_plane, &map_k, bar_full(st), c0, x0 - 1, y0 - 1, b);
+                    tma_load_4d(stage + L.v_off + pl * L.halo_plane, &map_v, bar_full(st), c0, x0 - 1, y0 - 1, b);
+                    tma_load_4d(stage + L.q_off + pl * L.tile_plane, &map_q, bar_full(st), c0, x0, y0, b);
+                    tma_load_4d(stage + L.g_off + pl * L.tile_plane, &map_g, bar_full(st), c0, x0, y0, b);
                 }
             }
-            for (int i = ct; i < 2 * npix; i += kConvertWarps * 32) {
-                const int sd = i >= npix, px = sd ? i - npix : i;
-                const int py = px / P.tw, pxx = px - py * P.tw;
-                const int y = y0 + py, x = x0 + pxx;
-                float f[kK2];
-                if (y < P.H && x < P.W) {
-                    const float* src = (sd ? P.ws_a : P.ws_dl) + (((size_t)(b * P.H + y) * P.W + x) * P.heads + h) * kK2;
-#pragma unroll
-                    for (int s = 0; s < kK2; ++s) f[s] = __ldg(src + s);
-                } else {
-#pragma unroll
-                    for (int s = 0; s < kK2; ++s) f[s] = 0.f;
-                }
-                // columns: 9 upper parts, 9 middle parts, 9 lower parts, zeros
-                float v[28];
-#pragma unroll
-                for (int s = 0; s < kK2; ++s) {
-                    v[s] = f[s];
-                    v[9 + s] = rest(v[s]);
-                    v[18 + s] = rest(v[9 + s]);
-                }
-                v[27] = 0.f;
-                unsigned char* dst = stage + L.split_off + (uint32_t)sd * L.split_side + (uint32_t)px * 64u;
-                const uint32_t swz = (uint32_t)(px >> 1) & 3u;
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    uint4 o;
-                    o.x = pack_upper(v[8 * c], v[8 * c + 1]); o.y = pack_upper(v[8 * c + 2], v[8 * c + 3]);
-                    o.z = c < 3 ? pack_upper(v[8 * c + 4], v[8 * c + 5]) : 0u;
-                    o.w = c < 3 ? pack_upper(v[8 * c + 6], v[8 * c + 7]) : 0u;
-                    *reinterpret_cast<uint4*>(dst + (((uint32_t)c ^ swz) << 4)) = o;
-                }
-            }
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar_full(st));
+            if (!ok) atomicExch(P.status, 1);
         }
+        __syncwarp();
     } else {
         // ---- products and sums ----------------------------------------------------------------------
 #pragma unroll
@@ -318,7 +286,7 @@ bwd_weight_mma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
 }
 
 template <typename T>
-cudaError_t launch_t(const Problem& p, const BackwardArgs& ga, const BwdParams& BP, int num_sms, cudaStream_t stream) {
+cudaError_t launch_t(const Problem& p, const BackwardArgs& ga, const BwdScratch& ws, int* d_status, int num_sms, cudaStream_t stream) {
     static bool done[64] = {};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -335,30 +303,40 @@ cudaError_t launch_t(const Problem& p, const BackwardArgs& ga, const BwdParams& 
         if (c <= cover) { cover = c; tw = t; }
     }
     WParams P;
-    P.ws_a = BP.ws_a; P.ws_dl = BP.ws_dl; P.dwk = BP.dwk; P.dwv = BP.dwv; P.status = BP.status;
+    P.dwk = ga.dwk; P.dwv = ga.dwv; P.status = d_status;
     P.B = p.B; P.H = p.H; P.W = p.W; P.heads = p.heads;
     P.tw = tw; P.tiles_x = (p.W + tw - 1) / tw; P.tiles_y = (p.H + kTH - 1) / kTH;
-    P.scale = BP.scale;
+    P.scale = 1.f / sqrtf((float)kHeadDim);
     const int Ctot = p.heads * kHeadDim, es = (int)sizeof(T), bc = kHeadDim / WTile<T>::planes;
-    CUtensorMap mq, mk, mv, mg;
+    CUtensorMap mq, mk, mv, mg, mdl, ma;
     if (!make_tile_map(&mq, p.q, es, p.B, p.H, p.W, Ctot, bc, tw, kTH) ||
         !make_tile_map(&mg, ga.dout, es, p.B, p.H, p.W, Ctot, bc, tw, kTH) ||
         !make_tile_map(&mk, p.k, es, p.B, p.H, p.W, Ctot, bc, tw + 2, kTH + 2) ||
-        !make_tile_map(&mv, p.v, es, p.B, p.H, p.W, Ctot, bc, tw + 2, kTH + 2))
+        !make_tile_map(&mv, p.v, es, p.B, p.H, p.W, Ctot, bc, tw + 2, kTH + 2) ||
+        !make_tile_map(&mdl, ws.rows_dl, 2, p.B, p.H, p.W, Ctot, 32, tw, kTH) || !make_tile_map(&ma, ws.rows_a, 2, p.B, p.H, p.W, Ctot, 32, tw, kTH))
         return cudaErrorInvalidValue;
     const long long tiles = (long long)P.tiles_x * P.tiles_y * p.B;
     if (tiles > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
     long long per_head = num_sms / p.heads;                          // one CTA per SM, all heads alike
     if (per_head > tiles) per_head = tiles;
     if (per_head < 1) per_head = 1;
-    bwd_weight_mma_kernel<T><<<(unsigned)(per_head * p.heads), kThreads, w_smem_bytes<T>(tw), stream>>>(mq, mk, mv, mg, P);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(per_head * p.heads));
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = w_smem_bytes<T>(tw);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, bwd_weight_mma_kernel<T>, mq, mk, mv, mg, mdl, ma, P);
 }
 
 }  // namespace
 
-cudaError_t launch_bwd_weight_mma(const Problem& p, const BackwardArgs& ga, const BwdParams& P, int num_sms, cudaStream_t stream) {
-    return p.dtype == SLIDE_ATTN_BF16 ? launch_t<__nv_bfloat16>(p, ga, P, num_sms, stream) : launch_t<float>(p, ga, P, num_sms, stream);
+cudaError_t launch_bwd_weight_mma(const Problem& p, const BackwardArgs& ga, const BwdScratch& ws, int* d_status, int num_sms, cudaStream_t stream) {
+    return p.dtype == SLIDE_ATTN_BF16 ? launch_t<__nv_bfloat16>(p, ga, ws, d_status, num_sms, stream) : launch_t<float>(p, ga, ws, d_status, num_sms, stream);
 }
 
 }  // namespace slide_attn

@@ -92,7 +92,7 @@ struct BackwardArgs {
 };
 bool backward_supports(int head_dim, int ksize);
 size_t backward_workspace_bytes(int B, int H, int W, int heads, int ksize);
-cudaError_t launch_backward(const Problem& p, const BackwardArgs& ga, const void* wt, void* ws, int* d_status,
+cudaError_t launch_backward(const Problem& p, const BackwardArgs& ga, void* wt, void* ws, int* d_status,
                             int num_sms, cudaStream_t stream);
 
 // MMA_WIDE variant: general weights with large windows on mma.sync tensor cores (bf16, head_dim 32,

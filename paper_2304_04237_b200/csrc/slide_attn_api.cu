@@ -342,12 +342,7 @@ slide_attn_status slide_attn_backward(slide_attn_ctx* c, const void* q, const vo
     p.ksize = c->ksize; p.has_bias = c->has_bias; p.dtype = c->dtype;
     p.q = q; p.k = k; p.v = v; p.wk = wk; p.wv = wv; p.bias = bias; p.out = nullptr;
     BackwardArgs ga = {dout, dq, dk, dv, dwk, dwv, dbias};
-    const size_t k2 = (size_t)c->ksize * c->ksize;
-    const size_t wbytes = (size_t)c->heads * c->head_dim * k2 * k2 * sizeof(float);
-    bool ok = cudaMemsetAsync(dwk, 0, wbytes, stream) == cudaSuccess && cudaMemsetAsync(dwv, 0, wbytes, stream) == cudaSuccess;
-    if (ok && dbias) ok = cudaMemsetAsync(dbias, 0, (size_t)c->heads * k2 * sizeof(float), stream) == cudaSuccess;
-    if (ok) ok = launch_strip_prep(p, c->strip_ws, stream) == cudaSuccess;
-    if (ok) ok = launch_backward(p, ga, c->strip_ws, c->bwd_ws, c->d_status, c->num_sms, stream) == cudaSuccess;
+    const bool ok = launch_backward(p, ga, c->strip_ws, c->bwd_ws, c->d_status, c->num_sms, stream) == cudaSuccess;
     if (!ok) { cudaGetLastError(); return SLIDE_ATTN_ERR_CUDA; }
     return SLIDE_ATTN_OK;
 }

@@ -158,6 +158,65 @@ __device__ __forceinline__ void expand_row(const float (&a)[kK2], uint32_t (&row
     row[14] = 0u; row[15] = 0u;
 }
 
+// ---- the same expansion for slot values of any magnitude (gradients): three bf16 parts each -----------------------------
+// SPLIT ROW: 64 bytes of a pixel and head, 32 bf16: 0 - 8 upper parts of the slots, 9 - 17 middle, 18 - 26 lower parts, 27, 28
+// the middle parts of slots 7 and 8 again.  In memory its four 16-byte pieces are swizzled by the pixel's column x (piece c
+// at c ^ ((x >> 1) & 3)), which makes reads of eight neighbouring pixels' pieces free of bank conflicts.
+// It meets an image of four 16-row K steps: rows 0 - 15 of the row with the upper parts of the weights, 16 - 31 likewise
+// (27, 28 with the middle parts of slots 7 and 8), 0 - 15 with the middle parts, 0 - 8 with the lower parts: everything down to
+// 2^-24 of the product.
+__host__ __device__ constexpr uint32_t expand3_bytes(int head_dim) { return (uint32_t)head_dim * 9u * 128u; }
+template <typename T>
+__device__ __forceinline__ void build_expand3_item(const float* __restrict__ w, unsigned char* img, int item) {
+    constexpr int CH = Cut<T>::channels;
+    const int n = item % CH, r = item / CH, dy = r % 3, dx = (r / 3) % 3, plane = r / 9;
+    const int c = plane * CH + (CH / 4) * ((n & 7) >> 1) + 2 * (n >> 3) + (n & 1), tap = dy * 3 + dx;
+    float hi[kK2], mid[kK2], lo[kK2];
+#pragma unroll
+    for (int s = 0; s < kK2; ++s) {
+        hi[s] = w[(c * kK2 + s) * kK2 + tap];
+        mid[s] = split::rest(hi[s]);
+        lo[s] = split::rest(mid[s]);
+    }
+    float v[64];
+#pragma unroll
+    for (int i = 0; i < 64; ++i) v[i] = 0.f;
+#pragma unroll
+    for (int s = 0; s < kK2; ++s) {
+        v[s] = hi[s]; v[9 + s] = hi[s]; v[18 + s] = hi[s];
+        v[32 + s] = mid[s]; v[48 + s] = lo[s];
+    }
+    v[27] = mid[7]; v[28] = mid[8];
+#pragma unroll
+    for (int s = 0; s < 7; ++s) v[41 + s] = mid[s];
+    unsigned char* col = img + (size_t)(item >> 3) * 1024 + (item & 7) * 16;
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+        *reinterpret_cast<uint4*>(col + j * 128) = make_uint4(split::pack_upper(v[8 * j], v[8 * j + 1]), split::pack_upper(v[8 * j + 2], v[8 * j + 3]),
+                                                              split::pack_upper(v[8 * j + 4], v[8 * j + 5]), split::pack_upper(v[8 * j + 6], v[8 * j + 7]));
+}
+// The split row of nine slot values: 16 registers of two.
+__device__ __forceinline__ void split_row(const float (&a)[kK2], uint32_t (&row)[16]) {
+    float v[28];
+#pragma unroll
+    for (int s = 0; s < kK2; ++s) { v[s] = a[s]; v[9 + s] = split::rest(v[s]); v[18 + s] = split::rest(v[9 + s]); }
+    v[27] = v[16];
+#pragma unroll
+    for (int i = 0; i < 14; ++i) row[i] = split::pack_upper(v[2 * i], v[2 * i + 1]);
+    row[14] = split::pack_upper(v[17], 0.f);
+    row[15] = 0u;
+}
+// Where a split row of N columns of D is issued: B at `b_smem` (of the image), A in 16 columns at `a_col`.
+template <int N>
+__device__ __forceinline__ void issue_expand3(uint32_t d_col, uint32_t a_col, uint32_t b_smem) {
+    constexpr uint32_t idesc = umma_idesc_bf16(128, N);
+    const uint64_t b = umma_smem_desc(b_smem, 128, 1024);
+    umma_bf16_ts(d_col, a_col, b, idesc, 0);
+    umma_bf16_ts(d_col, a_col + 8, b + 16, idesc, 1);                        // 256 bytes on: the next K step
+    umma_bf16_ts(d_col, a_col, b + 32, idesc, 1);
+    umma_bf16_ts(d_col, a_col, b + 48, idesc, 1);
+}
+
 // The images of one head by prep_parts(head_dim) blocks of 256 threads, of which this one is `part`: a warp per channel of
 // the expansion image, then a thread per item of the contraction image.  (Four blocks a head, each looking for the
 // channels' largest weights by itself, took 12 us, most of what a small map needs.)
@@ -180,12 +239,13 @@ __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity) {
 // Barriers of a team; kFull, kEmpty: its ring of planes.
 constexpr int kMaxRing = 5;
 enum : int { kPFull = 0, kPFree = 2, kLFull = 4, kAFull = 5, kDFull = 6, kDFree = 9, kFull = 12, kEmpty = kFull + kMaxRing,
-             kTeamBars = kEmpty + kMaxRing };
+             kLFree = kEmpty + kMaxRing, kTeamBars };
 
 __device__ __forceinline__ void init_team_bars(uint32_t base) {
     auto init = [&](int i, uint32_t count) { mbar_init_only(base + 8u * (uint32_t)i, count); };
     for (int i = 0; i < 2; ++i) { init(kPFull + i, kTeamWarps); init(kPFree + i, 1); }
     init(kLFull, 1);
+    init(kLFree, 4);
     init(kAFull, 4);
     for (int i = 0; i < 3; ++i) { init(kDFull + i, 1); init(kDFree + i, kTeamWarps); }
     for (int i = 0; i < kMaxRing; ++i) { init(kFull + i, 1); init(kEmpty + i, kTeamWarps); }
@@ -291,8 +351,9 @@ __device__ __forceinline__ void issue_expand(uint32_t d_col, uint32_t a_col, uin
     umma_bf16_ts(d_col, a_col + 8, umma_smem_desc(b_smem + 256, 128, 512), idesc, 1);
 }
 
-// acc[row][channel of the lane] += D chunk (three taps of column dx) at `t` times the halo rows of that column, which are
-// loaded while the chunk is on its way.
+// acc[row][channel of the lane] += D chunk (three taps of a column) at `t` times the halo rows of that column, which are
+// loaded while the chunk is on its way.  Tap dy meets halo row `row` + dy, or, in the transposed shift, `row` + 2 - dy.
+template <bool Transposed = false>
 __device__ __forceinline__ void sum_chunk(__nv_bfloat16, uint32_t t, const unsigned char* plane, int row, int col, int tig, float (&acc)[2][8]) {
     uint32_t d[48];
     tmem_ld3_16x256b_x4_nowait(t, t + 32, t + 64, d);
@@ -313,8 +374,9 @@ __device__ __forceinline__ void sum_chunk(__nv_bfloat16, uint32_t t, const unsig
 #pragma unroll
             for (int j = 0; j < 4; ++j)
                 ffma2(acc[r][2 * j], acc[r][2 * j + 1], __uint_as_float(d[16 * dy + 4 * j + 2 * r]), __uint_as_float(d[16 * dy + 4 * j + 2 * r + 1]),
-                      f[r + dy][2 * j], f[r + dy][2 * j + 1]);
+                      f[r + (Transposed ? 2 - dy : dy)][2 * j], f[r + (Transposed ? 2 - dy : dy)][2 * j + 1]);
 }
+template <bool Transposed = false>
 __device__ __forceinline__ void sum_chunk(float, uint32_t t, const unsigned char* plane, int row, int col, int tig, float (&acc)[2][4]) {
     uint32_t d[3][8];
 #pragma unroll
@@ -331,7 +393,7 @@ __device__ __forceinline__ void sum_chunk(float, uint32_t t, const unsigned char
 #pragma unroll
             for (int j = 0; j < 2; ++j)
                 ffma2(acc[r][2 * j], acc[r][2 * j + 1], __uint_as_float(d[dy][4 * j + 2 * r]), __uint_as_float(d[dy][4 * j + 2 * r + 1]),
-                      f4(y[r + dy], 2 * j), f4(y[r + dy], 2 * j + 1));
+                      f4(y[r + (Transposed ? 2 - dy : dy)], 2 * j), f4(y[r + (Transposed ? 2 - dy : dy)], 2 * j + 1));
     }
 }
 

@@ -90,10 +90,10 @@ def test_backward_no_bias_dense_weights_and_repeat(dtype):
 
 
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
-@pytest.mark.parametrize("shape", [(4, 21, 60, 8, 3), (2, 19, 57, 5, 3), (3, 6, 120, 4, 3)], ids=lambda s: "x".join(map(str, s)))
+@pytest.mark.parametrize("shape", [(4, 21, 60, 8, 3), (2, 19, 57, 5, 3), (3, 6, 120, 4, 3), (7, 28, 64, 8, 3)], ids=lambda s: "x".join(map(str, s)))
 def test_backward_several_tiles_per_cta(shape, dtype):
-    """More tiles than CTAs per head (both stages of the weight kernel used again), widths at the edges of its
-    tile widths, odd heights.  dq, dk, dv as elsewhere; the weight gradients are fp32 sums of about 5000 exact
+    """More tiles than CTAs per head (both stages of the weight kernel used again), two to four blocks per team of
+    the point and gather kernels, widths at the edges of the tile widths, odd heights.  dq, dk, dv as elsewhere; the weight gradients are fp32 sums of about 5000 exact
     products in two levels of accumulation: 1e-5 of the largest entry."""
     x, dout = inputs(shape, dtype)
     ref = ob.backward(x["q"], x["k"], x["v"], x["wk"], x["wv"], x["bias"], 3, dout)
