@@ -130,13 +130,23 @@ __device__ __forceinline__ void leave_seat(unsigned char* smem, const Seat& s) {
         tmem_dealloc(*reinterpret_cast<const volatile uint32_t*>(smem + Plan<Images>::bar_off + 8u * (kTeams * kTeamBars + 1)), 512);
     }
 }
-// One slot of the ring: a plane of the block's four strips.
-__device__ __forceinline__ void load_slot(const Seat& s, const CUtensorMap* map, int slot, int c0, const Strip (&st)[4]) {
-    const uint32_t full = s.bar(kFull + slot);
-    mbar_expect_tx(full, kSlot);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) tma_load_4d(smem_u32(s.ring) + (uint32_t)(slot * kSlot + i * kHaloPlane), map, full, c0, st[i].x0 - 1, st[i].y0 - 1, st[i].b);
-}
+// The pixels of a compute lane: two rows of column g of a strip.
+struct Place { size_t pix; bool in[2]; };
+struct Lane {
+    StripWalk walk;
+    int wq, half, g, tig;
+    __device__ __forceinline__ Lane(const Seat& s, const TeamParams& P)
+        : walk(P.strips, s.strip0(0) + (s.warp & 3), 4LL * s.step), wq(s.warp & 3), half(s.warp % kTeamWarps >> 2), g(s.lane >> 2), tig(s.lane & 3) {}
+    // pixel (row, column) of the walk's strip, which is strip `i`, and the one below it; nothing is inside past the last strip
+    __device__ __forceinline__ Place place(const TeamParams& P, long long i, int row, int col) const {
+        Place p;
+        const int y = walk.y0() + row, x = walk.x0() + col;
+        const bool in = i < P.strips.total && x < P.W;
+        p.in[0] = in && y < P.H; p.in[1] = in && y + 1 < P.H;
+        p.pix = ((size_t)walk.b * P.H + y) * P.W + x;
+        return p;
+    }
+};
 
 template <typename T>
 __global__ void __launch_bounds__(kThreads, 1)
@@ -164,13 +174,11 @@ bwd_point_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constan
         if (elect_one(leader)) {
             int slot = 0;
             uint32_t phase = 1;
-            for (int bi = 0; ok && bi < my_blocks; ++bi) {
-                Strip st[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) st[i] = P.strips.at(seat.strip0(bi) + i);
+            StripWalk at(P.strips, seat.strip0(0), 4LL * seat.step);
+            for (int bi = 0; ok && bi < my_blocks; ++bi, at.next()) {
                 for (int v = 0; v < 3 * NPL; ++v) {
                     if (!mbar_wait(bar(kEmpty + slot), phase)) { ok = false; break; }
-                    load_slot(seat, v / NPL == 1 ? &map_v : &map_k, slot, h * kHeadDim + (v % NPL) * CH, st);
+                    load_strips(smem_u32(seat.ring) + (uint32_t)(slot * kSlot), v / NPL == 1 ? &map_v : &map_k, bar(kFull + slot), h * kHeadDim + (v % NPL) * CH, at);
                     if (++slot == R) { slot = 0; phase ^= 1u; }
                 }
             }
@@ -220,10 +228,11 @@ bwd_point_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constan
         }
         __syncwarp();
     } else {
-        const int w = warp % kTeamWarps, wq = w & 3, half = w >> 2, g = lane >> 2, tig = lane & 3;
+        Lane me(seat, P);
+        const int wq = me.wq, half = me.half, g = me.g, tig = me.tig;
         const uint32_t quad = tmem + ((uint32_t)(32 * wq) << 16), mine = quad + ((uint32_t)(16 * half) << 16);
-        const int C = P.heads * kHeadDim;
-        auto strip_of = [&](int bi) { return P.strips.at(seat.strip0(bi) + wq); };
+        const int C = P.heads * kHeadDim, piece = h * kHeadDim + tig * PL;
+        const size_t row_pitch = (size_t)P.W * C;
         float dbias[kK2];
 #pragma unroll
         for (int s = 0; s < kK2; ++s) dbias[s] = 0.f;
@@ -231,20 +240,18 @@ bwd_point_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constan
         uint32_t phase = 0;
         auto release = [&]() {
             __syncwarp();
-            if (lane == 0) mbar_arrive(bar(kEmpty + slot));
+            mbar_arrive_lane0(bar(kEmpty + slot), lane);
             if (++slot == R) { slot = 0; phase ^= 1u; }
         };
-        auto load_x = [&](const Strip& s, int side, int plane, uint4 (&x)[2]) {
-            const T* src = static_cast<const T*>(side ? P.g : P.q);
+        auto load_x = [&](const Place& p, int side, int plane, uint4 (&x)[2]) {
+            const T* src = static_cast<const T*>(side ? P.g : P.q) + p.pix * C + piece + plane * CH;
 #pragma unroll
             for (int r = 0; r < 2; ++r) {
-                const int y = s.y0 + 2 * half + r;
                 x[r] = make_uint4(0u, 0u, 0u, 0u);
-                if (y < P.H && s.x0 + g < P.W)
-                    x[r] = __ldg(reinterpret_cast<const uint4*>(src + (((size_t)s.b * P.H + y) * P.W + s.x0 + g) * C + h * kHeadDim + plane * CH + tig * PL));
+                if (p.in[r]) x[r] = __ldg(reinterpret_cast<const uint4*>(src + r * row_pitch));
             }
         };
-        Strip st = strip_of(0);
+        Place st = me.place(P, seat.strip0(0) + wq, 2 * half, g);
         uint4 xn[2];
         if (my_blocks > 0) load_x(st, 0, 0, xn);
         for (int bi = 0; ok && bi < my_blocks; ++bi) {
@@ -270,7 +277,7 @@ bwd_point_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constan
                     tmem_wait_st();
                     tc_fence_before_sync();
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(bar(kPFull + pb));
+                    mbar_arrive_lane0(bar(kPFull + pb), lane);
                     // the logits: complete while the first chunk of the other side was made
                     if (dx == 0 && v == NPL && turn) {
                         if (!warp_wait(bar(kLFull), 0)) { ok = false; break; }
@@ -278,15 +285,14 @@ bwd_point_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constan
                         load_contraction<T>(quad, a);
                         tc_fence_before_sync();
                         __syncwarp();
-                        if (lane == 0) mbar_arrive(bar(kLFree));
+                        mbar_arrive_lane0(bar(kLFree), lane);
                     }
                 }
                 if (!ok) break;
                 release();
             }
             if (!ok) break;
-            const Strip cur = st;
-            if (bi + 1 < my_blocks) { st = strip_of(bi + 1); load_x(st, 0, 0, xn); }
+            const Place cur = st;
 
             // ---- a and dl: thread = pixel of the quadrant ------------------------------------------------
             if (turn) {
@@ -312,11 +318,11 @@ bwd_point_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constan
                 tmem_wait_st();
                 tc_fence_before_sync();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(bar(kAFull));
+                mbar_arrive_lane0(bar(kAFull), lane);
                 // lane = 8 row + column of the strip
-                const int y = cur.y0 + (lane >> 3), x = cur.x0 + (lane & 7);
-                if (cur.inside && y < P.H && x < P.W) {
-                    const size_t at = ((((size_t)cur.b * P.H + y) * P.W + x) * P.heads + h) * 64;
+                const Place px = me.place(P, seat.strip0(bi) + wq, lane >> 3, lane & 7);
+                if (px.in[0]) {
+                    const size_t at = (px.pix * P.heads + h) * 64;
                     const uint32_t swz = (uint32_t)(lane >> 1) & 3u;             // x0 is a multiple of 8
 #pragma unroll
                     for (uint32_t c = 0; c < 4; ++c)
@@ -329,6 +335,8 @@ bwd_point_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constan
                     for (int s = 0; s < kK2; ++s) dbias[s] += dl[s];
                 }
             }
+
+            if (bi + 1 < my_blocks) { me.walk.next(); st = me.place(P, seat.strip0(bi + 1) + wq, 2 * half, g); load_x(st, 0, 0, xn); }
 
             // ---- dq ----------------------------------------------------------------------------------
             for (int pl = 0; pl < NPL; ++pl) {
@@ -347,18 +355,13 @@ bwd_point_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constan
                     sum_chunk(T(), mine + kColD + (uint32_t)(db * 3 * CH), plane, 2 * half, g + dx, tig, acc);
                     tc_fence_before_sync();
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(bar(kDFree + db));
+                    mbar_arrive_lane0(bar(kDFree + db), lane);
                 }
                 if (!ok) break;
                 release();
-                if (cur.inside && cur.x0 + g < P.W) {
 #pragma unroll
-                    for (int r = 0; r < 2; ++r) {
-                        const int y = cur.y0 + 2 * half + r;
-                        if (y < P.H)
-                            store_piece(static_cast<T*>(P.dq) + (((size_t)cur.b * P.H + y) * P.W + cur.x0 + g) * C + h * kHeadDim + pl * CH + tig * PL, acc[r], P.scale);
-                    }
-                }
+                for (int r = 0; r < 2; ++r)
+                    if (cur.in[r]) store_piece(static_cast<T*>(P.dq) + cur.pix * C + piece + pl * CH + r * row_pitch, acc[r], P.scale);
             }
         }
         if (!ok && lane == 0) atomicExch(P.status, 1);
@@ -390,7 +393,6 @@ bwd_gather_kernel(const __grid_constant__ CUtensorMap map_dl, const __grid_const
     auto bar = [&](int i) { return seat.bar(i); };
     const int warp = seat.warp, lane = seat.lane, h = seat.h, my_blocks = seat.my_blocks;
     const uint32_t tmem = seat.tmem;
-    const int steps = my_blocks * 6;                                 // side, tap column
     bool ok = true;
 
     if (warp >= kTmaWarp) {
@@ -400,14 +402,13 @@ bwd_gather_kernel(const __grid_constant__ CUtensorMap map_dl, const __grid_const
             grid_dependency_wait();                                  // the rows come from the kernel before
             int slot = 0;
             uint32_t phase = 1;
-            for (int bi = 0; ok && bi < my_blocks; ++bi) {
-                Strip st[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) st[i] = P.strips.at(seat.strip0(bi) + i);
+            StripWalk at(P.strips, seat.strip0(0), 4LL * seat.step);
+            for (int bi = 0; ok && bi < my_blocks; ++bi, at.next()) {
                 for (int v = 0; v < 2 * (NPL + 1); ++v) {
                     const int side = v / (NPL + 1), pl = v % (NPL + 1) - 1;
                     if (!mbar_wait(bar(kEmpty + slot), phase)) { ok = false; break; }
-                    load_slot(seat, pl < 0 ? (side ? &map_a : &map_dl) : (side ? &map_g : &map_q), slot, h * kHeadDim + (pl < 0 ? 0 : pl * CH), st);
+                    load_strips(smem_u32(seat.ring) + (uint32_t)(slot * kSlot), pl < 0 ? (side ? &map_a : &map_dl) : (side ? &map_g : &map_q), bar(kFull + slot),
+                                h * kHeadDim + (pl < 0 ? 0 : pl * CH), at);
                     if (++slot == R) { slot = 0; phase ^= 1u; }
                 }
             }
@@ -426,7 +427,7 @@ bwd_gather_kernel(const __grid_constant__ CUtensorMap map_dl, const __grid_const
             }
             if (my_blocks > 0) ok = mbar_wait(seat.bar_weights, 0);
             int dn = 0;
-            for (int s = 0; ok && s < steps; ++s) {
+            for (int s = 0; ok && s < my_blocks * 6; ++s) {         // side, tap column
                 const int side = s / 3 & 1, dx = s % 3;
                 if (!mbar_wait(bar(kAFull), (uint32_t)s & 1u)) { ok = false; break; }
                 for (int pl = 0; pl < NPL; ++pl, ++dn) {
@@ -444,21 +445,23 @@ bwd_gather_kernel(const __grid_constant__ CUtensorMap map_dl, const __grid_const
         }
         __syncwarp();
     } else {
-        const int w = warp % kTeamWarps, wq = w & 3, half = w >> 2, g = lane >> 2, tig = lane & 3;
+        Lane me(seat, P);
+        const int wq = me.wq, half = me.half, g = me.g, tig = me.tig;
         const uint32_t quad = tmem + ((uint32_t)(32 * wq) << 16), mine = quad + ((uint32_t)(16 * half) << 16);
-        const int C = P.heads * kHeadDim;
+        const int C = P.heads * kHeadDim, piece = h * kHeadDim + tig * PL;
+        const size_t row_pitch = (size_t)P.W * C;
         // visit v of the stream of planes (NPL + 1 per side): slot v % R, phase v / R
         int rows_slot = 0;
         uint32_t rows_phase = 0;
         auto ahead = [](int& slot, uint32_t& phase, int by) { slot += by; if (slot >= R) { slot -= R; phase ^= 1u; } };
-        // the left operands of step s: pixel (row, column) of the strip reads halo pixel (row + 2 - dy, column + 2 - dx)
-        auto store_rows = [&](int s) -> bool {
-            const int dx = s % 3;
+        const uint32_t rows_at = (uint32_t)(wq * kHaloPlane) + (uint32_t)(((lane >> 3) + 2) * 10 + (lane & 7) + 2) * 64u;
+        // the left operands of a step (tap column dx; `turn`: this warp's): pixel (row, column) of the strip reads halo pixel
+        // (row + 2 - dy, column + 2 - dx)
+        auto store_rows = [&](int dx, bool turn) -> bool {
             if (dx == 0 && !warp_wait(bar(kFull + rows_slot), rows_phase)) return false;
-            if (half == (s & 1)) {
-                const int pr = lane >> 3, pc = lane & 7;
-                const uint32_t swz = (uint32_t)((pc + 1 - dx) >> 1) & 3u;
-                const unsigned char* src = seat.ring + (uint32_t)(rows_slot * kSlot + wq * kHaloPlane) + (uint32_t)((pr + 2) * 10 + pc + 2 - dx) * 64u;
+            if (turn) {
+                const uint32_t swz = (uint32_t)(((lane & 7) + 1 - dx) >> 1) & 3u;
+                const unsigned char* src = seat.ring + (uint32_t)(rows_slot * kSlot) + rows_at - dx * 64;
 #pragma unroll
                 for (int dy = 0; dy < 3; ++dy) {
                     uint32_t row[16];
@@ -472,64 +475,62 @@ bwd_gather_kernel(const __grid_constant__ CUtensorMap map_dl, const __grid_const
                 tmem_wait_st();
                 tc_fence_before_sync();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(bar(kAFull));
+                mbar_arrive_lane0(bar(kAFull), lane);
             }
             if (dx == 2) {
                 __syncwarp();
-                if (lane == 0) mbar_arrive(bar(kEmpty + rows_slot));
+                mbar_arrive_lane0(bar(kEmpty + rows_slot), lane);
                 ahead(rows_slot, rows_phase, NPL + 1);
             }
             return true;
         };
         int slot = 1, dn = 0;                                        // of the side's first plane
         uint32_t phase = 0;
-        if (steps > 0) ok = store_rows(0);
-        float acc[NPL][2][PL];
-        for (int s = 0; ok && s < steps; ++s) {
-            const int bi = s / 6, side = s / 3 & 1, dx = s % 3;
-            if (dx == 0) {
+        if (my_blocks > 0) ok = store_rows(0, half == 0);
+        for (int bs = 0; ok && bs < 2 * my_blocks; ++bs) {           // block, side
+            const int side = bs & 1;
+            const bool even = half == side;                          // step 3 bs + dx is this warp's if even == (dx != 1)
+            float acc[NPL][2][PL];
 #pragma unroll
-                for (int pl = 0; pl < NPL; ++pl)
+            for (int pl = 0; pl < NPL; ++pl)
 #pragma unroll
-                    for (int r = 0; r < 2; ++r)
+                for (int r = 0; r < 2; ++r)
 #pragma unroll
-                        for (int c = 0; c < PL; ++c) acc[pl][r][c] = 0.f;
-            }
-            int ps = slot;
-            uint32_t pp = phase;
+                    for (int c = 0; c < PL; ++c) acc[pl][r][c] = 0.f;
 #pragma unroll
-            for (int pl = 0; pl < NPL; ++pl, ++dn) {
-                const int db = dn % DB;
-                if (dx == 0 && !warp_wait(bar(kFull + ps), pp)) { ok = false; break; }
-                if (!warp_wait(bar(kDFull + db), (uint32_t)(dn / DB) & 1u)) { ok = false; break; }
-                tc_fence_after_sync();
-                // the last MMAs of this step are complete: its operands make room for the next ones
-                if (pl == NPL - 1 && s + 1 < steps && !store_rows(s + 1)) { ok = false; break; }
-                sum_chunk<true>(T(), mine + kColD + (uint32_t)(db * 3 * CH), seat.ring + (uint32_t)(ps * kSlot + wq * kHaloPlane), 2 * half, g + 2 - dx, tig, acc[pl]);
-                tc_fence_before_sync();
-                __syncwarp();
-                if (lane == 0) {
-                    mbar_arrive(bar(kDFree + db));
-                    if (dx == 2) mbar_arrive(bar(kEmpty + ps));
+            for (int dx = 0; dx < 3; ++dx) {
+                int ps = slot;
+                uint32_t pp = phase;
+#pragma unroll
+                for (int pl = 0; pl < NPL; ++pl, ++dn) {
+                    const int db = dn % DB;
+                    if (dx == 0 && !warp_wait(bar(kFull + ps), pp)) { ok = false; break; }
+                    if (!warp_wait(bar(kDFull + db), (uint32_t)(dn / DB) & 1u)) { ok = false; break; }
+                    tc_fence_after_sync();
+                    // the last MMAs of this step are complete: its operands make room for the next ones
+                    if (pl == NPL - 1) {
+                        if (dx < 2) { if (!store_rows(dx + 1, dx == 0 ? !even : even)) { ok = false; break; } }
+                        else if (bs + 1 < 2 * my_blocks) { if (!store_rows(0, !even)) { ok = false; break; } }
+                    }
+                    sum_chunk<true>(T(), mine + kColD + (uint32_t)(db * 3 * CH), seat.ring + (uint32_t)(ps * kSlot + wq * kHaloPlane), 2 * half, g + 2 - dx, tig, acc[pl]);
+                    tc_fence_before_sync();
+                    __syncwarp();
+                    mbar_arrive_lane0(bar(kDFree + db), lane);
+                    if (dx == 2) mbar_arrive_lane0(bar(kEmpty + ps), lane);
+                    ahead(ps, pp, 1);
                 }
-                ahead(ps, pp, 1);
+                if (!ok) break;
             }
             if (!ok) break;
-            if (dx == 2) {
-                ahead(slot, phase, NPL + 1);
-                const Strip st = P.strips.at(seat.strip0(bi) + wq);
-                if (st.inside && st.x0 + g < P.W) {
-                    T* out = static_cast<T*>(side ? P.dv : P.dk);
+            ahead(slot, phase, NPL + 1);
+            const Place p = me.place(P, seat.strip0(bs >> 1) + wq, 2 * half, g);
+            T* out = static_cast<T*>(side ? P.dv : P.dk) + p.pix * C + piece;
 #pragma unroll
-                    for (int r = 0; r < 2; ++r) {
-                        const int y = st.y0 + 2 * half + r;
-                        if (y < P.H)
+            for (int r = 0; r < 2; ++r)
+                if (p.in[r])
 #pragma unroll
-                            for (int pl = 0; pl < NPL; ++pl)
-                                store_piece(out + (((size_t)st.b * P.H + y) * P.W + st.x0 + g) * C + h * kHeadDim + pl * CH + tig * PL, acc[pl][r], side ? 1.f : P.scale);
-                    }
-                }
-            }
+                    for (int pl = 0; pl < NPL; ++pl) store_piece(out + r * row_pitch + pl * CH, acc[pl][r], side ? 1.f : P.scale);
+            if (side) me.walk.next();
         }
         if (!ok && lane == 0) atomicExch(P.status, 1);
     }

@@ -96,19 +96,13 @@ umma_split_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
         if (elect_one(leader)) {
             int slot = 0;
             uint32_t phase = 1;                                      // a fresh barrier is free
-            for (int bi = 0; ok && bi < my_blocks; ++bi) {
-                const long long s0 = 4LL * (first + (long long)bi * step);
-                Strip st[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) st[i] = P.strips.at(s0 + i);
+            StripWalk at(P.strips, 4LL * first, 4LL * step);
+            for (int bi = 0; ok && bi < my_blocks; ++bi, at.next()) {
                 for (int v = 0; v < 2 * NPL; ++v) {
                     if (!mbar_wait(bar(kEmpty + slot), phase)) { ok = false; break; }
-                    mbar_expect_tx(bar(kFull + slot), kSlot);
                     const CUtensorMap* map = v < NPL ? &map_k : &map_v;
                     const int c0 = h * D + (v < NPL ? v : v - NPL) * CH;
-#pragma unroll
-                    for (int i = 0; i < 4; ++i)
-                        tma_load_4d(smem_u32(ring) + (uint32_t)(slot * kSlot + i * kHaloPlane), map, bar(kFull + slot), c0, st[i].x0 - 1, st[i].y0 - 1, st[i].b);
+                    load_strips(smem_u32(ring) + (uint32_t)(slot * kSlot), map, bar(kFull + slot), c0, at);
                     if (++slot == R) { slot = 0; phase ^= 1u; }
                 }
             }
@@ -161,26 +155,34 @@ umma_split_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
         float bias[kK2];
 #pragma unroll
         for (int s = 0; s < kK2; ++s) bias[s] = P.bias ? P.bias[h * kK2 + s] * kLog2e : 0.f;
-        auto strip_of = [&](int bi) { return P.strips.at(4LL * (first + (long long)bi * step) + wq); };
 
         int slot = 0, pn = 0, dn = 0;
         uint32_t phase = 0;
         auto release = [&]() {                                       // the plane at `slot` has been read
             __syncwarp();
-            if (lane == 0) mbar_arrive(bar(kEmpty + slot));
+            mbar_arrive_lane0(bar(kEmpty + slot), lane);
             if (++slot == R) { slot = 0; phase ^= 1u; }
         };
-        auto load_q = [&](const Strip& s, int plane, uint4 (&x)[2]) {
+        // the lane's first pixel: element offset of its piece, and which of its two rows are inside (past the last strip: none)
+        const size_t row_pitch = (size_t)P.W * C;
+        StripWalk walk(P.strips, 4LL * first + wq, 4LL * step);
+        struct Place { size_t at; bool in[2]; };
+        auto place = [&](int bi) {
+            Place p;
+            const int y = walk.y0() + 2 * half, x = walk.x0() + g;
+            const bool in = 4LL * (first + (long long)bi * step) + wq < P.strips.total && x < P.W;
+            p.in[0] = in && y < P.H; p.in[1] = in && y + 1 < P.H;
+            p.at = (((size_t)walk.b * P.H + y) * P.W + x) * C + h * D + tig * PL;
+            return p;
+        };
+        auto load_q = [&](const Place& p, int plane, uint4 (&x)[2]) {
 #pragma unroll
             for (int r = 0; r < 2; ++r) {
-                const int y = s.y0 + 2 * half + r;
                 x[r] = make_uint4(0u, 0u, 0u, 0u);
-                if (y < P.H && s.x0 + g < P.W)
-                    x[r] = __ldg(reinterpret_cast<const uint4*>(static_cast<const T*>(P.q) + (((size_t)s.b * P.H + y) * P.W + s.x0 + g) * C +
-                                                                h * D + plane * CH + tig * PL));
+                if (p.in[r]) x[r] = __ldg(reinterpret_cast<const uint4*>(static_cast<const T*>(P.q) + p.at + r * row_pitch + plane * CH));
             }
         };
-        Strip st = strip_of(0);
+        Place st = place(0);
         uint4 qn[2];
         if (my_blocks > 0) load_q(st, 0, qn);
         for (int bi = 0; bi < my_blocks; ++bi) {
@@ -204,14 +206,14 @@ umma_split_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
                     tmem_wait_st();
                     tc_fence_before_sync();
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(bar(kPFull + pb));
+                    mbar_arrive_lane0(bar(kPFull + pb), lane);
                 }
                 if (!ok) break;
                 release();
             }
             if (!ok) break;
-            const Strip cur = st;
-            if (bi + 1 < my_blocks) { st = strip_of(bi + 1); load_q(st, 0, qn); }
+            const Place cur = st;
+            if (bi + 1 < my_blocks) { walk.next(); st = place(bi + 1); load_q(st, 0, qn); }
 
             // ---- softmax: thread = pixel of the quadrant; the two warps of a quadrant take turns -------------
             if (half == (bi & 1)) {
@@ -232,7 +234,7 @@ umma_split_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
                 tmem_wait_st();
                 tc_fence_before_sync();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(bar(kAFull));
+                mbar_arrive_lane0(bar(kAFull), lane);
             }
 
             // ---- values ----------------------------------------------------------------------------
@@ -253,7 +255,7 @@ umma_split_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
                     sum_chunk(T(), mine + kColD + (uint32_t)(db * 3 * CH), plane, 2 * half, g + dx, tig, acc);
                     tc_fence_before_sync();
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(bar(kDFree + db));
+                    mbar_arrive_lane0(bar(kDFree + db), lane);
                 }
                 if (!ok) break;
                 release();
@@ -261,23 +263,18 @@ umma_split_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
                 float sc[PL];
 #pragma unroll
                 for (int c = 0; c < PL; ++c) sc[c] = inv[c] * (1.f / kScaleA);
-                if (cur.inside && cur.x0 + g < P.W) {
 #pragma unroll
-                    for (int r = 0; r < 2; ++r) {
-                        const int y = cur.y0 + 2 * half + r;
-                        if (y < P.H) {
-                            T* op = static_cast<T*>(P.out) + (((size_t)cur.b * P.H + y) * P.W + cur.x0 + g) * C + h * D + pl * CH + tig * PL;
-                            uint4 o;
-                            if constexpr (sizeof(T) == 2) {
-                                o.x = pack_bf16(acc[r][0] * sc[0], acc[r][1] * sc[1]); o.y = pack_bf16(acc[r][2] * sc[2], acc[r][3] * sc[3]);
-                                o.z = pack_bf16(acc[r][4] * sc[4], acc[r][5] * sc[5]); o.w = pack_bf16(acc[r][6] * sc[6], acc[r][7] * sc[7]);
-                            } else {
-                                o.x = __float_as_uint(acc[r][0] * sc[0]); o.y = __float_as_uint(acc[r][1] * sc[1]);
-                                o.z = __float_as_uint(acc[r][2] * sc[2]); o.w = __float_as_uint(acc[r][3] * sc[3]);
-                            }
-                            *reinterpret_cast<uint4*>(op) = o;
-                        }
+                for (int r = 0; r < 2; ++r) {
+                    if (!cur.in[r]) continue;
+                    uint4 o;
+                    if constexpr (sizeof(T) == 2) {
+                        o.x = pack_bf16(acc[r][0] * sc[0], acc[r][1] * sc[1]); o.y = pack_bf16(acc[r][2] * sc[2], acc[r][3] * sc[3]);
+                        o.z = pack_bf16(acc[r][4] * sc[4], acc[r][5] * sc[5]); o.w = pack_bf16(acc[r][6] * sc[6], acc[r][7] * sc[7]);
+                    } else {
+                        o.x = __float_as_uint(acc[r][0] * sc[0]); o.y = __float_as_uint(acc[r][1] * sc[1]);
+                        o.z = __float_as_uint(acc[r][2] * sc[2]); o.w = __float_as_uint(acc[r][3] * sc[3]);
                     }
+                    *reinterpret_cast<uint4*>(static_cast<T*>(P.out) + cur.at + r * row_pitch + pl * CH) = o;
                 }
             }
             if (!ok) break;
