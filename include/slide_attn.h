@@ -100,9 +100,9 @@ typedef enum {
     SLIDE_ATTN_VARIANT_UMMA_SPLIT = 11, /* fp32 arithmetic on tcgen05: operands split into parts whose bf16 / fp16
                                          products are exact or good to 2^-22; ksize 3, head_dim 32 or 64, fp32 or
                                          bf16: what AUTO runs for fp32 storage and for head_dim 64             */
-    SLIDE_ATTN_VARIANT_MMA_WIDE = 9   /* large windows with general weights on tensor cores (mma.sync):
-                                         TMA-staged halo tile, weights streamed tap by tap from L2 as
-                                         register fragments; bf16, head_dim 32, ksize 3 / 5 / 7 / 9: what
+    SLIDE_ATTN_VARIANT_MMA_WIDE = 9   /* large windows with general weights: persistent warp-specialised
+                                         kernel, both contractions on tcgen05, weights resident in shared
+                                         memory (ksize <= 5) or streamed from L2; bf16, head_dim 32, ksize 3 / 5 / 7 / 9: what
                                          AUTO runs for bf16 with ksize >= 5                              */
 } slide_attn_variant;
 

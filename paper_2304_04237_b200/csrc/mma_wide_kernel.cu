@@ -2,305 +2,539 @@
 // paper's stated limitation, App. E-F: k > 3 costs "a huge increase on the inference time"): bf16,
 // head_dim 32, k = 5, 7, 9 (k = 3 compiles too and serves as a cross-check).
 //
-// Arithmetic (Eq. 2 with Eq. 12 inside; w = E + D, E the one-hot shift of Eq. 11, D the remainder):
-//   P[p,(t,c)]  = q[p,c] k[p+off(t),c]                    packed bf16 multiply, formed in registers as
-//                                                          the A fragment of mma.sync.m16n8k16
-//   Ld[p,s]    += sum_c P[p,(t,c)] D_k[c,s,t]             k^2 taps x 2 k-steps x k^2/8 n-tiles
-//   Lp[p,t]    += sum_c P[p,(t,c)]                        one more MMA per k-step against a 0/1 fragment:
-//                                                          the plain q.k sum of tap t, exact products
-//   logit[s]    = (Ld[s] + Lp[s]) scale + bias[s];  e = exp2(logit - max)    (quad shuffles)
-//   A'[p,(t,c)] = e[p,t] + sum_s e_hi[p,s] D_v[c,s,t]     accumulator initialised to the exact fp32 e[p,t];
-//                                                          the logits' C fragments ARE the A fragments
-//   out[p,c]    = (sum_t A'[p,t,c] v[p+off(t),c]) / sum_s e[p,s]             packed fp32 FMAs
+// Arithmetic (Eq. 2 with Eq. 12 inside; w = E + D, E the one-hot shift of Eq. 11, D the remainder), both contractions on
+// tcgen05 with their left operands in tensor memory:
+//   P[p,(t,c)]  = q[p,c] k[p+off(t),c]                    packed bf16 multiplies -> tensor memory
+//   L[p,s]     += sum_c P[p,(t,c)] D_k[c,s,t]             per tap M = 128, N = slots (rounded up to 16), K = 32
+//   L[p,t]     += sum_c P[p,(t,c)]                        one-hot part: N = 16 columns around t against a column of ones, which
+//                                                         a window sliding over [0 .. 0 1 0 .. 0] puts at any column
+//   a[s]        = softmax(L scale + bias), kept as a_hi + a_lo (two bf16)
+//   A'[p,(t,c)] = sum_s a_hi[p,s] D_v[c,s,t] + (a_hi + a_lo)[p,t]          N = 32 per tap, K = slots; then K = 16 around t, twice
+//   out[p,c]    = sum_t A'[p,t,c] v[p+off(t),c]           packed fp32 FMAs
 // 2 k^4 multiply-adds per pixel-channel go to the tensor cores; the CUDA cores keep 2 k^2.
 //
-// One CTA = one head of a 4 x 32 pixel tile: K / V halo tiles and the q tile by TMA (64-byte channel
-// planes, zero fill = the padding); eight compute warps, each 2 rows x 8 columns = the 16 rows of an
-// MMA (lane (g, tig): column g, both rows, channels 8 tig .. 8 tig + 7).  The weights do not fit on
-// chip for k >= 5 (2 x 32 k^4 bf16 per head: 100 KB at k = 5, 950 KB at k = 9), so a ninth warp
-// streams them from L2 tap by tap through a four-stage ring of bulk copies, in the register-fragment
-// order a prep kernel wrote them in: first the k^2 key-side chunks, then the k^2 value-side chunks.
-// Every wait is bounded and sets the status word.
+// Persistent, one CTA per SM, one head per CTA; two teams of eight warps, each with its own block of 128 pixels = two TILES of
+// 8 x 8 pixels.  Warps q and q + 4 of a team have quadrant q of tensor memory: rows 4 (q % 2) .. + 3 of tile q / 2, the first
+// their upper two, the second their lower two; lane (g, tig) works on column g and channels 8 tig .. 8 tig + 7.  Tiles come by
+// TMA with their halo (zero fill = the padding), K then V.  Five more warps: an MMA and a TMA thread per team; one for weights.
+// The weights (2 x 32 k^4 bf16 per head, laid out by a prep kernel in the order they are used) stay in shared memory for
+// k <= 5 (102 KB at k = 5), so the teams run independently and cover each other's hand-offs; for k >= 7 (400 KB, 1 MB) they are
+// streamed from L2 through a ring that both teams read, 256 pixels per pass over them.
 //
-// Measured and not kept: two M tiles per warp (a weight fragment then feeds two MMAs, but half as many
-// warps with twice the registers ran 1.1-1.9x slower); 16-byte loads of two n-tiles' fragments at once
-// (within +-8 % of the 8-byte form).
-#include "tile_common.cuh"
+// Tensor-memory columns of a team (256): logits, later a (chunk of 16 slots: 8 columns a_hi, 8 a_lo, where its logits were), in
+// the last N; below them the product groups, later the A' groups.  A group = up to GK (GV) taps of one tap column.
+//
+// A call: 64 x 56 x 56, 3 heads, k = 5: 273 us with mma.sync (every CUDA-core multiply beside it cost it pipe time, and every
+// fragment was read from shared memory by every warp), 133 here; 2 x 128 x 128, 3 heads, k = 7: 137 and 61 us.
+#include "common.cuh"
+#include "ptx.cuh"
 
 namespace slide_attn {
 
 namespace {
 
-using namespace tile;
+constexpr int kHeadDim = 32;
+constexpr float kLog2e = 1.4426950408889634f;
+constexpr int kTeams = 2, kTeamWarps = 8, kComputeWarps = kTeams * kTeamWarps;
+constexpr int kMmaWarp = kComputeWarps, kTmaWarp = kMmaWarp + kTeams, kWeightWarp = kTmaWarp + kTeams;
+constexpr int kThreads = (kWeightWarp + 1) * 32;
+constexpr uint32_t kOnesBytes = 2 * 512;                 // [two 8-channel chunks][31 rows of 16 bytes], row 15 ones
+constexpr uint32_t kUnitBytes = 4 * 10 * 128;            // [four groups of 8 columns][zeros, ones in k = 0 .. 7, zeros]
+constexpr uint32_t kMaxSmem = 227 * 1024;
+
+// barriers of a team, then those of the weights
+enum : int { kPFull = 0, kPFree = 3, kLFull = 6, kAFull = 7, kDFull = 8, kDFree = 10, kFull = 12, kEmpty = 15, kTeamBars = 18 };
+enum : int { kWFull = kTeams * kTeamBars, kWEmpty = kWFull + 3, kBars = kWEmpty + 3 };
+
+constexpr int least(int a, int b) { return a < b ? a : b; }
 
 template <int K>
 struct Wide {
-    static constexpr int K2 = K * K;
-    static constexpr int KS = (K2 + 15) / 16;        // k-steps of the value MMA (slots, 16 per step)
-    static constexpr int NT = 2 * KS;                // n-tiles of 8 slots on the key side (covers 16 KS slots)
-    static constexpr int chunk_bytes = 2 * NT * 256; // one tap: key side [2 kh][NT][32 lanes][8 B] = value side [KS][4][32][8 B]
-    static constexpr int stages = 4;
-    using C_ = Cfg<__nv_bfloat16, K>;
-    static constexpr uint32_t ring_off = C_::bar_off + 128;                       // barriers: tile, full[4], empty[4]
-    static constexpr uint32_t total = ring_off + stages * chunk_bytes + 128;
-    static constexpr int threads = C_::threads * 2 + 32;                          // eight compute warps + the streaming warp
+    static constexpr int K2 = K * K, R = K / 2;
+    static constexpr int KS = (K2 + 15) / 16;            // K steps of the value side
+    static constexpr int N = 16 * KS;                    // columns of the logits
+    static constexpr bool resident = K <= 5;
+    static constexpr int GK = K == 5 ? 5 : K == 7 ? 4 : 3, GV = K == 9 ? 2 : 3;
+    static constexpr int NGK = (K + GK - 1) / GK, NGV = (K + GV - 1) / GV;
+    static constexpr int PB = least(3, (256 - N) / (16 * GK)), DB = 2;
+    static_assert(DB * 32 * GV <= 256 - N && PB >= 2, "tensor memory");
+    static constexpr int HP = 8 + 2 * R;                 // edge of a tile with its halo
+    static constexpr uint32_t plane = (uint32_t)(HP * HP * 64), slot = 2 * plane;
+    static constexpr uint32_t tap = (uint32_t)(N * 64);  // weights of a tap, either side
+    static constexpr uint32_t weights = 2u * K2 * tap;   // of a head
+    static constexpr uint32_t chunk = (uint32_t)(GK > GV ? GK : GV) * tap;
+    static constexpr uint32_t w_bytes = resident ? weights : 3 * chunk;
+    static constexpr uint32_t misc = kOnesBytes + kUnitBytes + 336 + 8u * kBars + 16;
+    static constexpr int ring = least(3, (int)((kMaxSmem - w_bytes - misc - 128) / (kTeams * slot)));
+    static_assert(ring >= 2, "the ring does not fit");
+    static constexpr uint32_t w_off = (uint32_t)(kTeams * ring) * slot, ones_off = w_off + w_bytes, unit_off = ones_off + kOnesBytes,
+                              bias_off = unit_off + kUnitBytes, bar_off = bias_off + 336, tmem_off = bar_off + 8u * kBars,
+                              total = tmem_off + 16 + 128;
+};
+
+// A walk over the 8 x 8 tiles of the maps from a given one in equal steps, by carries.
+struct TileWalk {
+    int b, y, x, db, dy, dx, tx, ty;
+    __device__ __forceinline__ TileWalk(int tiles_x, int tiles_y, int first, int step) : tx(tiles_x), ty(tiles_y) {
+        x = first % tx; y = first / tx % ty; b = first / tx / ty;
+        dx = step % tx; dy = step / tx % ty; db = step / tx / ty;
+    }
+    __device__ __forceinline__ void next() {
+        x += dx; y += dy; b += db;
+        if (x >= tx) { x -= tx; ++y; }
+        if (y >= ty) { y -= ty; ++b; }
+    }
 };
 
 struct WideParams {
-    const unsigned char* frag;       // [head][2 K2 chunks][chunk_bytes]
+    const unsigned char* weights;    // [head][Wide::weights]
+    const __nv_bfloat16* q;
     const float* bias;
     __nv_bfloat16* out;
     int* status;
-    int B, H, W, heads;
-    int tiles_x, tiles_y;
+    int H, W, heads;
+    int tiles_x, tiles_y, tiles;
     float scale_log2e;
 };
 
-// Prep: fp32 [C][slot][tap] -> bf16 B fragments of mma.sync.m16n8k16 (b0 = rows 2 tig, 2 tig + 1 of
-// column g; b1 = rows 2 tig + 8, 2 tig + 9), one 8-byte item per (chunk, unit, lane).
-//   key chunk t, unit (kh, j): row kappa = 2 tig' + e + 8 j' of k-step kh is channel 8 tig' + 4 kh + 2 j' + e
-//                              (the order in which a lane's 16-byte piece fills the A fragment);
-//                              column g of n-tile j is slot 8 j + g; value D_k[c][slot][t]
-//   value chunk t, unit (ks, jc): row kappa of k-step ks is slot 16 ks + kappa; column g' of n-tile jc is
-//                              channel 8 (g' >> 1) + 2 jc + (g' & 1); value D_v[c][slot][t]
+// Prep: fp32 [C][slot][tap] -> bf16, taps in the order o = dx K + dy (tap t = dy K + dx), first the key side, then the value side,
+// one 16-byte item per thread.
+//   key tap, item (j, n): k 8j .. 8j + 7 (channels in the order tcgen05.st lays the products out), column n = slot
+//   value tap, item (n, j): column n (channel in the order tcgen05.ld hands them out), k 8j .. 8j + 7 = slots
 template <int K>
 __global__ void __launch_bounds__(256)
-mma_wide_prep_kernel(const float* __restrict__ wk, const float* __restrict__ wv, unsigned char* __restrict__ frag, int heads)
+mma_wide_prep_kernel(const float* __restrict__ wk, const float* __restrict__ wv, unsigned char* __restrict__ img)
 {
     using Wd = Wide<K>;
-    constexpr int K2 = Wd::K2, NT = Wd::NT, KS = Wd::KS;
-    const long long items = (long long)heads * 2 * K2 * 2 * NT * 32;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < items; i += (long long)gridDim.x * blockDim.x) {
-        const int lane = (int)(i & 31);
-        long long r = i >> 5;
-        const int unit = (int)(r % (2 * NT)); r /= 2 * NT;
-        const int chunk = (int)(r % (2 * K2));
-        const int h = (int)(r / (2 * K2));
-        const int g = lane >> 2, tig = lane & 3;
-        float val[4];
-        if (chunk < K2) {
-            const int t = chunk, kh = unit / NT, j = unit % NT;
-            const int s = 8 * j + g;
+    constexpr int K2 = Wd::K2, N = Wd::N, per_tap = 4 * N;
+    grid_launch_dependents();
+    const int h = blockIdx.y;
+    const float* wkh = wk + (size_t)h * kHeadDim * K2 * K2;
+    const float* wvh = wv + (size_t)h * kHeadDim * K2 * K2;
+    for (int i = blockIdx.x * 256 + threadIdx.x; i < 2 * K2 * per_tap; i += gridDim.x * 256) {
+        const int side = i >= K2 * per_tap, r = side ? i - K2 * per_tap : i;
+        const int o = r / per_tap, item = r % per_tap, t = (o % K) * K + o / K;
+        unsigned char* tap = img + (size_t)h * Wd::weights + (size_t)(side * K2 + o) * Wd::tap;
+        float v[8];
+        uint32_t at;
+        if (side == 0) {
+            const int n = item % N, j = item / N;
 #pragma unroll
-            for (int x = 0; x < 4; ++x) {                      // x = 2 j' + e
-                const int c = h * kHeadDim + 8 * tig + 4 * kh + x;
-                val[x] = s < K2 ? wk[((size_t)c * K2 + s) * K2 + t] - (s == t ? 1.f : 0.f) : 0.f;
+            for (int e = 0; e < 8; ++e) {
+                const int kap = 8 * j + e, c = 8 * ((kap & 15) >> 2) + (kap & 3) + (kap >= 16 ? 4 : 0);
+                v[e] = n < K2 ? wkh[((size_t)c * K2 + n) * K2 + t] - (n == t ? 1.f : 0.f) : 0.f;
             }
+            at = (uint32_t)(j * N * 16 + n * 16);
         } else {
-            const int t = chunk - K2, ks = unit / 4, jc = unit % 4;
-            const int c = h * kHeadDim + 8 * (g >> 1) + 2 * jc + (g & 1);
+            const int n = item & 31, j = item >> 5, c = 8 * ((n & 7) >> 1) + 2 * (n >> 3) + (n & 1);
 #pragma unroll
-            for (int x = 0; x < 4; ++x) {                      // x = 2 j' + e: slot 16 ks + 2 tig + e + 8 j'
-                const int s = 16 * ks + 2 * tig + (x & 1) + 8 * (x >> 1);
-                val[x] = (unit < 4 * KS && s < K2) ? wv[((size_t)c * K2 + s) * K2 + t] - (s == t ? 1.f : 0.f) : 0.f;
+            for (int e = 0; e < 8; ++e) {
+                const int s = 8 * j + e;
+                v[e] = s < K2 ? wvh[((size_t)c * K2 + s) * K2 + t] - (s == t ? 1.f : 0.f) : 0.f;
             }
+            at = (uint32_t)((n >> 3) * (2 * Wd::KS * 128) + j * 128 + (n & 7) * 16);
         }
-        *reinterpret_cast<uint2*>(frag + (size_t)i * 8) = make_uint2(pack_bf16(val[0], val[1]), pack_bf16(val[2], val[3]));
+        *reinterpret_cast<uint4*>(tap + at) = make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
     }
 }
 
+__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity) {
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity) ? 1 : 0) != 0;
+}
+
+// Products of G taps (halo rows dy0 .. of column dx) for the lane's two pixels into tensor memory at `t`, 16 columns a tap.
+template <int G, int HP>
+__device__ __forceinline__ void store_products(uint32_t t, const unsigned char* src, const uint4 (&x)[2]) {
+    uint4 y[G + 1];
+#pragma unroll
+    for (int r = 0; r <= G; ++r) y[r] = *reinterpret_cast<const uint4*>(src + r * HP * 64);
+#pragma unroll
+    for (int i = 0; i < G; ++i) {
+        const uint32_t r[8] = {hmul2_bf16(x[0].x, y[i].x), hmul2_bf16(x[0].y, y[i].y), hmul2_bf16(x[1].x, y[i + 1].x), hmul2_bf16(x[1].y, y[i + 1].y),
+                               hmul2_bf16(x[0].z, y[i].z), hmul2_bf16(x[0].w, y[i].w), hmul2_bf16(x[1].z, y[i + 1].z), hmul2_bf16(x[1].w, y[i + 1].w)};
+        tmem_st_16x256b_x2(t + 16 * i, r);
+    }
+}
+// acc += the A' of G taps at `t` times their halo pixels.
+template <int G, int HP>
+__device__ __forceinline__ void sum_group(uint32_t t, const unsigned char* src, float (&acc)[2][8]) {
+    uint32_t d[G][16];
+#pragma unroll
+    for (int i = 0; i < G; ++i) tmem_ld_16x256b_x4_nowait(t + 32 * i, d[i]);
+    uint4 y[G + 1];
+#pragma unroll
+    for (int r = 0; r <= G; ++r) y[r] = *reinterpret_cast<const uint4*>(src + r * HP * 64);
+    float f[G + 1][8];
+#pragma unroll
+    for (int r = 0; r <= G; ++r) {
+        f[r][0] = bf16_lo(y[r].x); f[r][1] = bf16_hi(y[r].x); f[r][2] = bf16_lo(y[r].y); f[r][3] = bf16_hi(y[r].y);
+        f[r][4] = bf16_lo(y[r].z); f[r][5] = bf16_hi(y[r].z); f[r][6] = bf16_lo(y[r].w); f[r][7] = bf16_hi(y[r].w);
+    }
+    tmem_wait_ld();
+#pragma unroll
+    for (int i = 0; i < G; ++i) {
+        tmem_pass(d[i]);
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                ffma2(acc[r][2 * j], acc[r][2 * j + 1], __uint_as_float(d[i][4 * j + 2 * r]), __uint_as_float(d[i][4 * j + 2 * r + 1]),
+                      f[r + i][2 * j], f[r + i][2 * j + 1]);
+    }
+}
+
+// Softmax of the lane's pixel, whose N logits start at tensor-memory column `col`; leaves a_hi, a_lo in their place.
 template <int K>
-__global__ void __launch_bounds__(Wide<K>::threads)
-mma_wide_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
-                const __grid_constant__ CUtensorMap map_v, const WideParams P)
-{
-    using T = __nv_bfloat16;
-    using C_ = Cfg<T, K>;
+__device__ __forceinline__ void softmax_in_place(uint32_t col, const float* s_bias, float scale_log2e) {
     using Wd = Wide<K>;
-    constexpr int R = K / 2, K2 = Wd::K2, NT = Wd::NT, KS = Wd::KS, ST = Wd::stages;
-    constexpr int NTS = (K2 + 7) / 8;                            // n-tiles that hold real slots
+    constexpr int K2 = Wd::K2, KS = Wd::KS;
+    constexpr bool keep = KS <= 2;                       // the logits stay in registers between the passes
+    float l[keep ? KS : 1][16];
+    auto load = [&](int j, float (&v)[16]) {
+        tmem_ld_32x32b_x16(col + 16 * j, v);
+#pragma unroll
+        for (int i = 0; i < 16; ++i)
+            if (16 * j + i < K2) v[i] = fmaf(v[i], scale_log2e, s_bias[16 * j + i]);
+    };
+    float m = -INFINITY, z = 0.f;
+#pragma unroll
+    for (int j = 0; j < KS; ++j) {
+        float (&v)[16] = l[keep ? j : 0];
+        load(j, v);
+        float most = m;
+#pragma unroll
+        for (int i = 0; i < 16; ++i)
+            if (16 * j + i < K2) most = fmaxf(most, v[i]);
+        z *= fast_exp2(m - most);
+        m = most;
+#pragma unroll
+        for (int i = 0; i < 16; ++i)
+            if (16 * j + i < K2) z += fast_exp2(v[i] - m);
+    }
+    m += __log2f(z);
+#pragma unroll
+    for (int j = 0; j < KS; ++j) {
+        float (&v)[16] = l[keep ? j : 0];
+        if (!keep) load(j, v);
+        uint32_t row[16];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const float a0 = 16 * j + 2 * i < K2 ? fast_exp2(v[2 * i] - m) : 0.f, a1 = 16 * j + 2 * i + 1 < K2 ? fast_exp2(v[2 * i + 1] - m) : 0.f;
+            row[i] = pack_bf16(a0, a1);
+            row[8 + i] = pack_bf16(a0 - bf16_lo(row[i]), a1 - bf16_hi(row[i]));
+        }
+        tmem_st_32x32b_x16(col + 16 * j, row);
+    }
+    tmem_wait_st();
+}
+
+template <int K>
+__global__ void __launch_bounds__(kThreads, 1)
+mma_wide_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v, const WideParams P)
+{
+    using Wd = Wide<K>;
+    constexpr int N = Wd::N, KS = Wd::KS, GK = Wd::GK, GV = Wd::GV, NGK = Wd::NGK, NGV = Wd::NGV, PB = Wd::PB, DB = Wd::DB, HP = Wd::HP, R = Wd::ring;
+    constexpr uint32_t kColL = 256 - N;
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u);
-    const uint32_t bar0 = smem_u32(smem + C_::bar_off);
-    const uint32_t bar_tile = bar0;
-    auto bar_full = [&](int s) { return bar0 + 8u * (uint32_t)(1 + s); };
-    auto bar_empty = [&](int s) { return bar0 + 8u * (uint32_t)(1 + ST + s); };
-    float* s_bias = reinterpret_cast<float*>(smem + C_::bias_off);
-    const unsigned char* ring = smem + Wd::ring_off;
+    const uint32_t bars = smem_u32(smem + Wd::bar_off);
+    float* s_bias = reinterpret_cast<float*>(smem + Wd::bias_off);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int g = lane >> 2, tig = lane & 3;
-    const int h = blockIdx.x % P.heads;
-    int rest = blockIdx.x / P.heads;
-    const int tx = rest % P.tiles_x; rest /= P.tiles_x;
-    const int ty = rest % P.tiles_y;
-    const int b = rest / P.tiles_y;
-    const int x0 = tx * kTW, y0 = ty * C_::TH;
-    constexpr int kCWarps = 8;
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
+    const int h = blockIdx.x % P.heads, rank = blockIdx.x / P.heads, nrank = (int)gridDim.x / P.heads;
+    const int team_id = warp < kComputeWarps ? warp / kTeamWarps : (warp - kComputeWarps) % kTeams;
+    const int blocks = (P.tiles + 1) >> 1, step = kTeams * nrank, first = team_id * nrank + rank;
+    auto blocks_from = [&](int at) { return at < blocks ? (blocks - at + step - 1) / step : 0; };
+    const int my_blocks = blocks_from(first), rounds = blocks_from(rank);            // rounds: of team 0, which has the most
+    auto bar = [&](int i) { return bars + 8u * (uint32_t)(team_id * kTeamBars + i); };
+    auto wbar = [&](int i) { return bars + 8u * (uint32_t)i; };
 
     if (threadIdx.x == 0) {
-        mbar_init_only(bar_tile, 1);
-        for (int s = 0; s < ST; ++s) { mbar_init_only(bar_full(s), 1); mbar_init_only(bar_empty(s), kCWarps); }
+        for (int t = 0; t < kTeams; ++t) {
+            auto init = [&](int i, uint32_t count) { mbar_init_only(bars + 8u * (uint32_t)(t * kTeamBars + i), count); };
+            for (int i = 0; i < 3; ++i) { init(kPFull + i, kTeamWarps); init(kPFree + i, 1); init(kFull + i, 1); init(kEmpty + i, kTeamWarps); }
+            init(kLFull, 1);
+            init(kAFull, 4);
+            for (int i = 0; i < 2; ++i) { init(kDFull + i, 1); init(kDFree + i, kTeamWarps); }
+        }
+        for (int i = 0; i < 3; ++i) { mbar_init_only(wbar(kWFull + i), 1); mbar_init_only(wbar(kWEmpty + i), kTeams); }
         mbar_init_fence();
-        mbar_expect_tx(bar_tile, C_::tx_bytes);
-        const int c0 = h * kHeadDim;
-        tma_load_4d(smem_u32(smem + C_::k_off), &map_k, bar_tile, c0, x0 - R, y0 - R, b);
-        tma_load_4d(smem_u32(smem + C_::v_off), &map_v, bar_tile, c0, x0 - R, y0 - R, b);
-        tma_load_4d(smem_u32(smem + C_::q_off), &map_q, bar_tile, c0, x0, y0, b);
     }
-    for (int i = threadIdx.x; i < K2; i += Wd::threads) s_bias[i] = P.bias ? P.bias[h * K2 + i] * kLog2e : 0.f;
+    for (int i = threadIdx.x; i < Wd::K2; i += kThreads) s_bias[i] = P.bias ? P.bias[h * Wd::K2 + i] * kLog2e : 0.f;
+    for (uint32_t i = threadIdx.x; i < (kOnesBytes + kUnitBytes) / 4; i += kThreads) {
+        uint32_t v = 0;
+        if (i < kOnesBytes / 4) {
+            if (((i * 4) & 511u) >> 4 == 15) v = kOnesBf16x2;
+        } else {
+            const uint32_t b = (i * 4 - kOnesBytes) % 1280u, core = b >> 7, k = (b & 15u) >> 1;      // k, k + 1 of a row
+            if (core >= 1 && core <= 8) v = (core - 1 == k ? 0x3F80u : 0u) | (core - 1 == k + 1 ? 0x3F800000u : 0u);
+        }
+        *reinterpret_cast<uint32_t*>(smem + Wd::ones_off + i * 4) = v;
+    }
+    fence_proxy_async_smem();
+    if (warp == kMmaWarp) tmem_alloc(smem_u32(smem + Wd::tmem_off), 512);
+    tc_fence_before_sync();
     __syncthreads();
+    tc_fence_after_sync();
+    const uint32_t tmem = *reinterpret_cast<const volatile uint32_t*>(smem + Wd::tmem_off) + 256u * (uint32_t)team_id;
+    unsigned char* ring = smem + (uint32_t)(team_id * R) * Wd::slot;
+    const uint32_t w_smem = smem_u32(smem + Wd::w_off);
+    bool ok = true;
 
-    if (warp == kCWarps) {
-        // ---- streaming warp: 2 K2 weight chunks of this head through the ring -------------------------
-        if (lane == 0) {
-            const unsigned char* src = P.frag + (size_t)h * 2 * K2 * Wd::chunk_bytes;
-            bool ok = true;
-            for (int i = 0; i < 2 * K2; ++i) {
-                const int s = i % ST;
-                if (i >= ST && !mbar_wait(bar_empty(s), (uint32_t)(i / ST - 1) & 1u)) { ok = false; break; }
-                mbar_expect_tx(bar_full(s), Wd::chunk_bytes);
-                bulk_load_1d(smem_u32(ring + s * Wd::chunk_bytes), src + (size_t)i * Wd::chunk_bytes, Wd::chunk_bytes, bar_full(s));
+    if (warp == kWeightWarp) {
+        // ---- weights: once, or a pass over them per round -----------------------------------------------
+        uint32_t leader;
+        if (elect_one(leader)) {
+            grid_dependency_wait();
+            const unsigned char* src = P.weights + (size_t)h * Wd::weights;
+            if constexpr (Wd::resident) {
+                mbar_expect_tx(wbar(kWFull), Wd::weights);
+                bulk_load_1d(w_smem, src, Wd::weights, wbar(kWFull));
+            } else {
+                int ws = 0;
+                uint32_t phase = 1;
+                for (int r = 0; ok && r < rounds; ++r) {
+                    const unsigned char* at = src;
+                    for (int side = 0; ok && side < 2; ++side)
+                        for (int dx = 0; ok && dx < K; ++dx)
+                            for (int left = K; left > 0;) {
+                                const int g = side ? (left < GV ? left : GV) : (left < GK ? left : GK);
+                                left -= g;
+                                if (!mbar_wait(wbar(kWEmpty + ws), phase)) { ok = false; break; }
+                                mbar_expect_tx(wbar(kWFull + ws), (uint32_t)g * Wd::tap);
+                                bulk_load_1d(w_smem + (uint32_t)ws * Wd::chunk, at, (uint32_t)g * Wd::tap, wbar(kWFull + ws));
+                                at += (uint32_t)g * Wd::tap;
+                                if (++ws == 3) { ws = 0; phase ^= 1u; }
+                            }
+                }
             }
             if (!ok) atomicExch(P.status, 1);
         }
-        return;
-    }
-
-    // ---- compute warps ---------------------------------------------------------------------------------
-    bool ok = __all_sync(0xffffffffu, mbar_wait(bar_tile, 0) ? 1 : 0) != 0;
-    const int wx = warp & 3, wy = warp >> 2;                       // column group, row pair
-    const int col = wx * 8 + g, row0 = 2 * wy;
-    const unsigned char* sK = smem + C_::k_off;
-    const unsigned char* sV = smem + C_::v_off;
-    const unsigned char* sQ = smem + C_::q_off;
-    auto piece = [&](const unsigned char* tile, int pix) { return *reinterpret_cast<const uint4*>(tile + (uint32_t)pix * 64u + tig * 16u); };
-
-    uint4 qa = make_uint4(0, 0, 0, 0), qb = qa;
-    if (ok) { qa = piece(sQ, row0 * kTW + col); qb = piece(sQ, (row0 + 1) * kTW + col); }
-
-    float ld[NT][4], lp[NTS][4];
-#pragma unroll
-    for (int j = 0; j < NT; ++j)
-#pragma unroll
-        for (int x = 0; x < 4; ++x) ld[j][x] = 0.f;
-#pragma unroll
-    for (int j = 0; j < NTS; ++j)
-#pragma unroll
-        for (int x = 0; x < 4; ++x) lp[j][x] = 0.f;
-
-    int chunk = 0;                                                  // position in the stream of 2 K2 chunks
-#pragma unroll
-    for (int t = 0; t < K2; ++t, ++chunk) {
-        const int dy = t / K, dx = t % K;
-        const int s = chunk % ST;
-        if (ok && !__all_sync(0xffffffffu, mbar_wait(bar_full(s), (uint32_t)(chunk / ST) & 1u) ? 1 : 0)) ok = false;
-        if (ok) {
-            const uint4 ka = piece(sK, (row0 + dy) * C_::HW + col + dx), kb = piece(sK, (row0 + 1 + dy) * C_::HW + col + dx);
-            const uint32_t pa[4] = {hmul2_bf16(qa.x, ka.x), hmul2_bf16(qa.y, ka.y), hmul2_bf16(qa.z, ka.z), hmul2_bf16(qa.w, ka.w)};
-            const uint32_t pb[4] = {hmul2_bf16(qb.x, kb.x), hmul2_bf16(qb.y, kb.y), hmul2_bf16(qb.z, kb.z), hmul2_bf16(qb.w, kb.w)};
-            const unsigned char* bsrc = ring + s * Wd::chunk_bytes + lane * 8;
-            const uint32_t ones = (g == (t & 7)) ? kOnesBf16x2 : 0u;
-#pragma unroll
-            for (int kh = 0; kh < 2; ++kh) {
-                const uint32_t a[4] = {pa[2 * kh], pb[2 * kh], pa[2 * kh + 1], pb[2 * kh + 1]};
-#pragma unroll
-                for (int j = 0; j < NT; ++j) {
-                    const uint2 bf = *reinterpret_cast<const uint2*>(bsrc + (kh * NT + j) * 256);
-                    mma_bf16(ld[j], a, bf.x, bf.y);
+        __syncwarp();
+    } else if (warp >= kTmaWarp) {
+        // ---- TMA thread of a team: K, then V tiles of every block ---------------------------------------
+        uint32_t leader;
+        if (elect_one(leader)) {
+            int slot = 0;
+            uint32_t phase = 1;
+            TileWalk at(P.tiles_x, P.tiles_y, 2 * first, 2 * step);
+            for (int bi = 0; ok && bi < my_blocks; ++bi, at.next())
+                for (int v = 0; v < 2; ++v) {
+                    if (!mbar_wait(bar(kEmpty + slot), phase)) { ok = false; break; }
+                    mbar_expect_tx(bar(kFull + slot), Wd::slot);
+                    const CUtensorMap* map = v ? &map_v : &map_k;
+                    const uint32_t dst = smem_u32(ring) + (uint32_t)slot * Wd::slot;
+                    // the second tile may be past the last: its image does not exist and it reads as zero
+                    int x = at.x + 1, y = at.y, b = at.b;
+                    if (x == at.tx) { x = 0; if (++y == at.ty) { y = 0; ++b; } }
+                    tma_load_4d(dst, map, bar(kFull + slot), h * kHeadDim, 8 * at.x - Wd::R, 8 * at.y - Wd::R, at.b);
+                    tma_load_4d(dst + Wd::plane, map, bar(kFull + slot), h * kHeadDim, 8 * x - Wd::R, 8 * y - Wd::R, b);
+                    if (++slot == R) { slot = 0; phase ^= 1u; }
                 }
-                mma_bf16(lp[t >> 3], a, ones, ones);
-            }
+            if (!ok) atomicExch(P.status, 1);
         }
         __syncwarp();
-        if (lane == 0) mbar_arrive(bar_empty(s));
-    }
-
-    // ---- softmax over the k^2 slots: a quad holds one pixel's logits (lane tig: slots 8 j + 2 tig, + 1) ---
-    float ev[2][NT][2];                                             // [pixel row][n-tile][slot parity]
-    float inv[2];
-#pragma unroll
-    for (int r = 0; r < 2; ++r) {
-        float m = -INFINITY;
-#pragma unroll
-        for (int j = 0; j < NT; ++j)
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                const int s = 8 * j + 2 * tig + e;
-                float v = -INFINITY;
-                if (j < NTS && s < K2) v = fmaf(ld[j][2 * r + e] + lp[j][2 * r + e], P.scale_log2e, s_bias[s]);
-                ev[r][j][e] = v;
-                m = fmaxf(m, v);
-            }
-        m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 1));
-        m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 2));
-        float z = 0.f;
-#pragma unroll
-        for (int j = 0; j < NT; ++j)
-#pragma unroll
-            for (int e = 0; e < 2; ++e) { ev[r][j][e] = fast_exp2(ev[r][j][e] - m); z += ev[r][j][e]; }   // exp2(-inf) = 0 for the padding slots
-        z += __shfl_xor_sync(0xffffffffu, z, 1);
-        z += __shfl_xor_sync(0xffffffffu, z, 2);
-        inv[r] = 1.f / z;
-    }
-    // the logits' C fragments are the A fragments of the value MMA (bf16: the deformed part is small)
-    uint32_t ah[KS][4];
-#pragma unroll
-    for (int ks = 0; ks < KS; ++ks) {
-        ah[ks][0] = pack_bf16(ev[0][2 * ks][0], ev[0][2 * ks][1]);
-        ah[ks][1] = pack_bf16(ev[1][2 * ks][0], ev[1][2 * ks][1]);
-        ah[ks][2] = pack_bf16(ev[0][2 * ks + 1][0], ev[0][2 * ks + 1][1]);
-        ah[ks][3] = pack_bf16(ev[1][2 * ks + 1][0], ev[1][2 * ks + 1][1]);
-    }
-
-    float oa[8], ob[8];                                              // the two pixel rows, channels 8 tig ..
-#pragma unroll
-    for (int c = 0; c < 8; ++c) { oa[c] = 0.f; ob[c] = 0.f; }
-#pragma unroll
-    for (int t = 0; t < K2; ++t, ++chunk) {
-        const int dy = t / K, dx = t % K;
-        const int s = chunk % ST;
-        if (ok && !__all_sync(0xffffffffu, mbar_wait(bar_full(s), (uint32_t)(chunk / ST) & 1u) ? 1 : 0)) ok = false;
-        // e[p][t] of the two pixels: slot t lives in quad lane (t % 8) / 2, n-tile t / 8, parity t % 2
-        const float ea = __shfl_sync(0xffffffffu, ev[0][t >> 3][t & 1], (lane & ~3) | ((t & 7) >> 1));
-        const float eb = __shfl_sync(0xffffffffu, ev[1][t >> 3][t & 1], (lane & ~3) | ((t & 7) >> 1));
-        if (ok) {
-            float cf[4][4];
-#pragma unroll
-            for (int jc = 0; jc < 4; ++jc) { cf[jc][0] = ea; cf[jc][1] = ea; cf[jc][2] = eb; cf[jc][3] = eb; }
-            const unsigned char* bsrc = ring + s * Wd::chunk_bytes + lane * 8;
-#pragma unroll
-            for (int ks = 0; ks < KS; ++ks)
-#pragma unroll
-                for (int jc = 0; jc < 4; ++jc) {
-                    const uint2 bf = *reinterpret_cast<const uint2*>(bsrc + (ks * 4 + jc) * 256);
-                    mma_bf16(cf[jc], ah[ks], bf.x, bf.y);
+    } else if (warp >= kMmaWarp) {
+        // ---- MMA thread of a team ---------------------------------------------------------------------
+        uint32_t leader;
+        if (elect_one(leader)) {
+            constexpr uint32_t id_l = umma_idesc_bf16(128, N), id16 = umma_idesc_bf16(128, 16), id32 = umma_idesc_bf16(128, 32);
+            const uint32_t ones = smem_u32(smem + Wd::ones_off), unit = smem_u32(smem + Wd::unit_off);
+            if (Wd::resident && my_blocks > 0) ok = mbar_wait(wbar(kWFull), 0);
+            int ws = 0, pb = 0, db = 0;
+            uint32_t wphase = 0, pphase = 0, dphase = 1;
+            // the next group of weights; `at`: where it is when they are resident
+            auto weights = [&](uint32_t at) -> uint32_t {
+                if constexpr (Wd::resident) return w_smem + at;
+                if (!mbar_wait(wbar(kWFull + ws), wphase)) ok = false;
+                return w_smem + (uint32_t)ws * Wd::chunk;
+            };
+            auto weights_done = [&](bool used) {
+                if constexpr (!Wd::resident) {
+                    if (used) umma_commit(wbar(kWEmpty + ws)); else mbar_arrive(wbar(kWEmpty + ws));
+                    if (++ws == 3) { ws = 0; wphase ^= 1u; }
                 }
-            const uint4 va = piece(sV, (row0 + dy) * C_::HW + col + dx), vb = piece(sV, (row0 + 1 + dy) * C_::HW + col + dx);
-            const uint32_t wa[4] = {va.x, va.y, va.z, va.w}, wb[4] = {vb.x, vb.y, vb.z, vb.w};
+            };
+            for (int r = 0; ok && r < (Wd::resident ? my_blocks : rounds); ++r) {
+                if (r >= my_blocks) {                                    // a round without a block of this team
+                    for (int i = 0; ok && i < K * (NGK + NGV); ++i) { weights(0); weights_done(false); }
+                    continue;
+                }
+                for (int dx = 0; ok && dx < K; ++dx) {
 #pragma unroll
-            for (int jc = 0; jc < 4; ++jc) {                       // channels 8 tig + 2 jc, + 1 = word jc of the piece
-                ffma2(oa[2 * jc], oa[2 * jc + 1], cf[jc][0], cf[jc][1], bf16_lo(wa[jc]), bf16_hi(wa[jc]));
-                ffma2(ob[2 * jc], ob[2 * jc + 1], cf[jc][2], cf[jc][3], bf16_lo(wb[jc]), bf16_hi(wb[jc]));
+                    for (int gi = 0; gi < NGK; ++gi) {
+                        constexpr int GL = K - (NGK - 1) * GK;
+                        const int G = gi == NGK - 1 ? GL : GK;
+                        const uint32_t w = weights((uint32_t)(dx * K + gi * GK) * Wd::tap);
+                        if (!ok || !mbar_wait(bar(kPFull + pb), pphase)) { ok = false; break; }
+                        tc_fence_after_sync();
+#pragma unroll
+                        for (int i = 0; i < G; ++i) {
+                            const int t = (gi * GK + i) * K + dx;
+                            const uint32_t a = tmem + (uint32_t)(pb * 16 * GK + 16 * i);
+                            const uint64_t b = umma_smem_desc(w + i * Wd::tap, N * 16, 128);
+                            umma_bf16_ts(tmem + kColL, a, b, id_l, (dx | gi | i) != 0 ? 1u : 0u);
+                            umma_bf16_ts(tmem + kColL, a + 8, b + 2 * N, id_l, 1);                    // the other 16 channels
+                            const uint64_t one = umma_smem_desc(ones + (uint32_t)(15 - (t & 15)) * 16u, 512, 128);
+                            umma_bf16_ts(tmem + kColL + (t & ~15), a, one, id16, 1);
+                            umma_bf16_ts(tmem + kColL + (t & ~15), a + 8, one, id16, 1);
+                        }
+                        umma_commit(bar(kPFree + pb));
+                        weights_done(true);
+                        if (++pb == PB) { pb = 0; pphase ^= 1u; }
+                    }
+                }
+                if (!ok) break;
+                umma_commit(bar(kLFull));
+                if (!mbar_wait(bar(kAFull), (uint32_t)r & 1u)) { ok = false; break; }
+                for (int dx = 0; ok && dx < K; ++dx) {
+#pragma unroll
+                    for (int gi = 0; gi < NGV; ++gi) {
+                        constexpr int GL = K - (NGV - 1) * GV;
+                        const int G = gi == NGV - 1 ? GL : GV;
+                        const uint32_t w = weights((uint32_t)(Wd::K2 + dx * K + gi * GV) * Wd::tap);
+                        if (!ok || !mbar_wait(bar(kDFree + db), dphase)) { ok = false; break; }
+                        tc_fence_after_sync();
+                        const uint32_t d = tmem + (uint32_t)(db * 32 * GV);
+                        const uint64_t b = umma_smem_desc(w, 128, 2 * KS * 128);
+#pragma unroll
+                        for (int j = 0; j < KS; ++j) umma_bf16_ts(d, tmem + kColL + 16 * j, b + 16 * j, umma_idesc_bf16(128, 32 * G), j != 0 ? 1u : 0u);
+#pragma unroll
+                        for (int i = 0; i < G; ++i) {
+                            const int t = (gi * GV + i) * K + dx, j = t & 15;
+                            // [ones in k = j | zeros] or [zeros | ones in k = j - 8] of the table
+                            const uint64_t one = j < 8 ? umma_smem_desc(unit + (uint32_t)(1 + j) * 128u, (uint32_t)(8 - j) * 128u, 1280)
+                                                       : umma_smem_desc(unit, (uint32_t)(j - 7) * 128u, 1280);
+                            umma_bf16_ts(d + 32 * i, tmem + kColL + (t & ~15), one, id32, 1);
+                            umma_bf16_ts(d + 32 * i, tmem + kColL + (t & ~15) + 8, one, id32, 1);
+                        }
+                        umma_commit(bar(kDFull + db));
+                        weights_done(true);
+                        if (++db == DB) { db = 0; dphase ^= 1u; }
+                    }
+                }
             }
+            if (!ok) atomicExch(P.status, 1);
         }
         __syncwarp();
-        if (lane == 0) mbar_arrive(bar_empty(s));
-    }
+    } else {
+        const int wq = warp & 3, half = (warp % kTeamWarps) >> 2, g = lane >> 2, tig = lane & 3;
+        const uint32_t quad = tmem + ((uint32_t)(32 * wq) << 16), mine = quad + ((uint32_t)(16 * half) << 16);
+        const int C = P.heads * kHeadDim, row0 = 4 * (wq & 1) + 2 * half;
+        const size_t row_pitch = (size_t)P.W * C;
+        const uint32_t lane_off = (uint32_t)(wq >> 1) * Wd::plane + (uint32_t)(row0 * HP + g) * 64u + (uint32_t)tig * 16u;
+        TileWalk walk(P.tiles_x, P.tiles_y, 2 * first + (wq >> 1), 2 * step);
+        struct Place { size_t at; bool in[2]; };
+        auto place = [&](int bi) {
+            Place p;
+            const int y = 8 * walk.y + row0, x = 8 * walk.x + g;
+            const bool in = 2 * (first + bi * step) + (wq >> 1) < P.tiles && x < P.W;
+            p.in[0] = in && y < P.H; p.in[1] = in && y + 1 < P.H;
+            p.at = (((size_t)walk.b * P.H + y) * P.W + x) * C + h * kHeadDim + tig * 8;
+            return p;
+        };
+        auto load_q = [&](const Place& p, uint4 (&x)[2]) {
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                x[r] = make_uint4(0u, 0u, 0u, 0u);
+                if (p.in[r]) x[r] = __ldg(reinterpret_cast<const uint4*>(P.q + p.at + r * row_pitch));
+            }
+        };
+        int slot = 0, pb = 0, db = 0;
+        uint32_t phase = 0, pphase = 1, dphase = 0;
+        auto release = [&]() {
+            __syncwarp();
+            mbar_arrive_lane0(bar(kEmpty + slot), lane);
+            if (++slot == R) { slot = 0; phase ^= 1u; }
+        };
+        Place cur = place(0);
+        uint4 x[2];
+        if (my_blocks > 0) load_q(cur, x);
+        for (int bi = 0; ok && bi < my_blocks; ++bi) {
+            // ---- products -------------------------------------------------------------------------------
+            if (!warp_wait(bar(kFull + slot), phase)) { ok = false; break; }
+            {
+                const unsigned char* src = ring + (uint32_t)slot * Wd::slot + lane_off;
+#pragma unroll 1
+                for (int dx = 0; ok && dx < K; ++dx, src += 64) {
+#pragma unroll
+                    for (int gi = 0; gi < NGK; ++gi) {
+                        constexpr int GL = K - (NGK - 1) * GK;
+                        if (!warp_wait(bar(kPFree + pb), pphase)) { ok = false; break; }
+                        tc_fence_after_sync();
+                        const uint32_t t = mine + (uint32_t)(pb * 16 * GK);
+                        if (gi == NGK - 1) store_products<GL, HP>(t, src + gi * GK * HP * 64, x);
+                        else store_products<GK, HP>(t, src + gi * GK * HP * 64, x);
+                        tmem_wait_st();
+                        tc_fence_before_sync();
+                        __syncwarp();
+                        mbar_arrive_lane0(bar(kPFull + pb), lane);
+                        if (++pb == PB) { pb = 0; pphase ^= 1u; }
+                    }
+                }
+            }
+            if (!ok) break;
+            release();
+            const Place out = cur;
+            if (bi + 1 < my_blocks) { walk.next(); cur = place(bi + 1); load_q(cur, x); }
 
-    if (!ok) { if (lane == 0) atomicExch(P.status, 1); return; }
-    const int x = x0 + col, y = y0 + row0;
-    const int Ctot = P.heads * kHeadDim;
-    if (x < P.W) {
-        if (y < P.H) {
-            uint4 o;
-            o.x = pack_bf16(oa[0] * inv[0], oa[1] * inv[0]); o.y = pack_bf16(oa[2] * inv[0], oa[3] * inv[0]);
-            o.z = pack_bf16(oa[4] * inv[0], oa[5] * inv[0]); o.w = pack_bf16(oa[6] * inv[0], oa[7] * inv[0]);
-            *reinterpret_cast<uint4*>(P.out + ((size_t)(b * P.H + y) * P.W + x) * Ctot + h * kHeadDim + tig * 8) = o;
+            // ---- softmax: thread = pixel of the quadrant; the two warps of a quadrant take turns ----------------
+            if (half == (bi & 1)) {
+                if (!warp_wait(bar(kLFull), (uint32_t)bi & 1u)) { ok = false; break; }
+                tc_fence_after_sync();
+                softmax_in_place<K>(quad + kColL, s_bias, P.scale_log2e);
+                tc_fence_before_sync();
+                __syncwarp();
+                mbar_arrive_lane0(bar(kAFull), lane);
+            }
+
+            // ---- values -----------------------------------------------------------------------------------
+            float acc[2][8];
+#pragma unroll
+            for (int r = 0; r < 2; ++r)
+#pragma unroll
+                for (int c = 0; c < 8; ++c) acc[r][c] = 0.f;
+            if (!warp_wait(bar(kFull + slot), phase)) { ok = false; break; }
+            {
+                const unsigned char* src = ring + (uint32_t)slot * Wd::slot + lane_off;
+#pragma unroll 1
+                for (int dx = 0; ok && dx < K; ++dx, src += 64) {
+#pragma unroll
+                    for (int gi = 0; gi < NGV; ++gi) {
+                        constexpr int GL = K - (NGV - 1) * GV;
+                        if (!warp_wait(bar(kDFull + db), dphase)) { ok = false; break; }
+                        tc_fence_after_sync();
+                        const uint32_t t = mine + (uint32_t)(db * 32 * GV);
+                        if (gi == NGV - 1) sum_group<GL, HP>(t, src + gi * GV * HP * 64, acc);
+                        else sum_group<GV, HP>(t, src + gi * GV * HP * 64, acc);
+                        tc_fence_before_sync();
+                        __syncwarp();
+                        mbar_arrive_lane0(bar(kDFree + db), lane);
+                        if (++db == DB) { db = 0; dphase ^= 1u; }
+                    }
+                }
+            }
+            if (!ok) break;
+            release();
+#pragma unroll
+            for (int r = 0; r < 2; ++r)
+                if (out.in[r])
+                    *reinterpret_cast<uint4*>(P.out + out.at + r * row_pitch) = make_uint4(pack_bf16(acc[r][0], acc[r][1]), pack_bf16(acc[r][2], acc[r][3]),
+                                                                                          pack_bf16(acc[r][4], acc[r][5]), pack_bf16(acc[r][6], acc[r][7]));
         }
-        if (y + 1 < P.H) {
-            uint4 o;
-            o.x = pack_bf16(ob[0] * inv[1], ob[1] * inv[1]); o.y = pack_bf16(ob[2] * inv[1], ob[3] * inv[1]);
-            o.z = pack_bf16(ob[4] * inv[1], ob[5] * inv[1]); o.w = pack_bf16(ob[6] * inv[1], ob[7] * inv[1]);
-            *reinterpret_cast<uint4*>(P.out + ((size_t)(b * P.H + y + 1) * P.W + x) * Ctot + h * kHeadDim + tig * 8) = o;
-        }
+        if (!ok && lane == 0) atomicExch(P.status, 1);
+    }
+    tc_fence_before_sync();
+    __syncthreads();
+    if (warp == kMmaWarp) {
+        tc_fence_after_sync();
+        tmem_dealloc(*reinterpret_cast<const volatile uint32_t*>(smem + Wd::tmem_off), 512);
     }
 }
 
 template <int K>
-cudaError_t launch_t(const Problem& p, void* workspace, int* d_status, cudaStream_t stream) {
+cudaError_t launch_t(const Problem& p, void* workspace, int* d_status, int num_sms, cudaStream_t stream) {
     using Wd = Wide<K>;
-    using C_ = Cfg<__nv_bfloat16, K>;
     static bool configured[64] = {};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -310,30 +544,40 @@ cudaError_t launch_t(const Problem& p, void* workspace, int* d_status, cudaStrea
         if (e != cudaSuccess) return e;
         if (dev < 64) configured[dev] = true;
     }
-    const long long items = (long long)p.heads * 2 * Wd::K2 * 2 * Wd::NT * 32;
-    long long pblocks = (items + 255) / 256;
-    if (pblocks > 2368) pblocks = 2368;
-    mma_wide_prep_kernel<K><<<(unsigned)pblocks, 256, 0, stream>>>(p.wk, p.wv, static_cast<unsigned char*>(workspace), p.heads);
+    WideParams P;
+    P.weights = static_cast<const unsigned char*>(workspace);
+    P.q = static_cast<const __nv_bfloat16*>(p.q); P.bias = p.bias; P.out = static_cast<__nv_bfloat16*>(p.out); P.status = d_status;
+    P.H = p.H; P.W = p.W; P.heads = p.heads;
+    P.tiles_x = (p.W + 7) / 8; P.tiles_y = (p.H + 7) / 8;
+    const long long tiles = (long long)P.tiles_x * P.tiles_y * p.B;
+    if (tiles > 0x3fffffffLL) return cudaErrorInvalidConfiguration;
+    P.tiles = (int)tiles;
+    P.scale_log2e = kLog2e / sqrtf((float)kHeadDim);
+    const int C = p.heads * kHeadDim;
+    CUtensorMap mk, mv;
+    if (!make_tile_map(&mk, p.k, 2, p.B, p.H, p.W, C, kHeadDim, Wd::HP, Wd::HP) ||
+        !make_tile_map(&mv, p.v, 2, p.B, p.H, p.W, C, kHeadDim, Wd::HP, Wd::HP))
+        return cudaErrorInvalidValue;
+    mma_wide_prep_kernel<K><<<dim3((unsigned)((2 * Wd::K2 * 4 * Wd::N + 255) / 256), (unsigned)p.heads), 256, 0, stream>>>(
+        p.wk, p.wv, static_cast<unsigned char*>(workspace));
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
 
-    WideParams P;
-    P.frag = static_cast<const unsigned char*>(workspace);
-    P.bias = p.bias; P.out = static_cast<__nv_bfloat16*>(p.out); P.status = d_status;
-    P.B = p.B; P.H = p.H; P.W = p.W; P.heads = p.heads;
-    P.tiles_x = (p.W + kTW - 1) / kTW;
-    P.tiles_y = (p.H + C_::TH - 1) / C_::TH;
-    P.scale_log2e = kLog2e / sqrtf((float)kHeadDim);
-    const int Ctot = p.heads * kHeadDim;
-    CUtensorMap mq, mk, mv;
-    if (!make_tile_map(&mq, p.q, 2, p.B, p.H, p.W, Ctot, kHeadDim, kTW, C_::TH) ||
-        !make_tile_map(&mk, p.k, 2, p.B, p.H, p.W, Ctot, kHeadDim, C_::HW, C_::HH) ||
-        !make_tile_map(&mv, p.v, 2, p.B, p.H, p.W, Ctot, kHeadDim, C_::HW, C_::HH))
-        return cudaErrorInvalidValue;
-    const long long ctas = (long long)P.tiles_x * P.tiles_y * p.B * p.heads;
-    if (ctas > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-    mma_wide_kernel<K><<<(unsigned)ctas, Wd::threads, Wd::total, stream>>>(mq, mk, mv, P);
-    return cudaGetLastError();
+    const long long blocks = (tiles + 1) / 2;
+    long long per_head = num_sms / p.heads;
+    if (per_head > blocks) per_head = blocks;
+    if (per_head < 1) per_head = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(per_head * p.heads));
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = Wd::total;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, mma_wide_kernel<K>, mk, mv, P);
 }
 
 }  // namespace
@@ -345,21 +589,21 @@ bool mma_wide_supports(slide_attn_dtype dtype, int head_dim, int ksize) {
 
 size_t mma_wide_workspace_bytes(int heads, int ksize) {
     switch (ksize) {
-        case 3: return (size_t)heads * 2 * 9 * Wide<3>::chunk_bytes;
-        case 5: return (size_t)heads * 2 * 25 * Wide<5>::chunk_bytes;
-        case 7: return (size_t)heads * 2 * 49 * Wide<7>::chunk_bytes;
-        case 9: return (size_t)heads * 2 * 81 * Wide<9>::chunk_bytes;
+        case 3: return (size_t)heads * Wide<3>::weights;
+        case 5: return (size_t)heads * Wide<5>::weights;
+        case 7: return (size_t)heads * Wide<7>::weights;
+        case 9: return (size_t)heads * Wide<9>::weights;
         default: return 0;
     }
 }
 
-// Prep launch (weights -> fragment-ordered chunks in `workspace`) followed by the fused kernel.
-cudaError_t launch_mma_wide(const Problem& p, void* workspace, int* d_status, cudaStream_t stream) {
+// Prep launch (weights -> images in the order of their use, in `workspace`) followed by the fused kernel.
+cudaError_t launch_mma_wide(const Problem& p, void* workspace, int* d_status, int num_sms, cudaStream_t stream) {
     switch (p.ksize) {
-        case 3: return launch_t<3>(p, workspace, d_status, stream);
-        case 5: return launch_t<5>(p, workspace, d_status, stream);
-        case 7: return launch_t<7>(p, workspace, d_status, stream);
-        case 9: return launch_t<9>(p, workspace, d_status, stream);
+        case 3: return launch_t<3>(p, workspace, d_status, num_sms, stream);
+        case 5: return launch_t<5>(p, workspace, d_status, num_sms, stream);
+        case 7: return launch_t<7>(p, workspace, d_status, num_sms, stream);
+        case 9: return launch_t<9>(p, workspace, d_status, num_sms, stream);
         default: return cudaErrorInvalidConfiguration;
     }
 }

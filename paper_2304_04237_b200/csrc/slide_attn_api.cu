@@ -19,7 +19,7 @@ struct slide_attn_ctx {
     void* strip_ws;                  // transposed weights of the STRIP variant
     void* umma_ws;                   // bf16 B images of the UMMA_TS variant
     void* split_ws;                  // weight images of the UMMA_SPLIT variant
-    void* wide_ws;                   // bf16 B fragments of the MMA_WIDE variant
+    void* wide_ws;                   // bf16 weight images of the MMA_WIDE variant
     void* bwd_ws;                    // attention weights and logit gradients between the two backward kernels (first backward)
     void* block_ws;                  // q, k, v, z of slide_attn_block_forward (first use)
     bool proj_ready;                 // the projection kernel's attributes are set on this device
@@ -124,7 +124,7 @@ slide_attn_status launch_problem(slide_attn_ctx* c, const Problem& p, cudaStream
             break;
         case SLIDE_ATTN_VARIANT_MMA_WIDE:
             if (ev) cudaEventRecord(ev[1], stream);          // the prep launch is issued inside launch_mma_wide
-            err = launch_mma_wide(p, c->wide_ws, c->d_status, stream);
+            err = launch_mma_wide(p, c->wide_ws, c->d_status, c->num_sms, stream);
             break;
         case SLIDE_ATTN_VARIANT_UMMA_SPLIT:
             if (ev) cudaEventRecord(ev[1], stream);          // the prep launch is issued inside launch_umma_split
@@ -504,7 +504,7 @@ slide_attn_status slide_attn_launches_per_forward(const slide_attn_ctx* c, int* 
         case SLIDE_ATTN_VARIANT_STRIP: *n = 2; break;    // weight transpose + fused kernel
         case SLIDE_ATTN_VARIANT_UMMA_TS: *n = 2; break;  // B-image prep + fused kernel
         case SLIDE_ATTN_VARIANT_TILE: *n = 2; break;     // weight transpose + fused kernel
-        case SLIDE_ATTN_VARIANT_MMA_WIDE: *n = 2; break; // weight fragments + fused kernel
+        case SLIDE_ATTN_VARIANT_MMA_WIDE: *n = 2; break; // weight images + fused kernel
         case SLIDE_ATTN_VARIANT_UMMA_SPLIT: *n = 2; break; // weight images + fused kernel
         default: *n = 1; break;
     }
