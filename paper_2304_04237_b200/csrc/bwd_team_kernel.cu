@@ -259,7 +259,8 @@ bwd_point_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constan
             float a[kK2];
             // ---- products of both sides ----------------------------------------------------------------
             for (int v = 0; v < 2 * NPL; ++v) {
-                const uint4 x[2] = {xn[0], xn[1]};
+                Factor<T> x;
+                x.set(xn);
                 if (v + 1 < 2 * NPL) load_x(st, (v + 1) / NPL, (v + 1) % NPL, xn);
                 if (!warp_wait(bar(kFull + slot), phase)) { ok = false; break; }
                 const unsigned char* plane = seat.ring + (uint32_t)(slot * kSlot + wq * kHaloPlane);
@@ -273,7 +274,7 @@ bwd_point_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constan
                     tc_fence_after_sync();
                     const uint32_t t = mine + kColP + (uint32_t)(pb * 3 * Cut<T>::tap_cols);
 #pragma unroll
-                    for (int dy = 0; dy < 3; ++dy) store_products(T(), t + dy * Cut<T>::tap_cols, x, y[dy], y[dy + 1]);
+                    for (int dy = 0; dy < 3; ++dy) store_products(x, t + dy * Cut<T>::tap_cols, y[dy], y[dy + 1]);
                     tmem_wait_st();
                     tc_fence_before_sync();
                     __syncwarp();
@@ -322,18 +323,34 @@ bwd_point_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constan
                 // lane = 8 row + column of the strip
                 const Place px = me.place(P, seat.strip0(bi) + wq, lane >> 3, lane & 7);
                 if (px.in[0]) {
-                    const size_t at = (px.pix * P.heads + h) * 64;
-                    const uint32_t swz = (uint32_t)(lane >> 1) & 3u;             // x0 is a multiple of 8
-#pragma unroll
-                    for (uint32_t c = 0; c < 4; ++c)
-                        *reinterpret_cast<uint4*>(P.rows_dl + at + ((c ^ swz) << 4)) = make_uint4(row[4 * c], row[4 * c + 1], row[4 * c + 2], row[4 * c + 3]);
-                    split_row(a, row);
-#pragma unroll
-                    for (uint32_t c = 0; c < 4; ++c)
-                        *reinterpret_cast<uint4*>(P.rows_a + at + ((c ^ swz) << 4)) = make_uint4(row[4 * c], row[4 * c + 1], row[4 * c + 2], row[4 * c + 3]);
 #pragma unroll
                     for (int s = 0; s < kK2; ++s) dbias[s] += dl[s];
                 }
+                // Lanes 2i and 2i + 1 write both pieces of a 32-byte sector together: piece c of the even lane's pixel and its
+                // neighbour c + 1, then of the odd one's (16 bytes of each sector at a time took 20 of the kernel's 132 us).
+                const size_t at = (px.pix * P.heads + h) * 64, pitch = (size_t)P.heads * 64;
+                const bool odd = lane & 1, other = __shfl_xor_sync(0xffffffffu, (int)px.in[0], 1) != 0;
+                const bool in_even = odd ? other : px.in[0], in_odd = odd ? px.in[0] : other;
+                const size_t at_even = odd ? at - pitch : at;
+                const uint32_t swz = (uint32_t)(lane >> 1) & 3u;                 // x0 is a multiple of 8
+                auto write = [&](unsigned char* rows, const uint32_t (&w)[16]) {
+#pragma unroll
+                    for (uint32_t m = 0; m < 2; ++m) {                           // pieces 2m, 2m + 1
+                        uint32_t e[4], o[4];
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            const uint32_t lo = w[8 * m + i], hi = w[8 * m + 4 + i], got = __shfl_xor_sync(0xffffffffu, odd ? lo : hi, 1);
+                            e[i] = odd ? got : lo;                               // of the even pixel: this lane's piece 2m + odd
+                            o[i] = odd ? hi : got;                               // of the odd pixel
+                        }
+                        const uint32_t c = ((2 * m + (odd ? 1u : 0u)) ^ swz) << 4;
+                        if (in_even) *reinterpret_cast<uint4*>(rows + at_even + c) = make_uint4(e[0], e[1], e[2], e[3]);
+                        if (in_odd) *reinterpret_cast<uint4*>(rows + at_even + pitch + c) = make_uint4(o[0], o[1], o[2], o[3]);
+                    }
+                };
+                write(P.rows_dl, row);
+                split_row(a, row);
+                write(P.rows_a, row);
             }
 
             if (bi + 1 < my_blocks) { me.walk.next(); st = me.place(P, seat.strip0(bi + 1) + wq, 2 * half, g); load_x(st, 0, 0, xn); }

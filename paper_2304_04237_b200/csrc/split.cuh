@@ -52,6 +52,16 @@ __device__ __forceinline__ float2 lds_f2(uint32_t addr) {
     return v;
 }
 
+// The same with -lo instead of lo, given nx = -x: a multiply and an FMA, no negation in between.
+__device__ __forceinline__ void product2n(uint32_t x, uint32_t nx, uint32_t y, uint32_t& hi, uint32_t& neg_lo) {
+    const __nv_bfloat162 a = *reinterpret_cast<const __nv_bfloat162*>(&x), na = *reinterpret_cast<const __nv_bfloat162*>(&nx),
+                         b = *reinterpret_cast<const __nv_bfloat162*>(&y);
+    const __nv_bfloat162 h = __hmul2_rn(a, b);
+    const __nv_bfloat162 l = __hfma2(na, b, h);
+    hi = *reinterpret_cast<const uint32_t*>(&h);
+    neg_lo = *reinterpret_cast<const uint32_t*>(&l);
+}
+
 // four 8 x 8 matrices of 16-bit elements, transposed: the B fragments of a row-major [K][N] tile.
 // lane i holds the address of row i % 8 of matrix i / 8.
 __device__ __forceinline__ void ldmatrix_x4_trans(uint32_t addr, uint32_t& r0, uint32_t& r1, uint32_t& r2, uint32_t& r3) {

@@ -294,16 +294,34 @@ __device__ __forceinline__ float f4(const uint4& v, int i) {
     return __uint_as_float(i == 0 ? v.x : i == 1 ? v.y : i == 2 ? v.z : v.w);
 }
 
+// A lane's two left factors of the products.  bf16 keeps their negatives too: hi = x y and -lo = -x y + hi then need no
+// negation in between, and the tensor core negates the low part (it was one instruction in seven of the products).
+template <typename T> struct Factor;
+template <> struct Factor<__nv_bfloat16> {
+    uint4 x[2], nx[2];
+    __device__ __forceinline__ void set(const uint4 (&v)[2]) {
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            x[r] = v[r];
+            nx[r] = make_uint4(v[r].x ^ 0x80008000u, v[r].y ^ 0x80008000u, v[r].z ^ 0x80008000u, v[r].w ^ 0x80008000u);
+        }
+    }
+};
+template <> struct Factor<float> {
+    uint4 x[2];
+    __device__ __forceinline__ void set(const uint4 (&v)[2]) { x[0] = v[0]; x[1] = v[1]; }
+};
 // Products of one tap of a plane for the lane's two pixels, split, into tensor memory at column `t`.
-__device__ __forceinline__ void store_products(__nv_bfloat16, uint32_t t, const uint4 (&x)[2], const uint4& y0, const uint4& y1) {
+__device__ __forceinline__ void store_products(const Factor<__nv_bfloat16>& f, uint32_t t, const uint4& y0, const uint4& y1) {
     uint32_t r[16];
-    split::product2(x[0].x, y0.x, r[0], r[8]); split::product2(x[0].y, y0.y, r[1], r[9]);
-    split::product2(x[1].x, y1.x, r[2], r[10]); split::product2(x[1].y, y1.y, r[3], r[11]);
-    split::product2(x[0].z, y0.z, r[4], r[12]); split::product2(x[0].w, y0.w, r[5], r[13]);
-    split::product2(x[1].z, y1.z, r[6], r[14]); split::product2(x[1].w, y1.w, r[7], r[15]);
+    split::product2n(f.x[0].x, f.nx[0].x, y0.x, r[0], r[8]); split::product2n(f.x[0].y, f.nx[0].y, y0.y, r[1], r[9]);
+    split::product2n(f.x[1].x, f.nx[1].x, y1.x, r[2], r[10]); split::product2n(f.x[1].y, f.nx[1].y, y1.y, r[3], r[11]);
+    split::product2n(f.x[0].z, f.nx[0].z, y0.z, r[4], r[12]); split::product2n(f.x[0].w, f.nx[0].w, y0.w, r[5], r[13]);
+    split::product2n(f.x[1].z, f.nx[1].z, y1.z, r[6], r[14]); split::product2n(f.x[1].w, f.nx[1].w, y1.w, r[7], r[15]);
     tmem_st_16x256b_x4(t, r);
 }
-__device__ __forceinline__ void store_products(float, uint32_t t, const uint4 (&x)[2], const uint4& y0, const uint4& y1) {
+__device__ __forceinline__ void store_products(const Factor<float>& f, uint32_t t, const uint4& y0, const uint4& y1) {
+    const uint4 (&x)[2] = f.x;
     float2 p[4];                                         // first row: channels 0 1, 2 3; second row
     p[0] = split::mul2(make_float2(f4(x[0], 0), f4(x[0], 1)), make_float2(f4(y0, 0), f4(y0, 1)));
     p[1] = split::mul2(make_float2(f4(x[0], 2), f4(x[0], 3)), make_float2(f4(y0, 2), f4(y0, 3)));
@@ -334,12 +352,13 @@ __device__ __forceinline__ void issue_contract(uint32_t tmem, uint32_t p_col, ui
     const uint32_t r = tmem + kColR, h = tmem + kColH<T>;
     if constexpr (sizeof(T) == 2) {
         constexpr uint32_t k1 = 96;                                          // 1536 bytes on: the next 16 k
+        constexpr uint32_t neg32 = id32 | kIdescNegateA;
         umma_bf16_ts(h, p_col, b, id16, fresh ? 0u : 1u);
         umma_bf16_ts(r, p_col, b + mid, id32, first ? 0u : 1u);              // upper . middle | upper . lower
         umma_bf16_ts(h + 16, p_col + 8, b + k1, id16, fresh ? 0u : 1u);
         umma_bf16_ts(r, p_col + 8, b + k1 + mid, id32, 1);
-        umma_bf16_ts(r, p_col + 16, b, id32, 1);                             // lower . upper | lower . middle
-        umma_bf16_ts(r, p_col + 24, b + k1, id32, 1);
+        umma_bf16_ts(r, p_col + 16, b, neg32, 1);                            // lower . upper | lower . middle
+        umma_bf16_ts(r, p_col + 24, b + k1, neg32, 1);
     } else {
         umma_bf16_ts(h + 16 * dx, p_col, b, id16, fresh ? 0u : 1u);
         umma_bf16_ts(r, p_col, b + mid, id32, first ? 0u : 1u);

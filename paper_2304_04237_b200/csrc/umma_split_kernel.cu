@@ -188,7 +188,8 @@ umma_split_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
         for (int bi = 0; bi < my_blocks; ++bi) {
             // ---- products -------------------------------------------------------------------------
             for (int pl = 0; pl < NPL; ++pl) {
-                const uint4 x[2] = {qn[0], qn[1]};
+                Factor<T> x;
+                x.set(qn);
                 if (pl + 1 < NPL) load_q(st, pl + 1, qn);
                 if (!warp_wait(bar(kFull + slot), phase)) { ok = false; break; }
                 const unsigned char* plane = ring + (uint32_t)(slot * kSlot + wq * kHaloPlane);
@@ -202,7 +203,7 @@ umma_split_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
                     tc_fence_after_sync();
                     const uint32_t t = mine + kColP + (uint32_t)(pb * 3 * Cut<T>::tap_cols);
 #pragma unroll
-                    for (int dy = 0; dy < 3; ++dy) store_products(T(), t + dy * Cut<T>::tap_cols, x, y[dy], y[dy + 1]);
+                    for (int dy = 0; dy < 3; ++dy) store_products(x, t + dy * Cut<T>::tap_cols, y[dy], y[dy + 1]);
                     tmem_wait_st();
                     tc_fence_before_sync();
                     __syncwarp();
