@@ -16,7 +16,8 @@ size_t bwd_team_workspace_bytes(int B, int H, int W, int heads);
 
 // Clears the weight and bias gradients and builds the images, then dq, dbias and the split rows, then dk and dv.
 cudaError_t launch_bwd_team(const Problem& p, const BackwardArgs& ga, const BwdScratch& ws, int* d_status, int num_sms, cudaStream_t stream);
-// dwk, dwv from the split rows.
+// dwk, dwv from the split rows: bf16 on tcgen05, fp32 on mma.sync.
+cudaError_t launch_bwd_weight_umma(const Problem& p, const BackwardArgs& ga, const BwdScratch& ws, int* d_status, int num_sms, cudaStream_t stream);
 cudaError_t launch_bwd_weight_mma(const Problem& p, const BackwardArgs& ga, const BwdScratch& ws, int* d_status, int num_sms, cudaStream_t stream);
 
 }  // namespace slide_attn

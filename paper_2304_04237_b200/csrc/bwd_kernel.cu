@@ -630,7 +630,9 @@ cudaError_t launch_backward(const Problem& p, const BackwardArgs& ga, void* wt, 
     if (p.ksize == 3) {
         const BwdScratch s = bwd_scratch(ws, p.B, p.H, p.W, p.heads);
         e = launch_bwd_team(p, ga, s, d_status, num_sms, stream);
-        return e == cudaSuccess ? launch_bwd_weight_mma(p, ga, s, d_status, num_sms, stream) : e;
+        if (e != cudaSuccess) return e;
+        return p.dtype == SLIDE_ATTN_BF16 ? launch_bwd_weight_umma(p, ga, s, d_status, num_sms, stream)
+                                          : launch_bwd_weight_mma(p, ga, s, d_status, num_sms, stream);
     }
     const size_t k2 = (size_t)p.ksize * p.ksize, wbytes = (size_t)p.heads * kHeadDim * k2 * k2 * sizeof(float);
     e = cudaMemsetAsync(ga.dwk, 0, wbytes, stream);

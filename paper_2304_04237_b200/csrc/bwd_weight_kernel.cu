@@ -1,28 +1,22 @@
-// Weight gradients of the backward pass for k = 3 (head_dim 32, fp32 or bf16 storage) on tensor cores:
+// Weight gradients of the backward pass for k = 3, fp32 storage (head_dim 32), on mma.sync (bf16: bwd_weight_umma_kernel):
 //
 //   dwk[c,s,t] = scale * sum over pixels of dl[s] (q[c] k_t[c])        dwv[c,s,t] = sum of a[s] (g[c] v_t[c])
 //
 // For one tap t and one side this is a matrix product over the pixels: [channels x pixels] . [pixels x slots],
 // with the elementwise products as the left operand.  mma.sync.m16n8k16, M = 16 channels, K = 16 pixels (2 rows
-// x 8 columns), N = 32 columns that hold the nine slots three times: the upper, middle and lower 8 bits of the
-// fp32 dl (a), so that a bf16 tensor-core product loses none of them.  The left operand is split too: bf16
-// inputs multiply exactly into hi + lo, fp32 products into hi + mid + lo; the pairs below 2^-24 are left out
-// (hi meets all four 8-column tiles, the next part the first three, the last part the first two).
+// x 8 columns), N = 32 columns of a split row: the nine slots three times, the upper, middle and lower 8 bits of the
+// fp32 dl (a).  The products are split into hi + mid + lo too; the pairs below 2^-24 are left out (hi meets all four
+// 8-column tiles, mid the first three, lo the first two).
 //
 // Persistent, one CTA per SM and one head per CTA.  Twelve compute warps = side x 16-channel half x tap row,
 // three per scheduler; a warp keeps the sums of its three taps in registers over all its tiles.  The tensor core
 // truncates when it accumulates, so the columns that hold upper parts move to a second set of fp32 registers
-// after every kFlush pixel groups (eight to twelve tensor-core steps).  Tiles (4 rows x up to 56 columns + halo)
-// come by TMA into two stages, in channel planes that give a conflict-free fragment load: bf16 eight channels
-// (16 bytes a pixel), so that one transposing ldmatrix is a whole left operand at any tap's offset; fp32, which
-// ldmatrix cannot transpose, 16 channels (four pixels x eight channel pairs = 256 contiguous bytes).  Four more
-// warps turn the attention weights and logit gradients into the split columns (64 bytes per pixel, 16-byte chunks
-// swizzled so that ldmatrix meets no bank conflict).
+// after every kFlush pixel groups (twelve tensor-core steps).  Tiles (4 rows x up to 32 columns + halo) come by TMA into
+// two stages, in planes of 16 channels (four pixels x eight channel pairs = 256 contiguous bytes: no bank conflict).
 //
 // Bound by the mma.sync pipe and the CUDA-core work beside it, which hardly overlap (measured: 8 cycles per MMA and
-// scheduler, and each packed bf16 multiply or fp32 add next to it adds 0.75 - 1.5): 252 MMAs (bf16; 324 for fp32) per
-// 16 pixels of a head.  64 x 56 x 56, 3 heads, bf16: 410 us with fp32 FMAs (lane = channel, 2 x 81 sums in registers),
-// 145 us here; 2 x 128 x 128, 3 heads, fp32: 76 and 49 us.
+// scheduler, and each packed bf16 multiply or fp32 add next to it adds 0.75 - 1.5): 324 MMAs per 16 pixels of a head.
+// 2 x 128 x 128, 3 heads: 76 us with fp32 FMAs (lane = channel, 2 x 81 sums in registers), 45 us here.
 #include "bwd_common.cuh"
 #include "split.cuh"
 
@@ -41,7 +35,6 @@ constexpr int kFlush = 4;
 constexpr uint32_t kSumBytes = 2u * kK2 * kHeadDim * 32u * 4u;        // the CTA's sums at its end, [side][tap][channel][32 columns]
 
 template <typename T> struct WTile;
-template <> struct WTile<__nv_bfloat16> { static constexpr int max_w = 56, planes = 4; };
 template <> struct WTile<float> { static constexpr int max_w = 32, planes = 2; };
 
 // Stage layout for tiles of tw columns (bytes); the channel planes of a tensor follow each other.
@@ -82,22 +75,10 @@ struct WParams {
     float scale;
 };
 
-// One 16-pixel (2 rows x 8 columns), 16-channel operand tile in registers: for bf16 the A fragment of the raw
-// values, for fp32 the values of channels 2g, 2g + 1 of the lane's four pixels.  `offset` and `col` say where a lane
-// reads, in a tile whose planes are `plane` bytes and whose rows are `pitch` bytes apart, and which column of the
-// group the K index k (of its row's eight) is.
+// One 16-pixel (2 rows x 8 columns), 16-channel operand tile in registers: the values of channels 2g, 2g + 1 of the lane's
+// four pixels.  `offset` and `col` say where a lane reads, in a tile whose planes are `plane` bytes and whose rows are `pitch`
+// bytes apart, and which column of the group the K index k (of its row's eight) is.
 template <typename T> struct Frag;
-template <> struct Frag<__nv_bfloat16> {
-    static constexpr uint32_t pixel_bytes = 16;
-    uint32_t a[4];
-    // lane i: row i % 8 of matrix i / 8 = (channels 0-7 row 0, channels 8-15 row 0, channels 0-7 row 1, ..)
-    static __device__ __forceinline__ uint32_t offset(int lane, int half, uint32_t plane, uint32_t pitch) {
-        return (uint32_t)(2 * half + ((lane >> 3) & 1)) * plane + (uint32_t)(lane >> 4) * pitch + (uint32_t)(lane & 7) * pixel_bytes;
-    }
-    static __device__ __forceinline__ int col(int k) { return k; }
-    static __device__ __forceinline__ int channel(int row) { return row; }
-    __device__ __forceinline__ void load(uint32_t p, uint32_t) { ldmatrix_x4_trans(p, a[0], a[1], a[2], a[3]); }
-};
 template <> struct Frag<float> {
     static constexpr uint32_t pixel_bytes = 64;
     float2 a[4];
@@ -113,16 +94,6 @@ template <> struct Frag<float> {
 };
 
 // acc += (x . y) times the split columns b[tile][2]
-__device__ __forceinline__ void accumulate(float (&acc)[4][4], const Frag<__nv_bfloat16>& x, const Frag<__nv_bfloat16>& y,
-                                           const uint32_t (&b)[4][2]) {
-    uint32_t hi[4], lo[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) product2(x.a[i], y.a[i], hi[i], lo[i]);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) mma_bf16(acc[j], hi, b[j][0], b[j][1]);
-#pragma unroll
-    for (int j = 0; j < 3; ++j) mma_bf16(acc[j], lo, b[j][0], b[j][1]);
-}
 __device__ __forceinline__ void accumulate(float (&acc)[4][4], const Frag<float>& x, const Frag<float>& y, const uint32_t (&b)[4][2]) {
     float2 p[4];
 #pragma unroll
@@ -336,7 +307,7 @@ cudaError_t launch_t(const Problem& p, const BackwardArgs& ga, const BwdScratch&
 }  // namespace
 
 cudaError_t launch_bwd_weight_mma(const Problem& p, const BackwardArgs& ga, const BwdScratch& ws, int* d_status, int num_sms, cudaStream_t stream) {
-    return p.dtype == SLIDE_ATTN_BF16 ? launch_t<__nv_bfloat16>(p, ga, ws, d_status, num_sms, stream) : launch_t<float>(p, ga, ws, d_status, num_sms, stream);
+    return launch_t<float>(p, ga, ws, d_status, num_sms, stream);
 }
 
 }  // namespace slide_attn

@@ -20,15 +20,6 @@ __device__ __forceinline__ uint32_t pack_upper(float a, float b) {
 // what truncation to bf16 leaves of x (exact)
 __device__ __forceinline__ float rest(float x) { return x - __uint_as_float(__float_as_uint(x) & 0xFFFF0000u); }
 
-// hi + lo = a * b exactly, per half of the register (barring underflow of the low part)
-__device__ __forceinline__ void product2(uint32_t a, uint32_t b, uint32_t& hi, uint32_t& lo) {
-    const __nv_bfloat162 x = *reinterpret_cast<const __nv_bfloat162*>(&a), y = *reinterpret_cast<const __nv_bfloat162*>(&b);
-    const __nv_bfloat162 h = __hmul2_rn(x, y);
-    const __nv_bfloat162 l = __hfma2(x, y, __hneg2(h));
-    hi = *reinterpret_cast<const uint32_t*>(&h);
-    lo = *reinterpret_cast<const uint32_t*>(&l);
-}
-
 // (a0, a1) * (b0, b1), and what truncation to bf16 leaves of a pair, as packed fp32 operations
 __device__ __forceinline__ float2 mul2(float2 a, float2 b) {
     float2 d;
@@ -52,7 +43,8 @@ __device__ __forceinline__ float2 lds_f2(uint32_t addr) {
     return v;
 }
 
-// The same with -lo instead of lo, given nx = -x: a multiply and an FMA, no negation in between.
+// hi - neg_lo = x * y exactly, per half of the register (barring underflow of the low part), given nx = -x: a multiply and an
+// FMA, no negation in between.
 __device__ __forceinline__ void product2n(uint32_t x, uint32_t nx, uint32_t y, uint32_t& hi, uint32_t& neg_lo) {
     const __nv_bfloat162 a = *reinterpret_cast<const __nv_bfloat162*>(&x), na = *reinterpret_cast<const __nv_bfloat162*>(&nx),
                          b = *reinterpret_cast<const __nv_bfloat162*>(&y);
