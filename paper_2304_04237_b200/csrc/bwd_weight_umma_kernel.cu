@@ -204,7 +204,7 @@ bwd_weight_umma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                 float v[16];
                 tmem_ld_32x32b_x16(quad + 16 * idx, v);
 #pragma unroll
-                for (int c = 0; c < 16; ++c) sum[i][c] += v[c];
+                for (int c = 0; c < 16; c += 2) fadd2(sum[i][c], sum[i][c + 1], v[c], v[c + 1]);
             }
             tc_fence_before_sync();
             __syncwarp();

@@ -102,6 +102,16 @@ __device__ __forceinline__ void ffma2(float& o0, float& o1, float a0, float a1, 
         : "+f"(o0), "+f"(o1) : "f"(a0), "f"(a1), "f"(b0), "f"(b1));
 }
 
+// (o0, o1) += (a0, a1)
+__device__ __forceinline__ void fadd2(float& o0, float& o1, float a0, float a1) {
+    asm("{\n\t.reg .b64 ra, rc;\n\t"
+        "mov.b64 ra, {%2, %3};\n\t"
+        "mov.b64 rc, {%0, %1};\n\t"
+        "add.rn.f32x2 rc, rc, ra;\n\t"
+        "mov.b64 {%0, %1}, rc;\n\t}"
+        : "+f"(o0), "+f"(o1) : "f"(a0), "f"(a1));
+}
+
 __device__ __forceinline__ uint32_t hmul2_bf16(uint32_t a, uint32_t b) {
     uint32_t d;
     asm("mul.rn.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
