@@ -62,6 +62,7 @@ template <typename T>
 __global__ void __launch_bounds__(256)
 bwd_prep_kernel(const float* __restrict__ wk, const float* __restrict__ wv, unsigned char* __restrict__ images, float* dwk, float* dwv, float* dbias)
 {
+    grid_dependency_wait();
     grid_launch_dependents();
     const size_t w = (size_t)blockIdx.x * kHeadDim * kK2 * kK2;
     unsigned char* img = images + (size_t)blockIdx.x * kImages;
@@ -554,21 +555,6 @@ bwd_gather_kernel(const __grid_constant__ CUtensorMap map_dl, const __grid_const
     leave_seat<kGatherImages>(smem, seat);
 }
 
-template <typename... Params, typename... Args>
-cudaError_t launch_chained(void (*kernel)(Params...), int grid, int threads, uint32_t smem, cudaStream_t stream, Args... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3((unsigned)threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, args...);
-}
-
 template <typename T>
 cudaError_t launch_t(const Problem& p, const BackwardArgs& ga, const BwdScratch& ws, int* d_status, int num_sms, cudaStream_t stream) {
     static bool configured[64] = {};
@@ -595,14 +581,13 @@ cudaError_t launch_t(const Problem& p, const BackwardArgs& ga, const BwdScratch&
         !make_tile_map(&mv, p.v, es, p.B, p.H, p.W, C, ch, 10, 6) || !make_tile_map(&mg, ga.dout, es, p.B, p.H, p.W, C, ch, 10, 6) ||
         !make_tile_map(&mdl, ws.rows_dl, 2, p.B, p.H, p.W, C, 32, 10, 6) || !make_tile_map(&ma, ws.rows_a, 2, p.B, p.H, p.W, C, 32, 10, 6))
         return cudaErrorInvalidValue;
-    bwd_prep_kernel<T><<<dim3((unsigned)p.heads, 9), 256, 0, stream>>>(p.wk, p.wv, ws.images, ga.dwk, ga.dwv, ga.dbias);
-    e = cudaGetLastError();
+    e = launch_chained(bwd_prep_kernel<T>, dim3((unsigned)p.heads, 9), 256, 0, stream, p.wk, p.wv, ws.images, ga.dwk, ga.dwv, ga.dbias);
     if (e != cudaSuccess) return e;
     const long long blocks = (P.strips.total + 3) / 4;
     long long per_head = num_sms / p.heads;
     if (per_head > blocks) per_head = blocks;
     if (per_head < 1) per_head = 1;
-    const int grid = (int)(per_head * p.heads);
+    const dim3 grid((unsigned)(per_head * p.heads));
     e = launch_chained(bwd_point_kernel<T>, grid, kThreads, Plan<kPointImages>::total, stream, mk, mv, P);
     if (e != cudaSuccess) return e;
     return launch_chained(bwd_gather_kernel<T>, grid, kThreads, Plan<kGatherImages>::total, stream, mdl, ma, mq, mg, P);

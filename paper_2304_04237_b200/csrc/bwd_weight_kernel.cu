@@ -291,17 +291,7 @@ cudaError_t launch_t(const Problem& p, const BackwardArgs& ga, const BwdScratch&
     long long per_head = num_sms / p.heads;                          // one CTA per SM, all heads alike
     if (per_head > tiles) per_head = tiles;
     if (per_head < 1) per_head = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(per_head * p.heads));
-    cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = w_smem_bytes<T>(tw);
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, bwd_weight_mma_kernel<T>, mq, mk, mv, mg, mdl, ma, P);
+    return launch_chained(bwd_weight_mma_kernel<T>, dim3((unsigned)(per_head * p.heads)), kThreads, w_smem_bytes<T>(tw), stream, mq, mk, mv, mg, mdl, ma, P);
 }
 
 }  // namespace

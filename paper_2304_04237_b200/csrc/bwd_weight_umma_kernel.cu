@@ -312,17 +312,7 @@ cudaError_t launch_bwd_weight_umma(const Problem& p, const BackwardArgs& ga, con
     long long per_head = num_sms / p.heads;                          // one CTA per SM, all heads alike
     if (per_head > tiles) per_head = tiles;
     if (per_head < 1) per_head = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(per_head * p.heads));
-    cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = smem_bytes(tw);
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, bwd_weight_umma_kernel, mq, mk, mv, mg, mdl, ma, P);
+    return launch_chained(bwd_weight_umma_kernel, dim3((unsigned)(per_head * p.heads)), kThreads, smem_bytes(tw), stream, mq, mk, mv, mg, mdl, ma, P);
 }
 
 }  // namespace slide_attn

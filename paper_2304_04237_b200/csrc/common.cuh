@@ -38,6 +38,25 @@ bool tensor_map_available();
 bool make_tile_map(CUtensorMap* map, const void* base, int elem_bytes, int B, int H, int W, int C,
                    int box_c, int box_w, int box_h);
 
+// Launches with programmatic stream serialisation: the kernel may start before the one ahead of it in the stream has finished and
+// has to execute griddepcontrol.wait before it touches anything that one may write or read.  The prep kernels wait first
+// of all and only then let the main kernel behind them start, so a main kernel never runs beside what was ahead of its prep
+// kernel.  Chained so, back-to-back forwards have no launch gap between them.
+template <typename... Params, typename... Args>
+inline cudaError_t launch_chained(void (*kernel)(Params...), dim3 grid, int threads, size_t smem, cudaStream_t stream, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 // Launchers.  Each returns cudaGetLastError() of its launch(es).
 cudaError_t launch_direct(const Problem& p, cudaStream_t stream);
 bool direct_supports(int head_dim, int ksize);

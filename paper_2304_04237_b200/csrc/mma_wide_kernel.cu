@@ -107,6 +107,7 @@ mma_wide_prep_kernel(const float* __restrict__ wk, const float* __restrict__ wv,
 {
     using Wd = Wide<K>;
     constexpr int K2 = Wd::K2, N = Wd::N, per_tap = 4 * N;
+    grid_dependency_wait();
     grid_launch_dependents();
     const int h = blockIdx.y;
     const float* wkh = wk + (size_t)h * kHeadDim * K2 * K2;
@@ -558,26 +559,15 @@ cudaError_t launch_t(const Problem& p, void* workspace, int* d_status, int num_s
     if (!make_tile_map(&mk, p.k, 2, p.B, p.H, p.W, C, kHeadDim, Wd::HP, Wd::HP) ||
         !make_tile_map(&mv, p.v, 2, p.B, p.H, p.W, C, kHeadDim, Wd::HP, Wd::HP))
         return cudaErrorInvalidValue;
-    mma_wide_prep_kernel<K><<<dim3((unsigned)((2 * Wd::K2 * 4 * Wd::N + 255) / 256), (unsigned)p.heads), 256, 0, stream>>>(
-        p.wk, p.wv, static_cast<unsigned char*>(workspace));
-    e = cudaGetLastError();
+    e = launch_chained(mma_wide_prep_kernel<K>, dim3((unsigned)((2 * Wd::K2 * 4 * Wd::N + 255) / 256), (unsigned)p.heads), 256, 0, stream, p.wk, p.wv,
+                       static_cast<unsigned char*>(workspace));
     if (e != cudaSuccess) return e;
 
     const long long blocks = (tiles + 1) / 2;
     long long per_head = num_sms / p.heads;
     if (per_head > blocks) per_head = blocks;
     if (per_head < 1) per_head = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(per_head * p.heads));
-    cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = Wd::total;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, mma_wide_kernel<K>, mk, mv, P);
+    return launch_chained(mma_wide_kernel<K>, dim3((unsigned)(per_head * p.heads)), kThreads, Wd::total, stream, mk, mv, P);
 }
 
 }  // namespace

@@ -180,6 +180,7 @@ shift_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ 
 // Sets the status word to 2 if any weight differs from the one-hot shift kernel w[c][s][t] = [s == t].
 __global__ void shift_check_kernel(const float* __restrict__ wk, const float* __restrict__ wv, long long n_per, int k2, int* status)
 {
+    grid_dependency_wait();
     grid_launch_dependents();        // the fixed-shift kernel does not read this kernel's result
     bool bad = false;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < 2 * n_per; i += (long long)gridDim.x * blockDim.x) {
@@ -259,8 +260,7 @@ cudaError_t launch_shift_check(const Problem& p, int* d_status, cudaStream_t str
     const int k2 = p.ksize * p.ksize;
     const long long n_per = (long long)p.heads * p.head_dim * k2 * k2;
     const int blocks = (int)((2 * n_per + 255) / 256 < 1184 ? (2 * n_per + 255) / 256 : 1184);
-    shift_check_kernel<<<blocks, 256, 0, stream>>>(p.wk, p.wv, n_per, k2, d_status);
-    return cudaGetLastError();
+    return launch_chained(shift_check_kernel, dim3((unsigned)blocks), 256, 0, stream, p.wk, p.wv, n_per, k2, d_status);
 }
 
 cudaError_t launch_shift(const Problem& p, int* d_status, cudaStream_t stream) {

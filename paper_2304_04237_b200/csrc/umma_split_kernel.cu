@@ -50,6 +50,7 @@ template <typename T, int D>
 __global__ void __launch_bounds__(256)
 umma_split_prep_kernel(const float* __restrict__ wk, const float* __restrict__ wv, unsigned char* __restrict__ img)
 {
+    grid_dependency_wait();
     grid_launch_dependents();        // the main kernel may start its own prologue now
     const size_t w = (size_t)blockIdx.x * D * kK2 * kK2;
     unsigned char* dst = img + (size_t)blockIdx.x * Fwd<T, D>::image;
@@ -314,25 +315,14 @@ cudaError_t launch_t(const Problem& p, void* workspace, int* d_status, int num_s
     if (!make_tile_map(&mk, p.k, (int)sizeof(T), p.B, p.H, p.W, C, Cut<T>::channels, 10, 6) ||
         !make_tile_map(&mv, p.v, (int)sizeof(T), p.B, p.H, p.W, C, Cut<T>::channels, 10, 6))
         return cudaErrorInvalidValue;
-    umma_split_prep_kernel<T, D><<<dim3((unsigned)p.heads, prep_parts(D)), 256, 0, stream>>>(p.wk, p.wv, static_cast<unsigned char*>(workspace));
-    e = cudaGetLastError();
+    e = launch_chained(umma_split_prep_kernel<T, D>, dim3((unsigned)p.heads, prep_parts(D)), 256, 0, stream, p.wk, p.wv, static_cast<unsigned char*>(workspace));
     if (e != cudaSuccess) return e;
 
     const long long blocks = (P.strips.total + 3) / 4;
     long long per_head = num_sms / p.heads;
     if (per_head > blocks) per_head = blocks;
     if (per_head < 1) per_head = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(per_head * p.heads));
-    cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = F::total;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, umma_split_kernel<T, D>, mk, mv, P);
+    return launch_chained(umma_split_kernel<T, D>, dim3((unsigned)(per_head * p.heads)), kThreads, F::total, stream, mk, mv, P);
 }
 
 }  // namespace

@@ -146,6 +146,7 @@ __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity) {
 __global__ void __launch_bounds__(256)
 umma_ts_prep_kernel(const float* __restrict__ wk, const float* __restrict__ wv, unsigned char* __restrict__ img)
 {
+    grid_dependency_wait();
     grid_launch_dependents();        // the main kernel may start its own prologue now
     const int h = blockIdx.x;
     const float* wks = wk + (size_t)h * kHeadDim * 81;
@@ -670,17 +671,7 @@ template <int TW>
 cudaError_t launch_one(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv, const UmmaParams& P,
                        int grid, cudaStream_t stream) {
     static_assert(v_stages_for(TW) >= 2, "tile width does not fit shared memory");
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = smem_layout(TW, v_stages_for(TW)).total;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, umma_ts_kernel<TW>, mq, mk, mv, P);
+    return launch_chained(umma_ts_kernel<TW>, dim3((unsigned)grid), kThreads, smem_layout(TW, v_stages_for(TW)).total, stream, mq, mk, mv, P);
 }
 
 }  // namespace
@@ -701,8 +692,7 @@ cudaError_t umma_ts_setup() {
 }
 
 cudaError_t launch_umma_ts_prep(const Problem& p, void* workspace, cudaStream_t stream) {
-    umma_ts_prep_kernel<<<dim3((unsigned)p.heads, 6), 256, 0, stream>>>(p.wk, p.wv, static_cast<unsigned char*>(workspace));
-    return cudaGetLastError();
+    return launch_chained(umma_ts_prep_kernel, dim3((unsigned)p.heads, 6), 256, 0, stream, p.wk, p.wv, static_cast<unsigned char*>(workspace));
 }
 
 cudaError_t launch_umma_ts(const Problem& p, const void* workspace, int* d_status, int num_sms, cudaStream_t stream) {
