@@ -98,6 +98,7 @@ cudaError_t launch_umma_split(const Problem& p, void* workspace, int* d_status, 
 bool shift_supports(int head_dim, int ksize);
 cudaError_t launch_shift_check(const Problem& p, int* d_status, cudaStream_t stream);
 cudaError_t launch_shift(const Problem& p, int* d_status, cudaStream_t stream);
+cudaError_t launch_shift_mma(const Problem& p, int* d_status, cudaStream_t stream);       // bf16, k = 5, 7, 9
 
 // Backward pass (head_dim 32, k = 1 or 3, both dtypes): gradients of the forward's inputs.
 struct BackwardArgs {

@@ -225,17 +225,7 @@ cudaError_t launch_t(const Problem& p, int* d_status, cudaStream_t stream) {
     if (ctas > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
     // programmatic stream serialisation: the kernel may run beside the weight check launched just
     // before it (it does not read the check's result; both only ever set the status word)
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)ctas);
-    cfg.blockDim = dim3(C_::threads);
-    cfg.dynamicSmemBytes = C_::total;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, shift_kernel<T, K>, mq, mk, mv, P);
+    return launch_chained(shift_kernel<T, K>, dim3((unsigned)ctas), C_::threads, C_::total, stream, mq, mk, mv, P);
 }
 
 template <typename T>
@@ -243,11 +233,17 @@ cudaError_t launch_k(const Problem& p, int* d_status, cudaStream_t stream) {
     switch (p.ksize) {
         case 1: return launch_t<T, 1>(p, d_status, stream);
         case 3: return launch_t<T, 3>(p, d_status, stream);
-        case 5: return launch_t<T, 5>(p, d_status, stream);
-        case 7: return launch_t<T, 7>(p, d_status, stream);
-        case 9: return launch_t<T, 9>(p, d_status, stream);
-        default: return cudaErrorInvalidConfiguration;
+        default: break;
     }
+    if constexpr (sizeof(T) == 4) {
+        switch (p.ksize) {
+            case 5: return launch_t<T, 5>(p, d_status, stream);
+            case 7: return launch_t<T, 7>(p, d_status, stream);
+            case 9: return launch_t<T, 9>(p, d_status, stream);
+            default: break;
+        }
+    }
+    return cudaErrorInvalidConfiguration;
 }
 
 }  // namespace
@@ -264,6 +260,8 @@ cudaError_t launch_shift_check(const Problem& p, int* d_status, cudaStream_t str
 }
 
 cudaError_t launch_shift(const Problem& p, int* d_status, cudaStream_t stream) {
+    // wide windows of bf16 on tensor cores; the sides of the line are measured there
+    if (p.dtype == SLIDE_ATTN_BF16 && p.ksize >= 5) return launch_shift_mma(p, d_status, stream);
     return p.dtype == SLIDE_ATTN_BF16 ? launch_k<__nv_bfloat16>(p, d_status, stream) : launch_k<float>(p, d_status, stream);
 }
 

@@ -152,3 +152,14 @@ def test_unsupported_shapes_keep_the_mode_off():
         assert e.value.status == sa.ERR_UNSUPPORTED
     finally:
         sa.slide_attn_destroy(ctx)
+
+
+@pytest.mark.parametrize("k", [5, 7, 9])
+@pytest.mark.parametrize("H,W", [(5, 31), (2, 32), (7, 64), (4, 8), (3, 65)])
+def test_fixed_shift_band_edges_keep_fp32_accuracy(H, W, k):
+    """The tensor-core band at the edges of its tiles.  Exact products, fp32 sums, weights as two bf16 (2^-17): beyond the one
+    rounding of the result (half an ulp of 8 bits, 2^-8 of the value at most) 1e-4 remains."""
+    x = synth.make_inputs(2, H, W, 2, 32, k, "bf16", 0.0, 0.3, True, seed=H * 1000 + W * 10 + k)
+    ref = oracle.forward(x["q"], x["k"], x["v"], x["wk"], x["wv"], x["bias"], k)
+    got = shift_forward(x, k, "bf16")
+    assert np.isfinite(got).all() and (np.abs(got - ref) <= 2.0 ** -8 * np.abs(ref) + 1e-4).all()
