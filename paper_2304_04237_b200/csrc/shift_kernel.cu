@@ -10,7 +10,7 @@
 // 2 k^2 multiply-adds per pixel-channel instead of 2 k^4 + 2 k^2: for small windows the pass is bound by
 // HBM, so it runs on the CUDA cores straight off a halo tile.
 //
-// One CTA = one head of a 4 x 32 pixel tile (four warps; several CTAs share an SM, so one CTA's loads
+// One CTA = one head of a 4 x tw pixel tile (a warp per 8 columns; several CTAs share an SM, so one CTA's loads
 // overlap another's arithmetic).  The K and V tile + floor(k/2) halo and the q tile come in
 // by TMA (out-of-map elements zero-filled: that IS the padding) as "planes" of 64 bytes of channels per
 // pixel (bf16: one plane of 32 channels; fp32: two planes of 16), so that a quad of lanes reads one
@@ -26,19 +26,50 @@ namespace slide_attn {
 namespace {
 
 using namespace tile;
-using ShiftParams = TileParams;
+struct ShiftParams {
+    const float* bias;
+    void* out;
+    int* status;
+    int B, H, W, heads;
+    int tw, tiles_x, tiles_y;
+    float scale_log2e;
+};
 
+// Widest tile (with 56 columns fewer CTAs share an SM and cover each other's loads: 64 x 56 x 56, 3 heads, 37.2 us against 35.8
+// although 32-wide tiles cover 64 columns there).
+constexpr int kMaxTW = 32;
+
+// Shared memory of a 4 x tw tile.
 template <typename T, int K>
-__global__ void __launch_bounds__(Cfg<T, K>::threads, (sizeof(T) == 2 && K <= 3) ? 6 : 4)
+struct ShiftLayout {
+    static constexpr int planes = Elem<T>::planes, HH = kR + K - 1;
+    int HW;
+    uint32_t halo_plane, q_plane, k_off, v_off, q_off, bias_off, bar_off, total, tx_bytes;
+    __host__ __device__ explicit ShiftLayout(int tw) {
+        HW = tw + K - 1;
+        halo_plane = ((uint32_t)(HW * HH) * 64u + 127u) & ~127u;
+        q_plane = (uint32_t)(tw * kR) * 64u;
+        k_off = 0; v_off = planes * halo_plane; q_off = 2 * planes * halo_plane;
+        bias_off = q_off + planes * q_plane;
+        bar_off = bias_off + ((K * K * 4 + 15) & ~15);
+        total = bar_off + 16 + 128;                                   // + alignment slack
+        tx_bytes = planes * (2u * (uint32_t)(HW * HH) * 64u + q_plane);
+    }
+};
+
+// TW: the tile width, or 0 for any (strides known at compile time are 2 % faster with wide windows).
+template <typename T, int K, int TW>
+__global__ void __launch_bounds__(kMaxTW * 4, sizeof(T) == 2 ? 6 : 4)
 shift_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
              const __grid_constant__ CUtensorMap map_v, const ShiftParams P)
 {
-    using C_ = Cfg<T, K>;
     constexpr int R = K / 2;
+    const int tw = TW ? TW : P.tw;
+    const ShiftLayout<T, K> L(tw);
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u);
-    const uint32_t bar = smem_u32(smem + C_::bar_off);
-    float* s_bias = reinterpret_cast<float*>(smem + C_::bias_off);
+    const uint32_t bar = smem_u32(smem + L.bar_off);
+    float* s_bias = reinterpret_cast<float*>(smem + L.bias_off);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = lane >> 2, tig = lane & 3;
@@ -47,32 +78,31 @@ shift_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ 
     const int tx = tile % P.tiles_x; tile /= P.tiles_x;
     const int ty = tile % P.tiles_y;
     const int b = tile / P.tiles_y;
-    const int x0 = tx * kTW, y0 = ty * C_::TH;
+    const int x0 = tx * tw, y0 = ty * kR;
     constexpr int chan_per_plane = 64 / (int)sizeof(T);
 
     if (threadIdx.x == 0) {
         mbar_init(bar, 1);
-        mbar_expect_tx(bar, C_::tx_bytes);
+        mbar_expect_tx(bar, L.tx_bytes);
 #pragma unroll
-        for (int pl = 0; pl < C_::planes; ++pl) {
+        for (int pl = 0; pl < L.planes; ++pl) {
             const int c0 = h * kHeadDim + pl * chan_per_plane;
-            tma_load_4d(smem_u32(smem + C_::k_off + pl * C_::halo_plane), &map_k, bar, c0, x0 - R, y0 - R, b);
-            tma_load_4d(smem_u32(smem + C_::v_off + pl * C_::halo_plane), &map_v, bar, c0, x0 - R, y0 - R, b);
-            tma_load_4d(smem_u32(smem + C_::q_off + pl * C_::q_plane), &map_q, bar, c0, x0, y0, b);
+            tma_load_4d(smem_u32(smem + L.k_off + pl * L.halo_plane), &map_k, bar, c0, x0 - R, y0 - R, b);
+            tma_load_4d(smem_u32(smem + L.v_off + pl * L.halo_plane), &map_v, bar, c0, x0 - R, y0 - R, b);
+            tma_load_4d(smem_u32(smem + L.q_off + pl * L.q_plane), &map_q, bar, c0, x0, y0, b);
         }
     }
-    for (int i = threadIdx.x; i < K * K; i += C_::threads) s_bias[i] = P.bias ? P.bias[h * K * K + i] * kLog2e : 0.f;
+    for (int i = threadIdx.x; i < K * K; i += tw * 4) s_bias[i] = P.bias ? P.bias[h * K * K + i] * kLog2e : 0.f;
     __syncthreads();
     if (!mbar_wait(bar, 0)) {                                  // bounded: about two seconds
         if (lane == 0) atomicExch(P.status, 1);
         return;
     }
 
-    const int wx = warp % (kTW / 8), wy = warp / (kTW / 8);
-    const int col = wx * 8 + g, row0 = wy * kR;                  // this lane's pixel column, first pixel row
-    const unsigned char* sK = smem + C_::k_off;
-    const unsigned char* sV = smem + C_::v_off;
-    const unsigned char* sQ = smem + C_::q_off;
+    const int col = warp * 8 + g;                                // this lane's pixel column
+    const unsigned char* sK = smem + L.k_off;
+    const unsigned char* sV = smem + L.v_off;
+    const unsigned char* sQ = smem + L.q_off;
 
     // Within a quad, lane tig also OWNS pixel row tig of the strip: the partial dot products of the
     // four lanes are summed so that each lane ends up with the k logits of its own pixel (a
@@ -82,7 +112,7 @@ shift_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ 
     const int qbase = lane & ~3;
     typename Piece<T>::Raw qr[kR];
 #pragma unroll
-    for (int r = 0; r < kR; ++r) qr[r] = Piece<T>::load(sQ, C_::q_plane, (uint32_t)((row0 + r) * kTW + col), tig);
+    for (int r = 0; r < kR; ++r) qr[r] = Piece<T>::load(sQ, L.q_plane, (uint32_t)(r * tw + col), tig);
     float m = -INFINITY, sum = 0.f;                              // of pixel row tig
     float acc[kR][8];
 #pragma unroll
@@ -96,7 +126,7 @@ shift_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ 
         float p[kR][K];
 #pragma unroll
         for (int j = 0; j < kR + K - 1; ++j) {
-            const typename Piece<T>::Raw kv = Piece<T>::load(sK, C_::halo_plane, (uint32_t)((row0 + j) * C_::HW + col + dx), tig);
+            const typename Piece<T>::Raw kv = Piece<T>::load(sK, L.halo_plane, (uint32_t)(j * L.HW + col + dx), tig);
 #pragma unroll
             for (int r = 0; r < kR; ++r) {
                 const int dy = j - r;
@@ -138,7 +168,7 @@ shift_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ 
 #pragma unroll
         for (int j = 0; j < kR + K - 1; ++j) {
             float vv[8];
-            Piece<T>::widen(Piece<T>::load(sV, C_::halo_plane, (uint32_t)((row0 + j) * C_::HW + col + dx), tig), vv);
+            Piece<T>::widen(Piece<T>::load(sV, L.halo_plane, (uint32_t)(j * L.HW + col + dx), tig), vv);
 #pragma unroll
             for (int r = 0; r < kR; ++r) {
                 const int dy = j - r;
@@ -159,7 +189,7 @@ shift_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ 
     const int Ctot = P.heads * kHeadDim;
 #pragma unroll
     for (int r = 0; r < kR; ++r) {
-        const int y = y0 + row0 + r;
+        const int y = y0 + r;
         if (x < P.W && y < P.H) {
             const float inv = invs[r];
             const size_t base = ((size_t)(b * P.H + y) * P.W + x) * Ctot + h * kHeadDim;
@@ -195,37 +225,42 @@ __global__ void shift_check_kernel(const float* __restrict__ wk, const float* __
 
 template <typename T, int K>
 cudaError_t launch_t(const Problem& p, int* d_status, cudaStream_t stream) {
-    using C_ = Cfg<T, K>;
     static bool configured[64] = {};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    if (dev < 64 && !configured[dev]) {
-        e = cudaFuncSetAttribute(shift_kernel<T, K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C_::total);
+    if (dev >= 64 || !configured[dev]) {
+        const int most = (int)ShiftLayout<T, K>(kMaxTW).total;
+        e = cudaFuncSetAttribute(shift_kernel<T, K, kMaxTW>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(shift_kernel<T, K, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
         if (e != cudaSuccess) return e;
-        configured[dev] = true;
-    } else if (dev >= 64) {
-        e = cudaFuncSetAttribute(shift_kernel<T, K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C_::total);
-        if (e != cudaSuccess) return e;
+        if (dev < 64) configured[dev] = true;
     }
+    // The tile width (a multiple of 8) that takes the fewest columns, four counted for a tile's halo and start; the widest of
+    // those.  32 x 28 x 42, 6 heads: 24 columns 17.9 us, 32 20.2; 10 x 106 x 15, 5 heads: 16 columns 8.3 us, 32 10.9.
+    int tw = 8, cost = 1 << 30;
+    for (int t = 8; t <= kMaxTW; t += 8) {
+        const int c = (p.W + t - 1) / t * (t + 4);
+        if (c <= cost) { cost = c; tw = t; }
+    }
+    const ShiftLayout<T, K> L(tw);
     ShiftParams P;
-    P.wt = nullptr; P.bias = p.bias; P.out = p.out; P.status = d_status;
+    P.bias = p.bias; P.out = p.out; P.status = d_status;
     P.B = p.B; P.H = p.H; P.W = p.W; P.heads = p.heads;
-    P.tiles_x = (p.W + kTW - 1) / kTW;
-    P.tiles_y = (p.H + C_::TH - 1) / C_::TH;
+    P.tw = tw; P.tiles_x = (p.W + tw - 1) / tw; P.tiles_y = (p.H + kR - 1) / kR;
     P.scale_log2e = kLog2e / sqrtf((float)kHeadDim);
     const int Ctot = p.heads * kHeadDim;
     const int cpp = 64 / (int)sizeof(T);
     CUtensorMap mq, mk, mv;
-    if (!make_tile_map(&mq, p.q, (int)sizeof(T), p.B, p.H, p.W, Ctot, cpp, kTW, C_::TH) ||
-        !make_tile_map(&mk, p.k, (int)sizeof(T), p.B, p.H, p.W, Ctot, cpp, C_::HW, C_::HH) ||
-        !make_tile_map(&mv, p.v, (int)sizeof(T), p.B, p.H, p.W, Ctot, cpp, C_::HW, C_::HH))
+    if (!make_tile_map(&mq, p.q, (int)sizeof(T), p.B, p.H, p.W, Ctot, cpp, tw, kR) ||
+        !make_tile_map(&mk, p.k, (int)sizeof(T), p.B, p.H, p.W, Ctot, cpp, L.HW, L.HH) ||
+        !make_tile_map(&mv, p.v, (int)sizeof(T), p.B, p.H, p.W, Ctot, cpp, L.HW, L.HH))
         return cudaErrorInvalidValue;
     const long long ctas = (long long)P.tiles_x * P.tiles_y * p.B * p.heads;
     if (ctas > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
     // programmatic stream serialisation: the kernel may run beside the weight check launched just
     // before it (it does not read the check's result; both only ever set the status word)
-    return launch_chained(shift_kernel<T, K>, dim3((unsigned)ctas), C_::threads, C_::total, stream, mq, mk, mv, P);
+    return launch_chained(tw == kMaxTW ? shift_kernel<T, K, kMaxTW> : shift_kernel<T, K, 0>, dim3((unsigned)ctas), tw * 4, L.total, stream, mq, mk, mv, P);
 }
 
 template <typename T>
