@@ -306,27 +306,8 @@ bwd_point_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constan
                 const float iz = 1.f / z;
 #pragma unroll
                 for (int s = 0; s < kK2; ++s) a[s] *= iz;
-                if (!warp_wait(bar(kLFull), 1)) { ok = false; break; }
-                tc_fence_after_sync();
-                float dl[kK2], mean = 0.f;
-                load_contraction<T>(quad, dl);                       // da
-#pragma unroll
-                for (int s = 0; s < kK2; ++s) mean = fmaf(a[s], dl[s], mean);
-#pragma unroll
-                for (int s = 0; s < kK2; ++s) dl[s] = a[s] * (dl[s] - mean);
-                uint32_t row[16];
-                split_row(dl, row);
-                tmem_st_32x32b_x16(quad + kColA, row);
-                tmem_wait_st();
-                tc_fence_before_sync();
-                __syncwarp();
-                mbar_arrive_lane0(bar(kAFull), lane);
                 // lane = 8 row + column of the strip
                 const Place px = me.place(P, seat.strip0(bi) + wq, lane >> 3, lane & 7);
-                if (px.in[0]) {
-#pragma unroll
-                    for (int s = 0; s < kK2; ++s) dbias[s] += dl[s];
-                }
                 // Lanes 2i and 2i + 1 write both pieces of a 32-byte sector together: piece c of the even lane's pixel and its
                 // neighbour c + 1, then of the odd one's (16 bytes of each sector at a time took 20 of the kernel's 132 us).
                 const size_t at = (px.pix * P.heads + h) * 64, pitch = (size_t)P.heads * 64;
@@ -349,9 +330,28 @@ bwd_point_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constan
                         if (in_odd) *reinterpret_cast<uint4*>(rows + at_even + pitch + c) = make_uint4(o[0], o[1], o[2], o[3]);
                     }
                 };
-                write(P.rows_dl, row);
+                uint32_t row[16];
                 split_row(a, row);
-                write(P.rows_a, row);
+                write(P.rows_a, row);                                // while the other side's last MMAs run
+                if (!warp_wait(bar(kLFull), 1)) { ok = false; break; }
+                tc_fence_after_sync();
+                float dl[kK2], mean = 0.f;
+                load_contraction<T>(quad, dl);                       // da
+#pragma unroll
+                for (int s = 0; s < kK2; ++s) mean = fmaf(a[s], dl[s], mean);
+#pragma unroll
+                for (int s = 0; s < kK2; ++s) dl[s] = a[s] * (dl[s] - mean);
+                split_row(dl, row);
+                tmem_st_32x32b_x16(quad + kColA, row);
+                tmem_wait_st();
+                tc_fence_before_sync();
+                __syncwarp();
+                mbar_arrive_lane0(bar(kAFull), lane);
+                if (px.in[0]) {
+#pragma unroll
+                    for (int s = 0; s < kK2; ++s) dbias[s] += dl[s];
+                }
+                write(P.rows_dl, row);
             }
 
             if (bi + 1 < my_blocks) { me.walk.next(); st = me.place(P, seat.strip0(bi + 1) + wq, 2 * half, g); load_x(st, 0, 0, xn); }
