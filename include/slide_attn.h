@@ -98,8 +98,8 @@ typedef enum {
                                          head_dim 32, ksize <= 9, fp32 or bf16: what AUTO runs for fp32
                                          storage with ksize 1 or >= 5                                    */
     SLIDE_ATTN_VARIANT_UMMA_SPLIT = 11, /* fp32 arithmetic on tcgen05: operands split into parts whose bf16 / fp16
-                                         products are exact or good to 2^-22; ksize 3, head_dim 32 or 64, fp32 or
-                                         bf16: what AUTO runs for fp32 storage and for head_dim 64             */
+                                         products are exact or good to 2^-22; ksize 3, head_dim 16, 32 or 64, fp32
+                                         or bf16: what AUTO runs for fp32 storage and for head_dim 16 and 64   */
     SLIDE_ATTN_VARIANT_MMA_WIDE = 9   /* large windows with general weights: persistent warp-specialised
                                          kernel, both contractions on tcgen05, weights resident in shared
                                          memory (ksize <= 5) or streamed from L2; bf16, head_dim 32, ksize 3 / 5 / 7 / 9: what

@@ -270,7 +270,7 @@ bwd_point_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constan
                     const int pb = pn & 1;
                     uint4 y[4];
 #pragma unroll
-                    for (int r = 0; r < 4; ++r) y[r] = halo_piece(plane, 2 * half + r, g + dx, tig);
+                    for (int r = 0; r < 4; ++r) y[r] = halo_piece<T>(plane, 2 * half + r, g + dx, tig);
                     if (!warp_wait(bar(kPFree + pb), ((uint32_t)(pn >> 1) & 1u) ^ 1u)) { ok = false; break; }
                     tc_fence_after_sync();
                     const uint32_t t = mine + kColP + (uint32_t)(pb * 3 * Cut<T>::tap_cols);

@@ -46,14 +46,29 @@ constexpr float kScaleA = 8192.f;                       // softmax weights (at m
 
 // How the channels of a storage type are cut: planes of 64 bytes, chunks of one plane and one tap column.
 template <typename T> struct Cut;
+// bf16 storage with 16 channels a head.  Its planes keep the 64-byte pitch: TMA brings the next head's channels (past the
+// last head: zeros) along, which nobody reads.
+struct NarrowBf16 { __nv_bfloat16 v; };
 template <> struct Cut<__nv_bfloat16> {
+    using piece = uint4;                                // a lane's channels of a pixel
     static constexpr int channels = 32;                 // of a plane
+    static constexpr int box = 32;                      // channels that a TMA box takes
     static constexpr int per_lane = 8;
     static constexpr int d_buffers = 2;                 // N = 96 columns per tap column of a plane
     static constexpr int tap_cols = 32, h_tiles = 2;    // products are hi + lo: 2 x 3 x 32 + 2 x 16 + 32 = 256 columns
 };
-template <> struct Cut<float> {
+template <> struct Cut<NarrowBf16> {
+    using piece = uint2;
     static constexpr int channels = 16;
+    static constexpr int box = 32;
+    static constexpr int per_lane = 4;
+    static constexpr int d_buffers = 3;                 // N = 48
+    static constexpr int tap_cols = 16, h_tiles = 3;    // hi + lo: 2 x 3 x 16 + 3 x 16 + 32 = 176 columns
+};
+template <> struct Cut<float> {
+    using piece = uint4;
+    static constexpr int channels = 16;
+    static constexpr int box = 16;
     static constexpr int per_lane = 4;
     static constexpr int d_buffers = 3;                 // N = 48
     static constexpr int tap_cols = 24, h_tiles = 3;    // hi + mid + lo: 2 x 3 x 24 + 3 x 16 + 32 = 224
@@ -286,9 +301,11 @@ __device__ __forceinline__ void load_strips(uint32_t dst, const CUtensorMap* map
     }
 }
 
-// The 16 bytes of piece tig at pixel (row, column) of a halo plane.
-__device__ __forceinline__ uint4 halo_piece(const unsigned char* plane, int row, int col, int tig) {
-    return *reinterpret_cast<const uint4*>(plane + (uint32_t)(row * 10 + col) * 64u + (uint32_t)tig * 16u);
+// Piece tig at pixel (row, column) of a halo plane.
+template <typename T>
+__device__ __forceinline__ typename Cut<T>::piece halo_piece(const unsigned char* plane, int row, int col, int tig) {
+    using Piece = typename Cut<T>::piece;
+    return *reinterpret_cast<const Piece*>(plane + (uint32_t)(row * 10 + col) * 64u + (uint32_t)tig * (uint32_t)sizeof(Piece));
 }
 __device__ __forceinline__ float f4(const uint4& v, int i) {
     return __uint_as_float(i == 0 ? v.x : i == 1 ? v.y : i == 2 ? v.z : v.w);
@@ -307,6 +324,13 @@ template <> struct Factor<__nv_bfloat16> {
         }
     }
 };
+template <> struct Factor<NarrowBf16> {
+    uint2 x[2], nx[2];
+    __device__ __forceinline__ void set(const uint2 (&v)[2]) {
+#pragma unroll
+        for (int r = 0; r < 2; ++r) { x[r] = v[r]; nx[r] = make_uint2(v[r].x ^ 0x80008000u, v[r].y ^ 0x80008000u); }
+    }
+};
 template <> struct Factor<float> {
     uint4 x[2];
     __device__ __forceinline__ void set(const uint4 (&v)[2]) { x[0] = v[0]; x[1] = v[1]; }
@@ -319,6 +343,12 @@ __device__ __forceinline__ void store_products(const Factor<__nv_bfloat16>& f, u
     split::product2n(f.x[0].z, f.nx[0].z, y0.z, r[4], r[12]); split::product2n(f.x[0].w, f.nx[0].w, y0.w, r[5], r[13]);
     split::product2n(f.x[1].z, f.nx[1].z, y1.z, r[6], r[14]); split::product2n(f.x[1].w, f.nx[1].w, y1.w, r[7], r[15]);
     tmem_st_16x256b_x4(t, r);
+}
+__device__ __forceinline__ void store_products(const Factor<NarrowBf16>& f, uint32_t t, const uint2& y0, const uint2& y1) {
+    uint32_t r[8];
+    split::product2n(f.x[0].x, f.nx[0].x, y0.x, r[0], r[4]); split::product2n(f.x[0].y, f.nx[0].y, y0.y, r[1], r[5]);
+    split::product2n(f.x[1].x, f.nx[1].x, y1.x, r[2], r[6]); split::product2n(f.x[1].y, f.nx[1].y, y1.y, r[3], r[7]);
+    tmem_st_16x256b_x2(t, r);
 }
 __device__ __forceinline__ void store_products(const Factor<float>& f, uint32_t t, const uint4& y0, const uint4& y1) {
     const uint4 (&x)[2] = f.x;
@@ -343,14 +373,14 @@ __device__ __forceinline__ uint64_t contract_desc(uint32_t img) { return umma_sm
 template <typename T> __host__ __device__ constexpr uint32_t contract_step(int plane, int tap) {
     return (uint32_t)((plane * kK2 + tap) * (Cut<T>::channels / 8) * 48);          // in 16-byte units
 }
-// The MMAs of one tap, issued by one thread.  `fresh`: the first tap of a block for its H tile (f32: tile dx; bf16: both
-// tiles, one per k-step); `first`: the first tap of the block.
+// The MMAs of one tap, issued by one thread.  `fresh`: the first tap of a block for its H tile (planes of 16 channels: tile
+// dx; of 32: both tiles, one per k-step); `first`: the first tap of the block.
 template <typename T>
 __device__ __forceinline__ void issue_contract(uint32_t tmem, uint32_t p_col, uint64_t b, int dx, bool fresh, bool first) {
     constexpr uint32_t id32 = umma_idesc_bf16(128, 32), id16 = umma_idesc_bf16(128, 16);
     constexpr uint32_t mid = 16;                                             // 256 bytes on: the columns of the middle parts
     const uint32_t r = tmem + kColR, h = tmem + kColH<T>;
-    if constexpr (sizeof(T) == 2) {
+    if constexpr (Cut<T>::channels == 32) {
         constexpr uint32_t k1 = 96;                                          // 1536 bytes on: the next 16 k
         constexpr uint32_t neg32 = id32 | kIdescNegateA;
         umma_bf16_ts(h, p_col, b, id16, fresh ? 0u : 1u);
@@ -359,6 +389,10 @@ __device__ __forceinline__ void issue_contract(uint32_t tmem, uint32_t p_col, ui
         umma_bf16_ts(r, p_col + 8, b + k1 + mid, id32, 1);
         umma_bf16_ts(r, p_col + 16, b, neg32, 1);                            // lower . upper | lower . middle
         umma_bf16_ts(r, p_col + 24, b + k1, neg32, 1);
+    } else if constexpr (sizeof(T) == 2) {
+        umma_bf16_ts(h + 16 * dx, p_col, b, id16, fresh ? 0u : 1u);
+        umma_bf16_ts(r, p_col, b + mid, id32, first ? 0u : 1u);
+        umma_bf16_ts(r, p_col + 8, b, id32 | kIdescNegateA, 1);
     } else {
         umma_bf16_ts(h + 16 * dx, p_col, b, id16, fresh ? 0u : 1u);
         umma_bf16_ts(r, p_col, b + mid, id32, first ? 0u : 1u);
@@ -398,7 +432,7 @@ __device__ __forceinline__ void sum_chunk(__nv_bfloat16, uint32_t t, const unsig
     tmem_ld3_16x256b_x4_nowait(t, t + 32, t + 64, d);
     uint4 y[4];
 #pragma unroll
-    for (int r = 0; r < 4; ++r) y[r] = halo_piece(plane, row + r, col, tig);
+    for (int r = 0; r < 4; ++r) y[r] = halo_piece<__nv_bfloat16>(plane, row + r, col, tig);
     float f[4][8];
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
@@ -415,14 +449,19 @@ __device__ __forceinline__ void sum_chunk(__nv_bfloat16, uint32_t t, const unsig
                 ffma2(acc[r][2 * j], acc[r][2 * j + 1], __uint_as_float(d[16 * dy + 4 * j + 2 * r]), __uint_as_float(d[16 * dy + 4 * j + 2 * r + 1]),
                       f[r + (Transposed ? 2 - dy : dy)][2 * j], f[r + (Transposed ? 2 - dy : dy)][2 * j + 1]);
 }
-template <bool Transposed = false>
-__device__ __forceinline__ void sum_chunk(float, uint32_t t, const unsigned char* plane, int row, int col, int tig, float (&acc)[2][4]) {
+// planes of 16 channels
+template <typename T, bool Transposed>
+__device__ __forceinline__ void sum_chunk16(uint32_t t, const unsigned char* plane, int row, int col, int tig, float (&acc)[2][4]) {
     uint32_t d[3][8];
 #pragma unroll
     for (int dy = 0; dy < 3; ++dy) tmem_ld_16x256b_x2_nowait(t + 16 * dy, d[dy]);
-    uint4 y[4];
+    float f[4][4];
 #pragma unroll
-    for (int r = 0; r < 4; ++r) y[r] = halo_piece(plane, row + r, col, tig);
+    for (int r = 0; r < 4; ++r) {
+        const typename Cut<T>::piece y = halo_piece<T>(plane, row + r, col, tig);
+        if constexpr (sizeof(T) == 2) { f[r][0] = bf16_lo(y.x); f[r][1] = bf16_hi(y.x); f[r][2] = bf16_lo(y.y); f[r][3] = bf16_hi(y.y); }
+        else { f[r][0] = f4(y, 0); f[r][1] = f4(y, 1); f[r][2] = f4(y, 2); f[r][3] = f4(y, 3); }
+    }
     tmem_wait_ld();
 #pragma unroll
     for (int dy = 0; dy < 3; ++dy) {
@@ -432,8 +471,16 @@ __device__ __forceinline__ void sum_chunk(float, uint32_t t, const unsigned char
 #pragma unroll
             for (int j = 0; j < 2; ++j)
                 ffma2(acc[r][2 * j], acc[r][2 * j + 1], __uint_as_float(d[dy][4 * j + 2 * r]), __uint_as_float(d[dy][4 * j + 2 * r + 1]),
-                      f4(y[r + (Transposed ? 2 - dy : dy)], 2 * j), f4(y[r + (Transposed ? 2 - dy : dy)], 2 * j + 1));
+                      f[r + (Transposed ? 2 - dy : dy)][2 * j], f[r + (Transposed ? 2 - dy : dy)][2 * j + 1]);
     }
+}
+template <bool Transposed = false>
+__device__ __forceinline__ void sum_chunk(float, uint32_t t, const unsigned char* plane, int row, int col, int tig, float (&acc)[2][4]) {
+    sum_chunk16<float, Transposed>(t, plane, row, col, tig, acc);
+}
+template <bool Transposed = false>
+__device__ __forceinline__ void sum_chunk(NarrowBf16, uint32_t t, const unsigned char* plane, int row, int col, int tig, float (&acc)[2][4]) {
+    sum_chunk16<NarrowBf16, Transposed>(t, plane, row, col, tig, acc);
 }
 
 }  // namespace team

@@ -1,4 +1,4 @@
-// UMMA_SPLIT variant (k = 3; fp32 storage or bf16; head_dim 32 or 64): the fused forward (Eq. 2 with Eq. 12 inside)
+// UMMA_SPLIT variant (k = 3; fp32 storage or bf16; head_dim 16, 32 or 64): the fused forward (Eq. 2 with Eq. 12 inside)
 // with fp32 arithmetic, both k^4 contractions on tcgen05.  Where UMMA_TS rounds the q.k products and the softmax
 // weights to bf16, this kernel splits them, and the weights, into parts whose tensor-core products are exact
 // (split.cuh), so fp32 storage keeps its 1e-4 - in fact 1e-6 - and wide heads the accuracy of an fp32 kernel.
@@ -11,8 +11,10 @@
 // come through the team's ring.
 //
 // Bound by instruction issue and the hand-offs between the warps and the tensor core (issue slots 51 % busy, tensor pipe
-// 15 - 24 %, DRAM 13 - 16 %).  A call: 2 x 128 x 128, 3 heads, fp32: 45.3 us in tile_kernel, 30.7 here; 32 x 28 x 28,
-// 3 heads of 64, bf16: 232 us in strip_kernel, 28.3 here; 1 x 14 x 14, 1 head, fp32: 14.7 and 11.2 us.
+// 15 - 24 %, DRAM 13 - 16 %).  A call, before (the CUDA-core kernel that took the shape) and here: 2 x 128 x 128, 3 heads,
+// fp32: 45.3 us in tile_kernel, 28.5; 32 x 28 x 28, 3 heads of 64, bf16: 232 us in strip_kernel, 25.3; 1 x 14 x 14, 1 head,
+// fp32: 14.7 and 8.0 us; heads of 16, strip_kernel before: 16 x 56 x 56 x 3, bf16 197 and 16.1, fp32 184 and 22.7 us;
+// 30 x 28 x 42 x 8, bf16 449 and 30.9; 1 x 7 x 7 x 1, bf16 18.3 and 10.4.
 #include "team.cuh"
 
 namespace slide_attn {
@@ -62,6 +64,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 umma_split_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v, const SplitParams P)
 {
     using F = Fwd<T, D>;
+    using Piece = typename Cut<T>::piece;
     constexpr int NPL = F::planes, CH = Cut<T>::channels, PL = Cut<T>::per_lane, DB = Cut<T>::d_buffers, R = F::ring;
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u);
@@ -132,7 +135,7 @@ umma_split_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
 #pragma unroll
                     for (int dy = 0; dy < 3; ++dy)
                         issue_contract<T>(tmem, p_col + dy * Cut<T>::tap_cols, kdesc + contract_step<T>(plane, dy * 3 + dx), dx,
-                                          dy == 0 && (sizeof(T) == 2 ? i == 0 : plane == 0), dy == 0 && i == 0);
+                                          dy == 0 && (CH == 32 ? i == 0 : plane == 0), dy == 0 && i == 0);
                     umma_commit(bar(kPFree + pb));
                 }
                 if (!ok) break;
@@ -176,15 +179,15 @@ umma_split_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
             p.at = (((size_t)walk.b * P.H + y) * P.W + x) * C + h * D + tig * PL;
             return p;
         };
-        auto load_q = [&](const Place& p, int plane, uint4 (&x)[2]) {
+        auto load_q = [&](const Place& p, int plane, Piece (&x)[2]) {
 #pragma unroll
             for (int r = 0; r < 2; ++r) {
-                x[r] = make_uint4(0u, 0u, 0u, 0u);
-                if (p.in[r]) x[r] = __ldg(reinterpret_cast<const uint4*>(static_cast<const T*>(P.q) + p.at + r * row_pitch + plane * CH));
+                x[r] = Piece();
+                if (p.in[r]) x[r] = __ldg(reinterpret_cast<const Piece*>(static_cast<const T*>(P.q) + p.at + r * row_pitch + plane * CH));
             }
         };
         Place st = place(0);
-        uint4 qn[2];
+        Piece qn[2];
         if (my_blocks > 0) load_q(st, 0, qn);
         for (int bi = 0; bi < my_blocks; ++bi) {
             // ---- products -------------------------------------------------------------------------
@@ -197,9 +200,9 @@ umma_split_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
 #pragma unroll
                 for (int dx = 0; dx < 3; ++dx, ++pn) {
                     const int pb = pn & 1;
-                    uint4 y[4];
+                    Piece y[4];
 #pragma unroll
-                    for (int r = 0; r < 4; ++r) y[r] = halo_piece(plane, 2 * half + r, g + dx, tig);
+                    for (int r = 0; r < 4; ++r) y[r] = halo_piece<T>(plane, 2 * half + r, g + dx, tig);
                     if (!warp_wait(bar(kPFree + pb), ((uint32_t)(pn >> 1) & 1u) ^ 1u)) { ok = false; break; }
                     tc_fence_after_sync();
                     const uint32_t t = mine + kColP + (uint32_t)(pb * 3 * Cut<T>::tap_cols);
@@ -268,15 +271,15 @@ umma_split_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
 #pragma unroll
                 for (int r = 0; r < 2; ++r) {
                     if (!cur.in[r]) continue;
-                    uint4 o;
+                    Piece o;
                     if constexpr (sizeof(T) == 2) {
                         o.x = pack_bf16(acc[r][0] * sc[0], acc[r][1] * sc[1]); o.y = pack_bf16(acc[r][2] * sc[2], acc[r][3] * sc[3]);
-                        o.z = pack_bf16(acc[r][4] * sc[4], acc[r][5] * sc[5]); o.w = pack_bf16(acc[r][6] * sc[6], acc[r][7] * sc[7]);
+                        if constexpr (PL == 8) { o.z = pack_bf16(acc[r][4] * sc[4], acc[r][5] * sc[5]); o.w = pack_bf16(acc[r][6] * sc[6], acc[r][7] * sc[7]); }
                     } else {
                         o.x = __float_as_uint(acc[r][0] * sc[0]); o.y = __float_as_uint(acc[r][1] * sc[1]);
                         o.z = __float_as_uint(acc[r][2] * sc[2]); o.w = __float_as_uint(acc[r][3] * sc[3]);
                     }
-                    *reinterpret_cast<uint4*>(static_cast<T*>(P.out) + cur.at + r * row_pitch + pl * CH) = o;
+                    *reinterpret_cast<Piece*>(static_cast<T*>(P.out) + cur.at + r * row_pitch + pl * CH) = o;
                 }
             }
             if (!ok) break;
@@ -312,8 +315,8 @@ cudaError_t launch_t(const Problem& p, void* workspace, int* d_status, int num_s
     P.scale_log2e = kLog2e / sqrtf((float)D);
     CUtensorMap mk, mv;
     const int C = p.heads * D;
-    if (!make_tile_map(&mk, p.k, (int)sizeof(T), p.B, p.H, p.W, C, Cut<T>::channels, 10, 6) ||
-        !make_tile_map(&mv, p.v, (int)sizeof(T), p.B, p.H, p.W, C, Cut<T>::channels, 10, 6))
+    if (!make_tile_map(&mk, p.k, (int)sizeof(T), p.B, p.H, p.W, C, Cut<T>::box, 10, 6) ||
+        !make_tile_map(&mv, p.v, (int)sizeof(T), p.B, p.H, p.W, C, Cut<T>::box, 10, 6))
         return cudaErrorInvalidValue;
     e = launch_chained(umma_split_prep_kernel<T, D>, dim3((unsigned)p.heads, prep_parts(D)), 256, 0, stream, p.wk, p.wv, static_cast<unsigned char*>(workspace));
     if (e != cudaSuccess) return e;
@@ -328,7 +331,7 @@ cudaError_t launch_t(const Problem& p, void* workspace, int* d_status, int num_s
 }  // namespace
 
 bool umma_split_supports(int head_dim, int ksize) {
-    return (head_dim == 32 || head_dim == 64) && ksize == 3 && tensor_map_available();
+    return (head_dim == 16 || head_dim == 32 || head_dim == 64) && ksize == 3 && tensor_map_available();
 }
 
 size_t umma_split_workspace_bytes(int heads, int head_dim) {
@@ -338,9 +341,11 @@ size_t umma_split_workspace_bytes(int heads, int head_dim) {
 // Prep launch (weights -> images in `workspace`) followed by the fused kernel.
 cudaError_t launch_umma_split(const Problem& p, void* workspace, int* d_status, int num_sms, cudaStream_t stream) {
     if (p.dtype == SLIDE_ATTN_BF16)
-        return p.head_dim == 32 ? launch_t<__nv_bfloat16, 32>(p, workspace, d_status, num_sms, stream)
+        return p.head_dim == 16 ? launch_t<NarrowBf16, 16>(p, workspace, d_status, num_sms, stream)
+             : p.head_dim == 32 ? launch_t<__nv_bfloat16, 32>(p, workspace, d_status, num_sms, stream)
                                 : launch_t<__nv_bfloat16, 64>(p, workspace, d_status, num_sms, stream);
-    return p.head_dim == 32 ? launch_t<float, 32>(p, workspace, d_status, num_sms, stream)
+    return p.head_dim == 16 ? launch_t<float, 16>(p, workspace, d_status, num_sms, stream)
+         : p.head_dim == 32 ? launch_t<float, 32>(p, workspace, d_status, num_sms, stream)
                             : launch_t<float, 64>(p, workspace, d_status, num_sms, stream);
 }
 

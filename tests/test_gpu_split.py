@@ -27,7 +27,7 @@ def inputs(shape, d, dtype, sigma_w, bias=True):
 
 
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
-@pytest.mark.parametrize("d", [32, 64])
+@pytest.mark.parametrize("d", [16, 32, 64])
 @pytest.mark.parametrize("shape", SHAPES, ids=lambda s: "x".join(map(str, s)))
 def test_split_variant_matches_oracle(shape, d, dtype):
     for sigma_w, bias in ((0.05, True), (0.4, False)):
