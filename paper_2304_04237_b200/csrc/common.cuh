@@ -127,10 +127,13 @@ bool tile_supports(int head_dim, int ksize);
 cudaError_t launch_tile(const Problem& p, const void* workspace, int* d_status, cudaStream_t stream);
 
 // Projections of a block (Eq. 1 / Eq. 3) as a tcgen05 GEMM: y[i] = x w[i] for nmat row-major fp32 [c_in][c_out]
-// matrices, x and y bf16 with channels contiguous.  proj_setup must have succeeded once on the device.
+// matrices, x and y bf16 with channels contiguous.
 bool proj_supports(int c_in, int c_out);
-cudaError_t proj_setup();
-cudaError_t launch_proj(const void* x, long long rows, int c_in, const float* w, int c_out, int nmat,
+// `image`: w as launch_proj_prep laid it out (proj_image_bytes; two sets of matrices per launch), or null.
+bool proj_wants_image(long long rows, int c_in, int c_out, int nmat, int num_sms);
+size_t proj_image_bytes(int c_in, int c_out, int nmat);
+cudaError_t launch_proj_prep(const float* wa, int nmat_a, void* image_a, const float* wb, int nmat_b, void* image_b, int c_in, int c_out, cudaStream_t stream);
+cudaError_t launch_proj(const void* x, long long rows, int c_in, const float* w, const void* image, int c_out, int nmat,
                         void* const* y, int* d_status, int num_sms, cudaStream_t stream);
 
 }  // namespace slide_attn

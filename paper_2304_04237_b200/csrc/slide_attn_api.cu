@@ -22,7 +22,6 @@ struct slide_attn_ctx {
     void* wide_ws;                   // bf16 weight images of the MMA_WIDE variant
     void* bwd_ws;                    // attention weights and logit gradients between the two backward kernels (first backward)
     void* block_ws;                  // q, k, v, z of slide_attn_block_forward (first use)
-    bool proj_ready;                 // the projection kernel's attributes are set on this device
     // staging buffers for slide_attn_forward_host, allocated on first use
     void* stage;
     size_t stage_bytes;
@@ -358,19 +357,15 @@ slide_attn_status proj_check(slide_attn_ctx* c) {
     const int C = c->heads * c->head_dim;
     if (c->dtype != SLIDE_ATTN_BF16 || !proj_supports(C, C)) return SLIDE_ATTN_ERR_UNSUPPORTED;
     if ((long long)c->B * c->H * c->W > 0x7fffff00LL) return SLIDE_ATTN_ERR_UNSUPPORTED;
-    if (!c->proj_ready) {
-        if (proj_setup() != cudaSuccess) { cudaGetLastError(); return SLIDE_ATTN_ERR_CUDA; }
-        c->proj_ready = true;
-    }
     return SLIDE_ATTN_OK;
 }
 
-// Scratch of the block: four bf16 token tensors (q, k, v, z).
+// Scratch of the block: four bf16 token tensors (q, k, v, z), then the weight images of its projections.
 slide_attn_status block_scratch(slide_attn_ctx* c) {
     slide_attn_status st = proj_check(c);
     if (st != SLIDE_ATTN_OK) return st;
     if (c->block_ws) return SLIDE_ATTN_OK;
-    const size_t total = 4 * block_tensor_bytes(c);
+    const size_t total = 4 * block_tensor_bytes(c) + proj_image_bytes(c->heads * c->head_dim, c->heads * c->head_dim, 4);
     if (cudaMalloc(&c->block_ws, total) != cudaSuccess) {
         cudaGetLastError();
         c->block_ws = nullptr;
@@ -396,7 +391,7 @@ slide_attn_status slide_attn_project(slide_attn_ctx* c, const void* x, const flo
     slide_attn_status st = proj_check(c);
     if (st != SLIDE_ATTN_OK) return st;
     const int C = c->heads * c->head_dim;
-    if (launch_proj(x, (long long)c->B * c->H * c->W, C, w, C, nmat, y, c->d_status, c->num_sms,
+    if (launch_proj(x, (long long)c->B * c->H * c->W, C, w, nullptr, C, nmat, y, c->d_status, c->num_sms,
                     static_cast<cudaStream_t>(cuda_stream)) != cudaSuccess) {
         cudaGetLastError();
         return SLIDE_ATTN_ERR_CUDA;
@@ -425,7 +420,11 @@ slide_attn_status slide_attn_block_forward(slide_attn_ctx* c, const void* x, con
     void* qkv[3] = {base, base + tb, base + 2 * tb};
     void* z = base + 3 * tb;
 
-    if (launch_proj(x, rows, C, w_qkv, C, 3, qkv, c->d_status, c->num_sms, stream) != cudaSuccess) {
+    const bool images = proj_wants_image(rows, C, C, 3, c->num_sms);
+    void* img_qkv = images ? base + 4 * tb : nullptr;
+    void* img_o = images ? base + 4 * tb + proj_image_bytes(C, C, 3) : nullptr;
+    if ((images && launch_proj_prep(w_qkv, 3, img_qkv, w_o, 1, img_o, C, C, stream) != cudaSuccess) ||
+        launch_proj(x, rows, C, w_qkv, img_qkv, C, 3, qkv, c->d_status, c->num_sms, stream) != cudaSuccess) {
         cudaGetLastError();
         return SLIDE_ATTN_ERR_CUDA;
     }
@@ -436,7 +435,7 @@ slide_attn_status slide_attn_block_forward(slide_attn_ctx* c, const void* x, con
     st = launch_problem(c, p, stream, false);
     if (st != SLIDE_ATTN_OK) return st;
     void* ys[1] = {out};
-    if (launch_proj(z, rows, C, w_o, C, 1, ys, c->d_status, c->num_sms, stream) != cudaSuccess) {
+    if (launch_proj(z, rows, C, w_o, img_o, C, 1, ys, c->d_status, c->num_sms, stream) != cudaSuccess) {
         cudaGetLastError();
         return SLIDE_ATTN_ERR_CUDA;
     }

@@ -156,6 +156,32 @@ def test_block_forward_full_size_every_element():
     print(f"block c2: worst error {worst:.3e}")
 
 
+@pytest.mark.parametrize("shape", [(1, 1, 1, 8, 32), (1, 14, 14, 8, 32), (1, 13, 19, 15, 16), (1, 170, 150, 7, 16), (1, 150, 170, 7, 32)],
+                         ids=lambda s: "x".join(map(str, s)))
+def test_block_is_its_three_stages(shape):
+    """The block lays its projection weights out in a launch of their own, slide_attn_project in every CTA: the same products
+    in the same order, so the block must equal project, forward, project bit for bit (both unit widths, one and several
+    column groups, several tiles per CTA)."""
+    B, H, W, heads, d = shape
+    C = heads * d
+    gen = torch.Generator(device="cuda").manual_seed(zlib.crc32(repr(shape).encode()))
+    x = torch.randn(B, H, W, C, device="cuda", generator=gen).to(torch.bfloat16)
+    w_qkv = torch.randn(3, C, C, device="cuda", generator=gen) / C ** 0.5
+    w_o = torch.randn(C, C, device="cuda", generator=gen) / C ** 0.5
+    wk, wv = (torch.randn(C, 9, 9, device="cuda", generator=gen) * 0.05 for _ in range(2))
+    got, q, k, v, z, want = (torch.full_like(x, float("nan")) for _ in range(6))
+    ctx = sa.slide_attn_create(B, H, W, heads, d, 3, torch.bfloat16, False)
+    try:
+        sa.slide_attn_block_forward(ctx, x, w_qkv, w_o, wk, wv, None, got)
+        sa.slide_attn_project(ctx, x, w_qkv, [q, k, v])
+        sa.slide_attn_forward(ctx, q, k, v, wk, wv, None, z)
+        sa.slide_attn_project(ctx, z, w_o.unsqueeze(0).contiguous(), [want])
+        assert sa.slide_attn_query_status(ctx) == sa.OK
+    finally:
+        sa.slide_attn_destroy(ctx)
+    assert torch.isfinite(got.float()).all() and torch.equal(got, want)
+
+
 def test_block_argument_errors():
     ctx = sa.slide_attn_create(1, 4, 4, 1, 32, 3, torch.bfloat16, False)
     x = torch.zeros((1, 4, 4, 32), dtype=torch.bfloat16, device="cuda")
