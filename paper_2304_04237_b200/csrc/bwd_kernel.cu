@@ -1,8 +1,9 @@
 // Backward pass of the fused forward (training through the module, Sec. 4.3 / Fig. 4 (1); the paper
 // prints no backward formulas: these are the derivatives of Eq. 2 with the depthwise convolution of
-// Eq. 12 inside).  head_dim 32, k = 1 or 3, fp32 or bf16 storage, fp32 arithmetic on the CUDA cores,
-// staged like tile_kernel (TMA halo tiles in 64-byte channel planes, lane = column g x the eight
-// channels of piece tig, a warp = 8 columns x 4 rows).  With g = d(loss)/d(out):
+// Eq. 12 inside).  head_dim 32, fp32 or bf16 storage.  The dispatch for k = 3 (bwd_team_kernel.cu, bwd_weight_umma_kernel.cu,
+// bwd_weight_kernel.cu) and the kernels for k = 1: fp32 arithmetic on the CUDA cores, staged like tile_kernel (TMA halo
+// tiles in 64-byte channel planes, lane = column g x the eight channels of piece tig, a warp = 8 columns x 4 rows).
+// With g = d(loss)/d(out):
 //
 //   forward again   a = softmax_s( scale * sum_{t,c} q[c] k_t[c] wk[c,s,t] + bias[s] )
 //   da[s]   = sum_{t,c} g[c] v_t[c] wv[c,s,t]                 (the logit contraction with g, v, wv)
@@ -16,9 +17,8 @@
 // Three kernels.  bwd_point_kernel does what belongs to the query pixel: a, dl (kept in a workspace for
 // the other two), dq and the bias gradient.  bwd_gather_kernel computes dk and dv per key / value pixel by
 // gathering from the k x k query pixels whose windows hold it (out-of-map queries contribute nothing:
-// their q, g tiles read as zero).  The weight gradients: for k = 3 on the tensor cores (bwd_weight_kernel.cu); for
-// k = 1, where there is nothing to contract, bwd_weight_kernel here (persistent CTAs, one head each) sums them over
-// the pixels with lane = channel, so that a lane's 2 k^4 accumulators live in registers over all its tiles; one
+// their q, g tiles read as zero).  bwd_weight_kernel (persistent CTAs, one head each) sums the weight gradients over the
+// pixels with lane = channel, so that a lane's 2 k^4 accumulators live in registers over all its tiles; one
 // addition per weight and CTA goes to global memory at its end.
 #include "bwd_common.cuh"
 #include "tile_common.cuh"

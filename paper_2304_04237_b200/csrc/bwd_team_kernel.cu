@@ -12,6 +12,10 @@
 // operand of tap t is the split rows of the block's pixels moved by -off(t): every tap has rows of its own, copied from a halo
 // in shared memory to tensor memory (out-of-map queries read as zero and contribute nothing), N = the channels of a plane.
 // Both persistent, one CTA per SM and one head per CTA, two teams; geometry and hand-offs as in umma_split_kernel.
+//
+// Bound by instruction issue on the CUDA cores: products and their splits, sums, the point kernel's softmax, dL and row splits
+// (62 M warp instructions at 64 x 56 x 56, 3 heads, bf16; gather 46 M).  There, in CUDA-core kernels before and here: point 333 and
+// 125 us, gather 227 and 82; 2 x 128 x 128, 3 heads, fp32: point 69 and 48, gather 54 and 24 us.
 #include "bwd_common.cuh"
 #include "team.cuh"
 
@@ -239,9 +243,15 @@ bwd_point_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constan
         for (int s = 0; s < kK2; ++s) dbias[s] = 0.f;
         int slot = 0, pn = 0, dn = 0;
         uint32_t phase = 0;
+        const uint32_t zero = (uint32_t)(P.H >> 31);
         auto release = [&]() {
             __syncwarp();
             mbar_arrive_lane0(bar(kEmpty + slot), lane);
+            if (++slot == R) { slot = 0; phase ^= 1u; }
+        };
+        auto release_after = [&](float a, float b) {                // the sums a and b hold what was read from it
+            __syncwarp();
+            mbar_arrive_lane0_after(bar(kEmpty + slot), lane, a, b, zero);
             if (++slot == R) { slot = 0; phase ^= 1u; }
         };
         auto load_x = [&](const Place& p, int side, int plane, uint4 (&x)[2]) {
@@ -376,7 +386,7 @@ bwd_point_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constan
                     mbar_arrive_lane0(bar(kDFree + db), lane);
                 }
                 if (!ok) break;
-                release();
+                release_after(acc[0][0], acc[1][0]);
 #pragma unroll
                 for (int r = 0; r < 2; ++r)
                     if (cur.in[r]) store_piece(static_cast<T*>(P.dq) + cur.pix * C + piece + pl * CH + r * row_pitch, acc[r], P.scale);
@@ -534,7 +544,7 @@ bwd_gather_kernel(const __grid_constant__ CUtensorMap map_dl, const __grid_const
                     tc_fence_before_sync();
                     __syncwarp();
                     mbar_arrive_lane0(bar(kDFree + db), lane);
-                    if (dx == 2) mbar_arrive_lane0(bar(kEmpty + ps), lane);
+                    if (dx == 2) mbar_arrive_lane0_after(bar(kEmpty + ps), lane, acc[pl][0][0], acc[pl][1][0], (uint32_t)(P.H >> 31));
                     ahead(ps, pp, 1);
                 }
                 if (!ok) break;

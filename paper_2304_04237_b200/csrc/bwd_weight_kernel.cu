@@ -225,8 +225,12 @@ bwd_weight_mma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
                     if (++pending == kFlush) { pending = 0; flush(); }
                 }
             }
+            // tiles 0 and 2 of a tap have taken in everything that was loaded for it (tile 0 may just have moved to its sum)
+            uint32_t read = 0;
+#pragma unroll
+            for (int t = 0; t < 3; ++t) read |= __float_as_uint(acc[t][0][0]) | __float_as_uint(sum[t][0][0]) | __float_as_uint(acc[t][2][0]);
             __syncwarp();
-            if (lane == 0) mbar_arrive(bar_empty(st));
+            mbar_arrive_lane0_after(bar_empty(st), lane, __uint_as_float(read), 0.f, (uint32_t)(P.H >> 31));
         }
         flush();
     }

@@ -443,9 +443,15 @@ mma_wide_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant
         };
         int slot = 0, pb = 0, db = 0;
         uint32_t phase = 0, pphase = 1, dphase = 0;
+        const uint32_t zero = (uint32_t)(P.H >> 31);
         auto release = [&]() {
             __syncwarp();
             mbar_arrive_lane0(bar(kEmpty + slot), lane);
+            if (++slot == R) { slot = 0; phase ^= 1u; }
+        };
+        auto release_after = [&](float a, float b) {                // the sums a and b hold what was read from it
+            __syncwarp();
+            mbar_arrive_lane0_after(bar(kEmpty + slot), lane, a, b, zero);
             if (++slot == R) { slot = 0; phase ^= 1u; }
         };
         Place cur = place(0);
@@ -516,7 +522,7 @@ mma_wide_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant
                 }
             }
             if (!ok) break;
-            release();
+            release_after(acc[0][0], acc[1][0]);
 #pragma unroll
             for (int r = 0; r < 2; ++r)
                 if (out.in[r])

@@ -67,6 +67,14 @@ __device__ __forceinline__ void mbar_arrive_lane0(uint32_t bar, int lane) {
         "@p mbarrier.arrive.shared::cta.b64 _, [%0];\n\t}" ::"r"(bar), "r"(lane) : "memory");
 }
 
+// The same once a and b have arrived in registers.  An arrival that hands shared memory back to TMA has to come after the
+// loads from it are DONE; sums that only registers wait for may be scheduled behind it, and with them the wait for the loads that
+// feed them (fp32 heads of 64 lost a few pixels of a plane in one of a hundred runs that way).  `zero` is 0, which the compiler
+// must not know.
+__device__ __forceinline__ void mbar_arrive_lane0_after(uint32_t bar, int lane, float a, float b, uint32_t zero) {
+    mbar_arrive_lane0(bar + ((__float_as_uint(a) | __float_as_uint(b)) & zero), lane);
+}
+
 __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map, uint32_t bar,
                                             int c0, int c1, int c2, int c3) {
     asm volatile(

@@ -1,5 +1,5 @@
-// STRIP variant: the generic fp32 path for every shape the tensor-core variants do not take (other
-// window sizes, other head widths, fp32 storage).  Same arithmetic as DIRECT (Eq. 2 with Eq. 12
+// STRIP variant: the generic fp32 path for every shape the tensor-core variants and TILE do not take (head
+// widths other than 32 with k != 3, widths other than 16, 32 and 64).  Same arithmetic as DIRECT (Eq. 2 with Eq. 12
 // inside, no re-association), organised so that the CUDA cores are fed from registers and
 // coalesced loads:
 //   * a prep kernel transposes both weight tensors from [C][slot][tap] to [slot][tap][C], so that a

@@ -2,8 +2,8 @@
 // head_dim 32, k <= 9, fp32 or bf16 storage, staged like the fixed-shift kernel: the K and V tile + halo
 // and the q tile come in by TMA into shared memory (zero fill = the padding), every access to them is a
 // conflict-free 16-byte load, the output goes out in 16-byte stores, and all arithmetic is fp32 on the
-// CUDA cores (packed FMAs).  It is what AUTO runs where the tensor-core kernel does not apply (fp32
-// storage, k >= 5).
+// CUDA cores (packed FMAs).  It is what AUTO runs where no tensor-core kernel applies (k = 1;
+// fp32 storage with k = 5, 7, 9).
 //
 // Per lane (column g, the eight channels of piece tig) and sub-strip of RS pixel rows, the convolution
 // is never formed per slot; it is re-associated with the q.k product and with the attention weights:

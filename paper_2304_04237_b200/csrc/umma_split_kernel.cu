@@ -162,9 +162,15 @@ umma_split_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
 
         int slot = 0, pn = 0, dn = 0;
         uint32_t phase = 0;
+        const uint32_t zero = (uint32_t)(P.H >> 31);
         auto release = [&]() {                                       // the plane at `slot` has been read
             __syncwarp();
             mbar_arrive_lane0(bar(kEmpty + slot), lane);
+            if (++slot == R) { slot = 0; phase ^= 1u; }
+        };
+        auto release_after = [&](float a, float b) {                // the sums a and b hold what was read from it
+            __syncwarp();
+            mbar_arrive_lane0_after(bar(kEmpty + slot), lane, a, b, zero);
             if (++slot == R) { slot = 0; phase ^= 1u; }
         };
         // the lane's first pixel: element offset of its piece, and which of its two rows are inside (past the last strip: none)
@@ -263,7 +269,7 @@ umma_split_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
                     mbar_arrive_lane0(bar(kDFree + db), lane);
                 }
                 if (!ok) break;
-                release();
+                release_after(acc[0][0], acc[1][0]);
                 const float* inv = reinterpret_cast<const float*>(smem + F::w_off + contract_bytes(D) + expand_image_bytes(D)) + pl * CH + tig * PL;
                 float sc[PL];
 #pragma unroll

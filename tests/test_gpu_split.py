@@ -7,6 +7,7 @@ import zlib
 
 import numpy as np
 import pytest
+import torch
 
 import oracle
 import paper_2304_04237_b200 as sa
@@ -56,3 +57,23 @@ def test_split_variant_is_repeatable(dtype):
     x = inputs((5, 30, 33, 3), 64, dtype, 0.05)
     a, b = (gpu_forward(x, 3, dtype, sa.VARIANT_UMMA_SPLIT) for _ in range(2))
     assert np.array_equal(a, b)
+
+
+def test_split_variant_many_calls_same_bits():
+    """Four planes a head through a ring of four slots: a slot handed back to TMA before its loads were done lost pixels of a
+    plane in one call of about a hundred."""
+    gen = torch.Generator(device="cuda").manual_seed(11)
+    q, k, v = (torch.randn(19, 28, 28, 8, 64, device="cuda", generator=gen) for _ in range(3))
+    wk, wv = (torch.randn(512, 9, 9, device="cuda", generator=gen) * 0.05 for _ in range(2))
+    ctx = sa.slide_attn_create(19, 28, 28, 8, 64, 3, torch.float32, False)
+    try:
+        sa.slide_attn_set_variant(ctx, sa.VARIANT_UMMA_SPLIT)
+        want, got = torch.empty_like(q), torch.empty_like(q)
+        sa.slide_attn_forward(ctx, q, k, v, wk, wv, None, want)
+        wrong = torch.zeros((), dtype=torch.int64, device="cuda")
+        for _ in range(1500):
+            sa.slide_attn_forward(ctx, q, k, v, wk, wv, None, got)
+            wrong += (got != want).any()
+        assert int(wrong) == 0 and sa.slide_attn_query_status(ctx) == sa.OK
+    finally:
+        sa.slide_attn_destroy(ctx)
