@@ -6,6 +6,8 @@
 
 using namespace slide_attn;
 
+constexpr int kArenas = 6;
+
 struct slide_attn_ctx {
     int B, H, W, heads, head_dim, ksize, has_bias;
     slide_attn_dtype dtype;
@@ -14,7 +16,7 @@ struct slide_attn_ctx {
     int device;
     int num_sms;
     int* d_status;                   // device status word (0 = ok)
-    void* arena;                     // one allocation: the status word and the five workspaces that follow
+    void* arena[kArenas];            // what holds the status word and the five workspaces that follow (see slide_attn_create)
     void* workspace;                 // weight fragments of the MMA variant
     void* strip_ws;                  // transposed weights of the STRIP variant
     void* umma_ws;                   // bf16 B images of the UMMA_TS variant
@@ -182,23 +184,34 @@ slide_attn_status slide_attn_create(slide_attn_ctx** ctx, int B, int H, int W, i
         slide_attn_destroy(c);
         return SLIDE_ATTN_ERR_CUDA;
     }
-    // the status word and every variant's workspace in one allocation: each cudaMalloc is tens of microseconds of a create
+    // The status word and every variant's workspace, in as few allocations as stay within 1 MB, or in one if a part is larger by
+    // itself: a cudaMalloc is microseconds of a create up to 1 MB, hundreds above.  (8 heads of 32, bf16, k = 3, 1.1 MB in all:
+    // 328 us in one, 19 in six, 16 here; 3 heads, k = 7: 630 in six, of which two are larger, 325 in one.)
     auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
-    const size_t b_mma = mma_supports(dtype, head_dim, ksize) ? up(mma_workspace_bytes(heads)) : 0;
-    const size_t b_umma = mma_supports(dtype, head_dim, ksize) ? up(umma_ts_workspace_bytes(heads)) : 0;
-    const size_t b_split = umma_split_supports(head_dim, ksize) ? up(umma_split_workspace_bytes(heads, head_dim)) : 0;
-    const size_t b_wide = mma_wide_supports(dtype, head_dim, ksize) ? up(mma_wide_workspace_bytes(heads, ksize)) : 0;
-    const size_t b_strip = strip_supports(head_dim, ksize) ? up(strip_workspace_bytes(heads, head_dim, ksize)) : 0;
-    if (cudaMalloc(&c->arena, 256 + b_mma + b_umma + b_split + b_wide + b_strip) != cudaSuccess) {
-        cudaGetLastError();
-        c->arena = nullptr;
-        slide_attn_destroy(c);
-        return SLIDE_ATTN_ERR_ALLOC;
+    const struct { void** at; size_t bytes; } parts[] = {
+        {reinterpret_cast<void**>(&c->d_status), 256},
+        {&c->workspace, mma_supports(dtype, head_dim, ksize) ? up(mma_workspace_bytes(heads)) : 0},
+        {&c->umma_ws, mma_supports(dtype, head_dim, ksize) ? up(umma_ts_workspace_bytes(heads)) : 0},
+        {&c->split_ws, umma_split_supports(head_dim, ksize) ? up(umma_split_workspace_bytes(heads, head_dim)) : 0},
+        {&c->wide_ws, mma_wide_supports(dtype, head_dim, ksize) ? up(mma_wide_workspace_bytes(heads, ksize)) : 0},
+        {&c->strip_ws, strip_supports(head_dim, ksize) ? up(strip_workspace_bytes(heads, head_dim, ksize)) : 0}};
+    constexpr int kParts = (int)(sizeof(parts) / sizeof(parts[0]));
+    static_assert(kParts == kArenas, "an allocation per part at most");
+    size_t limit = 1u << 20;
+    for (const auto& part : parts)
+        if (part.bytes > limit) limit = ~(size_t)0;
+    for (int i = 0, n = 0, j; i < kParts; i = j, ++n) {
+        size_t bytes = parts[i].bytes;
+        for (j = i + 1; j < kParts && bytes + parts[j].bytes <= limit; ++j) bytes += parts[j].bytes;
+        if (cudaMalloc(&c->arena[n], bytes) != cudaSuccess) {
+            cudaGetLastError();
+            c->arena[n] = nullptr;
+            slide_attn_destroy(c);
+            return SLIDE_ATTN_ERR_ALLOC;
+        }
+        unsigned char* at = static_cast<unsigned char*>(c->arena[n]);
+        for (int k = i; k < j; ++k) { *parts[k].at = parts[k].bytes ? at : nullptr; at += parts[k].bytes; }
     }
-    unsigned char* at = static_cast<unsigned char*>(c->arena);
-    c->d_status = reinterpret_cast<int*>(at); at += 256;
-    auto take = [&](size_t bytes) { void* w = bytes ? at : nullptr; at += bytes; return w; };
-    c->workspace = take(b_mma); c->umma_ws = take(b_umma); c->split_ws = take(b_split); c->wide_ws = take(b_wide); c->strip_ws = take(b_strip);
     if (cudaMemset(c->d_status, 0, sizeof(int)) != cudaSuccess) {
         cudaGetLastError();
         slide_attn_destroy(c);
@@ -573,7 +586,8 @@ slide_attn_status slide_attn_destroy(slide_attn_ctx* c)
 {
     if (!c) return SLIDE_ATTN_OK;
     bool ok = true;
-    if (c->arena) ok &= cudaFree(c->arena) == cudaSuccess;
+    for (void* a : c->arena)
+        if (a) ok &= cudaFree(a) == cudaSuccess;
     if (c->bwd_ws) ok &= cudaFree(c->bwd_ws) == cudaSuccess;
     if (c->block_ws) ok &= cudaFree(c->block_ws) == cudaSuccess;
     if (c->stage) ok &= cudaFree(c->stage) == cudaSuccess;
