@@ -8,9 +8,12 @@
 //   L[p,s]     += sum_c P[p,(t,c)] D_k[c,s,t]             per tap M = 128, N = slots (rounded up to 16), K = 32
 //   L[p,t]     += sum_c P[p,(t,c)]                        one-hot part: N = 16 columns around t against a column of ones, which
 //                                                         a window sliding over [0 .. 0 1 0 .. 0] puts at any column
-//   a[s]        = softmax(L scale + bias), kept as a_hi + a_lo (two bf16)
-//   A'[p,(t,c)] = sum_s a_hi[p,s] D_v[c,s,t] + (a_hi + a_lo)[p,t]          N = 32 per tap, K = slots; then K = 16 around t, twice
-//   out[p,c]    = sum_t A'[p,t,c] v[p+off(t),c]           packed fp32 FMAs
+//   e[s]        = exp(L scale + bias - the largest of them), kept as e_hi + e_lo (two bf16)
+//   A'[p,(t,c)] = sum_s e_hi[p,s] D_v[c,s,t] + (e_hi + e_lo)[p,t]          N = 32 per tap, K = slots; then K = 16 around t, twice
+//   out[p,c]    = (sum_t A'[p,t,c] v[p+off(t),c]) / sum_s e[s]              packed fp32 FMAs
+// The weights are divided by their sum at the end only: the largest e is 1, which bf16 holds exactly, whereas a normalised
+// weight is rounded like any other (error of the result against 64 bits, 2 x 56 x 56 x 2, k = 7, one-hot weights + N(0, 0.21): 3.61e-3,
+// with normalised weights 3.78e-3).
 // 2 k^4 multiply-adds per pixel-channel go to the tensor cores; the CUDA cores keep 2 k^2.
 //
 // Persistent, one CTA per SM, one head per CTA; two teams of eight warps, each with its own block of 128 pixels = two TILES of
@@ -21,7 +24,7 @@
 // k <= 5 (102 KB at k = 5), so the teams run independently and cover each other's hand-offs; for k >= 7 (400 KB, 1 MB) they are
 // streamed from L2 through a ring that both teams read, 256 pixels per pass over them.
 //
-// Tensor-memory columns of a team (256): logits, later a (chunk of 16 slots: 8 columns a_hi, 8 a_lo, where its logits were), in
+// Tensor-memory columns of a team (256): logits, later e (chunk of 16 slots: 8 columns e_hi, 8 e_lo, where its logits were), in
 // the last N; below them the product groups, later the A' groups.  A group = up to GK (GV) taps of one tap column.
 //
 // A call: 64 x 56 x 56, 3 heads, k = 5: 273 us with mma.sync (every CUDA-core multiply beside it cost it pipe time, and every
@@ -40,6 +43,7 @@ constexpr int kMmaWarp = kComputeWarps, kTmaWarp = kMmaWarp + kTeams, kWeightWar
 constexpr int kThreads = (kWeightWarp + 1) * 32;
 constexpr uint32_t kOnesBytes = 2 * 512;                 // [two 8-channel chunks][31 rows of 16 bytes], row 15 ones
 constexpr uint32_t kUnitBytes = 4 * 10 * 128;            // [four groups of 8 columns][zeros, ones in k = 0 .. 7, zeros]
+constexpr uint32_t kInvBytes = kTeams * 128 * 4;         // 1 / sum of the weights of each pixel
 constexpr uint32_t kMaxSmem = 227 * 1024;
 
 // barriers of a team, then those of the weights
@@ -64,11 +68,11 @@ struct Wide {
     static constexpr uint32_t weights = 2u * K2 * tap;   // of a head
     static constexpr uint32_t chunk = (uint32_t)(GK > GV ? GK : GV) * tap;
     static constexpr uint32_t w_bytes = resident ? weights : 3 * chunk;
-    static constexpr uint32_t misc = kOnesBytes + kUnitBytes + 336 + 8u * kBars + 16;
+    static constexpr uint32_t misc = kOnesBytes + kUnitBytes + 336 + kInvBytes + 8u * kBars + 16;
     static constexpr int ring = least(3, (int)((kMaxSmem - w_bytes - misc - 128) / (kTeams * slot)));
     static_assert(ring >= 2, "the ring does not fit");
     static constexpr uint32_t w_off = (uint32_t)(kTeams * ring) * slot, ones_off = w_off + w_bytes, unit_off = ones_off + kOnesBytes,
-                              bias_off = unit_off + kUnitBytes, bar_off = bias_off + 336, tmem_off = bar_off + 8u * kBars,
+                              bias_off = unit_off + kUnitBytes, inv_off = bias_off + 336, bar_off = inv_off + kInvBytes, tmem_off = bar_off + 8u * kBars,
                               total = tmem_off + 16 + 128;
 };
 
@@ -184,9 +188,9 @@ __device__ __forceinline__ void sum_group(uint32_t t, const unsigned char* src, 
     }
 }
 
-// Softmax of the lane's pixel, whose N logits start at tensor-memory column `col`; leaves a_hi, a_lo in their place.
+// Softmax of the lane's pixel, whose N logits start at tensor-memory column `col`; leaves e_hi, e_lo in their place, returns 1 / sum.
 template <int K>
-__device__ __forceinline__ void softmax_in_place(uint32_t col, const float* s_bias, float scale_log2e) {
+__device__ __forceinline__ float softmax_in_place(uint32_t col, const float* s_bias, float scale_log2e) {
     using Wd = Wide<K>;
     constexpr int K2 = Wd::K2, KS = Wd::KS;
     constexpr bool keep = KS <= 2;                       // the logits stay in registers between the passes
@@ -212,7 +216,6 @@ __device__ __forceinline__ void softmax_in_place(uint32_t col, const float* s_bi
         for (int i = 0; i < 16; ++i)
             if (16 * j + i < K2) z += fast_exp2(v[i] - m);
     }
-    m += __log2f(z);
 #pragma unroll
     for (int j = 0; j < KS; ++j) {
         float (&v)[16] = l[keep ? j : 0];
@@ -227,6 +230,7 @@ __device__ __forceinline__ void softmax_in_place(uint32_t col, const float* s_bi
         tmem_st_32x32b_x16(col + 16 * j, row);
     }
     tmem_wait_st();
+    return 1.f / z;
 }
 
 template <int K>
@@ -444,6 +448,7 @@ mma_wide_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant
         int slot = 0, pb = 0, db = 0;
         uint32_t phase = 0, pphase = 1, dphase = 0;
         const uint32_t zero = (uint32_t)(P.H >> 31);
+        float* inv = reinterpret_cast<float*>(smem + Wd::inv_off) + 128 * team_id + 32 * wq;      // of the quadrant's pixels
         auto release = [&]() {
             __syncwarp();
             mbar_arrive_lane0(bar(kEmpty + slot), lane);
@@ -489,7 +494,7 @@ mma_wide_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant
             if (half == (bi & 1)) {
                 if (!warp_wait(bar(kLFull), (uint32_t)bi & 1u)) { ok = false; break; }
                 tc_fence_after_sync();
-                softmax_in_place<K>(quad + kColL, s_bias, P.scale_log2e);
+                inv[lane] = softmax_in_place<K>(quad + kColL, s_bias, P.scale_log2e);
                 tc_fence_before_sync();
                 __syncwarp();
                 mbar_arrive_lane0(bar(kAFull), lane);
@@ -523,11 +528,15 @@ mma_wide_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant
             }
             if (!ok) break;
             release_after(acc[0][0], acc[1][0]);
+            if (!warp_wait(bar(kAFull), (uint32_t)bi & 1u)) { ok = false; break; }        // long complete: orders the reads of inv
 #pragma unroll
             for (int r = 0; r < 2; ++r)
-                if (out.in[r])
-                    *reinterpret_cast<uint4*>(P.out + out.at + r * row_pitch) = make_uint4(pack_bf16(acc[r][0], acc[r][1]), pack_bf16(acc[r][2], acc[r][3]),
-                                                                                          pack_bf16(acc[r][4], acc[r][5]), pack_bf16(acc[r][6], acc[r][7]));
+                if (out.in[r]) {
+                    const float s = inv[16 * half + 8 * r + g];
+                    *reinterpret_cast<uint4*>(P.out + out.at + r * row_pitch) =
+                        make_uint4(pack_bf16(acc[r][0] * s, acc[r][1] * s), pack_bf16(acc[r][2] * s, acc[r][3] * s),
+                                   pack_bf16(acc[r][4] * s, acc[r][5] * s), pack_bf16(acc[r][6] * s, acc[r][7] * s));
+                }
         }
         if (!ok && lane == 0) atomicExch(P.status, 1);
     }
