@@ -201,20 +201,16 @@ __device__ __forceinline__ float softmax_in_place(uint32_t col, const float* s_b
         for (int i = 0; i < 16; ++i)
             if (16 * j + i < K2) v[i] = fmaf(v[i], scale_log2e, s_bias[16 * j + i]);
     };
+    // the largest of all slots first: a running one is -inf while all slots so far are masked by a bias of -inf, and exp2(-inf + inf)
+    // is not a number
     float m = -INFINITY, z = 0.f;
 #pragma unroll
     for (int j = 0; j < KS; ++j) {
         float (&v)[16] = l[keep ? j : 0];
         load(j, v);
-        float most = m;
 #pragma unroll
         for (int i = 0; i < 16; ++i)
-            if (16 * j + i < K2) most = fmaxf(most, v[i]);
-        z *= fast_exp2(m - most);
-        m = most;
-#pragma unroll
-        for (int i = 0; i < 16; ++i)
-            if (16 * j + i < K2) z += fast_exp2(v[i] - m);
+            if (16 * j + i < K2) m = fmaxf(m, v[i]);
     }
 #pragma unroll
     for (int j = 0; j < KS; ++j) {
@@ -223,9 +219,10 @@ __device__ __forceinline__ float softmax_in_place(uint32_t col, const float* s_b
         uint32_t row[16];
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
-            const float a0 = 16 * j + 2 * i < K2 ? fast_exp2(v[2 * i] - m) : 0.f, a1 = 16 * j + 2 * i + 1 < K2 ? fast_exp2(v[2 * i + 1] - m) : 0.f;
-            row[i] = pack_bf16(a0, a1);
-            row[8 + i] = pack_bf16(a0 - bf16_lo(row[i]), a1 - bf16_hi(row[i]));
+            const float e0 = 16 * j + 2 * i < K2 ? fast_exp2(v[2 * i] - m) : 0.f, e1 = 16 * j + 2 * i + 1 < K2 ? fast_exp2(v[2 * i + 1] - m) : 0.f;
+            z += e0; z += e1;
+            row[i] = pack_bf16(e0, e1);
+            row[8 + i] = pack_bf16(e0 - bf16_lo(row[i]), e1 - bf16_hi(row[i]));
         }
         tmem_st_32x32b_x16(col + 16 * j, row);
     }
