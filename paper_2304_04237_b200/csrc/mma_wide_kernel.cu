@@ -203,8 +203,9 @@ __device__ __forceinline__ float softmax_in_place(uint32_t col, const float* s_b
     };
     // the largest of all slots first: a running one is -inf while all slots so far are masked by a bias of -inf, and exp2(-inf + inf)
     // is not a number
+    // (k >= 7, unrolled: registers spill, 61.6 us instead of 60.0 at 2 x 128 x 128, 3 heads, k = 7)
     float m = -INFINITY, z = 0.f;
-#pragma unroll
+#pragma unroll (keep ? KS : 1)
     for (int j = 0; j < KS; ++j) {
         float (&v)[16] = l[keep ? j : 0];
         load(j, v);
@@ -212,7 +213,7 @@ __device__ __forceinline__ float softmax_in_place(uint32_t col, const float* s_b
         for (int i = 0; i < 16; ++i)
             if (16 * j + i < K2) m = fmaxf(m, v[i]);
     }
-#pragma unroll
+#pragma unroll (keep ? KS : 1)
     for (int j = 0; j < KS; ++j) {
         float (&v)[16] = l[keep ? j : 0];
         if (!keep) load(j, v);
