@@ -26,7 +26,7 @@ namespace {
 using namespace team;
 
 constexpr int kHeadDim = 32;
-constexpr uint32_t kContract = contract_bytes(kHeadDim), kExpand = expand3_bytes(kHeadDim);
+constexpr uint32_t kContract = contract_bytes(kHeadDim), kExpand = expand_bytes(kHeadDim);
 // per head: contraction images of wk and wv, expansion images of wk and wv
 constexpr uint32_t kImages = 2 * kContract + 2 * kExpand;
 constexpr uint32_t kPointImages = 2 * kContract + kExpand, kGatherImages = 2 * kExpand, kGatherFrom = 2 * kContract;
@@ -76,7 +76,7 @@ bwd_prep_kernel(const float* __restrict__ wk, const float* __restrict__ wv, unsi
         const int side = i >= contract_items + expand_items, j = side ? i - contract_items - expand_items : i;
         const float* src = (side ? wv : wk) + w;
         if (j < contract_items) build_contract_item<T>(src, img + side * kContract, j);
-        else build_expand3_item<T>(src, img + 2 * kContract + side * kExpand, j - contract_items);
+        else build_expand_item<T>(src, img + 2 * kContract + side * kExpand, j - contract_items);
     }
     for (int i = at; i < kHeadDim * kK2 * kK2; i += step) { dwk[w + i] = 0.f; dwv[w + i] = 0.f; }
     if (dbias && at < kK2) dbias[blockIdx.x * kK2 + at] = 0.f;
@@ -225,7 +225,7 @@ bwd_point_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constan
                     const int db = dn % DB;
                     if (!mbar_wait(bar(kDFree + db), ((uint32_t)(dn / DB) & 1u) ^ 1u)) { ok = false; break; }
                     tc_fence_after_sync();
-                    issue_expand3<3 * CH>(tmem + kColD + (uint32_t)(db * 3 * CH), tmem + kColA, dsrc + (uint32_t)(i * 3 * CH * 128));
+                    issue_expand<3 * CH>(tmem + kColD + (uint32_t)(db * 3 * CH), tmem + kColA, dsrc + (uint32_t)(i * 3 * CH * 128));
                     umma_commit(bar(kDFull + db));
                 }
             }
@@ -464,7 +464,7 @@ bwd_gather_kernel(const __grid_constant__ CUtensorMap map_dl, const __grid_const
                     tc_fence_after_sync();
 #pragma unroll
                     for (int dy = 0; dy < 3; ++dy)
-                        issue_expand3<CH>(tmem + kColD + (uint32_t)(db * 3 * CH + dy * CH), tmem + kColRows + 16 * dy,
+                        issue_expand<CH>(tmem + kColD + (uint32_t)(db * 3 * CH + dy * CH), tmem + kColRows + 16 * dy,
                                           w + side * kExpand + (uint32_t)(((pl * 3 + dx) * 3 + dy) * CH * 128));
                     umma_commit(bar(kDFull + db));
                 }

@@ -17,15 +17,13 @@
 //               tile for everything: relative error 8.4e-7 of the forward, so: 2.1e-7) -, everything that is 2^-8
 //               smaller in the first half of a tile R, 2^-16 smaller in the second; they meet in registers.
 //   softmax     one thread has a pixel's nine slots
-//   expansion   D[p][(tap, channel)] = A'[p][32] . Bv[32][(tap, channel)], fp16 operands: upper and middle part of the
-//               slot value against upper and middle part of the weight (middle . middle is below 2^-22 and left out)
+//   expansion   D[p][(tap, channel)] = A'[p][32] . Bv[64][(tap, channel)]: the three parts of the slot value against the three
+//               parts of the weight, without the pairs below 2^-24 of the product
 //   sum         sum_t D[p][t][c] y_t[p][c] with packed fp32 FMAs
 //
 // Tensor-memory columns of a team: product chunks, H tiles, R tile (32 columns at the end); later D in 0 - 191 and A' in
 // the last 16.
 #pragma once
-#include <cuda_fp16.h>
-
 #include "common.cuh"
 #include "ptx.cuh"
 #include "split.cuh"
@@ -42,7 +40,6 @@ constexpr int kHaloPlane = 60 * 64;                     // bytes of one plane of
 constexpr int kSlot = 4 * kHaloPlane;                   // of a block: a slot of the team's ring
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr uint32_t kCols = 256, kColP = 0, kColR = 224, kColA = 240, kColD = 0;
-constexpr float kScaleA = 8192.f;                       // softmax weights (at most 1) enter fp16 times 2^13
 
 // How the channels of a storage type are cut: planes of 64 bytes, chunks of one plane and one tap column.
 template <typename T> struct Cut;
@@ -82,10 +79,9 @@ template <typename T> __host__ __device__ constexpr int channel_of_k(int kappa) 
 }
 
 // Weight images of one head (bytes).  Contraction: [plane][tap][K / 8][48 n][8 k] bf16.  Expansion: [plane][tap
-// column dx][dy][n][32 k] fp16 in core matrices, then one float per channel that undoes the channel's scale.
+// column dx][dy][n][64 k] bf16 in core matrices.
 __host__ __device__ constexpr uint32_t contract_bytes(int head_dim) { return (uint32_t)head_dim * 9u * 96u; }
-__host__ __device__ constexpr uint32_t expand_image_bytes(int head_dim) { return (uint32_t)head_dim * 9u * 64u; }
-__host__ __device__ constexpr uint32_t expand_bytes(int head_dim) { return expand_image_bytes(head_dim) + (uint32_t)head_dim * 4u; }
+__host__ __device__ constexpr uint32_t expand_bytes(int head_dim) { return (uint32_t)head_dim * 9u * 128u; }
 
 // Contraction image item: 16 bytes = 8 k of column n.  w: fp32 [head_dim][slot][tap] of the head.
 template <typename T>
@@ -109,80 +105,18 @@ __device__ __forceinline__ void build_contract_item(const float* __restrict__ w,
         make_uint4(split::pack_upper(v[0], v[1]), split::pack_upper(v[2], v[3]), split::pack_upper(v[4], v[5]), split::pack_upper(v[6], v[7]));
 }
 
-// A power of two that brings `most` (the largest magnitude of what it will multiply) to [2^13, 2^14), and its inverse.
-__device__ __forceinline__ void fp16_scale(float most, float& scale, float& inverse) {
-    int e = (int)(__float_as_uint(most) >> 23) & 0xff;
-    e = e < 14 ? 14 : e;
-    scale = __uint_as_float((uint32_t)(267 - e) << 23);
-    inverse = __uint_as_float((uint32_t)(e - 13) << 23);
-}
-// x = hi + mid to 2^-22 of x (as far as 2^-24 allows)
-__device__ __forceinline__ void split_fp16(float x, __half& hi, __half& mid) {
-    hi = __float2half_rn(x);
-    mid = __float2half_rn(x - __half2float(hi));
-}
-__device__ __forceinline__ uint32_t pack_half(__half a, __half b) {
-    return (uint32_t)__half_as_ushort(a) | ((uint32_t)__half_as_ushort(b) << 16);
-}
-
-// Expansion image of one channel by one warp (w: the channel's fp32 [slot][tap]).  Column ((plane 3 + dx) 3 + dy)
-// channels + n; its K rows: 0 - 7 upper parts of slots 0 - 7, 8 - 15 their middle parts, 16 - 23 the upper parts again,
-// 24 - 26 slot 8: upper, middle, upper.
-template <typename T>
-__device__ __forceinline__ void build_expand_channel(const float* __restrict__ w, unsigned char* img, int head_dim, int c, int lane) {
-    constexpr int CH = Cut<T>::channels;
-    float most = 0.f, v[kK2];
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-        if (lane + 32 * i < kK2 * kK2) most = fmaxf(most, fabsf(w[lane + 32 * i]));
-#pragma unroll
-    for (int s = 0; s < kK2; ++s) v[s] = lane < kK2 ? w[s * kK2 + lane] : 0.f;      // lane = tap
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) most = fmaxf(most, __shfl_xor_sync(0xffffffffu, most, o));
-    float scale, inverse;
-    fp16_scale(most, scale, inverse);
-    if (lane == 0) reinterpret_cast<float*>(img + expand_image_bytes(head_dim))[c] = inverse;
-    if (lane >= kK2) return;
-    const int plane = c / CH, ch = c % CH, dy = lane / 3, dx = lane % 3;
-    const int q4 = CH / 4, n = 8 * ((ch % q4) >> 1) + 2 * (ch / q4) + (ch & 1);      // the column of this channel
-    const int item = ((plane * 3 + dx) * 3 + dy) * CH + n;
-    __half hi[kK2], mid[kK2];
-#pragma unroll
-    for (int s = 0; s < kK2; ++s) split_fp16(v[s] * scale, hi[s], mid[s]);
-    unsigned char* col = img + (size_t)(item >> 3) * 512 + (item & 7) * 16;
-    const uint4 h = make_uint4(pack_half(hi[0], hi[1]), pack_half(hi[2], hi[3]), pack_half(hi[4], hi[5]), pack_half(hi[6], hi[7]));
-    *reinterpret_cast<uint4*>(col) = h;
-    *reinterpret_cast<uint4*>(col + 128) = make_uint4(pack_half(mid[0], mid[1]), pack_half(mid[2], mid[3]), pack_half(mid[4], mid[5]), pack_half(mid[6], mid[7]));
-    *reinterpret_cast<uint4*>(col + 256) = h;
-    const __half zero = __float2half_rn(0.f);
-    *reinterpret_cast<uint4*>(col + 384) = make_uint4(pack_half(hi[8], mid[8]), pack_half(hi[8], zero), 0u, 0u);
-}
-// The A' row that meets it, from nine slot values already scaled: 16 registers of two halves.
-__device__ __forceinline__ void expand_row(const float (&a)[kK2], uint32_t (&row)[16]) {
-    __half hi[kK2], mid[kK2];
-#pragma unroll
-    for (int s = 0; s < kK2; ++s) split_fp16(a[s], hi[s], mid[s]);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        row[i] = pack_half(hi[2 * i], hi[2 * i + 1]);
-        row[4 + i] = row[i];
-        row[8 + i] = pack_half(mid[2 * i], mid[2 * i + 1]);
-    }
-    row[12] = pack_half(hi[8], hi[8]);
-    row[13] = pack_half(mid[8], __float2half_rn(0.f));
-    row[14] = 0u; row[15] = 0u;
-}
-
-// ---- the same expansion for slot values of any magnitude (gradients): three bf16 parts each -----------------------------
+// ---- the expansion's operands ----------------------------------------------------------------------------------------------
+// Slot values (softmax weights, gradients) and weights have three bf16 parts each, so their magnitude does not matter.  (With
+// two fp16 parts each, scaled to that type's range, a forward took half the MMAs and was not faster (2 x 128 x 128, 3 heads, fp32: 29.1 us,
+// 26.7 here), and values above 2^100 overflowed before the scale was undone.)
 // SPLIT ROW: 64 bytes of a pixel and head, 32 bf16: 0 - 8 upper parts of the slots, 9 - 17 middle, 18 - 26 lower parts, 27, 28
 // the middle parts of slots 7 and 8 again.  In memory its four 16-byte pieces are swizzled by the pixel's column x (piece c
 // at c ^ ((x >> 1) & 3)), which makes reads of eight neighbouring pixels' pieces free of bank conflicts.
 // It meets an image of four 16-row K steps: rows 0 - 15 of the row with the upper parts of the weights, 16 - 31 likewise
 // (27, 28 with the middle parts of slots 7 and 8), 0 - 15 with the middle parts, 0 - 8 with the lower parts: everything down to
 // 2^-24 of the product.
-__host__ __device__ constexpr uint32_t expand3_bytes(int head_dim) { return (uint32_t)head_dim * 9u * 128u; }
 template <typename T>
-__device__ __forceinline__ void build_expand3_item(const float* __restrict__ w, unsigned char* img, int item) {
+__device__ __forceinline__ void build_expand_item(const float* __restrict__ w, unsigned char* img, int item) {
     constexpr int CH = Cut<T>::channels;
     const int n = item % CH, r = item / CH, dy = r % 3, dx = (r / 3) % 3, plane = r / 9;
     const int c = plane * CH + (CH / 4) * ((n & 7) >> 1) + 2 * (n >> 3) + (n & 1), tap = dy * 3 + dx;
@@ -221,29 +155,29 @@ __device__ __forceinline__ void split_row(const float (&a)[kK2], uint32_t (&row)
     row[14] = split::pack_upper(v[17], 0.f);
     row[15] = 0u;
 }
-// Where a split row of N columns of D is issued: B at `b_smem` (of the image), A in 16 columns at `a_col`.
+// The MMAs of N columns of D: B at `b_smem` (of the image), A = a split row in 16 columns at `a_col`.  The smallest products come
+// first, so that the tensor core, which truncates whatever it adds to, truncates at full magnitude once.
 template <int N>
-__device__ __forceinline__ void issue_expand3(uint32_t d_col, uint32_t a_col, uint32_t b_smem) {
+__device__ __forceinline__ void issue_expand(uint32_t d_col, uint32_t a_col, uint32_t b_smem) {
     constexpr uint32_t idesc = umma_idesc_bf16(128, N);
-    const uint64_t b = umma_smem_desc(b_smem, 128, 1024);
-    umma_bf16_ts(d_col, a_col, b, idesc, 0);
-    umma_bf16_ts(d_col, a_col + 8, b + 16, idesc, 1);                        // 256 bytes on: the next K step
+    const uint64_t b = umma_smem_desc(b_smem, 128, 1024);                    // a K step further: 256 bytes = 16
+    umma_bf16_ts(d_col, a_col, b + 48, idesc, 0);
+    umma_bf16_ts(d_col, a_col + 8, b + 16, idesc, 1);
     umma_bf16_ts(d_col, a_col, b + 32, idesc, 1);
-    umma_bf16_ts(d_col, a_col, b + 48, idesc, 1);
+    umma_bf16_ts(d_col, a_col, b, idesc, 1);
 }
 
-// The images of one head by prep_parts(head_dim) blocks of 256 threads, of which this one is `part`: a warp per channel of
-// the expansion image, then a thread per item of the contraction image.  (Four blocks a head, each looking for the
-// channels' largest weights by itself, took 12 us, most of what a small map needs.)
-__host__ __device__ constexpr int prep_parts(int head_dim) { return head_dim / 8 + (head_dim / 8 * 9 * 48 + 255) / 256; }
+// The images of one head by prep_parts(head_dim) blocks of 256 threads, of which this one is `part`: a thread per item of the
+// expansion image, then of the contraction image.  (Four blocks a head took 12 us, most of what a small map needs.)
+__host__ __device__ constexpr int expand_parts(int head_dim) { return (head_dim * kK2 + 255) / 256; }
+__host__ __device__ constexpr int prep_parts(int head_dim) { return expand_parts(head_dim) + (head_dim / 8 * kK2 * 48 + 255) / 256; }
 template <typename T>
 __device__ __forceinline__ void build_images(const float* wc, unsigned char* cimg, const float* we, unsigned char* eimg, int head_dim, int part) {
-    if (part < head_dim / 8) {
-        const int c = part * 8 + (threadIdx.x >> 5);
-        build_expand_channel<T>(we + c * kK2 * kK2, eimg, head_dim, c, threadIdx.x & 31);
-    } else {
-        const int i = (part - head_dim / 8) * 256 + threadIdx.x;
-        if (i < head_dim / 8 * 9 * 48) build_contract_item<T>(wc, cimg, i);
+    const int ce = part - expand_parts(head_dim), i = (ce < 0 ? part : ce) * 256 + threadIdx.x;
+    if (ce < 0) {
+        if (i < head_dim * kK2) build_expand_item<T>(we, eimg, i);
+    } else if (i < head_dim / 8 * kK2 * 48) {
+        build_contract_item<T>(wc, cimg, i);
     }
 }
 
@@ -416,14 +350,6 @@ __device__ __forceinline__ void load_contraction(uint32_t quad, float (&l)[kK2])
 #pragma unroll
     for (int s = 0; s < kK2; ++s) l[s] += r[s] + r[16 + s];
 }
-// The MMAs of one D chunk (plane, dx): [128 x 32] . [32 x 3 channels].
-template <typename T>
-__device__ __forceinline__ void issue_expand(uint32_t d_col, uint32_t a_col, uint32_t b_smem) {
-    constexpr uint32_t idesc = umma_idesc_f16(128, 3 * Cut<T>::channels);
-    umma_bf16_ts(d_col, a_col, umma_smem_desc(b_smem, 128, 512), idesc, 0);
-    umma_bf16_ts(d_col, a_col + 8, umma_smem_desc(b_smem + 256, 128, 512), idesc, 1);
-}
-
 // acc[row][channel of the lane] += D chunk (three taps of a column) at `t` times the halo rows of that column, which are
 // loaded while the chunk is on its way.  Tap dy meets halo row `row` + dy, or, in the transposed shift, `row` + 2 - dy.
 template <bool Transposed = false>

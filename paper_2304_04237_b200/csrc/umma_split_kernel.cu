@@ -145,7 +145,7 @@ umma_split_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
                     const int db = dn % DB;
                     if (!mbar_wait(bar(kDFree + db), ((uint32_t)(dn / DB) & 1u) ^ 1u)) { ok = false; break; }
                     tc_fence_after_sync();
-                    issue_expand<T>(tmem + kColD + (uint32_t)(db * 3 * CH), tmem + kColA, dsrc + (uint32_t)(i * 3 * CH * 64));
+                    issue_expand<3 * CH>(tmem + kColD + (uint32_t)(db * 3 * CH), tmem + kColA, dsrc + (uint32_t)(i * 3 * CH * 128));
                     umma_commit(bar(kDFull + db));
                 }
             }
@@ -236,11 +236,11 @@ umma_split_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
                 for (int s = 0; s < kK2; ++s) { a[s] = fmaf(a[s], P.scale_log2e, bias[s]); m = fmaxf(m, a[s]); }
 #pragma unroll
                 for (int s = 0; s < kK2; ++s) { a[s] = fast_exp2(a[s] - m); z += a[s]; }
-                const float iz = kScaleA / z;
+                const float iz = 1.f / z;
 #pragma unroll
                 for (int s = 0; s < kK2; ++s) a[s] *= iz;
                 uint32_t row[16];
-                expand_row(a, row);
+                split_row(a, row);
                 tmem_st_32x32b_x16(quad + kColA, row);
                 tmem_wait_st();
                 tc_fence_before_sync();
@@ -249,7 +249,6 @@ umma_split_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
             }
 
             // ---- values ----------------------------------------------------------------------------
-            if (bi == 0 && !warp_wait(bar_weights, 0)) { ok = false; break; }     // for the channel scales
             for (int pl = 0; pl < NPL; ++pl) {
                 float acc[2][PL];
 #pragma unroll
@@ -270,20 +269,16 @@ umma_split_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
                 }
                 if (!ok) break;
                 release_after(acc[0][0], acc[1][0]);
-                const float* inv = reinterpret_cast<const float*>(smem + F::w_off + contract_bytes(D) + expand_image_bytes(D)) + pl * CH + tig * PL;
-                float sc[PL];
-#pragma unroll
-                for (int c = 0; c < PL; ++c) sc[c] = inv[c] * (1.f / kScaleA);
 #pragma unroll
                 for (int r = 0; r < 2; ++r) {
                     if (!cur.in[r]) continue;
                     Piece o;
                     if constexpr (sizeof(T) == 2) {
-                        o.x = pack_bf16(acc[r][0] * sc[0], acc[r][1] * sc[1]); o.y = pack_bf16(acc[r][2] * sc[2], acc[r][3] * sc[3]);
-                        if constexpr (PL == 8) { o.z = pack_bf16(acc[r][4] * sc[4], acc[r][5] * sc[5]); o.w = pack_bf16(acc[r][6] * sc[6], acc[r][7] * sc[7]); }
+                        o.x = pack_bf16(acc[r][0], acc[r][1]); o.y = pack_bf16(acc[r][2], acc[r][3]);
+                        if constexpr (PL == 8) { o.z = pack_bf16(acc[r][4], acc[r][5]); o.w = pack_bf16(acc[r][6], acc[r][7]); }
                     } else {
-                        o.x = __float_as_uint(acc[r][0] * sc[0]); o.y = __float_as_uint(acc[r][1] * sc[1]);
-                        o.z = __float_as_uint(acc[r][2] * sc[2]); o.w = __float_as_uint(acc[r][3] * sc[3]);
+                        o.x = __float_as_uint(acc[r][0]); o.y = __float_as_uint(acc[r][1]);
+                        o.z = __float_as_uint(acc[r][2]); o.w = __float_as_uint(acc[r][3]);
                     }
                     *reinterpret_cast<Piece*>(static_cast<T*>(P.out) + cur.at + r * row_pitch + pl * CH) = o;
                 }

@@ -41,7 +41,7 @@ def test_split_variant_matches_oracle(shape, d, dtype):
 
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 def test_split_variant_weights_of_any_scale(dtype):
-    """Channels whose value weights differ by 2^40 (each is scaled by its own power of two for the fp16 split)."""
+    """Channels whose value weights differ by 2^40."""
     x = inputs((1, 9, 10, 2), 32, dtype, 0.4)
     scale = np.exp2(np.arange(64) % 41 - 20).astype(np.float32)
     x["wv"] = x["wv"] * scale[:, None, None]
@@ -50,6 +50,17 @@ def test_split_variant_weights_of_any_scale(dtype):
     s = scale.reshape(2, 32)
     err = np.abs(got - ref) / s / np.maximum(1.0, np.abs(ref) / s)
     assert err.max() <= TIGHT[dtype], float(err.max())
+
+
+@pytest.mark.parametrize("power", [-100, 110, 120])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("d", [16, 32, 64])
+def test_split_variant_values_of_any_scale(d, dtype, power):
+    """Values near both ends of the type's range; the result scales with them exactly."""
+    x = inputs((1, 9, 10, 2), d, dtype, 0.4)
+    plain = gpu_forward(x, 3, dtype, sa.VARIANT_UMMA_SPLIT)
+    x["v"] = x["v"] * np.float32(2.0 ** power)
+    assert np.array_equal(gpu_forward(x, 3, dtype, sa.VARIANT_UMMA_SPLIT), plain * 2.0 ** power)
 
 
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
