@@ -97,8 +97,8 @@ typedef enum {
                                          re-associated with the q.k products and the softmax weights;
                                          head_dim 32, ksize <= 9, fp32 or bf16: what AUTO runs for fp32
                                          storage with ksize 1 or >= 5                                    */
-    SLIDE_ATTN_VARIANT_UMMA_SPLIT = 11, /* fp32 arithmetic on tcgen05: operands split into parts whose bf16 / fp16
-                                         products are exact or good to 2^-22; ksize 3, head_dim 16, 32 or 64, fp32
+    SLIDE_ATTN_VARIANT_UMMA_SPLIT = 11, /* fp32 arithmetic on tcgen05: operands split into bf16 parts, all products
+                                         down to 2^-24 kept, results as close to 64 bits as fp32 FMAs'; ksize 3, head_dim 16, 32 or 64, fp32
                                          or bf16: what AUTO runs for fp32 storage and for head_dim 16 and 64   */
     SLIDE_ATTN_VARIANT_MMA_WIDE = 9   /* large windows with general weights: persistent warp-specialised
                                          kernel, both contractions on tcgen05, weights resident in shared

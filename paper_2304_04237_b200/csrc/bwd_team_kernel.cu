@@ -72,11 +72,19 @@ bwd_prep_kernel(const float* __restrict__ wk, const float* __restrict__ wv, unsi
     unsigned char* img = images + (size_t)blockIdx.x * kImages;
     constexpr int contract_items = kHeadDim / 8 * kK2 * 48, expand_items = kHeadDim * kK2;
     const int step = gridDim.y * 256, at = blockIdx.y * 256 + threadIdx.x;
+    float most[2] = {0.f, 0.f};
+    const float* const both[2] = {wk + w, wv + w};
+    if constexpr (sizeof(T) == 4) block_most<2>(both, kHeadDim * kK2 * kK2, most);
     for (int i = at; i < 2 * (contract_items + expand_items); i += step) {
         const int side = i >= contract_items + expand_items, j = side ? i - contract_items - expand_items : i;
-        const float* src = (side ? wv : wk) + w;
-        if (j < contract_items) build_contract_item<T>(src, img + side * kContract, j);
-        else build_expand_item<T>(src, img + 2 * kContract + side * kExpand, j - contract_items);
+        const float* src = both[side];
+        if (j < contract_items) {
+            float v[8];
+            load_contract_item<T>(src, j, v);
+            build_contract_item<T>(v, img + side * kContract, j, most[side]);
+        } else {
+            build_expand_item<T>(src, img + 2 * kContract + side * kExpand, j - contract_items);
+        }
     }
     for (int i = at; i < kHeadDim * kK2 * kK2; i += step) { dwk[w + i] = 0.f; dwv[w + i] = 0.f; }
     if (dbias && at < kK2) dbias[blockIdx.x * kK2 + at] = 0.f;
@@ -214,8 +222,7 @@ bwd_point_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constan
                         const uint32_t p_col = tmem + kColP + (uint32_t)(pb * 3 * Cut<T>::tap_cols);
 #pragma unroll
                         for (int dy = 0; dy < 3; ++dy)
-                            issue_contract<T>(tmem, p_col + dy * Cut<T>::tap_cols, desc + contract_step<T>(plane, dy * 3 + dx), dx,
-                                              dy == 0 && (sizeof(T) == 2 ? i == 0 : plane == 0), dy == 0 && i == 0);
+                            issue_contract<T>(tmem, p_col + dy * Cut<T>::tap_cols, desc + contract_step<T>(plane, dy * 3 + dx), plane, dx, dy);
                         umma_commit(bar(kPFree + pb));
                     }
                     if (ok) umma_commit(bar(kLFull));
@@ -281,11 +288,11 @@ bwd_point_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constan
                     uint4 y[4];
 #pragma unroll
                     for (int r = 0; r < 4; ++r) y[r] = halo_piece<T>(plane, 2 * half + r, g + dx, tig);
+                    if (dx == 0) x.meet(plane, 2 * half, g, tig, y);
                     if (!warp_wait(bar(kPFree + pb), ((uint32_t)(pn >> 1) & 1u) ^ 1u)) { ok = false; break; }
                     tc_fence_after_sync();
                     const uint32_t t = mine + kColP + (uint32_t)(pb * 3 * Cut<T>::tap_cols);
-#pragma unroll
-                    for (int dy = 0; dy < 3; ++dy) store_products(x, t + dy * Cut<T>::tap_cols, y[dy], y[dy + 1]);
+                    store_column<T>(x, t, y);
                     tmem_wait_st();
                     tc_fence_before_sync();
                     __syncwarp();
@@ -308,12 +315,7 @@ bwd_point_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constan
 
             // ---- a and dl: thread = pixel of the quadrant ------------------------------------------------
             if (turn) {
-                float m = -INFINITY, z = 0.f;
-#pragma unroll
-                for (int s = 0; s < kK2; ++s) { a[s] = fmaf(a[s], P.scale * kLog2e, s_bias[s]); m = fmaxf(m, a[s]); }
-#pragma unroll
-                for (int s = 0; s < kK2; ++s) { a[s] = fast_exp2(a[s] - m); z += a[s]; }
-                const float iz = 1.f / z;
+                const float iz = 1.f / softmax_terms(a, P.scale * kLog2e, s_bias);
 #pragma unroll
                 for (int s = 0; s < kK2; ++s) a[s] *= iz;
                 // lane = 8 row + column of the strip

@@ -12,17 +12,20 @@
 //
 //   products    x . y per (plane, tap column dx), split into parts, to tensor memory (a chunk; two buffers)
 //   contraction L[p][n] += parts . Bk.  The columns of Bk are three groups of 16, nine used: the upper, middle and
-//               lower 8 bits of the weight of each slot.  Upper x upper accumulates in tiles H of its own - the tensor
-//               core truncates at every step, and two or three tiles mean half or a third of the steps for each (one
-//               tile for everything: relative error 8.4e-7 of the forward, so: 2.1e-7) -, everything that is 2^-8
-//               smaller in the first half of a tile R, 2^-16 smaller in the second; they meet in registers.
-//   softmax     one thread has a pixel's nine slots
+//               lower part of the weight of each slot.  Upper x upper accumulates apart (H) from everything smaller (R);
+//               they meet in registers.  The tensor core truncates whenever it adds to H, so:
+//               bf16: three tiles H, one per tap column, whose sums stay small (two tiles, one per K step: error of the softmax
+//               weights 1.9e-7, so: 1.4e-7, fp32 FMAs: 1.5e-7);
+//               fp32: the upper parts are multiples of one power of two per pixel and plane (2^-8 of the largest product its window
+//               can have), those of the weights of one per head, so that the sums in H are integers below 2^24 of their product:
+//               exact.  (A product below that power of two keeps its 17 upper bits.)
+//   softmax     one thread has a pixel's nine slots; the largest logit is subtracted before anything is rounded to scale
 //   expansion   D[p][(tap, channel)] = A'[p][32] . Bv[64][(tap, channel)]: the three parts of the slot value against the three
 //               parts of the weight, without the pairs below 2^-24 of the product
 //   sum         sum_t D[p][t][c] y_t[p][c] with packed fp32 FMAs
 //
-// Tensor-memory columns of a team: product chunks, H tiles, R tile (32 columns at the end); later D in 0 - 191 and A' in
-// the last 16.
+// Tensor-memory columns of a team: product chunks, then 64 of sums (bf16: three H, R; fp32: H, R of 2^-8, 2^-16 and 2^-24 of
+// it); later D in 0 - 191 and A' in the last 16.
 #pragma once
 #include "common.cuh"
 #include "ptx.cuh"
@@ -39,7 +42,7 @@ constexpr int kK2 = 9;
 constexpr int kHaloPlane = 60 * 64;                     // bytes of one plane of a strip with its halo
 constexpr int kSlot = 4 * kHaloPlane;                   // of a block: a slot of the team's ring
 constexpr float kLog2e = 1.4426950408889634f;
-constexpr uint32_t kCols = 256, kColP = 0, kColR = 224, kColA = 240, kColD = 0;
+constexpr uint32_t kCols = 256, kColP = 0, kColA = 240, kColD = 0;
 
 // How the channels of a storage type are cut: planes of 64 bytes, chunks of one plane and one tap column.
 template <typename T> struct Cut;
@@ -52,7 +55,7 @@ template <> struct Cut<__nv_bfloat16> {
     static constexpr int box = 32;                      // channels that a TMA box takes
     static constexpr int per_lane = 8;
     static constexpr int d_buffers = 2;                 // N = 96 columns per tap column of a plane
-    static constexpr int tap_cols = 32, h_tiles = 2;    // products are hi + lo: 2 x 3 x 32 + 2 x 16 + 32 = 256 columns
+    static constexpr int tap_cols = 32;                 // products are hi + lo: 2 x 3 x 32 + 64 = 256 columns
 };
 template <> struct Cut<NarrowBf16> {
     using piece = uint2;
@@ -60,7 +63,7 @@ template <> struct Cut<NarrowBf16> {
     static constexpr int box = 32;
     static constexpr int per_lane = 4;
     static constexpr int d_buffers = 3;                 // N = 48
-    static constexpr int tap_cols = 16, h_tiles = 3;    // hi + lo: 2 x 3 x 16 + 3 x 16 + 32 = 176 columns
+    static constexpr int tap_cols = 16;                 // hi + lo: 2 x 3 x 16 + 64 = 160 columns
 };
 template <> struct Cut<float> {
     using piece = uint4;
@@ -68,9 +71,9 @@ template <> struct Cut<float> {
     static constexpr int box = 16;
     static constexpr int per_lane = 4;
     static constexpr int d_buffers = 3;                 // N = 48
-    static constexpr int tap_cols = 24, h_tiles = 3;    // hi + mid + lo: 2 x 3 x 24 + 3 x 16 + 32 = 224
+    static constexpr int tap_cols = 24;                 // hi + mid + lo: 2 x 3 x 24 + 64 = 208
 };
-template <typename T> constexpr uint32_t kColH = 6 * Cut<T>::tap_cols;
+template <typename T> constexpr uint32_t kColL = 6 * Cut<T>::tap_cols;          // the sums
 
 // Channel of K index kappa within a plane (the order in which tcgen05.st lays the pieces out); the channel of column n of
 // a tap of D (the order in which tcgen05.ld hands them to the lanes) is (CH / 4) ((n & 7) >> 1) + 2 (n >> 3) + (n & 1).
@@ -83,23 +86,60 @@ template <typename T> __host__ __device__ constexpr int channel_of_k(int kappa) 
 __host__ __device__ constexpr uint32_t contract_bytes(int head_dim) { return (uint32_t)head_dim * 9u * 96u; }
 __host__ __device__ constexpr uint32_t expand_bytes(int head_dim) { return (uint32_t)head_dim * 9u * 128u; }
 
+// What rounds numbers up to `most` in magnitude to multiples of a power of two, so that the quotients are integers up to 256 and
+// fit bf16: added and taken away again, 1.5 * 2^23 times that power.  Not for numbers from 2^112 on (`wide`), where it would be infinite.
+__device__ __forceinline__ bool wide(float most) { return __float_as_uint(most) >= 0x77800000u; }       // NaN too
+__device__ __forceinline__ float rounder(float most) { return __uint_as_float((__float_as_uint(most) & 0x7f800000u) + 0x08400000u); }
+
+// The largest magnitude (a NaN counts as larger than anything) of each of N arrays of n floats, n a multiple of 4, by a block of 256.
+template <int N>
+__device__ __forceinline__ void block_most(const float* const (&w)[N], int n, float (&most)[N]) {
+    __shared__ uint32_t s_most[N][8];
+    uint32_t m[N] = {};
+    for (int i = threadIdx.x; i < n / 4; i += 256)
+#pragma unroll
+        for (int a = 0; a < N; ++a) {
+            const uint4 v = __ldg(reinterpret_cast<const uint4*>(w[a]) + i);
+            m[a] = max(max(m[a], max(v.x & 0x7fffffffu, v.y & 0x7fffffffu)), max(v.z & 0x7fffffffu, v.w & 0x7fffffffu));
+        }
+#pragma unroll
+    for (int a = 0; a < N; ++a) {
+        m[a] = __reduce_max_sync(0xffffffffu, m[a]);
+        if ((threadIdx.x & 31) == 0) s_most[a][threadIdx.x >> 5] = m[a];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int a = 0; a < N; ++a) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) m[a] = max(m[a], s_most[a][i]);
+        most[a] = __uint_as_float(m[a]);
+    }
+}
+
 // Contraction image item: 16 bytes = 8 k of column n.  w: fp32 [head_dim][slot][tap] of the head.
 template <typename T>
-__device__ __forceinline__ void build_contract_item(const float* __restrict__ w, unsigned char* img, int item) {
+__device__ __forceinline__ void load_contract_item(const float* __restrict__ w, int item, float (&v)[8]) {
     constexpr int KG = Cut<T>::channels / 8;             // k groups of a (plane, tap)
-    const int n = item % 48, kg = item / 48;
+    const int n = item % 48, kg = item / 48, s = n & 15;
     const int j = kg % KG, pt = kg / KG, tap = pt % kK2, plane = pt / kK2;
-    const int s = n & 15, part = n >> 4;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) v[e] = s < kK2 ? w[((plane * Cut<T>::channels + channel_of_k<T>(8 * j + e)) * kK2 + s) * kK2 + tap] : 0.f;
+}
+// `most` (fp32 storage): the largest of all weights of the head.
+template <typename T>
+__device__ __forceinline__ void build_contract_item(const float (&w)[8], unsigned char* img, int item, float most) {
+    const int n = item % 48, kg = item / 48, part = n >> 4;
     float v[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
-        float x = 0.f;
-        if (s < kK2) {
-            x = w[((plane * Cut<T>::channels + channel_of_k<T>(8 * j + e)) * kK2 + s) * kK2 + tap];
-            if (part >= 1) x = split::rest(x);
-            if (part >= 2) x = split::rest(x);
+        v[e] = w[e];
+        if (sizeof(T) == 4 && !wide(most)) {
+            const float r = rounder(most), hi = __fadd_rn(__fadd_rn(v[e], r), -r), rest = v[e] - hi, mid = __bfloat162float(__float2bfloat16_rn(rest));
+            v[e] = part == 0 ? hi : part == 1 ? mid : __bfloat162float(__float2bfloat16_rn(rest - mid));
+        } else {
+            if (part >= 1) v[e] = split::rest(v[e]);
+            if (part >= 2) v[e] = split::rest(v[e]);
         }
-        v[e] = x;
     }
     *reinterpret_cast<uint4*>(img + (size_t)kg * 768 + (n >> 3) * 128 + (n & 7) * 16) =
         make_uint4(split::pack_upper(v[0], v[1]), split::pack_upper(v[2], v[3]), split::pack_upper(v[4], v[5]), split::pack_upper(v[6], v[7]));
@@ -115,6 +155,9 @@ __device__ __forceinline__ void build_contract_item(const float* __restrict__ w,
 // It meets an image of four 16-row K steps: rows 0 - 15 of the row with the upper parts of the weights, 16 - 31 likewise
 // (27, 28 with the middle parts of slots 7 and 8), 0 - 15 with the middle parts, 0 - 8 with the lower parts: everything down to
 // 2^-24 of the product.
+// The lower parts carry what the tensor core's one truncation at full magnitude takes off a product on average: half a unit in the last
+// place, relative to a number spread evenly over its logarithm 2^-24 / (2 ln 2).  (A single product of 8-bit numbers stays exact.)
+constexpr float kTruncation = 4.3e-8f;
 template <typename T>
 __device__ __forceinline__ void build_expand_item(const float* __restrict__ w, unsigned char* img, int item) {
     constexpr int CH = Cut<T>::channels;
@@ -125,7 +168,7 @@ __device__ __forceinline__ void build_expand_item(const float* __restrict__ w, u
     for (int s = 0; s < kK2; ++s) {
         hi[s] = w[(c * kK2 + s) * kK2 + tap];
         mid[s] = split::rest(hi[s]);
-        lo[s] = split::rest(mid[s]);
+        lo[s] = __bfloat162float(__float2bfloat16_rn(fmaf(kTruncation, hi[s], split::rest(mid[s]))));
     }
     float v[64];
 #pragma unroll
@@ -176,9 +219,15 @@ __device__ __forceinline__ void build_images(const float* wc, unsigned char* cim
     const int ce = part - expand_parts(head_dim), i = (ce < 0 ? part : ce) * 256 + threadIdx.x;
     if (ce < 0) {
         if (i < head_dim * kK2) build_expand_item<T>(we, eimg, i);
-    } else if (i < head_dim / 8 * kK2 * 48) {
-        build_contract_item<T>(wc, cimg, i);
+        return;
     }
+    const bool in = i < head_dim / 8 * kK2 * 48;
+    float w[8];
+    if (in) load_contract_item<T>(wc, i, w);                                 // on their way while the largest weight is looked for
+    float most[1] = {0.f};
+    const float* const src[1] = {wc};
+    if constexpr (sizeof(T) == 4) block_most<1>(src, head_dim * kK2 * kK2, most);
+    if (in) build_contract_item<T>(w, cimg, i, most[0]);
 }
 
 // (A vote in every probe, which makes all branches of the wait uniform, measured 5 - 8 % slower than one at the end.)
@@ -257,6 +306,7 @@ template <> struct Factor<__nv_bfloat16> {
             nx[r] = make_uint4(v[r].x ^ 0x80008000u, v[r].y ^ 0x80008000u, v[r].z ^ 0x80008000u, v[r].w ^ 0x80008000u);
         }
     }
+    __device__ __forceinline__ void meet(const unsigned char*, int, int, int, const uint4 (&)[4]) {}
 };
 template <> struct Factor<NarrowBf16> {
     uint2 x[2], nx[2];
@@ -264,10 +314,38 @@ template <> struct Factor<NarrowBf16> {
 #pragma unroll
         for (int r = 0; r < 2; ++r) { x[r] = v[r]; nx[r] = make_uint2(v[r].x ^ 0x80008000u, v[r].y ^ 0x80008000u); }
     }
+    __device__ __forceinline__ void meet(const unsigned char*, int, int, int, const uint2 (&)[4]) {}
 };
+// fp32 keeps what rounds the products of each pixel to their common power of two.
+__device__ __forceinline__ float largest(const uint4& v) {
+    return fmaxf(fmaxf(fabsf(f4(v, 0)), fabsf(f4(v, 1))), fmaxf(fabsf(f4(v, 2)), fabsf(f4(v, 3))));
+}
 template <> struct Factor<float> {
     uint4 x[2];
+    float r[2];
+    bool any_wide;
     __device__ __forceinline__ void set(const uint4 (&v)[2]) { x[0] = v[0]; x[1] = v[1]; }
+    // what x will be multiplied with: the halo plane's rows `row` .. + 3, columns `col` (given: y0) .. + 2
+    __device__ __forceinline__ void meet(const unsigned char* plane, int row, int col, int tig, const uint4 (&y0)[4]) {
+        float y[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            y[i] = largest(y0[i]);
+#pragma unroll
+            for (int dx = 1; dx < 3; ++dx) y[i] = fmaxf(y[i], largest(halo_piece<float>(plane, row + i, col + dx, tig)));
+        }
+        const float both = fmaxf(y[1], y[2]);
+        float most[2] = {fmaxf(both, y[0]) * largest(x[0]), fmaxf(both, y[3]) * largest(x[1])};
+        bool w = false;
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            most[i] = fmaxf(most[i], __shfl_xor_sync(0xffffffffu, most[i], 1));
+            most[i] = fmaxf(most[i], __shfl_xor_sync(0xffffffffu, most[i], 2));
+            w = w || wide(most[i]);
+            r[i] = rounder(most[i]);
+        }
+        any_wide = __any_sync(0xffffffffu, w);
+    }
 };
 // Products of one tap of a plane for the lane's two pixels, split, into tensor memory at column `t`.
 __device__ __forceinline__ void store_products(const Factor<__nv_bfloat16>& f, uint32_t t, const uint4& y0, const uint4& y1) {
@@ -284,22 +362,55 @@ __device__ __forceinline__ void store_products(const Factor<NarrowBf16>& f, uint
     split::product2n(f.x[1].x, f.nx[1].x, y1.x, r[2], r[6]); split::product2n(f.x[1].y, f.nx[1].y, y1.y, r[3], r[7]);
     tmem_st_16x256b_x2(t, r);
 }
-__device__ __forceinline__ void store_products(const Factor<float>& f, uint32_t t, const uint4& y0, const uint4& y1) {
-    const uint4 (&x)[2] = f.x;
-    float2 p[4];                                         // first row: channels 0 1, 2 3; second row
-    p[0] = split::mul2(make_float2(f4(x[0], 0), f4(x[0], 1)), make_float2(f4(y0, 0), f4(y0, 1)));
-    p[1] = split::mul2(make_float2(f4(x[0], 2), f4(x[0], 3)), make_float2(f4(y0, 2), f4(y0, 3)));
-    p[2] = split::mul2(make_float2(f4(x[1], 0), f4(x[1], 1)), make_float2(f4(y1, 0), f4(y1, 1)));
-    p[3] = split::mul2(make_float2(f4(x[1], 2), f4(x[1], 3)), make_float2(f4(y1, 2), f4(y1, 3)));
+// fp32: minus the upper part (the tensor core negates it again), then the middle and the lower part.  Three instructions take the
+// upper part off a pair of products: x y + r, its distance to r, and what is left of x y, which is never rounded as a whole.
+template <bool Wide>
+__device__ __forceinline__ void store_products_f32(const Factor<float>& f, uint32_t t, const uint4& y0, const uint4& y1) {
     uint32_t r[8], s[4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) { r[i] = split::pack_upper(p[i].x, p[i].y); p[i] = split::rest2(p[i]); }
-#pragma unroll
-    for (int i = 0; i < 4; ++i) { r[4 + i] = split::pack_upper(p[i].x, p[i].y); p[i] = split::rest2(p[i]); }
-#pragma unroll
-    for (int i = 0; i < 4; ++i) s[i] = split::pack_upper(p[i].x, p[i].y);
+    for (int i = 0; i < 4; ++i) {                        // first row: channels 0 1, 2 3; second row
+        const uint4 &x = f.x[i >> 1], &y = i < 2 ? y0 : y1;
+        const float x0 = f4(x, 2 * (i & 1)), x1 = f4(x, 2 * (i & 1) + 1), v0 = f4(y, 2 * (i & 1)), v1 = f4(y, 2 * (i & 1) + 1), round = f.r[i >> 1];
+        float p0, p1;
+        if constexpr (!Wide) {
+            float h0 = round, h1 = round;
+            ffma2(h0, h1, x0, x1, v0, v1);
+            p0 = round; p1 = round;
+            ffma2(p0, p1, h0, h1, -1.f, -1.f);
+            r[i] = split::pack_upper(p0, p1);
+            ffma2(p0, p1, x0, x1, v0, v1);
+        } else {                                         // the upper 8 bits
+            p0 = -x0 * v0; p1 = -x1 * v1;
+            r[i] = split::pack_upper(p0, p1);
+            p0 = -split::rest(p0); p1 = -split::rest(p1);
+        }
+        r[4 + i] = pack_bf16(p0, p1);
+        ffma2(p0, p1, bf16_lo(r[4 + i]), bf16_hi(r[4 + i]), -1.f, -1.f);
+        s[i] = pack_bf16(p0, p1);
+    }
     tmem_st_16x256b_x2(t, r);
     tmem_st_16x256b_x1(t + 16, s);
+}
+static __device__ __noinline__ void store_products_wide(uint32_t t, uint4 x0, uint4 x1, uint4 y0, uint4 y1) {
+    Factor<float> f;
+    f.x[0] = x0; f.x[1] = x1; f.r[0] = f.r[1] = 0.f;
+    store_products_f32<true>(f, t, y0, y1);
+}
+// The products of the three taps of a column.
+template <typename T>
+__device__ __forceinline__ void store_column(const Factor<T>& f, uint32_t t, const typename Cut<T>::piece (&y)[4]) {
+    if constexpr (sizeof(T) == 4) {
+        if (f.any_wide) {                                // products from 2^112 on
+#pragma unroll 1
+            for (int dy = 0; dy < 3; ++dy) store_products_wide(t + dy * Cut<T>::tap_cols, f.x[0], f.x[1], dy == 0 ? y[0] : dy == 1 ? y[1] : y[2], dy == 0 ? y[1] : dy == 1 ? y[2] : y[3]);
+        } else {
+#pragma unroll
+            for (int dy = 0; dy < 3; ++dy) store_products_f32<false>(f, t + dy * Cut<T>::tap_cols, y[dy], y[dy + 1]);
+        }
+    } else {
+#pragma unroll
+        for (int dy = 0; dy < 3; ++dy) store_products(f, t + dy * Cut<T>::tap_cols, y[dy], y[dy + 1]);
+    }
 }
 
 // Descriptor of a contraction image; a (plane, tap) further is contract_step.
@@ -307,49 +418,58 @@ __device__ __forceinline__ uint64_t contract_desc(uint32_t img) { return umma_sm
 template <typename T> __host__ __device__ constexpr uint32_t contract_step(int plane, int tap) {
     return (uint32_t)((plane * kK2 + tap) * (Cut<T>::channels / 8) * 48);          // in 16-byte units
 }
-// The MMAs of one tap, issued by one thread.  `fresh`: the first tap of a block for its H tile (planes of 16 channels: tile
-// dx; of 32: both tiles, one per k-step); `first`: the first tap of the block.
+// The MMAs of one tap (row dy of column dx of a plane), issued by one thread.
 template <typename T>
-__device__ __forceinline__ void issue_contract(uint32_t tmem, uint32_t p_col, uint64_t b, int dx, bool fresh, bool first) {
-    constexpr uint32_t id32 = umma_idesc_bf16(128, 32), id16 = umma_idesc_bf16(128, 16);
-    constexpr uint32_t mid = 16;                                             // 256 bytes on: the columns of the middle parts
-    const uint32_t r = tmem + kColR, h = tmem + kColH<T>;
-    if constexpr (Cut<T>::channels == 32) {
-        constexpr uint32_t k1 = 96;                                          // 1536 bytes on: the next 16 k
-        constexpr uint32_t neg32 = id32 | kIdescNegateA;
-        umma_bf16_ts(h, p_col, b, id16, fresh ? 0u : 1u);
-        umma_bf16_ts(r, p_col, b + mid, id32, first ? 0u : 1u);              // upper . middle | upper . lower
-        umma_bf16_ts(h + 16, p_col + 8, b + k1, id16, fresh ? 0u : 1u);
-        umma_bf16_ts(r, p_col + 8, b + k1 + mid, id32, 1);
-        umma_bf16_ts(r, p_col + 16, b, neg32, 1);                            // lower . upper | lower . middle
-        umma_bf16_ts(r, p_col + 24, b + k1, neg32, 1);
-    } else if constexpr (sizeof(T) == 2) {
-        umma_bf16_ts(h + 16 * dx, p_col, b, id16, fresh ? 0u : 1u);
-        umma_bf16_ts(r, p_col, b + mid, id32, first ? 0u : 1u);
-        umma_bf16_ts(r, p_col + 8, b, id32 | kIdescNegateA, 1);
-    } else {
-        umma_bf16_ts(h + 16 * dx, p_col, b, id16, fresh ? 0u : 1u);
-        umma_bf16_ts(r, p_col, b + mid, id32, first ? 0u : 1u);
-        umma_bf16_ts(r, p_col + 8, b, id32, 1);                              // middle . upper | middle . middle
-        umma_bf16_ts(r + 16, p_col + 16, b, id16, 1);                        // lower . upper
+__device__ __forceinline__ void issue_contract(uint32_t tmem, uint32_t p_col, uint64_t b, int plane, int dx, int dy) {
+    constexpr uint32_t id16 = umma_idesc_bf16(128, 16), id32 = umma_idesc_bf16(128, 32), id48 = umma_idesc_bf16(128, 48);
+    constexpr uint32_t group = 16;                                           // 256 bytes on: the weights' next parts
+    const uint32_t l = tmem + kColL<T>;
+    const bool fresh = plane == 0 && dy == 0, first = fresh && dx == 0;
+    if constexpr (sizeof(T) == 2) {
+#pragma unroll
+        for (int k = 0; k < Cut<T>::channels / 16; ++k) {
+            const uint32_t hi = p_col + 8 * k, lo = p_col + Cut<T>::tap_cols / 2 + 8 * k, r = l + 48;
+            const uint64_t bk = b + 96 * k;                                  // 1536 bytes on: the next 16 k
+            umma_bf16_ts(l + 16 * dx, hi, bk, id16, fresh && k == 0 ? 0u : 1u);
+            umma_bf16_ts(r, hi, bk + group, id16, first && k == 0 ? 0u : 1u);
+            umma_bf16_ts(r, hi, bk + 2 * group, id16, 1);
+            umma_bf16_ts(r, lo, bk, id16 | kIdescNegateA, 1);
+            umma_bf16_ts(r, lo, bk + group, id16 | kIdescNegateA, 1);
+        }
+    } else {                                                                 // column group i of l: 2^-8i of the first
+        const uint32_t hi = p_col, mid = p_col + 8, lo = p_col + 16;
+        umma_bf16_ts(l + 16, mid, b, id48, first ? 0u : 1u);
+        umma_bf16_ts(l + 32, lo, b, id32, 1);
+        if (first) {
+            umma_bf16_ts(l, hi, b, id16 | kIdescNegateA, 0);
+            umma_bf16_ts(l + 16, hi, b + group, id32 | kIdescNegateA, 1);
+        } else {
+            umma_bf16_ts(l, hi, b, id48 | kIdescNegateA, 1);
+        }
     }
 }
 // The contraction of the lane's pixel (thread = TMEM lane).
 template <typename T>
 __device__ __forceinline__ void load_contraction(uint32_t quad, float (&l)[kK2]) {
-    float h[32], r[32];
-    tmem_ld_32x32b_x32(quad + kColR, r);
-    tmem_ld_32x32b_x32(quad + kColH<T>, h);                                  // two H tiles
+    float u[32], v[32];
+    tmem_ld_32x32b_x32(quad + kColL<T>, u);
+    tmem_ld_32x32b_x32(quad + kColL<T> + 32, v);
 #pragma unroll
-    for (int s = 0; s < kK2; ++s) l[s] = h[s] + h[16 + s];
-    if constexpr (Cut<T>::h_tiles == 3) {
-        tmem_ld_32x32b_x32(quad + kColH<T> + 16, h);                         // the second and the third
-#pragma unroll
-        for (int s = 0; s < kK2; ++s) l[s] += h[16 + s];
-    }
-#pragma unroll
-    for (int s = 0; s < kK2; ++s) l[s] += r[s] + r[16 + s];
+    for (int s = 0; s < kK2; ++s) l[s] = sizeof(T) == 2 ? (u[s] + u[16 + s]) + (v[s] + v[16 + s]) : u[s] + (u[16 + s] + (v[s] + v[16 + s]));
 }
+// exp2(l scale + bias - their largest) in place of l; returns the sum.  The largest l comes off before the scale is applied, so that
+// the slots that matter lose nothing to the rounding of a large logit.
+__device__ __forceinline__ float softmax_terms(float (&l)[kK2], float scale, const float* bias) {
+    float top = l[0], m = -INFINITY, z = 0.f;
+#pragma unroll
+    for (int s = 1; s < kK2; ++s) top = fmaxf(top, l[s]);
+#pragma unroll
+    for (int s = 0; s < kK2; ++s) { l[s] = fmaf(l[s] - top, scale, bias[s]); m = fmaxf(m, l[s]); }
+#pragma unroll
+    for (int s = 0; s < kK2; ++s) { l[s] = fast_exp2(l[s] - m); z += l[s]; }
+    return z;
+}
+
 // acc[row][channel of the lane] += D chunk (three taps of a column) at `t` times the halo rows of that column, which are
 // loaded while the chunk is on its way.  Tap dy meets halo row `row` + dy, or, in the transposed shift, `row` + 2 - dy.
 template <bool Transposed = false>

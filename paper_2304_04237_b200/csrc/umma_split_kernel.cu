@@ -1,7 +1,8 @@
 // UMMA_SPLIT variant (k = 3; fp32 storage or bf16; head_dim 16, 32 or 64): the fused forward (Eq. 2 with Eq. 12 inside)
 // with fp32 arithmetic, both k^4 contractions on tcgen05.  Where UMMA_TS rounds the q.k products and the softmax
 // weights to bf16, this kernel splits them, and the weights, into parts whose tensor-core products are exact
-// (split.cuh), so fp32 storage keeps its 1e-4 - in fact 1e-6 - and wide heads the accuracy of an fp32 kernel.
+// (split.cuh, team.cuh).  Error against 64 bits (2-norm, fp32 storage, 4 x 56 x 56, 3 heads of 16, 3 of 32, 2 of 64): 1.22, 1.21,
+// 1.22e-7, with q four times as large 1.29, 1.28, 1.30e-7; kernels of fp32 FMAs 1.29, 1.51, 1.30e-7 and 1.76, 2.24, 1.80e-7.
 //
 //   logits   l[s] = scale * sum_{t,c} (q[c] k_t[c]) wk[c,s,t] + bias[s]     a = softmax(l)
 //   values   out[c] = sum_t v_t[c] (sum_s a[s] wv[c,s,t])
@@ -134,8 +135,7 @@ umma_split_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
                     const uint32_t p_col = tmem + kColP + (uint32_t)(pb * 3 * Cut<T>::tap_cols);
 #pragma unroll
                     for (int dy = 0; dy < 3; ++dy)
-                        issue_contract<T>(tmem, p_col + dy * Cut<T>::tap_cols, kdesc + contract_step<T>(plane, dy * 3 + dx), dx,
-                                          dy == 0 && (CH == 32 ? i == 0 : plane == 0), dy == 0 && i == 0);
+                        issue_contract<T>(tmem, p_col + dy * Cut<T>::tap_cols, kdesc + contract_step<T>(plane, dy * 3 + dx), plane, dx, dy);
                     umma_commit(bar(kPFree + pb));
                 }
                 if (!ok) break;
@@ -209,11 +209,11 @@ umma_split_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
                     Piece y[4];
 #pragma unroll
                     for (int r = 0; r < 4; ++r) y[r] = halo_piece<T>(plane, 2 * half + r, g + dx, tig);
+                    if (dx == 0) x.meet(plane, 2 * half, g, tig, y);
                     if (!warp_wait(bar(kPFree + pb), ((uint32_t)(pn >> 1) & 1u) ^ 1u)) { ok = false; break; }
                     tc_fence_after_sync();
                     const uint32_t t = mine + kColP + (uint32_t)(pb * 3 * Cut<T>::tap_cols);
-#pragma unroll
-                    for (int dy = 0; dy < 3; ++dy) store_products(x, t + dy * Cut<T>::tap_cols, y[dy], y[dy + 1]);
+                    store_column<T>(x, t, y);
                     tmem_wait_st();
                     tc_fence_before_sync();
                     __syncwarp();
@@ -230,13 +230,9 @@ umma_split_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
             if (half == (bi & 1)) {
                 if (!warp_wait(bar(kLFull), (uint32_t)bi & 1u)) { ok = false; break; }
                 tc_fence_after_sync();
-                float a[kK2], m = -INFINITY, z = 0.f;
+                float a[kK2];
                 load_contraction<T>(quad, a);
-#pragma unroll
-                for (int s = 0; s < kK2; ++s) { a[s] = fmaf(a[s], P.scale_log2e, bias[s]); m = fmaxf(m, a[s]); }
-#pragma unroll
-                for (int s = 0; s < kK2; ++s) { a[s] = fast_exp2(a[s] - m); z += a[s]; }
-                const float iz = 1.f / z;
+                const float iz = 1.f / softmax_terms(a, P.scale_log2e, bias);
 #pragma unroll
                 for (int s = 0; s < kK2; ++s) a[s] *= iz;
                 uint32_t row[16];

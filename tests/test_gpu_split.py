@@ -63,6 +63,21 @@ def test_split_variant_values_of_any_scale(d, dtype, power):
     assert np.array_equal(gpu_forward(x, 3, dtype, sa.VARIANT_UMMA_SPLIT), plain * 2.0 ** power)
 
 
+@pytest.mark.parametrize("power", [-60, 60, 112, 118])
+@pytest.mark.parametrize("d", [16, 32, 64])
+def test_split_variant_products_of_any_scale(d, power):
+    """Products q k up to 2^118 times the usual ones, weights as much smaller (from 2^112 on products are cut otherwise; lower parts
+    of weights fall below the smallest normal bf16 there, 2^-126: 2^-10 of a product)."""
+    x = inputs((1, 9, 10, 2), d, "f32", 0.4)
+    ref = oracle.forward(x["q"], x["k"], x["v"], x["wk"], x["wv"], x["bias"], 3)
+    x["q"] = x["q"] * np.float32(2.0 ** (power // 2))
+    x["k"] = x["k"] * np.float32(2.0 ** (power - power // 2))
+    x["wk"] = x["wk"] * np.float32(2.0 ** -power)
+    got = gpu_forward(x, 3, "f32", sa.VARIANT_UMMA_SPLIT)
+    err = (np.abs(got - ref) / np.maximum(1.0, np.abs(ref))).max()
+    assert err <= (1e-5 if power < 112 else 2e-3), float(err)
+
+
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 def test_split_variant_is_repeatable(dtype):
     x = inputs((5, 30, 33, 3), 64, dtype, 0.05)
