@@ -10,8 +10,9 @@
 //
 // Persistent, one CTA per SM and one head per CTA.  Twelve compute warps = side x 16-channel half x tap row,
 // three per scheduler; a warp keeps the sums of its three taps in registers over all its tiles.  The tensor core
-// truncates when it accumulates, so the columns that hold upper parts move to a second set of fp32 registers
-// after every kFlush pixel groups (twelve tensor-core steps).  Tiles (4 rows x up to 32 columns + halo) come by TMA into
+// truncates when it accumulates, so the columns that hold upper parts are added up in fp32 registers after every pixel group, and
+// within one the smallest products come first: one truncation at full magnitude (after four groups, largest first: twelve, error of
+// dwv against 64 bits 4.4e-7, so 2.4e-7, with fp32 FMAs 2.7e-7; the same time).  Tiles (4 rows x up to 32 columns + halo) come by TMA into
 // two stages, in planes of 16 channels (four pixels x eight channel pairs = 256 contiguous bytes: no bank conflict).
 //
 // Bound by the mma.sync pipe and the CUDA-core work beside it, which hardly overlap (measured: 8 cycles per MMA and
@@ -31,7 +32,7 @@ constexpr int kK2 = 9;
 constexpr int kTH = 4;                         // tile rows
 constexpr int kComputeWarps = 12;
 constexpr int kThreads = (kComputeWarps + 1) * 32;
-constexpr int kFlush = 4;
+constexpr float kTruncation = 4.3e-8f;         // what one truncation takes off on average (team.cuh): half of 2^-23 / (2 ln 2)
 constexpr uint32_t kSumBytes = 2u * kK2 * kHeadDim * 32u * 4u;        // the CTA's sums at its end, [side][tap][channel][32 columns]
 
 template <typename T> struct WTile;
@@ -93,20 +94,32 @@ template <> struct Frag<float> {
     }
 };
 
-// acc += (x . y) times the split columns b[tile][2]
-__device__ __forceinline__ void accumulate(float (&acc)[4][4], const Frag<float>& x, const Frag<float>& y, const uint32_t (&b)[4][2]) {
+// sum += (x . y) times the split columns b[tile][2]
+__device__ __forceinline__ void accumulate(float (&sum)[4][4], const Frag<float>& x, const Frag<float>& y, const uint32_t (&b)[4][2]) {
     float2 p[4];
+    uint32_t a[3][4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) p[i] = mul2(x.a[i], y.a[i]);
 #pragma unroll
     for (int part = 0; part < 3; ++part) {
-        const uint32_t a[4] = {pack_upper(p[0].x, p[1].x), pack_upper(p[0].y, p[1].y), pack_upper(p[2].x, p[3].x), pack_upper(p[2].y, p[3].y)};
-#pragma unroll
-        for (int j = 0; j < 4 - part; ++j) mma_bf16(acc[j], a, b[j][0], b[j][1]);
+        a[part][0] = pack_upper(p[0].x, p[1].x); a[part][1] = pack_upper(p[0].y, p[1].y);
+        a[part][2] = pack_upper(p[2].x, p[3].x); a[part][3] = pack_upper(p[2].y, p[3].y);
         if (part < 2)
 #pragma unroll
             for (int i = 0; i < 4; ++i) p[i] = rest2(p[i]);
     }
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {                                    // columns of upper (and some middle) parts
+        float c[4];
+        mma_bf16_c(c, a[2], b[j][0], b[j][1], 0.f, 0.f, 0.f, 0.f);
+        mma_bf16(c, a[1], b[j][0], b[j][1]);
+        mma_bf16(c, a[0], b[j][0], b[j][1]);
+        fadd2(sum[j][0], sum[j][1], c[0], c[1]);
+        fadd2(sum[j][2], sum[j][3], c[2], c[3]);
+    }
+    mma_bf16(sum[2], a[1], b[2][0], b[2][1]);
+    mma_bf16(sum[2], a[0], b[2][0], b[2][1]);
+    mma_bf16(sum[3], a[0], b[3][0], b[3][1]);
 }
 
 template <typename T>
@@ -137,7 +150,7 @@ bwd_weight_mma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
     }
     __syncthreads();
 
-    float acc[3][4][4], sum[3][2][4];
+    float sum[3][4][4];
     bool ok = true;
     const int side = warp / 6, half = (warp / 3) & 1, ty = warp % 3;  // of a compute warp
 
@@ -174,24 +187,11 @@ bwd_weight_mma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
     } else {
         // ---- products and sums ----------------------------------------------------------------------
 #pragma unroll
-        for (int t = 0; t < 3; ++t) {
+        for (int t = 0; t < 3; ++t)
 #pragma unroll
             for (int j = 0; j < 4; ++j)
 #pragma unroll
-                for (int x = 0; x < 4; ++x) acc[t][j][x] = 0.f;
-#pragma unroll
-            for (int j = 0; j < 2; ++j)
-#pragma unroll
                 for (int x = 0; x < 4; ++x) sum[t][j][x] = 0.f;
-        }
-        auto flush = [&]() {
-#pragma unroll
-            for (int t = 0; t < 3; ++t)
-#pragma unroll
-                for (int j = 0; j < 2; ++j)
-#pragma unroll
-                    for (int x = 0; x < 4; ++x) { sum[t][j][x] += acc[t][j][x]; acc[t][j][x] = 0.f; }
-        };
         // lane i of the ldmatrix of the split columns: K index i % 8 of row (i / 8) % 2, 16-byte chunk i / 16 (+ 2)
         const int kcol = Frag<T>::col(lane & 7);
         const uint32_t b_off = L.split_off + (uint32_t)side * L.split_side + (uint32_t)(((lane >> 3) & 1) * P.tw + kcol) * 64u;
@@ -200,7 +200,7 @@ bwd_weight_mma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
         const uint32_t x_pitch = (uint32_t)P.tw * PB, y_pitch = (uint32_t)HW * PB;
         const uint32_t x_off = (side ? L.g_off : L.q_off) + Frag<T>::offset(lane, half, L.tile_plane, x_pitch);
         const uint32_t y_off = (side ? L.v_off : L.k_off) + (uint32_t)ty * y_pitch + Frag<T>::offset(lane, half, L.halo_plane, y_pitch);
-        int it = 0, pending = 0;
+        int it = 0;
         for (int tile = rank; tile < tiles; tile += nrank, ++it) {
             const int st = it & 1;
             int rest_ = tile;
@@ -221,18 +221,16 @@ bwd_weight_mma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
 #pragma unroll
                     for (int t = 0; t < 3; ++t) y[t].load(ya + t * PB, y_pitch);
 #pragma unroll
-                    for (int t = 0; t < 3; ++t) accumulate(acc[t], x, y[t], b);
-                    if (++pending == kFlush) { pending = 0; flush(); }
+                    for (int t = 0; t < 3; ++t) accumulate(sum[t], x, y[t], b);
                 }
             }
-            // tiles 0 and 2 of a tap have taken in everything that was loaded for it (tile 0 may just have moved to its sum)
+            // the sums have taken in everything that was loaded: tile 0 of a tap its products and the first split columns, tile 2 the others
             uint32_t read = 0;
 #pragma unroll
-            for (int t = 0; t < 3; ++t) read |= __float_as_uint(acc[t][0][0]) | __float_as_uint(sum[t][0][0]) | __float_as_uint(acc[t][2][0]);
+            for (int t = 0; t < 3; ++t) read |= __float_as_uint(sum[t][0][0]) | __float_as_uint(sum[t][2][0]);
             __syncwarp();
             mbar_arrive_lane0_after(bar_empty(st), lane, __uint_as_float(read), 0.f, (uint32_t)(P.H >> 31));
         }
-        flush();
     }
     if (!ok && lane == 0) atomicExch(P.status, 1);
     __syncthreads();                                                 // every load has been waited for: the stages are free
@@ -245,8 +243,7 @@ bwd_weight_mma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
 #pragma unroll
                 for (int x = 0; x < 4; ++x) {
                     const int ch = half * 16 + Frag<T>::channel(g + 8 * (x >> 1));
-                    const float v = j < 2 ? sum[t][j & 1][x] : acc[t][j][x];
-                    s_sum[((side * kK2 + ty * 3 + t) * kHeadDim + ch) * 32 + 8 * j + 2 * tig + (x & 1)] = v;
+                    s_sum[((side * kK2 + ty * 3 + t) * kHeadDim + ch) * 32 + 8 * j + 2 * tig + (x & 1)] = sum[t][j][x];
                 }
     }
     __syncthreads();
@@ -255,7 +252,7 @@ bwd_weight_mma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
         const int ch = rem / (kK2 * kK2), st = rem - ch * kK2 * kK2;
         const int s = st / kK2, t = st - s * kK2;
         const float* p = s_sum + ((sd * kK2 + t) * kHeadDim + ch) * 32 + s;
-        const float v = p[0] + (p[9] + p[18]);
+        const float v = fmaf(kTruncation, p[0], p[0] + (p[9] + p[18]));
         atomicAdd((sd ? P.dwv : P.dwk) + (size_t)(h * kHeadDim) * kK2 * kK2 + rem, sd ? v : v * P.scale);
     }
 }
