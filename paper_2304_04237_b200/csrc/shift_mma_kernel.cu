@@ -4,8 +4,8 @@
 //   l[s] = (q[p] . k[p + off(s)]) / sqrt(d) + bias[s]     a = softmax_s(l)     out[p,c] = sum_s a[s] v[p + off(s), c]
 //
 // as a banded attention in mma.sync.m16n8k16 tiles.  M = 16 queries = 2 rows x 8 columns; their windows cover k + 1 rows of 16
-// keys, two n-tiles a row, of which k + 1 <= 10 columns of each row are inside a query's window.  A table of biases in registers
-// holds -inf for the others, so one FMA scales, adds the bias and masks.  The logits' C fragments are the A fragments of
+// keys, two n-tiles a row, of which k + 1 <= 10 columns of each row are inside a query's window; the logits of the others become
+// -inf.  The logits' C fragments are the A fragments of
 // the product with V.  The softmax weights go in as hi + lo (two bf16): the products of q and k are exact, V is exact, so
 // the result has fp32 accuracy up to its own rounding, as the CUDA-core kernel has.
 //
@@ -15,12 +15,13 @@
 //
 // One CTA = one head of a 4 x tw pixel tile (tw <= 32: with 56 columns, or 8 rows, fewer CTAs share an SM and cover each other's
 // loads, 61 -> 65, 97 us at 64 x 56 x 56, 3 heads, k = 5), one warp per 8 columns; K and V tile + halo and the q tile by TMA
-// (out-of-map elements zero-filled: that IS the padding).  Keys up to seven columns outside a window enter the products with
-// weight 0 (a NaN there would spread; the CUDA-core kernel never touches them).
+// (out-of-map elements zero-filled: that IS the padding).  Values up to seven columns outside a window enter the products with weight
+// 0, and 0 times an infinity or a NaN would spread to queries that do not see it: a warp whose sums are not all finite takes them
+// again, window by window (plain_rows; with the test k = 9 is 2 % slower).
 //
 // k = 5, 7, 9: with k = 3 nine tenths of the band are masked, and the CUDA-core kernel is faster (64 x 56 x 56, 3 heads: 36 us
-// against 44).  CUDA cores and this kernel at 64 x 56 x 56, 3 heads: k = 5 70 and 61 us, k = 7 124 and 81; 16 x 56 x 56, 3 heads,
-// k = 9: 62 and 36 us.
+// against 44).  A call (weight check and kernel) on CUDA cores and here, 64 x 56 x 56, 3 heads: k = 5 70 and 59 us, k = 7 124 and 75; 16 x
+// 56 x 56, 3 heads, k = 9: 62 and 34 us.
 #include "common.cuh"
 #include "ptx.cuh"
 #include "split.cuh"
@@ -57,6 +58,54 @@ struct Plan {
     }
 };
 
+// The queries of the lane's column in rows r0 and r0 + 1 of the tile over their own windows only, in fp32.  `keys`, `values`, `queries`: the
+// lane's 16-byte piece at the first pixel of its column; row pitches in bytes.
+template <int K>
+__device__ __noinline__ void plain_rows(const unsigned char* keys, const unsigned char* values, const unsigned char* queries, uint32_t key_pitch,
+                                        uint32_t query_pitch, const float* bias, float scale_log2e, __nv_bfloat16* out, size_t out_pitch, int rows)
+{
+    auto widen = [](const unsigned char* p, float (&f)[8]) {
+        const uint4 v = *reinterpret_cast<const uint4*>(p);
+        f[0] = bf16_lo(v.x); f[1] = bf16_hi(v.x); f[2] = bf16_lo(v.y); f[3] = bf16_hi(v.y);
+        f[4] = bf16_lo(v.z); f[5] = bf16_hi(v.z); f[6] = bf16_lo(v.w); f[7] = bf16_hi(v.w);
+    };
+#pragma unroll 1
+    for (int r = 0; r < 2; ++r) {
+        float q[8], acc[8], m = -INFINITY, z = 0.f;
+        widen(queries + (uint32_t)r * query_pitch, q);
+#pragma unroll
+        for (int c = 0; c < 8; ++c) acc[c] = 0.f;
+        auto logit = [&](int u, int v) {
+            float k[8], l = 0.f;
+            widen(keys + (uint32_t)(r + u) * key_pitch + (uint32_t)v * 64u, k);
+#pragma unroll
+            for (int c = 0; c < 8; ++c) l = fmaf(q[c], k[c], l);
+            l += __shfl_xor_sync(0xffffffffu, l, 1);
+            l += __shfl_xor_sync(0xffffffffu, l, 2);
+            return fmaf(l, scale_log2e, bias ? bias[u * K + v] * kLog2e : 0.f);
+        };
+#pragma unroll 1
+        for (int u = 0; u < K; ++u)
+#pragma unroll 1
+            for (int v = 0; v < K; ++v) m = fmaxf(m, logit(u, v));
+#pragma unroll 1
+        for (int u = 0; u < K; ++u)
+#pragma unroll 1
+            for (int v = 0; v < K; ++v) {
+                const float p = fast_exp2(logit(u, v) - m);
+                float f[8];
+                widen(values + (uint32_t)(r + u) * (key_pitch >> 1) + (uint32_t)v * 32u, f);
+                z += p;
+#pragma unroll
+                for (int c = 0; c < 8; ++c) acc[c] = fmaf(p, f[c], acc[c]);
+            }
+        const float inv = 1.f / z;
+        if (r < rows)
+            *reinterpret_cast<uint4*>(out + (size_t)r * out_pitch) = make_uint4(pack_bf16(acc[0] * inv, acc[1] * inv), pack_bf16(acc[2] * inv, acc[3] * inv),
+                                                                                pack_bf16(acc[4] * inv, acc[5] * inv), pack_bf16(acc[6] * inv, acc[7] * inv));
+    }
+}
+
 template <int K>
 __global__ void __launch_bounds__(kMaxW * 4, K <= 5 ? 4 : 3)
 shift_mma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
@@ -86,12 +135,13 @@ shift_mma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     }
     // column n = 8 j + 2 tig + e of a row of keys is window column v = n - g of the lane's queries
     float tab[K][4];
+    bool in[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         const int v = 8 * (i >> 1) + 2 * tig + (i & 1) - g;
-        const bool in = v >= 0 && v < K;
+        in[i] = v >= 0 && v < K;
 #pragma unroll
-        for (int u = 0; u < K; ++u) tab[u][i] = in ? (P.bias ? P.bias[(h * K + u) * K + v] * kLog2e : 0.f) : -INFINITY;
+        for (int u = 0; u < K; ++u) tab[u][i] = in[i] && P.bias ? P.bias[(h * K + u) * K + v] * kLog2e : 0.f;
     }
     __syncthreads();
     if (!mbar_wait(bar, 0)) {                                        // bounded
@@ -127,7 +177,7 @@ shift_mma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     float& v = s[u + q][i >> 1][2 * q + (i & 1)];
-                    v = fmaf(v, P.scale_log2e, tab[u][i]);
+                    v = in[i] ? fmaf(v, P.scale_log2e, tab[u][i]) : -INFINITY;
                     m = fmaxf(m, v);
                 }
             m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 1));
@@ -170,6 +220,20 @@ shift_mma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                 mma_bf16(o[2 * p], lo, v[0], v[1]);
                 mma_bf16(o[2 * p + 1], lo, v[2], v[3]);
             }
+        }
+        float finite = 0.f, unused = 0.f;                            // 0 times a sum: 0 unless one is not finite
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            ffma2(finite, unused, o[c][0], o[c][1], 0.f, 0.f);
+            ffma2(finite, unused, o[c][2], o[c][3], 0.f, 0.f);
+        }
+        if (__any_sync(0xffffffffu, !(finite + unused == 0.f))) {
+            const int y = y0 + r0;
+            plain_rows<K>(keys + (uint32_t)(r0 * HW) * 64u,
+                          smem + L.v_off + (uint32_t)(tig >> 1) * L.v_plane + (uint32_t)(r0 * HW + 8 * warp + g) * 32u + (uint32_t)(tig & 1) * 16u,
+                          queries + (uint32_t)(r0 * P.tw) * 64u, (uint32_t)HW * 64u, (uint32_t)P.tw * 64u, P.bias ? P.bias + h * K * K : nullptr, P.scale_log2e,
+                          P.out + ((size_t)(b * P.H + y) * P.W + x) * C + h * kHeadDim + tig * 8, (size_t)P.W * C, x < P.W ? (y + 1 < P.H ? 2 : 1) : 0);
+            continue;
         }
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
