@@ -19,6 +19,8 @@
 // column dx the warp walks the 4 + k - 1 halo rows of that column once: each row vector serves every
 // pixel of the strip whose window holds it.  The softmax runs online over the window columns (running
 // maximum, sum and accumulator per pixel), so registers do not grow with k^2.
+#include <float.h>
+
 #include "tile_common.cuh"
 
 namespace slide_attn {
@@ -113,7 +115,8 @@ shift_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ 
     typename Piece<T>::Raw qr[kR];
 #pragma unroll
     for (int r = 0; r < kR; ++r) qr[r] = Piece<T>::load(sQ, L.q_plane, (uint32_t)(r * tw + col), tig);
-    float m = -INFINITY, sum = 0.f;                              // of pixel row tig
+    // of pixel row tig; m is finite, as -inf less -inf, after window columns that a bias of -inf masks, is not a number
+    float m = -FLT_MAX, sum = 0.f;
     float acc[kR][8];
 #pragma unroll
     for (int r = 0; r < kR; ++r)
@@ -148,7 +151,7 @@ shift_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ 
 #pragma unroll
         for (int dy = 0; dy < K; ++dy) { l[dy] = fmaf(l[dy], P.scale_log2e, s_bias[dy * K + dx]); cm = fmaxf(cm, l[dy]); }
         const float mn = fmaxf(m, cm);
-        const float corr = fast_exp2(m - mn);                    // 0 for the first column (m = -inf)
+        const float corr = fast_exp2(m - mn);                    // 0 for the first column
         m = mn;
         sum *= corr;
 #pragma unroll

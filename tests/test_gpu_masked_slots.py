@@ -10,6 +10,7 @@ import oracle
 import paper_2304_04237_b200 as sa
 from paper_2304_04237_b200 import synth
 
+from test_gpu_fixed_shift import shift_forward
 from util import VARIANTS, assert_close, gpu_forward
 
 pytestmark = pytest.mark.gpu
@@ -48,3 +49,11 @@ def test_masked_slots_every_variant(k, dtype):
             assert_close(got, ref, dtype, f"{name}, variant {variant}")
             ran += 1
     assert ran >= 3 * len(masks(k))
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("k", [3, 5, 7, 9])
+def test_masked_slots_fixed_shift(k, dtype):
+    for name, mask in masks(k).items():
+        x, ref = masked((1, 9, 37, 2, 32), k, dtype, mask, 0.0)
+        assert_close(shift_forward(x, k, dtype), ref, dtype, name)
