@@ -39,9 +39,9 @@ bool make_tile_map(CUtensorMap* map, const void* base, int elem_bytes, int B, in
                    int box_c, int box_w, int box_h);
 
 // Launches with programmatic stream serialisation: the kernel may start before the one ahead of it in the stream has finished and
-// has to execute griddepcontrol.wait before it touches anything that one may write or read.  The prep kernels wait first
-// of all and only then let the main kernel behind them start, so a main kernel never runs beside what was ahead of its prep
-// kernel.  Chained so, back-to-back forwards have no launch gap between them.
+// has to execute griddepcontrol.wait before it touches anything that one may write or read, and in any case before it completes:
+// whoever waits for it takes all that was launched earlier as complete.  The prep kernels wait first of all and only then let the
+// main kernel behind them start, so a main kernel never runs beside what was ahead of its prep kernel.  Chained so, back-to-back forwards have no launch gap between them.
 // (The main kernels do not let theirs start early: waiting beside them, the next prep kernel's blocks made a 2 x 128 x 128 x 3 heads
 // call with k = 7 take 70 us instead of 59, others up to 6 % longer.)
 template <typename... Params, typename... Args>

@@ -98,6 +98,7 @@ shift_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ 
     __syncthreads();
     if (!mbar_wait(bar, 0)) {                                  // bounded: about two seconds
         if (lane == 0) atomicExch(P.status, 1);
+        if (threadIdx.x == 0) grid_dependency_wait();
         return;
     }
 
@@ -208,13 +209,14 @@ shift_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ 
             }
         }
     }
+    if (threadIdx.x == 0) grid_dependency_wait();              // not complete before the weight check (see launch_chained)
 }
 
 // Sets the status word to 2 if any weight differs from the one-hot shift kernel w[c][s][t] = [s == t].
 __global__ void shift_check_kernel(const float* __restrict__ wk, const float* __restrict__ wv, long long n_per, int k2, int* status)
 {
     grid_dependency_wait();
-    grid_launch_dependents();        // the fixed-shift kernel does not read this kernel's result
+    grid_launch_dependents();        // the fixed-shift kernel runs beside this one and waits for it at its end
     bool bad = false;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < 2 * n_per; i += (long long)gridDim.x * blockDim.x) {
         const long long j = i < n_per ? i : i - n_per;
@@ -261,8 +263,7 @@ cudaError_t launch_t(const Problem& p, int* d_status, cudaStream_t stream) {
         return cudaErrorInvalidValue;
     const long long ctas = (long long)P.tiles_x * P.tiles_y * p.B * p.heads;
     if (ctas > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-    // programmatic stream serialisation: the kernel may run beside the weight check launched just
-    // before it (it does not read the check's result; both only ever set the status word)
+    // the kernel runs beside the weight check launched just before it; both only ever set the status word
     return launch_chained(tw == kMaxTW ? shift_kernel<T, K, kMaxTW> : shift_kernel<T, K, 0>, dim3((unsigned)ctas), tw * 4, L.total, stream, mq, mk, mv, P);
 }
 

@@ -146,6 +146,7 @@ shift_mma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     __syncthreads();
     if (!mbar_wait(bar, 0)) {                                        // bounded
         if (lane == 0) atomicExch(P.status, 1);
+        if (threadIdx.x == 0) grid_dependency_wait();
         return;
     }
 
@@ -257,6 +258,7 @@ shift_mma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                 *reinterpret_cast<uint4*>(P.out + ((size_t)(b * P.H + y) * P.W + x) * C + h * kHeadDim + tig * 8) = make_uint4(w[0], w[1], w[2], w[3]);
         }
     }
+    if (threadIdx.x == 0) grid_dependency_wait();                    // not complete before the weight check (see launch_chained)
 }
 
 template <int K>
@@ -289,7 +291,7 @@ cudaError_t launch_t(const Problem& p, int* d_status, cudaStream_t stream) {
         return cudaErrorInvalidValue;
     const long long ctas = (long long)P.tiles_x * P.tiles_y * p.B * p.heads;
     if (ctas > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-    // beside the weight check launched just before it (it does not read the check's result; both only ever set the status word)
+    // beside the weight check launched just before it; both only ever set the status word
     return launch_chained(shift_mma_kernel<K>, dim3((unsigned)ctas), tw * 4, Plan<K>(tw).total, stream, mq, mk, mv, P);
 }
 

@@ -163,3 +163,28 @@ def test_fixed_shift_band_edges_keep_fp32_accuracy(H, W, k):
     ref = oracle.forward(x["q"], x["k"], x["v"], x["wk"], x["wv"], x["bias"], k)
     got = shift_forward(x, k, "bf16")
     assert np.isfinite(got).all() and (np.abs(got - ref) <= 2.0 ** -8 * np.abs(ref) + 1e-4).all()
+
+
+@pytest.mark.parametrize("k", [3, 9])
+def test_weights_may_change_right_behind_a_forward(k):
+    """The weight check of a small map takes longer than its attention (k = 9, 8 heads: 6.7 MB a tensor).  What follows in the stream,
+    the next forward and a copy over the weights, must find it complete: every call reports its own weights."""
+    B, H, W, heads = 1, 4, 8, 8
+    x = synth.make_inputs(B, H, W, heads, 32, k, "bf16", 0.0, 0.3, True, seed=3)
+    dev = to_device(x, "bf16")
+    good = dev["wv"].clone()
+    bad = good.clone()
+    bad.view(-1)[-1] = 0.5
+    ctx = sa.slide_attn_create(B, H, W, heads, 32, k, torch.bfloat16, True)
+    try:
+        sa.slide_attn_set_fixed_shift(ctx, True)
+        out = torch.empty_like(dev["q"])
+        for first, then in ((bad, good), (good, bad)) * 20:
+            dev["wv"].copy_(first)
+            sa.slide_attn_forward(ctx, dev["q"], dev["k"], dev["v"], dev["wk"], dev["wv"], dev["bias"], out)
+            if first is bad:
+                sa.slide_attn_forward(ctx, dev["q"], dev["k"], dev["v"], dev["wk"], good, dev["bias"], out)
+            dev["wv"].copy_(then)
+            assert sa.slide_attn_query_status(ctx) == (sa.ERR_NOT_FIXED_SHIFT if first is bad else sa.OK)
+    finally:
+        sa.slide_attn_destroy(ctx)
