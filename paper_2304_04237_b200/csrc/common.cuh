@@ -92,7 +92,8 @@ cudaError_t launch_umma_ts(const Problem& p, const void* workspace, int* d_statu
 // launch writes the weight images of every head to `workspace`.
 bool umma_split_supports(int head_dim, int ksize);
 size_t umma_split_workspace_bytes(int heads, int head_dim);
-cudaError_t launch_umma_split(const Problem& p, void* workspace, int* d_status, int num_sms, cudaStream_t stream);
+cudaError_t launch_umma_split_prep(const Problem& p, void* workspace, cudaStream_t stream);
+cudaError_t launch_umma_split(const Problem& p, const void* workspace, int* d_status, int num_sms, cudaStream_t stream);
 
 // Fixed-shift fast path: plain k x k local attention for weights that are exactly the one-hot shift
 // kernels (head_dim 32, k <= 9, fp32 or bf16).  launch_shift_check sets the status word to 2 when a
@@ -121,7 +122,8 @@ cudaError_t launch_backward(const Problem& p, const BackwardArgs& ga, void* wt, 
 // launch writes the weights as shared-memory images into `workspace`.
 bool mma_wide_supports(slide_attn_dtype dtype, int head_dim, int ksize);
 size_t mma_wide_workspace_bytes(int heads, int ksize);
-cudaError_t launch_mma_wide(const Problem& p, void* workspace, int* d_status, int num_sms, cudaStream_t stream);
+cudaError_t launch_mma_wide_prep(const Problem& p, void* workspace, cudaStream_t stream);
+cudaError_t launch_mma_wide(const Problem& p, const void* workspace, int* d_status, int num_sms, cudaStream_t stream);
 
 // TILE variant: generic weights, CUDA cores, TMA-staged halo tiles (head_dim 32, k <= 9, both dtypes).
 // Reads the transposed weights that launch_strip_prep writes.

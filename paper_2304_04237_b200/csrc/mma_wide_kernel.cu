@@ -547,7 +547,13 @@ mma_wide_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant
 }
 
 template <int K>
-cudaError_t launch_t(const Problem& p, void* workspace, int* d_status, int num_sms, cudaStream_t stream) {
+cudaError_t launch_prep_t(const Problem& p, void* workspace, cudaStream_t stream) {
+    return launch_chained(mma_wide_prep_kernel<K>, dim3((unsigned)((2 * Wide<K>::K2 * 4 * Wide<K>::N + 255) / 256), (unsigned)p.heads), 256, 0, stream, p.wk, p.wv,
+                          static_cast<unsigned char*>(workspace));
+}
+
+template <int K>
+cudaError_t launch_t(const Problem& p, const void* workspace, int* d_status, int num_sms, cudaStream_t stream) {
     using Wd = Wide<K>;
     static bool configured[64] = {};
     int dev = 0;
@@ -572,10 +578,6 @@ cudaError_t launch_t(const Problem& p, void* workspace, int* d_status, int num_s
     if (!make_tile_map(&mk, p.k, 2, p.B, p.H, p.W, C, kHeadDim, Wd::HP, Wd::HP) ||
         !make_tile_map(&mv, p.v, 2, p.B, p.H, p.W, C, kHeadDim, Wd::HP, Wd::HP))
         return cudaErrorInvalidValue;
-    e = launch_chained(mma_wide_prep_kernel<K>, dim3((unsigned)((2 * Wd::K2 * 4 * Wd::N + 255) / 256), (unsigned)p.heads), 256, 0, stream, p.wk, p.wv,
-                       static_cast<unsigned char*>(workspace));
-    if (e != cudaSuccess) return e;
-
     const long long blocks = (tiles + 1) / 2;
     long long per_head = num_sms / p.heads;
     if (per_head > blocks) per_head = blocks;
@@ -600,8 +602,18 @@ size_t mma_wide_workspace_bytes(int heads, int ksize) {
     }
 }
 
-// Prep launch (weights -> images in the order of their use, in `workspace`) followed by the fused kernel.
-cudaError_t launch_mma_wide(const Problem& p, void* workspace, int* d_status, int num_sms, cudaStream_t stream) {
+// Weights -> images in the order of their use, in `workspace`.
+cudaError_t launch_mma_wide_prep(const Problem& p, void* workspace, cudaStream_t stream) {
+    switch (p.ksize) {
+        case 3: return launch_prep_t<3>(p, workspace, stream);
+        case 5: return launch_prep_t<5>(p, workspace, stream);
+        case 7: return launch_prep_t<7>(p, workspace, stream);
+        case 9: return launch_prep_t<9>(p, workspace, stream);
+        default: return cudaErrorInvalidConfiguration;
+    }
+}
+
+cudaError_t launch_mma_wide(const Problem& p, const void* workspace, int* d_status, int num_sms, cudaStream_t stream) {
     switch (p.ksize) {
         case 3: return launch_t<3>(p, workspace, d_status, num_sms, stream);
         case 5: return launch_t<5>(p, workspace, d_status, num_sms, stream);

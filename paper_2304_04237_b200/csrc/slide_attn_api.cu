@@ -124,12 +124,14 @@ slide_attn_status launch_problem(slide_attn_ctx* c, const Problem& p, cudaStream
             if (err == cudaSuccess) err = launch_umma_ts(p, c->umma_ws, c->d_status, c->num_sms, stream);
             break;
         case SLIDE_ATTN_VARIANT_MMA_WIDE:
-            if (ev) cudaEventRecord(ev[1], stream);          // the prep launch is issued inside launch_mma_wide
-            err = launch_mma_wide(p, c->wide_ws, c->d_status, c->num_sms, stream);
+            err = launch_mma_wide_prep(p, c->wide_ws, stream);
+            if (ev) cudaEventRecord(ev[1], stream);
+            if (err == cudaSuccess) err = launch_mma_wide(p, c->wide_ws, c->d_status, c->num_sms, stream);
             break;
         case SLIDE_ATTN_VARIANT_UMMA_SPLIT:
-            if (ev) cudaEventRecord(ev[1], stream);          // the prep launch is issued inside launch_umma_split
-            err = launch_umma_split(p, c->split_ws, c->d_status, c->num_sms, stream);
+            err = launch_umma_split_prep(p, c->split_ws, stream);
+            if (ev) cudaEventRecord(ev[1], stream);
+            if (err == cudaSuccess) err = launch_umma_split(p, c->split_ws, c->d_status, c->num_sms, stream);
             break;
         case SLIDE_ATTN_VARIANT_TILE:
             err = launch_strip_prep(p, c->strip_ws, stream);

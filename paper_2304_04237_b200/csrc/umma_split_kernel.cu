@@ -292,7 +292,7 @@ umma_split_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
 }
 
 template <typename T, int D>
-cudaError_t launch_t(const Problem& p, void* workspace, int* d_status, int num_sms, cudaStream_t stream) {
+cudaError_t launch_t(const Problem& p, const void* workspace, int* d_status, int num_sms, cudaStream_t stream) {
     using F = Fwd<T, D>;
     static bool configured[64] = {};
     int dev = 0;
@@ -315,14 +315,20 @@ cudaError_t launch_t(const Problem& p, void* workspace, int* d_status, int num_s
     if (!make_tile_map(&mk, p.k, (int)sizeof(T), p.B, p.H, p.W, C, Cut<T>::box, 10, 6) ||
         !make_tile_map(&mv, p.v, (int)sizeof(T), p.B, p.H, p.W, C, Cut<T>::box, 10, 6))
         return cudaErrorInvalidValue;
-    e = launch_chained(umma_split_prep_kernel<T, D>, dim3((unsigned)p.heads, prep_parts(D)), 256, 0, stream, p.wk, p.wv, static_cast<unsigned char*>(workspace));
-    if (e != cudaSuccess) return e;
-
     const long long blocks = (P.strips.total + 3) / 4;
     long long per_head = num_sms / p.heads;
     if (per_head > blocks) per_head = blocks;
     if (per_head < 1) per_head = 1;
     return launch_chained(umma_split_kernel<T, D>, dim3((unsigned)(per_head * p.heads)), kThreads, F::total, stream, mk, mv, P);
+}
+
+template <typename T, int D> struct Heads { using type = T; static constexpr int dim = D; };
+
+// f(the instance of p's storage type and head width)
+template <typename F>
+cudaError_t of_heads(const Problem& p, F f) {
+    if (p.dtype == SLIDE_ATTN_BF16) return p.head_dim == 16 ? f(Heads<NarrowBf16, 16>()) : p.head_dim == 32 ? f(Heads<__nv_bfloat16, 32>()) : f(Heads<__nv_bfloat16, 64>());
+    return p.head_dim == 16 ? f(Heads<float, 16>()) : p.head_dim == 32 ? f(Heads<float, 32>()) : f(Heads<float, 64>());
 }
 
 }  // namespace
@@ -335,15 +341,20 @@ size_t umma_split_workspace_bytes(int heads, int head_dim) {
     return (size_t)heads * (contract_bytes(head_dim) + expand_bytes(head_dim));
 }
 
-// Prep launch (weights -> images in `workspace`) followed by the fused kernel.
-cudaError_t launch_umma_split(const Problem& p, void* workspace, int* d_status, int num_sms, cudaStream_t stream) {
-    if (p.dtype == SLIDE_ATTN_BF16)
-        return p.head_dim == 16 ? launch_t<NarrowBf16, 16>(p, workspace, d_status, num_sms, stream)
-             : p.head_dim == 32 ? launch_t<__nv_bfloat16, 32>(p, workspace, d_status, num_sms, stream)
-                                : launch_t<__nv_bfloat16, 64>(p, workspace, d_status, num_sms, stream);
-    return p.head_dim == 16 ? launch_t<float, 16>(p, workspace, d_status, num_sms, stream)
-         : p.head_dim == 32 ? launch_t<float, 32>(p, workspace, d_status, num_sms, stream)
-                            : launch_t<float, 64>(p, workspace, d_status, num_sms, stream);
+// Weights -> images in `workspace`.
+cudaError_t launch_umma_split_prep(const Problem& p, void* workspace, cudaStream_t stream) {
+    return of_heads(p, [&](auto heads) {
+        using H = decltype(heads);
+        return launch_chained(umma_split_prep_kernel<typename H::type, H::dim>, dim3((unsigned)p.heads, prep_parts(H::dim)), 256, 0, stream, p.wk, p.wv,
+                              static_cast<unsigned char*>(workspace));
+    });
+}
+
+cudaError_t launch_umma_split(const Problem& p, const void* workspace, int* d_status, int num_sms, cudaStream_t stream) {
+    return of_heads(p, [&](auto heads) {
+        using H = decltype(heads);
+        return launch_t<typename H::type, H::dim>(p, workspace, d_status, num_sms, stream);
+    });
 }
 
 }  // namespace slide_attn
