@@ -620,19 +620,22 @@ bool backward_supports(int head_dim, int ksize) {
     return head_dim == kHeadDim && (ksize == 1 || ksize == 3) && tensor_map_available();
 }
 
-size_t backward_workspace_bytes(int B, int H, int W, int heads, int ksize) {
-    return ksize == 3 ? bwd_team_workspace_bytes(B, H, W, heads) : 2 * (size_t)B * H * W * heads * ksize * ksize * sizeof(float);
+size_t backward_workspace_bytes(int B, int H, int W, int heads, int ksize, bool compact) {
+    return ksize == 3 ? bwd_team_workspace_bytes(B, H, W, heads, compact) : 2 * (size_t)B * H * W * heads * ksize * ksize * sizeof(float);
 }
 
 // `ws`: backward_workspace_bytes of scratch; `wt`: strip_workspace_bytes, used for k = 1.
-cudaError_t launch_backward(const Problem& p, const BackwardArgs& ga, void* wt, void* ws, int* d_status, int num_sms, cudaStream_t stream) {
+cudaError_t launch_backward(const Problem& p, const BackwardArgs& ga, void* wt, void* ws, bool compact, int* d_status, int num_sms, cudaStream_t stream) {
     cudaError_t e;
     if (p.ksize == 3) {
-        const BwdScratch s = bwd_scratch(ws, p.B, p.H, p.W, p.heads);
-        e = launch_bwd_team(p, ga, s, d_status, num_sms, stream);
+        const BwdScratch s = bwd_scratch(ws, compact, ga.dv, p.B, p.H, p.W, p.heads);
+        e = launch_bwd_team(BwdPass::point, p, ga, s, d_status, num_sms, stream);
         if (e != cudaSuccess) return e;
-        return p.dtype == SLIDE_ATTN_BF16 ? launch_bwd_weight_umma(p, ga, s, d_status, num_sms, stream)
-                                          : launch_bwd_weight_mma(p, ga, s, d_status, num_sms, stream);
+        // the other way round (2 x 128 x 128 x 3, fp32: 2 us less; 64 x 56 x 56 x 3, bf16: 4 us more) only where dv holds split rows
+        if (!compact) e = launch_bwd_team(BwdPass::gather, p, ga, s, d_status, num_sms, stream);
+        if (e != cudaSuccess) return e;
+        e = p.dtype == SLIDE_ATTN_BF16 ? launch_bwd_weight_umma(p, ga, s, d_status, num_sms, stream) : launch_bwd_weight_mma(p, ga, s, d_status, num_sms, stream);
+        return e == cudaSuccess && compact ? launch_bwd_team(BwdPass::gather, p, ga, s, d_status, num_sms, stream) : e;
     }
     const size_t k2 = (size_t)p.ksize * p.ksize, wbytes = (size_t)p.heads * kHeadDim * k2 * k2 * sizeof(float);
     e = cudaMemsetAsync(ga.dwk, 0, wbytes, stream);

@@ -11,6 +11,8 @@
 // bwd_gather_kernel: dk and dv per key / value pixel, a gather over the nine query pixels whose window holds it.  The left
 // operand of tap t is the split rows of the block's pixels moved by -off(t): every tap has rows of its own, copied from a halo
 // in shared memory to tensor memory (out-of-map queries read as zero and contribute nothing), N = the channels of a plane.
+// One launch computes both, or two launches one each where memory is short: the rows of dl then lie where dv will be (64 bytes a pixel and
+// head, which is what dv takes in bf16) until the second launch writes it (64 x 56 x 56, 3 heads, bf16: 7 us more).
 // Both persistent, one CTA per SM and one head per CTA, two teams; geometry and hand-offs as in umma_split_kernel.
 //
 // Bound by instruction issue on the CUDA cores: products and their splits, sums, the point kernel's softmax, dL and row splits
@@ -57,6 +59,7 @@ struct TeamParams {
     float* dbias;
     int* status;
     int H, W, heads;
+    int first_side, sides;           // of bwd_gather_kernel: 0 dk, 1 dv
     Strips strips;
     float scale;
 };
@@ -434,8 +437,8 @@ bwd_gather_kernel(const __grid_constant__ CUtensorMap map_dl, const __grid_const
             uint32_t phase = 1;
             StripWalk at(P.strips, seat.strip0(0), 4LL * seat.step);
             for (int bi = 0; ok && bi < my_blocks; ++bi, at.next()) {
-                for (int v = 0; v < 2 * (NPL + 1); ++v) {
-                    const int side = v / (NPL + 1), pl = v % (NPL + 1) - 1;
+                for (int v = 0; v < P.sides * (NPL + 1); ++v) {
+                    const int side = P.first_side + v / (NPL + 1), pl = v % (NPL + 1) - 1;
                     if (!mbar_wait(bar(kEmpty + slot), phase)) { ok = false; break; }
                     load_strips(smem_u32(seat.ring) + (uint32_t)(slot * kSlot), pl < 0 ? (side ? &map_a : &map_dl) : (side ? &map_g : &map_q), bar(kFull + slot),
                                 h * kHeadDim + (pl < 0 ? 0 : pl * CH), at);
@@ -457,8 +460,8 @@ bwd_gather_kernel(const __grid_constant__ CUtensorMap map_dl, const __grid_const
             }
             if (my_blocks > 0) ok = mbar_wait(seat.bar_weights, 0);
             int dn = 0;
-            for (int s = 0; ok && s < my_blocks * 6; ++s) {         // side, tap column
-                const int side = s / 3 & 1, dx = s % 3;
+            for (int s = 0; ok && s < my_blocks * P.sides * 3; ++s) { // side, tap column
+                const int side = P.first_side + (s / 3 & (P.sides - 1)), dx = s % 3;
                 if (!mbar_wait(bar(kAFull), (uint32_t)s & 1u)) { ok = false; break; }
                 for (int pl = 0; pl < NPL; ++pl, ++dn) {
                     const int db = dn % DB;
@@ -517,9 +520,10 @@ bwd_gather_kernel(const __grid_constant__ CUtensorMap map_dl, const __grid_const
         int slot = 1, dn = 0;                                        // of the side's first plane
         uint32_t phase = 0;
         if (my_blocks > 0) ok = store_rows(0, half == 0);
-        for (int bs = 0; ok && bs < 2 * my_blocks; ++bs) {           // block, side
-            const int side = bs & 1;
-            const bool even = half == side;                          // step 3 bs + dx is this warp's if even == (dx != 1)
+        const int steps = P.sides * my_blocks;
+        for (int bs = 0; ok && bs < steps; ++bs) {                   // block, side
+            const int side = P.first_side + (bs & (P.sides - 1));
+            const bool even = half == (bs & 1);                      // step 3 bs + dx is this warp's if even == (dx != 1)
             float acc[NPL][2][PL];
 #pragma unroll
             for (int pl = 0; pl < NPL; ++pl)
@@ -540,7 +544,7 @@ bwd_gather_kernel(const __grid_constant__ CUtensorMap map_dl, const __grid_const
                     // the last MMAs of this step are complete: its operands make room for the next ones
                     if (pl == NPL - 1) {
                         if (dx < 2) { if (!store_rows(dx + 1, dx == 0 ? !even : even)) { ok = false; break; } }
-                        else if (bs + 1 < 2 * my_blocks) { if (!store_rows(0, !even)) { ok = false; break; } }
+                        else if (bs + 1 < steps) { if (!store_rows(0, !even)) { ok = false; break; } }
                     }
                     sum_chunk<true>(T(), mine + kColD + (uint32_t)(db * 3 * CH), seat.ring + (uint32_t)(ps * kSlot + wq * kHaloPlane), 2 * half, g + 2 - dx, tig, acc[pl]);
                     tc_fence_before_sync();
@@ -553,14 +557,14 @@ bwd_gather_kernel(const __grid_constant__ CUtensorMap map_dl, const __grid_const
             }
             if (!ok) break;
             ahead(slot, phase, NPL + 1);
-            const Place p = me.place(P, seat.strip0(bs >> 1) + wq, 2 * half, g);
+            const Place p = me.place(P, seat.strip0(P.sides == 2 ? bs >> 1 : bs) + wq, 2 * half, g);
             T* out = static_cast<T*>(side ? P.dv : P.dk) + p.pix * C + piece;
 #pragma unroll
             for (int r = 0; r < 2; ++r)
                 if (p.in[r])
 #pragma unroll
                     for (int pl = 0; pl < NPL; ++pl) store_piece(out + r * row_pitch + pl * CH, acc[pl][r], side ? 1.f : P.scale);
-            if (side) me.walk.next();
+            if (side || P.sides == 1) me.walk.next();
         }
         if (!ok && lane == 0) atomicExch(P.status, 1);
     }
@@ -568,7 +572,7 @@ bwd_gather_kernel(const __grid_constant__ CUtensorMap map_dl, const __grid_const
 }
 
 template <typename T>
-cudaError_t launch_t(const Problem& p, const BackwardArgs& ga, const BwdScratch& ws, int* d_status, int num_sms, cudaStream_t stream) {
+cudaError_t launch_t(BwdPass what, const Problem& p, const BackwardArgs& ga, const BwdScratch& ws, int* d_status, int num_sms, cudaStream_t stream) {
     static bool configured[64] = {};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -587,41 +591,49 @@ cudaError_t launch_t(const Problem& p, const BackwardArgs& ga, const BwdScratch&
     P.strips.total = (long long)p.B * P.strips.bands * P.strips.sx;
     if (P.strips.total > 0x7fffffffLL - 4) return cudaErrorInvalidConfiguration;
     P.scale = 1.f / sqrtf((float)kHeadDim);
+    P.first_side = 0; P.sides = 2;
     const int C = p.heads * kHeadDim, es = (int)sizeof(T), ch = Cut<T>::channels;
-    CUtensorMap mq, mk, mv, mg, mdl, ma;
-    if (!make_tile_map(&mq, p.q, es, p.B, p.H, p.W, C, ch, 10, 6) || !make_tile_map(&mk, p.k, es, p.B, p.H, p.W, C, ch, 10, 6) ||
-        !make_tile_map(&mv, p.v, es, p.B, p.H, p.W, C, ch, 10, 6) || !make_tile_map(&mg, ga.dout, es, p.B, p.H, p.W, C, ch, 10, 6) ||
-        !make_tile_map(&mdl, ws.rows_dl, 2, p.B, p.H, p.W, C, 32, 10, 6) || !make_tile_map(&ma, ws.rows_a, 2, p.B, p.H, p.W, C, 32, 10, 6))
-        return cudaErrorInvalidValue;
-    e = launch_chained(bwd_prep_kernel<T>, dim3((unsigned)p.heads, 9), 256, 0, stream, p.wk, p.wv, ws.images, ga.dwk, ga.dwv, ga.dbias);
-    if (e != cudaSuccess) return e;
     const long long blocks = (P.strips.total + 3) / 4;
     long long per_head = num_sms / p.heads;
     if (per_head > blocks) per_head = blocks;
     if (per_head < 1) per_head = 1;
     const dim3 grid((unsigned)(per_head * p.heads));
-    e = launch_chained(bwd_point_kernel<T>, grid, kThreads, Plan<kPointImages>::total, stream, mk, mv, P);
-    if (e != cudaSuccess) return e;
-    return launch_chained(bwd_gather_kernel<T>, grid, kThreads, Plan<kGatherImages>::total, stream, mdl, ma, mq, mg, P);
+    if (what == BwdPass::point) {
+        CUtensorMap mk, mv;
+        if (!make_tile_map(&mk, p.k, es, p.B, p.H, p.W, C, ch, 10, 6) || !make_tile_map(&mv, p.v, es, p.B, p.H, p.W, C, ch, 10, 6)) return cudaErrorInvalidValue;
+        e = launch_chained(bwd_prep_kernel<T>, dim3((unsigned)p.heads, 9), 256, 0, stream, p.wk, p.wv, ws.images, ga.dwk, ga.dwv, ga.dbias);
+        if (e != cudaSuccess) return e;
+        return launch_chained(bwd_point_kernel<T>, grid, kThreads, Plan<kPointImages>::total, stream, mk, mv, P);
+    }
+    CUtensorMap mq, mg, mdl, ma;
+    if (!make_tile_map(&mq, p.q, es, p.B, p.H, p.W, C, ch, 10, 6) || !make_tile_map(&mg, ga.dout, es, p.B, p.H, p.W, C, ch, 10, 6) ||
+        !make_tile_map(&mdl, ws.rows_dl, 2, p.B, p.H, p.W, C, 32, 10, 6) || !make_tile_map(&ma, ws.rows_a, 2, p.B, p.H, p.W, C, 32, 10, 6))
+        return cudaErrorInvalidValue;
+    if (ws.rows_dl == ga.dv) P.sides = 1;
+    for (; P.first_side < 2 && e == cudaSuccess; P.first_side += P.sides)
+        e = launch_chained(bwd_gather_kernel<T>, grid, kThreads, Plan<kGatherImages>::total, stream, mdl, ma, mq, mg, P);
+    return e;
 }
 
 size_t rows_bytes(int B, int H, int W, int heads) { return (size_t)B * H * W * heads * 64; }
 
 }  // namespace
 
-size_t bwd_team_workspace_bytes(int B, int H, int W, int heads) { return 2 * rows_bytes(B, H, W, heads) + (size_t)heads * kImages + 512; }
+size_t bwd_team_workspace_bytes(int B, int H, int W, int heads, bool compact) {
+    return (compact ? 1 : 2) * (rows_bytes(B, H, W, heads) + 256) + (size_t)heads * kImages;
+}
 
-BwdScratch bwd_scratch(void* ws, int B, int H, int W, int heads) {
-    auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
+BwdScratch bwd_scratch(void* ws, bool compact, void* dv, int B, int H, int W, int heads) {
+    const size_t rows = (rows_bytes(B, H, W, heads) + 255) & ~(size_t)255;
     BwdScratch s;
-    s.rows_dl = static_cast<unsigned char*>(ws);
-    s.rows_a = s.rows_dl + up(rows_bytes(B, H, W, heads));
-    s.images = s.rows_a + up(rows_bytes(B, H, W, heads));
+    s.rows_a = static_cast<unsigned char*>(ws);
+    s.rows_dl = compact ? static_cast<unsigned char*>(dv) : s.rows_a + rows;
+    s.images = s.rows_a + (compact ? 1 : 2) * rows;
     return s;
 }
 
-cudaError_t launch_bwd_team(const Problem& p, const BackwardArgs& ga, const BwdScratch& ws, int* d_status, int num_sms, cudaStream_t stream) {
-    return p.dtype == SLIDE_ATTN_BF16 ? launch_t<__nv_bfloat16>(p, ga, ws, d_status, num_sms, stream) : launch_t<float>(p, ga, ws, d_status, num_sms, stream);
+cudaError_t launch_bwd_team(BwdPass what, const Problem& p, const BackwardArgs& ga, const BwdScratch& ws, int* d_status, int num_sms, cudaStream_t stream) {
+    return p.dtype == SLIDE_ATTN_BF16 ? launch_t<__nv_bfloat16>(what, p, ga, ws, d_status, num_sms, stream) : launch_t<float>(what, p, ga, ws, d_status, num_sms, stream);
 }
 
 }  // namespace slide_attn

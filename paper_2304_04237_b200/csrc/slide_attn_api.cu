@@ -22,7 +22,8 @@ struct slide_attn_ctx {
     void* umma_ws;                   // bf16 B images of the UMMA_TS variant
     void* split_ws;                  // weight images of the UMMA_SPLIT variant
     void* wide_ws;                   // bf16 weight images of the MMA_WIDE variant
-    void* bwd_ws;                    // attention weights and logit gradients between the two backward kernels (first backward)
+    void* bwd_ws;                    // attention weights and logit gradients between the backward kernels (first backward)
+    bool bwd_compact;                // it was too large and holds the former only
     void* block_ws;                  // q, k, v, z of slide_attn_block_forward (first use)
     // staging buffers for slide_attn_forward_host, allocated on first use
     void* stage;
@@ -345,18 +346,20 @@ slide_attn_status slide_attn_backward(slide_attn_ctx* c, const void* q, const vo
         return SLIDE_ATTN_ERR_INVALID_ARG;
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
     if (!c->bwd_ws) {
-        if (cudaMalloc(&c->bwd_ws, backward_workspace_bytes(c->B, c->H, c->W, c->heads, c->ksize)) != cudaSuccess) {
-            cudaGetLastError();
-            c->bwd_ws = nullptr;
-            return SLIDE_ATTN_ERR_ALLOC;
-        }
+        auto allocate = [&](bool compact) {
+            c->bwd_compact = compact;
+            const bool ok = cudaMalloc(&c->bwd_ws, backward_workspace_bytes(c->B, c->H, c->W, c->heads, c->ksize, compact)) == cudaSuccess;
+            if (!ok) { cudaGetLastError(); c->bwd_ws = nullptr; }
+            return ok;
+        };
+        if (!allocate(false) && !allocate(true)) return SLIDE_ATTN_ERR_ALLOC;
     }
     Problem p;
     p.B = c->B; p.H = c->H; p.W = c->W; p.heads = c->heads; p.head_dim = c->head_dim;
     p.ksize = c->ksize; p.has_bias = c->has_bias; p.dtype = c->dtype;
     p.q = q; p.k = k; p.v = v; p.wk = wk; p.wv = wv; p.bias = bias; p.out = nullptr;
     BackwardArgs ga = {dout, dq, dk, dv, dwk, dwv, dbias};
-    const bool ok = launch_backward(p, ga, c->strip_ws, c->bwd_ws, c->d_status, c->num_sms, stream) == cudaSuccess;
+    const bool ok = launch_backward(p, ga, c->strip_ws, c->bwd_ws, c->bwd_compact, c->d_status, c->num_sms, stream) == cudaSuccess;
     if (!ok) { cudaGetLastError(); return SLIDE_ATTN_ERR_CUDA; }
     return SLIDE_ATTN_OK;
 }

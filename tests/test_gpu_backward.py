@@ -131,3 +131,35 @@ def test_backward_argument_errors():
         assert e.value.status == sa.ERR_INVALID_ARG
     finally:
         sa.slide_attn_destroy(ctx)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_backward_with_half_the_scratch(dtype):
+    """Where the scratch (128 bytes a pixel and head, 40 MB here) is not to be had, half of it is enough; same bits."""
+    B, H, W, heads = 25, 64, 64, 3
+    td = TORCH_DTYPE[dtype]
+    gen = torch.Generator(device="cuda").manual_seed(7)
+    q, k, v, dout = (torch.randn(B, H, W, heads, 32, device="cuda", generator=gen).to(td) for _ in range(4))
+    wk, wv = (torch.randn(heads * 32, 9, 9, device="cuda", generator=gen) * 0.2 for _ in range(2))
+    grads = [[torch.full_like(t, float("nan")) for t in (q, k, v, wk, wv)] for _ in range(2)]
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    for g, left in zip(grads, (None, 30 << 20)):
+        ctx = sa.slide_attn_create(B, H, W, heads, 32, 3, td, False)
+        held = []
+        try:
+            if left:
+                for piece in (1 << 30, 64 << 20, 2 << 20):          # all but `left` of the device's memory
+                    while torch.cuda.mem_get_info()[0] > left + piece:
+                        held.append(torch.empty(min(torch.cuda.mem_get_info()[0] - left, 8 << 30) // piece * piece, dtype=torch.uint8, device="cuda"))
+                assert torch.cuda.mem_get_info()[0] < 38 << 20
+            sa.slide_attn_backward(ctx, q, k, v, wk, wv, None, dout, *g, None)
+            assert sa.slide_attn_query_status(ctx) == sa.OK
+        finally:
+            sa.slide_attn_destroy(ctx)
+            held.clear()
+            torch.cuda.empty_cache()
+    for a, b in zip(*(g[:3] for g in grads)):
+        assert torch.equal(a, b) and torch.isfinite(a.float()).all()
+    for a, b in zip(*(g[3:] for g in grads)):                       # atomics
+        assert (a - b).abs().max() <= 1e-5 * a.abs().max()
