@@ -109,9 +109,11 @@ def _host_ptr(t):
 
 def _stream_ptr(stream):
     if stream is None:
-        # torch.cuda.current_stream() builds a stream object, 3 of the 13 us that a small call takes; the raw handle costs 0.3
-        if torch.cuda.is_initialized():
-            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+        # torch.cuda.current_stream() builds a stream object, 3 of the 13 us that a small call takes; the raw handle, where this
+        # torch gives it out, costs 0.3
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        if raw is not None and torch.cuda.is_initialized():
+            return raw(torch.cuda.current_device())
         stream = torch.cuda.current_stream()
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 

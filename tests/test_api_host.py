@@ -79,3 +79,17 @@ def test_product_package_does_not_import_the_oracle():
                 src = open(os.path.join(dirpath, f)).read()
                 assert "import oracle" not in src and "from oracle" not in src, f
                 assert "slide_attn_oracle" not in src, f
+
+
+def test_current_stream_without_the_raw_handle(monkeypatch):
+    """torch gives the current stream's raw handle out through a private function; without it the stream object has it."""
+    import types
+
+    import torch
+
+    from paper_2304_04237_b200 import binding
+    monkeypatch.delattr(torch._C, "_cuda_getCurrentRawStream", raising=False)
+    monkeypatch.setattr(torch.cuda, "is_initialized", lambda: True)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda *a: types.SimpleNamespace(cuda_stream=1234))
+    assert binding._stream_ptr(None) == 1234
+    assert binding._stream_ptr(types.SimpleNamespace(cuda_stream=5)) == 5 and binding._stream_ptr(7) == 7
