@@ -201,8 +201,8 @@ slide_attn_status slide_attn_launches_per_forward(const slide_attn_ctx* ctx, int
  * forward state is needed.  Supported: head_dim 32, ksize 1 or 3, both dtypes
  * (SLIDE_ATTN_ERR_UNSUPPORTED otherwise).  Arithmetic is fp32; dq, dk, dv are rounded to the dtype
  * once; dwk, dwv, dbias are summed over pixels with floating-point atomics, so their last bits may
- * differ from run to run.  The FIRST backward on a context allocates a scratch buffer (cudaMalloc,
- * synchronous) of 2 * B*H*W*heads*4 bytes for ksize 1 and about 2 * B*H*W*heads*64 for ksize 3, or half of that
+ * differ from run to run.  With ksize 3 the FIRST backward on a context allocates a scratch
+ * buffer (cudaMalloc, synchronous, typically 0.3 ms) of about 2 * B*H*W*heads*64 bytes, or half of that
  * where the whole is not to be had (dv's memory then holds intermediate results until dv is written, at the
  * price of one more launch); later calls allocate nothing.
  */

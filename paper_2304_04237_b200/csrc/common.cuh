@@ -114,9 +114,9 @@ struct BackwardArgs {
     float* dbias;        // [heads][k*k] or nullptr
 };
 bool backward_supports(int head_dim, int ksize);
-// `compact` (k = 3): scratch for half of the intermediate results only; the others lie in dv until it is written.
+// Scratch: none for k = 1.  `compact` (k = 3): for half of the intermediate results only; the others lie in dv until it is written.
 size_t backward_workspace_bytes(int B, int H, int W, int heads, int ksize, bool compact);
-cudaError_t launch_backward(const Problem& p, const BackwardArgs& ga, void* wt, void* ws, bool compact, int* d_status,
+cudaError_t launch_backward(const Problem& p, const BackwardArgs& ga, void* ws, bool compact, int* d_status,
                             int num_sms, cudaStream_t stream);
 
 // MMA_WIDE variant: general weights with large windows on tcgen05 (bf16, head_dim 32, k = 3, 5, 7, 9); a prep

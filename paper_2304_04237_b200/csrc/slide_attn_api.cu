@@ -337,7 +337,7 @@ slide_attn_status slide_attn_backward(slide_attn_ctx* c, const void* q, const vo
     if (!c || !q || !k || !v || !wk || !wv || !dout || !dq || !dk || !dv || !dwk || !dwv) return SLIDE_ATTN_ERR_INVALID_ARG;
     if ((c->has_bias != 0) != (bias != nullptr) || (c->has_bias != 0) != (dbias != nullptr)) return SLIDE_ATTN_ERR_INVALID_ARG;
     if (!on_ctx_device(c)) return SLIDE_ATTN_ERR_INVALID_ARG;
-    if (!backward_supports(c->head_dim, c->ksize) || !c->strip_ws) return SLIDE_ATTN_ERR_UNSUPPORTED;
+    if (!backward_supports(c->head_dim, c->ksize)) return SLIDE_ATTN_ERR_UNSUPPORTED;
     const void* ptrs[] = {q, k, v, wk, wv, dout, dq, dk, dv, dwk, dwv};
     for (const void* p : ptrs) if (!aligned16(p)) return SLIDE_ATTN_ERR_ALIGNMENT;
     if ((bias && !aligned16(bias)) || (dbias && !aligned16(dbias))) return SLIDE_ATTN_ERR_ALIGNMENT;
@@ -345,7 +345,7 @@ slide_attn_status slide_attn_backward(slide_attn_ctx* c, const void* q, const vo
         dv == q || dv == k || dv == v || dv == dout || dq == dk || dq == dv || dk == dv)
         return SLIDE_ATTN_ERR_INVALID_ARG;
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-    if (!c->bwd_ws) {
+    if (!c->bwd_ws && c->ksize != 1) {
         auto allocate = [&](bool compact) {
             c->bwd_compact = compact;
             const bool ok = cudaMalloc(&c->bwd_ws, backward_workspace_bytes(c->B, c->H, c->W, c->heads, c->ksize, compact)) == cudaSuccess;
@@ -359,7 +359,7 @@ slide_attn_status slide_attn_backward(slide_attn_ctx* c, const void* q, const vo
     p.ksize = c->ksize; p.has_bias = c->has_bias; p.dtype = c->dtype;
     p.q = q; p.k = k; p.v = v; p.wk = wk; p.wv = wv; p.bias = bias; p.out = nullptr;
     BackwardArgs ga = {dout, dq, dk, dv, dwk, dwv, dbias};
-    const bool ok = launch_backward(p, ga, c->strip_ws, c->bwd_ws, c->bwd_compact, c->d_status, c->num_sms, stream) == cudaSuccess;
+    const bool ok = launch_backward(p, ga, c->bwd_ws, c->bwd_compact, c->d_status, c->num_sms, stream) == cudaSuccess;
     if (!ok) { cudaGetLastError(); return SLIDE_ATTN_ERR_CUDA; }
     return SLIDE_ATTN_OK;
 }
