@@ -35,8 +35,9 @@ constexpr int kThreads = (kComputeWarps + 1) * 32;
 constexpr float kTruncation = 4.3e-8f;         // what one truncation takes off on average (team.cuh): half of 2^-23 / (2 ln 2)
 constexpr uint32_t kSumBytes = 2u * kK2 * kHeadDim * 32u * 4u;        // the CTA's sums at its end, [side][tap][channel][32 columns]
 
-template <typename T> struct WTile;
-template <> struct WTile<float> { static constexpr int max_w = 32, planes = 2; };
+constexpr int kMaxW = 32;                      // tile columns
+constexpr int kPlanes = 2;                     // planes of 16 channels
+constexpr uint32_t kPixel = 64;                // bytes of a pixel in a plane
 
 // Stage layout for tiles of tw columns (bytes); the channel planes of a tensor follow each other.
 struct WLayout {
@@ -46,9 +47,8 @@ struct WLayout {
     uint32_t stage;                            // bytes of a stage
     uint32_t tx_bytes;
 };
-template <typename T>
 __host__ __device__ inline WLayout w_layout(int tw) {
-    constexpr uint32_t np = (uint32_t)WTile<T>::planes, pb = 32u / np * (uint32_t)sizeof(T);
+    constexpr uint32_t np = kPlanes, pb = kPixel;
     auto up = [](uint32_t x) { return (x + 127u) & ~127u; };
     WLayout L;
     const uint32_t halo = (uint32_t)((kTH + 2) * (tw + 2)) * pb, tile = (uint32_t)(kTH * tw) * pb;
@@ -61,9 +61,8 @@ __host__ __device__ inline WLayout w_layout(int tw) {
     return L;
 }
 
-template <typename T>
 uint32_t w_smem_bytes(int tw) {
-    const uint32_t stages = 2 * w_layout<T>(tw).stage;
+    const uint32_t stages = 2 * w_layout(tw).stage;
     return (stages > kSumBytes ? stages : kSumBytes) + 64 + 128;      // + barriers + alignment slack
 }
 
@@ -77,25 +76,23 @@ struct WParams {
 };
 
 // One 16-pixel (2 rows x 8 columns), 16-channel operand tile in registers: the values of channels 2g, 2g + 1 of the lane's
-// four pixels.  `offset` and `col` say where a lane reads, in a tile whose planes are `plane` bytes and whose rows are `pitch`
-// bytes apart, and which column of the group the K index k (of its row's eight) is.
-template <typename T> struct Frag;
-template <> struct Frag<float> {
-    static constexpr uint32_t pixel_bytes = 64;
+// four pixels.  `offset`: where a lane reads in a tile whose planes are `plane` bytes apart; `col`: which column of the group the K index
+// k (of its row's eight) is; `channel`: which of the 16 channels the row is.
+struct Frag {
     float2 a[4];
-    static __device__ __forceinline__ uint32_t offset(int lane, int half, uint32_t plane, uint32_t) {
-        return (uint32_t)half * plane + (uint32_t)(lane & 3) * pixel_bytes + (uint32_t)(lane >> 2) * 8u;
+    static __device__ __forceinline__ uint32_t offset(int lane, int half, uint32_t plane) {
+        return (uint32_t)half * plane + (uint32_t)(lane & 3) * kPixel + (uint32_t)(lane >> 2) * 8u;
     }
     static __device__ __forceinline__ int col(int k) { return (k & 1) * 4 + (k >> 1); }
     static __device__ __forceinline__ int channel(int row) { return 2 * (row & 7) + (row >> 3); }
     __device__ __forceinline__ void load(uint32_t p, uint32_t pitch) {
-        a[0] = lds_f2(p); a[1] = lds_f2(p + 4 * pixel_bytes);
-        a[2] = lds_f2(p + pitch); a[3] = lds_f2(p + pitch + 4 * pixel_bytes);
+        a[0] = lds_f2(p); a[1] = lds_f2(p + 4 * kPixel);
+        a[2] = lds_f2(p + pitch); a[3] = lds_f2(p + pitch + 4 * kPixel);
     }
 };
 
 // sum += (x . y) times the split columns b[tile][2]
-__device__ __forceinline__ void accumulate(float (&sum)[4][4], const Frag<float>& x, const Frag<float>& y, const uint32_t (&b)[4][2]) {
+__device__ __forceinline__ void accumulate(float (&sum)[4][4], const Frag& x, const Frag& y, const uint32_t (&b)[4][2]) {
     float2 p[4];
     uint32_t a[3][4];
 #pragma unroll
@@ -122,16 +119,14 @@ __device__ __forceinline__ void accumulate(float (&sum)[4][4], const Frag<float>
     mma_bf16(sum[3], a[0], b[3][0], b[3][1]);
 }
 
-template <typename T>
 __global__ void __launch_bounds__(kThreads, 1)
 bwd_weight_mma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                       const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_g,
                       const __grid_constant__ CUtensorMap map_dl, const __grid_constant__ CUtensorMap map_a, const WParams P)
 {
-    constexpr uint32_t PB = Frag<T>::pixel_bytes;                    // of one plane
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u);
-    const WLayout L = w_layout<T>(P.tw);
+    const WLayout L = w_layout(P.tw);
     const uint32_t stages = 2 * L.stage;
     const uint32_t bar0 = smem_u32(smem) + (stages > kSumBytes ? stages : kSumBytes);
     auto bar_full = [&](int s) { return bar0 + 8u * (uint32_t)s; };
@@ -173,8 +168,8 @@ bwd_weight_mma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
                 tma_load_4d(stage + L.split_off, &map_dl, bar_full(st), h * 32, x0, y0, b);
                 tma_load_4d(stage + L.split_off + L.split_side, &map_a, bar_full(st), h * 32, x0, y0, b);
 #pragma unroll
-                for (int pl = 0; pl < WTile<T>::planes; ++pl) {
-                    const int c0 = h * kHeadDim + pl * (32 / WTile<T>::planes);
+                for (int pl = 0; pl < kPlanes; ++pl) {
+                    const int c0 = h * kHeadDim + pl * (32 / kPlanes);
                     tma_load_4d(stage + L.k_off + pl * L.halo_plane, &map_k, bar_full(st), c0, x0 - 1, y0 - 1, b);
                     tma_load_4d(stage + L.v_off + pl * L.halo_plane, &map_v, bar_full(st), c0, x0 - 1, y0 - 1, b);
                     tma_load_4d(stage + L.q_off + pl * L.tile_plane, &map_q, bar_full(st), c0, x0, y0, b);
@@ -193,13 +188,13 @@ bwd_weight_mma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
 #pragma unroll
                 for (int x = 0; x < 4; ++x) sum[t][j][x] = 0.f;
         // lane i of the ldmatrix of the split columns: K index i % 8 of row (i / 8) % 2, 16-byte chunk i / 16 (+ 2)
-        const int kcol = Frag<T>::col(lane & 7);
+        const int kcol = Frag::col(lane & 7);
         const uint32_t b_off = L.split_off + (uint32_t)side * L.split_side + (uint32_t)(((lane >> 3) & 1) * P.tw + kcol) * 64u;
         const uint32_t b_chunk0 = (((uint32_t)lane >> 4) ^ ((uint32_t)kcol >> 1)) << 4;
         const uint32_t b_chunk1 = ((2u + ((uint32_t)lane >> 4)) ^ ((uint32_t)kcol >> 1)) << 4;
-        const uint32_t x_pitch = (uint32_t)P.tw * PB, y_pitch = (uint32_t)HW * PB;
-        const uint32_t x_off = (side ? L.g_off : L.q_off) + Frag<T>::offset(lane, half, L.tile_plane, x_pitch);
-        const uint32_t y_off = (side ? L.v_off : L.k_off) + (uint32_t)ty * y_pitch + Frag<T>::offset(lane, half, L.halo_plane, y_pitch);
+        const uint32_t x_pitch = (uint32_t)P.tw * kPixel, y_pitch = (uint32_t)HW * kPixel;
+        const uint32_t x_off = (side ? L.g_off : L.q_off) + Frag::offset(lane, half, L.tile_plane);
+        const uint32_t y_off = (side ? L.v_off : L.k_off) + (uint32_t)ty * y_pitch + Frag::offset(lane, half, L.halo_plane);
         int it = 0;
         for (int tile = rank; tile < tiles; tile += nrank, ++it) {
             const int st = it & 1;
@@ -212,14 +207,14 @@ bwd_weight_mma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
             for (int r = 0; r < gy; r += 2) {
                 uint32_t ba = stage + b_off + (uint32_t)(r * P.tw) * 64u;
                 uint32_t xa = stage + x_off + (uint32_t)r * x_pitch, ya = stage + y_off + (uint32_t)r * y_pitch;
-                for (int c = 0; c < gx; c += 8, ba += 8 * 64, xa += 8 * PB, ya += 8 * PB) {
+                for (int c = 0; c < gx; c += 8, ba += 8 * 64, xa += 8 * kPixel, ya += 8 * kPixel) {
                     uint32_t b[4][2];
                     ldmatrix_x4_trans(ba + b_chunk0, b[0][0], b[0][1], b[1][0], b[1][1]);
                     ldmatrix_x4_trans(ba + b_chunk1, b[2][0], b[2][1], b[3][0], b[3][1]);
-                    Frag<T> x, y[3];
+                    Frag x, y[3];
                     x.load(xa, x_pitch);
 #pragma unroll
-                    for (int t = 0; t < 3; ++t) y[t].load(ya + t * PB, y_pitch);
+                    for (int t = 0; t < 3; ++t) y[t].load(ya + t * kPixel, y_pitch);
 #pragma unroll
                     for (int t = 0; t < 3; ++t) accumulate(sum[t], x, y[t], b);
                 }
@@ -242,7 +237,7 @@ bwd_weight_mma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
             for (int j = 0; j < 4; ++j)
 #pragma unroll
                 for (int x = 0; x < 4; ++x) {
-                    const int ch = half * 16 + Frag<T>::channel(g + 8 * (x >> 1));
+                    const int ch = half * 16 + Frag::channel(g + 8 * (x >> 1));
                     s_sum[((side * kK2 + ty * 3 + t) * kHeadDim + ch) * 32 + 8 * j + 2 * tig + (x & 1)] = sum[t][j][x];
                 }
     }
@@ -257,20 +252,21 @@ bwd_weight_mma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
     }
 }
 
-template <typename T>
-cudaError_t launch_t(const Problem& p, const BackwardArgs& ga, const BwdScratch& ws, int* d_status, int num_sms, cudaStream_t stream) {
+}  // namespace
+
+cudaError_t launch_bwd_weight_mma(const Problem& p, const BackwardArgs& ga, const BwdScratch& ws, int* d_status, int num_sms, cudaStream_t stream) {
     static bool done[64] = {};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev >= 64 || !done[dev]) {
-        e = cudaFuncSetAttribute(bwd_weight_mma_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)w_smem_bytes<T>(WTile<T>::max_w));
+        e = cudaFuncSetAttribute(bwd_weight_mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)w_smem_bytes(kMaxW));
         if (e != cudaSuccess) return e;
         if (dev < 64) done[dev] = true;
     }
     // the tile width (a multiple of 8) that covers the map with the fewest columns, the widest of those
     int tw = 8, cover = 1 << 30;
-    for (int t = 8; t <= WTile<T>::max_w; t += 8) {
+    for (int t = 8; t <= kMaxW; t += 8) {
         const int c = (p.W + t - 1) / t * t;
         if (c <= cover) { cover = c; tw = t; }
     }
@@ -279,7 +275,7 @@ cudaError_t launch_t(const Problem& p, const BackwardArgs& ga, const BwdScratch&
     P.B = p.B; P.H = p.H; P.W = p.W; P.heads = p.heads;
     P.tw = tw; P.tiles_x = (p.W + tw - 1) / tw; P.tiles_y = (p.H + kTH - 1) / kTH;
     P.scale = 1.f / sqrtf((float)kHeadDim);
-    const int Ctot = p.heads * kHeadDim, es = (int)sizeof(T), bc = kHeadDim / WTile<T>::planes;
+    const int Ctot = p.heads * kHeadDim, es = (int)sizeof(float), bc = kHeadDim / kPlanes;
     CUtensorMap mq, mk, mv, mg, mdl, ma;
     if (!make_tile_map(&mq, p.q, es, p.B, p.H, p.W, Ctot, bc, tw, kTH) ||
         !make_tile_map(&mg, ga.dout, es, p.B, p.H, p.W, Ctot, bc, tw, kTH) ||
@@ -292,13 +288,7 @@ cudaError_t launch_t(const Problem& p, const BackwardArgs& ga, const BwdScratch&
     long long per_head = num_sms / p.heads;                          // one CTA per SM, all heads alike
     if (per_head > tiles) per_head = tiles;
     if (per_head < 1) per_head = 1;
-    return launch_chained(bwd_weight_mma_kernel<T>, dim3((unsigned)(per_head * p.heads)), kThreads, w_smem_bytes<T>(tw), stream, mq, mk, mv, mg, mdl, ma, P);
-}
-
-}  // namespace
-
-cudaError_t launch_bwd_weight_mma(const Problem& p, const BackwardArgs& ga, const BwdScratch& ws, int* d_status, int num_sms, cudaStream_t stream) {
-    return launch_t<float>(p, ga, ws, d_status, num_sms, stream);
+    return launch_chained(bwd_weight_mma_kernel, dim3((unsigned)(per_head * p.heads)), kThreads, w_smem_bytes(tw), stream, mq, mk, mv, mg, mdl, ma, P);
 }
 
 }  // namespace slide_attn
