@@ -33,16 +33,6 @@
 
 namespace slide_attn {
 
-// Time-line build (-DSLIDE_ATTN_TIMELINE, `python -m paper_2304_04237_b200.build --timeline`): CTA 0 stamps clock64 at
-// six points of its role loops, per chunk; slide_attn_proj_timeline copies the stamps out.  The stamps cost a few
-// instructions and skip no work; the library proper is built without them.
-#ifdef SLIDE_ATTN_TIMELINE
-__device__ long long g_proj_timeline[6][256];
-#define PROJ_TL(role, idx) do { if (blockIdx.x == 0 && (idx) < 256) g_proj_timeline[role][idx] = clock64(); } while (0)
-#else
-#define PROJ_TL(role, idx) do {} while (0)
-#endif
-
 namespace {
 
 constexpr int kLoadWarps = 8, kStoreWarps = 8, kMmaWarp = kLoadWarps + kStoreWarps;
@@ -175,16 +165,13 @@ proj_kernel(const ProjParams P)
             for (int t = 0; ok && t < my_tiles; ++t) {
                 if (!mbar_wait(bar(kXFull + xb), xphase)) { ok = false; break; }
                 for (int ch = 0; ch < nchunks; ++ch, ++it) {
-                    PROJ_TL(0, it);                              // MMA thread turns to the chunk
                     if (!mbar_wait(bar(kDFree + db), dphase)) { ok = false; break; }
-                    PROJ_TL(1, it);                              // its accumulator is free
                     tc_fence_after_sync();
                     const uint32_t n = (uint32_t)(ncols - ch * kChunk < kChunk ? ncols - ch * kChunk : kChunk);
                     const uint32_t idesc = umma_idesc_bf16(128, n), d = tmem + kColD + (uint32_t)(db * kChunk), a = tmem + (uint32_t)(xb * 32 * NS);
                     const uint64_t b = umma_smem_desc(w_smem + (uint32_t)(ch * kChunk) * (uint32_t)P.K * 2u, 128, (uint32_t)P.K * 16u);
                     for (int kk = 0; kk < (P.K >> 4); ++kk) umma_bf16_ts(d, a + 8u * (uint32_t)kk, b + 16u * (uint32_t)kk, idesc, kk > 0 ? 1u : 0u);
                     umma_commit(bar(kDFull + db));
-                    PROJ_TL(2, it);                              // MMAs and commit issued
                     if (++db == kAccs) { db = 0; dphase ^= 1u; }
                 }
                 if (ok) umma_commit(bar(kXFree + xb));
@@ -247,9 +234,7 @@ proj_kernel(const ProjParams P)
             const size_t at = (size_t)row * P.ycols + tig * (U / 4);
             int mat = mat0, col = col0;
             for (int ch = 0; ch < nchunks; ++ch, ++it) {
-                if (w == 0 && lane == 0) PROJ_TL(3, it);         // the first of these warps turns to the chunk
                 if (!warp_wait(bar(kDFull + db), dphase)) { ok = false; break; }
-                if (w == 0 && lane == 0) PROJ_TL(4, it);         // accumulator seen
                 tc_fence_after_sync();
                 const uint32_t d = mine + (uint32_t)(db * kChunk);
                 uint32_t v[CU][U / 2];
@@ -281,7 +266,6 @@ proj_kernel(const ProjParams P)
                     }
                     if ((col += U) == P.ycols) { col = 0; ++mat; }
                 }
-                if (w == 0 && lane == 0) PROJ_TL(5, it);         // stored
                 if (++db == kAccs) { db = 0; dphase ^= 1u; }
             }
         }
@@ -379,10 +363,3 @@ cudaError_t launch_proj(const void* x, long long rows, int c_in, const float* w,
 }
 
 }  // namespace slide_attn
-
-#ifdef SLIDE_ATTN_TIMELINE
-// host [6][256]: per chunk of CTA 0 the clock64 stamps listed at PROJ_TL; returns the cudaError_t of the copy
-extern "C" int slide_attn_proj_timeline(long long* host) {
-    return (int)cudaMemcpyFromSymbol(host, slide_attn::g_proj_timeline, sizeof(long long) * 6 * 256);
-}
-#endif
