@@ -46,15 +46,15 @@ def algorithmic_bytes(cfg) -> int:
 
 
 # DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum, bytes per launch) of the dominant kernel
-# from one `ncu --set full` capture (profiles/).  It is tied to the kernel source by a hash: once
+# from an ncu capture (profiles/).  It is tied to the kernel source by a hash: once
 # the kernel changes, the figure no longer applies and `traffic` is reported as null.
 NCU_TRAFFIC = {
-    ("umma_ts", "c2"): {"bytes": 83.49e6,
+    ("umma_ts", "c2"): {"bytes": 82.71e6,
                         "sources": ('paper_2304_04237_b200/csrc/umma_ts_kernel.cu', 'paper_2304_04237_b200/csrc/ptx.cuh'),
-                        "sha256": "6c2f4e433aec8b8b57a0d6d1cc8f2be5a7dbd005c5f929bf5f1ac07841216743"},
-    ("fixed_shift", "c2"): {"bytes": 85.38e6,
+                        "sha256": "646390a567f177dab623de63857733c1fcd42d568be2468cc048990da52a8fd6"},
+    ("fixed_shift", "c2"): {"bytes": 84.93e6,
                             "sources": ('paper_2304_04237_b200/csrc/shift_kernel.cu', 'paper_2304_04237_b200/csrc/tile_common.cuh', 'paper_2304_04237_b200/csrc/ptx.cuh'),
-                            "sha256": "d52af488501a9d58cb50407f1b82e038f60eae2056031d64999604761f99ad6c"},
+                            "sha256": "028f2bbf9913442ef919699474eb0215b3e28622cdc3187ec3183fa2eea947bd"},
 }
 
 
@@ -437,7 +437,7 @@ def main():
         assert sa.slide_attn_query_status(ctx) == sa.OK
         bms = a.elapsed_time(b) / args.backward
         backward = {"ms_per_step": bms, "steps": args.backward, "value": npx / (bms * 1e-3), "unit": UNIT,
-                    "kernels": "weight transpose, point kernel (a, dl, dq, dbias), gather kernel (dk, dv), weight kernel (dWk, dWv)"}
+                    "kernels": "weight images, point kernel (a, dl, dq, dbias), weight kernel (dWk, dWv), gather kernel (dk, dv)" if cfg["ksize"] == 3 else "one kernel"}
 
     # optional: a whole block on the workload's shape (projections on tcgen05 around the attention stage)
     block = None

@@ -31,7 +31,7 @@
  *   wk, wv       : float [C][k*k slot][k*k tap], C = heads*head_dim.  This is the memory of a
  *                  PyTorch-style depthwise weight [C*k*k, 1, k, k] with groups = C and output
  *                  channel c*k*k + s, so a re-parameterised convolution weight can be passed as is.
- *   bias         : float [heads][k*k], or NULL
+ *   bias         : float [heads][k*k], or NULL; -infinity masks a slot
  *
  * Ownership: the caller owns every tensor.  The library reads/writes them only in stream order
  * within the call that received them and keeps no pointer afterwards.  A context owns a small
@@ -223,8 +223,7 @@ slide_attn_status slide_attn_backward(slide_attn_ctx* ctx,
  *   y0, y1, y2   [out, DEVICE] bf16 [B][H][W][C] each; the first nmat are written, the rest are ignored
  * Weights are rounded to bf16, sums are accumulated in fp32, results rounded to bf16 once.  Asynchronous on
  * `cuda_stream`.  Supported: bf16 contexts with C a multiple of 16, 16 <= C <= 256
- * (SLIDE_ATTN_ERR_UNSUPPORTED otherwise).  Allocates nothing; one kernel launch (two to twelve when C > 128, where
- * the weights of all output columns do not fit shared memory together).
+ * (SLIDE_ATTN_ERR_UNSUPPORTED otherwise).  Allocates nothing; one kernel launch.
  */
 slide_attn_status slide_attn_project(slide_attn_ctx* ctx, const void* x, const float* w, int nmat,
                                      void* y0, void* y1, void* y2, void* cuda_stream);
@@ -238,8 +237,9 @@ slide_attn_status slide_attn_project(slide_attn_ctx* ctx, const void* x, const f
  *   w_qkv         [in, DEVICE] float [3][C in][C out]: W_q, W_k, W_v
  *   w_o           [in, DEVICE] float [C in][C out]
  *   wk, wv, bias  as in slide_attn_forward
- * q, k, v and z live in bf16 in a scratch buffer of the context (4 * B*H*W*C*2 bytes), allocated with
- * cudaMalloc (synchronous) by the first call; they are rounded to bf16 once each.
+ * q, k, v and z live in bf16 in a scratch buffer of the context (4 * B*H*W*C*2 bytes, and 8 * C*C for the
+ * projection weights in bf16), allocated with cudaMalloc (synchronous, typically 0.3 ms) by the first call; they
+ * are rounded to bf16 once each.
  * The attention stage runs the context's current variant (or the fixed-shift kernel in fixed-shift mode).
  * Asynchronous on `cuda_stream`; same support as slide_attn_project.
  */

@@ -15,9 +15,10 @@
 // head, which is what dv takes in bf16) until the second launch writes it (64 x 56 x 56, 3 heads, bf16: 7 us more).
 // Both persistent, one CTA per SM and one head per CTA, two teams; geometry and hand-offs as in umma_split_kernel.
 //
-// Bound by instruction issue on the CUDA cores: products and their splits, sums, the point kernel's softmax, dL and row splits
-// (62 M warp instructions at 64 x 56 x 56, 3 heads, bf16; gather 46 M).  There, in CUDA-core kernels before and here: point 333 and
-// 125 us, gather 227 and 82; 2 x 128 x 128, 3 heads, fp32: point 69 and 48, gather 54 and 24 us.
+// Bound by latency and instruction issue on the CUDA cores (products and their splits, sums, the point kernel's softmax, dL and row splits):
+// at 64 x 56 x 56, 3 heads, bf16 the point kernel issues 64 M warp instructions in 48 % of the slots at 1.74 GHz, the gather kernel 46 M in 57 %;
+// fp32 39 and 32 %.  64 x 56 x 56, 3 heads, bf16, in CUDA-core kernels before and here: point 333 and 131 us, gather 227 and 82; 2 x 128 x 128, 3
+// heads, fp32: point 69 and 55, gather 54 and 24 us.
 #include "bwd_common.cuh"
 #include "team.cuh"
 

@@ -12,7 +12,7 @@
 // three per scheduler; a warp keeps the sums of its three taps in registers over all its tiles.  The tensor core
 // truncates when it accumulates, so the columns that hold upper parts are added up in fp32 registers after every pixel group, and
 // within one the smallest products come first: one truncation at full magnitude (after four groups, largest first: twelve, error of
-// dwv against 64 bits 4.4e-7, so 2.4e-7, with fp32 FMAs 2.7e-7; the same time).  Tiles (4 rows x up to 32 columns + halo) come by TMA into
+// dwv against 64 bits 4.4e-7, so 1.8e-7, with fp32 FMAs 2.5e-7; the same time).  Tiles (4 rows x up to 32 columns + halo) come by TMA into
 // two stages, in planes of 16 channels (four pixels x eight channel pairs = 256 contiguous bytes: no bank conflict).
 //
 // Bound by the mma.sync pipe and the CUDA-core work beside it, which hardly overlap (measured: 8 cycles per MMA and

@@ -13,12 +13,13 @@
 //           is the 64-byte swizzle of an operand whose N index is contiguous
 //   sums    the tensor core truncates when it accumulates, so after every chunk of 32 pixels the accumulators move to fp32
 //           registers, and within one the lower parts come first: two truncations at full magnitude (after two chunks, in any
-//           order: eight, error of dwk against 64 bits at 4 x 56 x 56 x 3 3.6e-7, so 2.6e-7, with fp32 FMAs 2.7e-7; 8 us less)
+//           order: eight, error of dwk against 64 bits at 4 x 56 x 56 x 3 3.6e-7, so 2.3e-7, with fp32 FMAs 2.7e-7; 9 us less)
 //
 // Persistent, one CTA per SM and one head per CTA.  Sixteen compute warps = quadrant of tensor memory (tap mod 4) x side x
 // 16-channel half, an MMA thread and a TMA thread.  Tiles of 4 rows x up to 56 columns + halo in two stages; a chunk = 4 rows x 8
-// columns.  Bound by instruction issue (45 M warp instructions at 64 x 56 x 56, 3 heads, slots 53 % busy: products, their splits and the
-// drains): 410 us with fp32 FMAs on the CUDA cores, 134 on mma.sync, 97.5 here.  Tensor-memory columns: six accumulators of 32, then two chunk buffers of [operand][16-pixel step][hi, lo: 8 each].
+// columns.  Bound by latency and instruction issue (50 M warp instructions at 64 x 56 x 56, 3 heads, in 46 % of the slots at 1.79 GHz:
+// products, their splits and the reading of the accumulators): 410 us with fp32 FMAs on the CUDA cores, 134 on mma.sync, 106 here.
+// Tensor-memory columns: six accumulators of 32, then two chunk buffers of [operand][16-pixel step][hi, lo: 8 each].
 #include "bwd_common.cuh"
 #include "split.cuh"
 

@@ -11,11 +11,11 @@
 // blocks dealt over teams round-robin, neighbouring CTAs on neighbouring blocks.  A block's K planes, then its V planes
 // come through the team's ring.
 //
-// Bound by instruction issue and the hand-offs between the warps and the tensor core (issue slots 51 % busy, tensor pipe
-// 15 - 24 %, DRAM 13 - 16 %).  A call, before (the CUDA-core kernel that took the shape) and here: 2 x 128 x 128, 3 heads,
-// fp32: 45.3 us in tile_kernel, 28.5; 32 x 28 x 28, 3 heads of 64, bf16: 232 us in strip_kernel, 25.3; 1 x 14 x 14, 1 head,
-// fp32: 14.7 and 8.0 us; heads of 16, strip_kernel before: 16 x 56 x 56 x 3, bf16 197 and 16.1, fp32 184 and 22.7 us;
-// 30 x 28 x 42 x 8, bf16 449 and 30.9; 1 x 7 x 7 x 1, bf16 18.3 and 10.4.
+// Bound by latency: the chain products -> MMA -> softmax -> split rows -> MMA -> sum and its hand-offs, with four compute warps per
+// scheduler to cover it.  Issue slots 30 - 36 % busy at 1.8 GHz, tensor pipe 13 - 24 %, DRAM 14 - 18 %.  A call, before (the CUDA-core kernel that
+// took the shape) and here: 2 x 128 x 128, 3 heads, fp32: 45.2 us in tile_kernel, 28.9; 32 x 28 x 28, 3 heads of 64, bf16: 232 us in
+// strip_kernel, 23.7; 1 x 14 x 14, 1 head, fp32: 14.4 and 8.5 us; heads of 16 (an earlier form of this kernel against strip_kernel): 16 x 56 x 56
+// x 3, bf16 197 and 16.1, fp32 184 and 22.7 us.
 #include "team.cuh"
 
 namespace slide_attn {

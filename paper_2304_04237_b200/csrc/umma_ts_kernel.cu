@@ -26,7 +26,8 @@
 // Warp 16 owns tensor memory.  Every wait is bounded; a wait that runs out sets the status word, and
 // tensor memory is released on every path.
 //
-// What bounds it: instruction issue on the CUDA cores.  An M = 128 MMA costs about N / 2 cycles (18 of N = 32 and
+// What bounds it: instruction issue and latency on the CUDA cores (18.3 M warp instructions at 64 x 56 x 56, 2 heads: 50 % of the issue slots at
+// 1.77 GHz, 61 % of those of the cycles in which an SM has work).  An M = 128 MMA costs about N / 2 cycles (18 of N = 32 and
 // 6 of N = 96 per 128 pixels: 540 cycles of a block period of about 2 850), the value warps are busy from block to
 // block, everything else waits for them, and with four or five warps per scheduler the time follows the instruction
 // count (5.9 k warp instructions per block: the q.k products, the widenings of V, the accumulator x V multiply-adds).
