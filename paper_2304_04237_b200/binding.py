@@ -30,6 +30,9 @@ EXPORTS = ("slide_attn_create", "slide_attn_forward", "slide_attn_forward_host",
 
 _lib = None
 
+# the current stream's handle and device without the objects around them, where this torch gives them out
+_raw_stream, _raw_device = (getattr(torch._C, n, None) for n in ("_cuda_getCurrentRawStream", "_cuda_getDevice"))
+
 
 class SlideAttnError(RuntimeError):
     def __init__(self, status: int, where: str):
@@ -109,11 +112,9 @@ def _host_ptr(t):
 
 def _stream_ptr(stream):
     if stream is None:
-        # torch.cuda.current_stream() builds a stream object, 3 of the 13 us that a small call takes; the raw handle, where this
-        # torch gives it out, costs 0.3
-        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
-        if raw is not None and torch.cuda.is_initialized():
-            return raw(torch.cuda.current_device())
+        # torch.cuda.current_stream() builds a stream object, 3 of the 13 us that a small call takes; the raw handle costs 0.3
+        if _raw_stream and _raw_device and torch.cuda.is_initialized():
+            return _raw_stream(_raw_device())
         stream = torch.cuda.current_stream()
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 

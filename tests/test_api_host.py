@@ -88,7 +88,8 @@ def test_current_stream_without_the_raw_handle(monkeypatch):
     import torch
 
     from paper_2304_04237_b200 import binding
-    monkeypatch.delattr(torch._C, "_cuda_getCurrentRawStream", raising=False)
+    monkeypatch.delattr(torch._C, "_cuda_getCurrentRawStream", raising=False)       # both where it would be looked up
+    monkeypatch.setattr(binding, "_raw_stream", None, raising=False)
     monkeypatch.setattr(torch.cuda, "is_initialized", lambda: True)
     monkeypatch.setattr(torch.cuda, "current_stream", lambda *a: types.SimpleNamespace(cuda_stream=1234))
     assert binding._stream_ptr(None) == 1234
