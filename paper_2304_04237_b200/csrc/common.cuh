@@ -80,8 +80,8 @@ cudaError_t launch_mma_prep(const Problem& p, void* workspace, cudaStream_t stre
 cudaError_t launch_mma_main(const Problem& p, const void* workspace, int* d_status, cudaStream_t stream);
 
 
-// UMMA_TS variant: both contractions on tcgen05 with their A operands in tensor memory.  A prep launch
-// writes the bf16 B images of every head (umma_ts_workspace_bytes) that the main launch's CTAs copy in.
+// UMMA_TS variant: both contractions on tcgen05 with their A operands in tensor memory.  The CTAs of the main launch lay out
+// their head's weights themselves, or copy in what a prep launch left in `workspace` (umma_ts_workspace_bytes; null: none did).
 bool umma_ts_supports(slide_attn_dtype dtype, int head_dim, int ksize);
 cudaError_t umma_ts_setup();
 size_t umma_ts_workspace_bytes(int heads);

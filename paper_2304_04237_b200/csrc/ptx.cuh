@@ -36,8 +36,19 @@ __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
 
 // Bounded wait: false if the phase did not complete within the limit (about two seconds).  Each
 // probe may park the thread for up to 100 us (the hardware wakes it when the phase completes), so
-// a waiting warp issues next to no instructions.
+// a waiting warp issues next to no instructions.  `Small`: a loop that the compiler may not unroll, in kernels of which many waits
+// would otherwise fill the instruction cache (41 instead of 63 KB of one of them); elsewhere it costs up to 3 %.
+template <bool Small = false>
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
+    auto probe = [&]() {
+        uint32_t done;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(done) : "r"(bar), "r"(parity), "r"(100000u) : "memory");
+        return done != 0;
+    };
     {   // a phase that is already complete costs about 30 cycles less without the time hint
         uint32_t done;
         asm volatile(
@@ -47,17 +58,34 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
             : "=r"(done) : "r"(bar), "r"(parity) : "memory");
         if (done) return true;
     }
-    for (int spin = 0; spin < 20000; ++spin) {
-        uint32_t done;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(done) : "r"(bar), "r"(parity), "r"(100000u) : "memory");
-        if (done) return true;
+    if constexpr (Small) {
+#pragma unroll 1
+        for (int spin = 0; spin < 20000; ++spin)
+            if (probe()) return true;
+    } else {
+        for (int spin = 0; spin < 20000; ++spin)
+            if (probe()) return true;
     }
     return false;
 }
+
+// A wait of a whole warp without a vote: a lane whose wait runs out carries on with `ok` cleared and waits no more, so that the
+// warp stays together whatever happens, and says so at its end.  (With a vote and a way out behind every wait, a wait on a phase that
+// is already complete took 124 cycles, without 76.)
+__device__ __forceinline__ void wait_or_give_up(uint32_t bar, uint32_t parity, bool& ok) {
+    uint32_t done;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(done) : "r"(bar), "r"(parity) : "memory");
+    if (!done && ok) ok = mbar_wait<true>(bar, parity);
+    __syncwarp();
+}
+
+// Moves registers between the warpgroups of a block (all four warps of one execute it).
+template <int N> __device__ __forceinline__ void reg_take() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
+template <int N> __device__ __forceinline__ void reg_give() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
 
 // One arrival by lane 0 of a converged warp, without a branch.
 __device__ __forceinline__ void mbar_arrive_lane0(uint32_t bar, int lane) {
@@ -308,6 +336,19 @@ __device__ __forceinline__ void tmem_ld_32x32b_x16(uint32_t taddr, float (&v)[16
         : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]) : "r"(taddr) : "memory");
 #pragma unroll
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+// thread i <- TMEM lane (base + i), 18 consecutive columns (waits for the data)
+__device__ __forceinline__ void tmem_ld_32x32b_18(uint32_t taddr, float (&v)[18]) {
+    uint32_t r[18];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%18];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x2.b32 {%16,%17}, [%19];\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17])
+        : "r"(taddr), "r"(taddr + 16) : "memory");
+#pragma unroll
+    for (int i = 0; i < 18; ++i) v[i] = __uint_as_float(r[i]);
 }
 
 // registers -> 16 TMEM lanes x 16 columns, laid out like the A fragments of two mma.sync.m16n8k16: of each four registers,

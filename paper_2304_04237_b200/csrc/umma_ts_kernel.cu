@@ -6,624 +6,517 @@
 //   product warps   P[p,(t,c)] = q[p,c] k[p+off(t),c]   packed bf16 multiply -> tcgen05.st (TMEM)
 //   key MMA         L[p,n]     = sum_{t,c} P[p,(t,c)] Bk[(t,c),n]       tcgen05.mma, A from TMEM
 //                   n = 0..8: deformed part D_k of slot n;  n = 9..17: plain q.k sum of tap n-9
-//   product warps   logit[s] = (L[s] + L[9+s]) scale + bias[s];  e = exp2(logit - max) / sum_s exp2(logit - max)
+//   softmax warps   logit[s] = (L[s] + L[9+s]) scale + bias[s];  e = exp2(logit - max) / sum_s exp2(logit - max)
 //                   (tcgen05.ld.32x32b: one thread holds all logits of one pixel, no shuffles)
 //                   A' row = e_hi | e_hi | e_lo | e8_hi e8_hi e8_lo 0..   -> tcgen05.st (TMEM)
 //   value MMA       D[p,(t,c)] = sum_k A'[p,k] Bv[k,(t,c)]                     A from TMEM
 //   value warps     out[p,c] = sum_t D[p,t,c] v[p+off(t),c]
 //
-// Tensor memory (512 columns): two value-chunk slots 112 columns apart, 96 used (chunk c = 3 blk + dx -> slot
-// c & 1), four P chunks of 48 (3 taps x 32 bf16, chunk -> buffer c & 3), two logit tiles of 32, two A' tiles of 16.
+// Persistent, one CTA per SM, CTA c -> head c mod heads.  A block is 128 pixels = four strips of 4 rows x 8 columns (team.cuh), which
+// TMA brings with their halo (zero fill = the padding); blocks are dealt round-robin.  24 warps:
+//   value warps    two sets of four; a set takes every other block, warp q of it strip q = quadrant q of tensor memory: lane (g, tig)
+//                  works on column g and channels 8 tig .. of all four rows, so that each halo row is widened once for up to three of them
+//   product warps  two sets likewise
+//   softmax warps  four: thread = pixel
+//   control warps  one thread each for the key MMAs, the value MMAs, the K and q strips, the head's weights and the V strips
+// Registers move from the others to the value warps (setmaxnreg).  Waits of the compute warps have no vote and no way out (see
+// wait_or_give_up).  Every wait is bounded; one that runs out sets the status word, and tensor memory is released on every path.
+// Every CTA lays out its head's weights itself, in the value and softmax warps, while the first products are made: a prep launch in
+// front cost 1 us at 64 x 56 x 56, 2 heads, and 1.7 us at 32 x 28 x 42, 6 heads.
 //
-// Warps (20, 86 registers): 0-7 value warps (quadrant = warp % 4, pixel-row pair = warp / 4, every
-// block), 8-15 product warps (quadrant, pixel-row pair: P of their 16 pixels of every block; the
-// softmax of a block is done for the whole quadrant by the warp whose pair index equals the block's
-// parity, after it has stored the P of the next block), 16 and 18 key-side control (the 18 key MMAs
-// of the even / odd blocks, taking turns through two barriers so that the P-ready barriers are
-// waited on strictly in chunk order), 17 value-side control
-// (value MMAs), 19 TMA thread (K/q and V rings).  The MMA threads have one thing to wait for at a
-// time and park in mbarrier waits instead of polling: that alone was worth 10 % of the kernel time.
-// Warp 16 owns tensor memory.  Every wait is bounded; a wait that runs out sets the status word, and
-// tensor memory is released on every path.
+// Tensor memory: three value chunks of 96 columns (dx), three P chunks of 48 (3 taps x 32 bf16), two logit tiles of 32, A' of 16.
 //
-// What bounds it: instruction issue and latency on the CUDA cores (18.3 M warp instructions at 64 x 56 x 56, 2 heads: 50 % of the issue slots at
-// 1.77 GHz, 61 % of those of the cycles in which an SM has work).  An M = 128 MMA costs about N / 2 cycles (18 of N = 32 and
-// 6 of N = 96 per 128 pixels: 540 cycles of a block period of about 2 850), the value warps are busy from block to
-// block, everything else waits for them, and with four or five warps per scheduler the time follows the instruction
-// count (5.9 k warp instructions per block: the q.k products, the widenings of V, the accumulator x V multiply-adds).
+// What bounds it: instruction issue and latency on the CUDA cores.  14.5 M warp instructions at 64 x 56 x 56, 2 heads, in 53 % of the
+// slots; the value warps wait for 40 % of the time, the product warps for 50 %, so that no stage alone is the bound.  With value
+// and product warps of two rows each on tiles of 4 rows x up to 64 columns it was 18.3 M (every halo row widened for two output rows
+// instead of three, twice the hand-offs).  Calls, a few hundred / for seconds, when the power limit takes clocks down to 1.69 GHz here
+// and 1.84 before: 64 x 56 x 56, 2 heads 32.3 / 33.2 -> 27.6 / 31.4 us, 32 x 28 x 42, 6 heads 23.5 / 23.4 -> 19.7 / 20.9.
+// The code has to stay small: the instruction cache holds 32 KB, and a build of 112 KB (waits' spin loops and tile loops unrolled by
+// the compiler) took 47 us.  Loops over tap columns not unrolled: 37 us.  fma.rn.f32x2 as two FMAs each: 3 % slower.  One set of
+// product warps: 28.8; all of a chunk's accumulators read at once (160 registers): 29.6; two value chunks instead of three: the same.
 #include "common.cuh"
 #include "ptx.cuh"
+#include "team.cuh"
 
 namespace slide_attn {
 
 namespace {
 
+using team::Strips; using team::StripWalk; using team::kHaloPlane; using team::kSlot; using team::kLog2e;
+
 constexpr int kHeadDim = 32;
-constexpr int kVWarps = 8;
-constexpr int kPWarps = 8;
-constexpr int kCtlK = kVWarps + kPWarps;                // warp 16: key MMAs of the even blocks, TMEM owner
-constexpr int kCtlV = kCtlK + 1;                        // warp 17: value MMAs
-constexpr int kCtlK2 = kCtlV + 1;                       // warp 18: key MMAs of the odd blocks
-constexpr int kCtlT = kCtlK2 + 1;                       // warp 19: TMA thread, K/q and V tiles
-constexpr int kThreads = (kCtlT + 1) * 32;
-constexpr int kKStages = 2;
-constexpr int kMaxVStages = 4;
+constexpr int kVSets = 2, kPSets = 2;                    // of four value warps, of four product warps: they take the blocks in turn
+constexpr int kPWarp0 = 4 * kVSets, kSWarp0 = kPWarp0 + 4 * kPSets, kCtlK = kSWarp0 + 4, kCtlV = kCtlK + 1, kCtlTK = kCtlK + 2, kCtlTV = kCtlK + 3;
+constexpr int kThreads = (kCtlTV + 1) * 32;
+constexpr int kValueRegs = 128, kProductRegs = 64, kSoftmaxRegs = 56, kControlRegs = 40;      // 480 over the six warpgroups: 80 each at the launch
+constexpr int kKSlots = 4, kVSlots = 6;
+constexpr uint32_t kQStrip = 4 * 8 * 64;                // bytes of a strip of q
+constexpr uint32_t kKSlot = kSlot + 4 * kQStrip;        // K with its halo, then q, of a block
 constexpr int kBCols = 288;                             // value columns: (tap, channel)
 constexpr int kBBytes = kBCols * 64;
 constexpr int kBkBytes = 36 * 512;                      // key-side B: 288 K x 32 N bf16
 constexpr int kImgBytes = kBBytes + kBkBytes;           // both B images of one head, as the prep kernel leaves them
-constexpr float kLog2e = 1.4426950408889634f;
+constexpr int kWeightFloats = kHeadDim * 81;             // of a head, either side
 constexpr uint32_t kTmemCols = 512;
 // tensor-memory columns
-constexpr uint32_t kColD = 0;                           // two value-chunk slots of 112 columns (chunk c -> slot c & 1)
-constexpr uint32_t kColP = 224;                         // four P chunks of 48 columns (3 taps x 32 bf16)
-constexpr uint32_t kColL = 416;                         // two logit tiles of 32 columns
-constexpr uint32_t kColE = 480;                         // two A' tiles of 16 columns (32 bf16)
+constexpr uint32_t kColD = 0;                           // three value chunks of 96 columns
+constexpr uint32_t kColP = 288;                         // three P chunks of 48 columns (3 taps x 32 bf16)
+constexpr uint32_t kColL = 432, kOtherL = 96;           // two logit tiles of 32 columns, 432 and 432 ^ 96
+constexpr uint32_t kColE = 496;                         // the A' tile of 16 columns (32 bf16)
 constexpr uint32_t kIdesc96 = umma_idesc_bf16(128, 96);
 constexpr uint32_t kIdesc32 = umma_idesc_bf16(128, 32);
 
 struct UmmaParams {
-    const unsigned char* bimg;       // per head: value-side B image (kBBytes) then key-side B image (kBkBytes)
+    const float* wk;
+    const float* wv;
+    const unsigned char* bimg;       // per head: value-side B image (kBBytes) then key-side B image (kBkBytes); null: built here
     const float* bias;
     __nv_bfloat16* out;
     int* status;
-    int B, H, W, heads;
-    int tiles_x, tiles_y;
+    int H, W, heads;
+    Strips strips;
     float scale_log2e;
 };
 
-struct Smem {
-    uint32_t halo_pad, kstage_bytes, v_off, b_off, bk_off, tmem_off, bar_off, total;
-};
+// shared memory
+constexpr uint32_t kVOff = kKSlots * kKSlot, kBOff = kVOff + kVSlots * (uint32_t)kSlot, kBkOff = kBOff + kBBytes, kBarOff = kBkOff + kBkBytes;
 
-__host__ __device__ constexpr Smem smem_layout(int TW, int vstages) {
-    Smem s{};
-    s.halo_pad = ((uint32_t)(6 * (TW + 2) * 64) + 1023u) & ~1023u;
-    s.kstage_bytes = s.halo_pad + (((uint32_t)(4 * TW * 64) + 1023u) & ~1023u);
-    s.v_off = kKStages * s.kstage_bytes;
-    s.b_off = s.v_off + vstages * s.halo_pad;
-    s.bk_off = s.b_off + kBBytes;
-    s.tmem_off = s.bk_off + kBkBytes;
-    s.bar_off = s.tmem_off + 16;
-    s.total = s.bar_off + 40 * 8 + 1024;
-    return s;
-}
+// barriers; those of a pair are told apart by bit 3 of their address
+enum : int { kBarKFull = 0, kBarKEmpty = kBarKFull + kKSlots, kBarVFull = kBarKEmpty + kKSlots, kBarVEmpty = kBarVFull + kVSlots,
+             kBarLFull = kBarVEmpty + kVSlots,           // [2] logits of a block complete
+             kBarLFree = kBarLFull + 2,                  // [2] count 4: logits read
+             kBarEReady = kBarLFree + 2, kBarEFree,      // count 4: A' rows stored; value MMAs of the block complete
+             kBarDFree,                                  // [dx] count 4: value chunk read
+             kBarDFull = kBarDFree + 3,                  // [set][dx] value chunk complete
+             kBarPFree = kBarDFull + 3 * kVSets,         // [set][dx] key MMAs reading the chunk are complete
+             kBarPReady = kBarPFree + 3 * kPSets,        // [dx] count 4: P chunk stored
+             kBarWeights = kBarPReady + 3,               // count: the warps that build the images, or one for their copy
+             kBarRaw,                                    // fp32 weights of the head
+             kBars };
+static_assert(kBarLFull % 2 == 0 && kKSlots % kPSets == 0 && kVSlots % kVSets == 0, "pairs of barriers; a slot has one set of readers");
+constexpr uint32_t kTmemOff = kBarOff + 8 * kBars, kSmemBytes = kTmemOff + 16 + 128;
+static_assert(kSmemBytes <= 227 * 1024, "shared memory");
+// the fp32 weights wait in the last two slots of V, which V does not need before
+constexpr int kRawSlots = 2;
+constexpr uint32_t kRawOff = kVOff + (kVSlots - kRawSlots) * (uint32_t)kSlot;
+static_assert(2 * kWeightFloats * 4 <= kRawSlots * kSlot, "fp32 weights");
+constexpr int kBuilders = 4 * kVSets + 4;               // value and softmax warps, which have nothing else to do yet
 
-constexpr size_t kMaxSmem = 227 * 1024;
-
-// V stages that fit beside everything else for a tile width (the kernel is instantiated per width,
-// so that every shared-memory offset and stride is a compile-time constant)
-__host__ __device__ constexpr int v_stages_for(int TW) {
-    for (int st = kMaxVStages; st >= 2; --st)
-        if (smem_layout(TW, st).total <= kMaxSmem) return st;
-    return 0;
-}
-
-constexpr int kBarKFull = 0;         // [2]
-constexpr int kBarKEmpty = 2;        // [2]  count 8 (product warps)
-constexpr int kBarVFull = 4;         // [4]
-constexpr int kBarVEmpty = 8;        // [4]  count 8
-constexpr int kBarWeights = 12;      // both B images have landed (one bulk copy)
-constexpr int kBarPReady = 14;       // [4]  count 8: P chunk stored by the eight product warps
-constexpr int kBarPFree = 18;        // [4]  key MMAs reading the chunk are complete
-constexpr int kBarLFull = 22;        // [2]  logits of a block complete
-constexpr int kBarLFree = 24;        // [2]  count 4: logits read (one product warp per quadrant)
-constexpr int kBarEReady = 26;       // [2]  count 4: A' rows stored
-constexpr int kBarEFree = 28;        // [2]  value MMAs of the block complete
-constexpr int kBarDFull = 30;        // [2]  value chunk complete
-constexpr int kBarDFree = 32;        // [2]  count 8: value chunk read
-constexpr int kBarVDone = 34;        // count 8
-constexpr int kBarTurn = 35;         // [2]  the other key-control thread has taken the last chunk of its block
-
-__device__ __forceinline__ uint4 lds_u4(const unsigned char* base, uint32_t off) {
-    return *reinterpret_cast<const uint4*>(base + off);
-}
 // Hand-offs of tensor memory between threads: the side that has read or written TMEM issues
 // tcgen05.wait::ld / ::st (the accesses are then complete) and arrives on an mbarrier; the side that
 // takes over waits on it and issues tcgen05.fence::after_thread_sync before its own tcgen05 work.
-__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity) {
-    return __all_sync(0xffffffffu, mbar_wait(bar, parity) ? 1 : 0) != 0;
-}
 
 // ---------------------------------------------------------------------------------------------
-// Prep kernel: the two B images of every head, in the shared-memory layout the MMAs read
-// (K-major core matrices of 8 rows x 16 bytes, no swizzle), written to the context workspace once per
-// forward.  Block (h, part) builds a share of head h's items.
+// The two B images of a head, in the shared-memory layout the MMAs read (K-major core matrices of 8 rows x 16 bytes, no
+// swizzle), from its fp32 weights [channel][slot][tap]; items of 16 bytes times 4 (value side) or 1 (key side).
 //   value side  [288 columns][32 K] bf16: column n = (tap-column-major tap, channel); K rows
 //               0..7 D_v[c][s][t], 8..15 and 16..23 the one-hot [s = t], 24 D_v[c][8][t], 25, 26 [t = 8]
 //               (the A' row is e_hi | e_hi | e_lo | e8_hi e8_hi e8_lo)
 //   key side    [288 K][32 N] bf16: K = 32 tap + kappa (kappa -> channel as tcgen05.st lays P out),
 //               N 0..8 D_k[c][n][t], 9..17 the one-hot [n - 9 = t]
+constexpr int kItems = kBCols + 36 * 32;
+__device__ __forceinline__ void build_item(const float* wks, const float* wvs, unsigned char* sB, int item) {
+    if (item < kBCols) {
+        const int n = item;
+        unsigned char* col = sB + (n >> 3) * 512 + (n & 7) * 16;
+        uint32_t w[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) w[i] = 0u;
+        {
+            const int ts = n >> 5, t = (ts % 3) * 3 + ts / 3;
+            const int cn = n & 31, j = cn >> 3, wi = cn & 7;
+            const float* wc = wvs + (8 * (wi >> 1) + 2 * j + (wi & 1)) * 81 + t;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int s0 = 2 * i, s1 = 2 * i + 1;
+                w[i] = pack_bf16(wc[s0 * 9] - (s0 == t ? 1.f : 0.f), wc[s1 * 9] - (s1 == t ? 1.f : 0.f));
+                const uint32_t oh = pack_bf16(s0 == t ? 1.f : 0.f, s1 == t ? 1.f : 0.f);
+                w[4 + i] = oh; w[8 + i] = oh;
+            }
+            const float o8 = t == 8 ? 1.f : 0.f;
+            w[12] = pack_bf16(wc[72] - o8, o8); w[13] = pack_bf16(o8, 0.f);
+        }
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+            *reinterpret_cast<uint4*>(col + c * 128) = make_uint4(w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
+    } else {
+        const int it = item - kBCols;
+        const int n = it & 31, kg = it >> 5;
+        const int t = kg >> 2, kap0 = (kg & 3) * 8;
+        float val[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            const int kap = kap0 + e;
+            const int c = 8 * ((kap & 15) >> 2) + (kap & 3) + (kap >= 16 ? 4 : 0);
+            float x = 0.f;
+            if (n < 9) x = wks[c * 81 + n * 9 + t] - (n == t ? 1.f : 0.f);
+            else if (n < 18) x = (n - 9 == t) ? 1.f : 0.f;
+            val[e] = x;
+        }
+        *reinterpret_cast<uint4*>(sB + kBBytes + kg * 512 + (n >> 3) * 128 + (n & 7) * 16) =
+            make_uint4(pack_bf16(val[0], val[1]), pack_bf16(val[2], val[3]), pack_bf16(val[4], val[5]), pack_bf16(val[6], val[7]));
+    }
+}
+
+// The images of every head into the context workspace.  Only kernel timing launches this, which has to tell the attention from
+// the layout of its weights; otherwise every CTA of the main kernel lays out its head's weights itself.
 __global__ void __launch_bounds__(256)
 umma_ts_prep_kernel(const float* __restrict__ wk, const float* __restrict__ wv, unsigned char* __restrict__ img)
 {
     grid_dependency_wait();
     grid_launch_dependents();        // the main kernel may start its own prologue now
     const int h = blockIdx.x;
-    const float* wks = wk + (size_t)h * kHeadDim * 81;
-    const float* wvs = wv + (size_t)h * kHeadDim * 81;
-    unsigned char* sB = img + (size_t)h * kImgBytes;
-    unsigned char* sBk = sB + kBBytes;
-    for (int item = blockIdx.y * blockDim.x + threadIdx.x; item < kBCols + 36 * 32; item += gridDim.y * blockDim.x) {
-        if (item < kBCols) {
-            const int n = item;
-            unsigned char* col = sB + (n >> 3) * 512 + (n & 7) * 16;
-            uint32_t w[16];
-#pragma unroll
-            for (int i = 0; i < 16; ++i) w[i] = 0u;
-            {
-                const int ts = n >> 5, t = (ts % 3) * 3 + ts / 3;
-                const int cn = n & 31, j = cn >> 3, wi = cn & 7;
-                const float* wc = wvs + (8 * (wi >> 1) + 2 * j + (wi & 1)) * 81 + t;
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int s0 = 2 * i, s1 = 2 * i + 1;
-                    w[i] = pack_bf16(wc[s0 * 9] - (s0 == t ? 1.f : 0.f), wc[s1 * 9] - (s1 == t ? 1.f : 0.f));
-                    const uint32_t oh = pack_bf16(s0 == t ? 1.f : 0.f, s1 == t ? 1.f : 0.f);
-                    w[4 + i] = oh; w[8 + i] = oh;
-                }
-                const float o8 = t == 8 ? 1.f : 0.f;
-                w[12] = pack_bf16(wc[72] - o8, o8); w[13] = pack_bf16(o8, 0.f);
-            }
-#pragma unroll
-            for (int c = 0; c < 4; ++c)
-                *reinterpret_cast<uint4*>(col + c * 128) = make_uint4(w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
-        } else {
-            const int it = item - kBCols;
-            const int n = it & 31, kg = it >> 5;
-            const int t = kg >> 2, kap0 = (kg & 3) * 8;
-            float val[8];
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const int kap = kap0 + e;
-                const int c = 8 * ((kap & 15) >> 2) + (kap & 3) + (kap >= 16 ? 4 : 0);
-                float x = 0.f;
-                if (n < 9) x = wks[c * 81 + n * 9 + t] - (n == t ? 1.f : 0.f);
-                else if (n < 18) x = (n - 9 == t) ? 1.f : 0.f;
-                val[e] = x;
-            }
-            *reinterpret_cast<uint4*>(sBk + kg * 512 + (n >> 3) * 128 + (n & 7) * 16) =
-                make_uint4(pack_bf16(val[0], val[1]), pack_bf16(val[2], val[3]), pack_bf16(val[4], val[5]), pack_bf16(val[6], val[7]));
-        }
-    }
+    for (int item = blockIdx.y * blockDim.x + threadIdx.x; item < kItems; item += gridDim.y * blockDim.x)
+        build_item(wk + (size_t)h * kWeightFloats, wv + (size_t)h * kWeightFloats, img + (size_t)h * kImgBytes, item);
 }
 
-template <int TW>
 __global__ void __launch_bounds__(kThreads, 1)
 umma_ts_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
-             const __grid_constant__ CUtensorMap map_v, const UmmaParams P)
+               const __grid_constant__ CUtensorMap map_v, const UmmaParams P)
 {
     extern __shared__ unsigned char smem_raw[];
-    unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
-    constexpr int SV = v_stages_for(TW);
-    constexpr Smem L = smem_layout(TW, SV);
-    const uint32_t bar0 = smem_u32(smem + L.bar_off);
+    unsigned char* smem = smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u);
+    const uint32_t bar0 = smem_u32(smem + kBarOff);
     auto bar = [&](int i) { return bar0 + 8u * (uint32_t)i; };
 
     // the warp index through a shuffle: the compiler then knows it is the same in every lane
     const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
-    const int g = lane >> 2, tig = lane & 3;
-    constexpr int U = TW >> 3;
-    constexpr int HW2 = TW + 2;
-
-    const int h = blockIdx.x % P.heads;
-    const int rank = blockIdx.x / P.heads;
-    const int nrank = ((int)gridDim.x - h + P.heads - 1) / P.heads;
-    const int tiles_per_head = P.B * P.tiles_y * P.tiles_x;
-    // tiles are dealt round-robin: neighbouring CTAs work on neighbouring tiles at the same time, which
-    // keeps the halos they share in L2
-    const int my_tiles = rank < tiles_per_head ? (tiles_per_head - rank + nrank - 1) / nrank : 0;
-    const int my_units = my_tiles * U;
-    const int my_blocks = (my_units + 3) >> 2;
-    const int C = P.heads * kHeadDim;
+    const int h = blockIdx.x % P.heads, rank = blockIdx.x / P.heads, nrank = ((int)gridDim.x - h + P.heads - 1) / P.heads;
+    const int blocks = (int)((P.strips.total + 3) >> 2);
+    // blocks are dealt round-robin: neighbouring CTAs work on neighbouring blocks at the same time, which keeps the halos they
+    // share in L2
+    const int my_blocks = rank < blocks ? (blocks - rank + nrank - 1) / nrank : 0;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < kKStages; ++s) { mbar_init_only(bar(kBarKFull + s), 1); mbar_init_only(bar(kBarKEmpty + s), kPWarps); }
-        for (int s = 0; s < kMaxVStages; ++s) { mbar_init_only(bar(kBarVFull + s), 1); mbar_init_only(bar(kBarVEmpty + s), kVWarps); }
-        mbar_init_only(bar(kBarWeights), 1);
-        for (int i = 0; i < 4; ++i) { mbar_init_only(bar(kBarPReady + i), kPWarps); mbar_init_only(bar(kBarPFree + i), 1); }
-        for (int i = 0; i < 2; ++i) {
-            mbar_init_only(bar(kBarLFull + i), 1);
-            mbar_init_only(bar(kBarLFree + i), 4);
-            mbar_init_only(bar(kBarEReady + i), 4);
-            mbar_init_only(bar(kBarEFree + i), 1);
-        }
-        for (int i = 0; i < 2; ++i) { mbar_init_only(bar(kBarDFull + i), 1); mbar_init_only(bar(kBarDFree + i), kVWarps); }
-        mbar_init_only(bar(kBarVDone), kVWarps);
-        mbar_init_only(bar(kBarTurn + 0), 1);
-        mbar_init_only(bar(kBarTurn + 1), 1);
+#pragma unroll 1
+        for (int i = 0; i < kKSlots; ++i) { mbar_init_only(bar(kBarKFull + i), 1); mbar_init_only(bar(kBarKEmpty + i), 4); }
+#pragma unroll 1
+        for (int i = 0; i < kVSlots; ++i) { mbar_init_only(bar(kBarVFull + i), 1); mbar_init_only(bar(kBarVEmpty + i), 4); }
+        for (int i = 0; i < 2; ++i) { mbar_init_only(bar(kBarLFull + i), 1); mbar_init_only(bar(kBarLFree + i), 4); }
+        mbar_init_only(bar(kBarEReady), 4);
+        mbar_init_only(bar(kBarEFree), 1);
+#pragma unroll 1
+        for (int i = 0; i < 3 * kVSets; ++i) mbar_init_only(bar(kBarDFull + i), 1);
+#pragma unroll 1
+        for (int i = 0; i < 3 * kPSets; ++i) mbar_init_only(bar(kBarPFree + i), 1);
+#pragma unroll 1
+        for (int i = 0; i < 3; ++i) { mbar_init_only(bar(kBarPReady + i), 4); mbar_init_only(bar(kBarDFree + i), 4); }
+        mbar_init_only(bar(kBarWeights), P.bimg ? 1 : kBuilders);
+        mbar_init_only(bar(kBarRaw), 1);
         mbar_init_fence();
     }
-    if (warp == kCtlK) tmem_alloc(smem_u32(smem + L.tmem_off), kTmemCols);
+    if (warp == kCtlK) tmem_alloc(smem_u32(smem + kTmemOff), kTmemCols);
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    const uint32_t tmem = *reinterpret_cast<const volatile uint32_t*>(smem + L.tmem_off);
-
-    struct TileWalk { int tx, ty, b, stage, round; };
-    const int step_tx = nrank % P.tiles_x, step_ty = (nrank / P.tiles_x) % P.tiles_y,
-              step_b = nrank / (P.tiles_x * P.tiles_y);
-    auto walk_begin = [&]() {
-        TileWalk w;
-        w.tx = rank % P.tiles_x;
-        w.ty = (rank / P.tiles_x) % P.tiles_y;
-        w.b = rank / (P.tiles_x * P.tiles_y);
-        w.stage = 0; w.round = 0;
-        return w;
-    };
-    auto walk_next = [&](TileWalk& w, int nstages) {
-        w.tx += step_tx;
-        if (w.tx >= P.tiles_x) { w.tx -= P.tiles_x; ++w.ty; }
-        w.ty += step_ty;
-        if (w.ty >= P.tiles_y) { w.ty -= P.tiles_y; ++w.b; }
-        w.b += step_b;
-        if (++w.stage == nstages) { w.stage = 0; ++w.round; }
-    };
-    auto issue_k_tile = [&](const TileWalk& w) {
-        const uint32_t base = smem_u32(smem + (size_t)w.stage * L.kstage_bytes);
-        const uint32_t fb = bar(kBarKFull + w.stage);
-        mbar_expect_tx(fb, (uint32_t)(6 * HW2 * 64 + 4 * TW * 64));
-        tma_load_4d(base, &map_k, fb, h * kHeadDim, w.tx * TW - 1, w.ty * 4 - 1, w.b);
-        tma_load_4d(base + L.halo_pad, &map_q, fb, h * kHeadDim, w.tx * TW, w.ty * 4, w.b);
-    };
-    auto issue_v_tile = [&](const TileWalk& w) {
-        const uint32_t fb = bar(kBarVFull + w.stage);
-        mbar_expect_tx(fb, (uint32_t)(6 * HW2 * 64));
-        tma_load_4d(smem_u32(smem + L.v_off + (size_t)w.stage * L.halo_pad), &map_v, fb, h * kHeadDim,
-                    w.tx * TW - 1, w.ty * 4 - 1, w.b);
+    const uint32_t tmem = *reinterpret_cast<const volatile uint32_t*>(smem + kTmemOff);
+    bool ok = true;
+    // the images of the weights, by the warps that wait for them to be used
+    auto build_images = [&](int builder) {
+        if (P.bimg) return;
+        wait_or_give_up(bar(kBarRaw), 0, ok);
+        const float* raw = reinterpret_cast<const float*>(smem + kRawOff);
+#pragma unroll 1
+        for (int item = 32 * builder + lane; item < kItems; item += 32 * kBuilders) build_item(raw, raw + kWeightFloats, smem + kBOff, item);
+        fence_proxy_async_smem();
+        __syncwarp();
+        mbar_arrive_lane0(bar(kBarWeights), lane);
     };
 
-    // The B images of this CTA's head were laid out by the prep kernel of the same forward; they come
-    // in with one bulk copy, sent for together with the first K/q and V tiles.  Only the MMA threads
-    // wait for them.  The prep kernel may still be running when this kernel starts (programmatic
-    // dependent launch), so the thread that reads its output waits for that grid first; nothing
-    // else in this kernel depends on it.
-    int k_issued = 0, v_issued = 0;
-    TileWalk kq = walk_begin(), vq = kq;
-    if (my_tiles > 0 && warp == kCtlT) {
-        // the same lane is elected here and in the refill loop below (the election is deterministic for
-        // a given member mask), so the ring positions it advances here are the ones it continues from
-        uint32_t leader;
-        if (elect_one(leader)) {
-            while (k_issued < my_tiles && k_issued < kKStages) { issue_k_tile(kq); walk_next(kq, kKStages); ++k_issued; }
-            while (v_issued < my_tiles && v_issued < SV) { issue_v_tile(vq); walk_next(vq, SV); ++v_issued; }
+    if (warp < kPWarp0) {
+        // =====================================================================================
+        // value warps: set s takes blocks s, s + sets, ..; warp q of it strip q of the block
+        // =====================================================================================
+        reg_take<kValueRegs>();
+        build_images(warp);
+        const int q = warp & 3, set = warp >> 2, g = lane >> 2, tig = lane & 3;
+        const uint32_t tq = tmem + kColD + ((uint32_t)(32 * q) << 16);
+        const uint32_t full = bar(kBarDFull + 3 * set);
+        const int C = P.heads * kHeadDim;
+        const size_t row_pitch = (size_t)P.W * C;
+        StripWalk walk(P.strips, 4LL * (rank + set * nrank) + q, 4LL * kVSets * nrank);
+        const unsigned char* ring = smem + kVOff + (uint32_t)(q * kHaloPlane) + (uint32_t)g * 64u + (uint32_t)tig * 16u;
+        const int last = (int)P.strips.total - q;
+        const uint32_t zero = (uint32_t)(P.H >> 31);
+        int slot = set;
+        uint32_t phase = 0, parity = 0;                            // of the slot; of the chunks
+#pragma unroll 1
+        for (int blk = set; blk < my_blocks; blk += kVSets) {
+            const unsigned char* src = ring + (uint32_t)slot * kSlot;
+            wait_or_give_up(bar(kBarVFull + slot), phase, ok);
+            float acc[4][8];
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int c = 0; c < 8; ++c) acc[i][c] = 0.f;
+            uint4 vp[6];
+#pragma unroll
+            for (int r = 0; r < 6; ++r) vp[r] = lds128(src, (uint32_t)(r * 10) * 64u);
+#pragma unroll
+            for (int dx = 0; dx < 3; ++dx) {
+                wait_or_give_up(full + 8u * dx, parity, ok);
+                tc_fence_after_sync();
+                const uint32_t ta = tq + 96u * dx, tb = ta + (16u << 16);
+                uint32_t d[48];
+                tmem_ld3_16x256b_x4_nowait(ta, ta + 32, ta + 64, d);
+                float vf[6][8];
+                auto widen = [&](int r) {
+                    const uint4 v = vp[r];
+                    vf[r][0] = bf16_lo(v.x); vf[r][1] = bf16_hi(v.x); vf[r][2] = bf16_lo(v.y); vf[r][3] = bf16_hi(v.y);
+                    vf[r][4] = bf16_lo(v.z); vf[r][5] = bf16_hi(v.z); vf[r][6] = bf16_lo(v.w); vf[r][7] = bf16_hi(v.w);
+                };
+                auto sum = [&](int m) {                            // pixel rows 2m, 2m + 1
+#pragma unroll
+                    for (int dy = 0; dy < 3; ++dy)
+#pragma unroll
+                        for (int i = 0; i < 2; ++i)
+#pragma unroll
+                            for (int j = 0; j < 4; ++j)
+                                ffma2(acc[2 * m + i][2 * j], acc[2 * m + i][2 * j + 1], __uint_as_float(d[16 * dy + 4 * j + 2 * i]),
+                                      __uint_as_float(d[16 * dy + 4 * j + 2 * i + 1]), vf[2 * m + dy + i][2 * j], vf[2 * m + dy + i][2 * j + 1]);
+                };
+#pragma unroll
+                for (int r = 0; r < 4; ++r) widen(r);
+                tmem_wait_ld48(d);
+                sum(0);
+                tmem_ld3_16x256b_x4_nowait(tb, tb + 32, tb + 64, d);
+                widen(4); widen(5);
+                if (dx < 2)
+#pragma unroll
+                    for (int r = 0; r < 6; ++r) vp[r] = lds128(src, (uint32_t)(r * 10 + dx + 1) * 64u);
+                tmem_wait_ld48(d);
+                tc_fence_before_sync();
+                mbar_arrive_lane0(bar(kBarDFree + dx), lane);
+                sum(1);
+            }
+            mbar_arrive_lane0_after(bar(kBarVEmpty + slot), lane, acc[0][0], acc[3][0], zero);
+            if ((slot += kVSets) >= kVSlots) { slot = set; phase ^= 1u; }
+            parity ^= 1u;
+            const int x = walk.x0() + g, y = walk.y0(), left = P.H - y;
+            if (x < P.W && 4 * (rank + blk * nrank) < last) {
+                __nv_bfloat16* op = P.out + (((size_t)walk.b * P.H + y) * P.W + x) * C + h * kHeadDim + tig * 8;
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (i < left)
+                        *reinterpret_cast<uint4*>(op + i * row_pitch) = make_uint4(pack_bf16(acc[i][0], acc[i][1]), pack_bf16(acc[i][2], acc[i][3]),
+                                                                                   pack_bf16(acc[i][4], acc[i][5]), pack_bf16(acc[i][6], acc[i][7]));
+            }
+            walk.next();
         }
-    }
-    if (my_tiles > 0 && warp == kCtlV && lane == 0) {
+    } else if (warp < kSWarp0) {
+        // =====================================================================================
+        // product warps: as the value warps
+        // =====================================================================================
+        reg_give<kProductRegs>();
+        const int q = warp & 3, set = (warp - kPWarp0) >> 2, g = lane >> 2, tig = lane & 3;
+        const uint32_t tq = tmem + kColP + ((uint32_t)(32 * q) << 16);
+        const unsigned char* ring = smem + (uint32_t)g * 64u + (uint32_t)tig * 16u;
+        // a chunk's buffer is free once the MMAs of the block before have read it, which the other set's barriers say
+        const uint32_t free = bar(kBarPFree + 3 * ((set + kPSets - 1) % kPSets)), ready = bar(kBarPReady);
+        int slot = set;
+        uint32_t phase = 0, parity = set == 0 ? 1u : 0u;
+#pragma unroll 1
+        for (int blk = set; blk < my_blocks; blk += kPSets) {
+            const unsigned char* sK = ring + (uint32_t)slot * kKSlot + (uint32_t)(q * kHaloPlane);
+            const unsigned char* sQ = ring + (uint32_t)slot * kKSlot + (uint32_t)kSlot + (uint32_t)q * kQStrip;
+            wait_or_give_up(bar(kBarKFull + slot), phase, ok);
+            uint4 qf[4], kc[6];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) qf[i] = lds128(sQ, (uint32_t)(i * 8) * 64u);
+#pragma unroll
+            for (int r = 0; r < 6; ++r) kc[r] = lds128(sK, (uint32_t)(r * 10) * 64u);
+#pragma unroll
+            for (int dx = 0; dx < 3; ++dx) {
+                wait_or_give_up(free + 8u * dx, parity, ok);
+                tc_fence_after_sync();
+#pragma unroll
+                for (int dy = 0; dy < 3; ++dy)
+#pragma unroll
+                    for (int m = 0; m < 2; ++m) {
+                        const uint4 q0 = qf[2 * m], q1 = qf[2 * m + 1], k0 = kc[2 * m + dy], k1 = kc[2 * m + dy + 1];
+                        const uint32_t r[8] = {hmul2_bf16(q0.x, k0.x), hmul2_bf16(q0.y, k0.y), hmul2_bf16(q1.x, k1.x), hmul2_bf16(q1.y, k1.y),
+                                               hmul2_bf16(q0.z, k0.z), hmul2_bf16(q0.w, k0.w), hmul2_bf16(q1.z, k1.z), hmul2_bf16(q1.w, k1.w)};
+                        tmem_st_16x256b_x2(tq + ((uint32_t)(16 * m) << 16) + 48 * dx + 16 * dy, r);
+                    }
+                if (dx < 2)
+#pragma unroll
+                    for (int r = 0; r < 6; ++r) kc[r] = lds128(sK, (uint32_t)(r * 10 + dx + 1) * 64u);
+                tmem_wait_st();
+                tc_fence_before_sync();
+                mbar_arrive_lane0(ready + 8u * dx, lane);
+            }
+            // the products that were made of what was read are in tensor memory
+            mbar_arrive_lane0(bar(kBarKEmpty + slot), lane);
+            if ((slot += kPSets) >= kKSlots) { slot = set; phase ^= 1u; }
+            parity ^= 1u;
+        }
+    } else if (warp < kCtlK) {
+        // =====================================================================================
+        // softmax warps: thread = pixel = TMEM lane 32 q + lane, every block
+        // =====================================================================================
+        reg_give<kSoftmaxRegs>();
+        build_images(4 * kVSets + warp - kSWarp0);
+        const uint32_t tq = tmem + ((uint32_t)(32 * (warp & 3)) << 16);
         grid_dependency_wait();
-        mbar_expect_tx(bar(kBarWeights), kImgBytes);
-        bulk_load_1d(smem_u32(smem + L.b_off), P.bimg + (size_t)h * kImgBytes, kImgBytes, bar(kBarWeights));
-    }
-    __syncwarp();
-    bool ok = my_tiles > 0;
-
-    if (warp >= kVWarps && warp < kCtlK) {
-        // =====================================================================================
-        // product warps: warp (q, pm) takes pixel rows 2pm, 2pm+1 of unit 4 blk + q of every block
-        // =====================================================================================
-        const int q = (warp - kVWarps) & 3;                        // == warp % 4
-        const int pm = (warp - kVWarps) >> 2;                      // pixel-row pair of the unit; softmax of blocks = pm mod 2
-        const uint32_t tq = tmem + ((uint32_t)(32 * q) << 16);
         float biasl[9];
 #pragma unroll
         for (int s = 0; s < 9; ++s) biasl[s] = P.bias ? P.bias[h * 9 + s] * kLog2e : 0.f;
-
-        // softmax of block sb (thread = pixel = TMEM lane 32 q + lane); `valid`: the unit exists
-        auto softmax_block = [&](int sb, bool valid) -> bool {
-            const int lb = sb & 1;
-            if (!warp_wait(bar(kBarLFull + lb), (sb >> 1) & 1)) return false;
+        uint32_t full = bar(kBarLFull), parity = 0, tl = tq + kColL;
+#pragma unroll 1
+        for (int blk = 0; blk < my_blocks; ++blk) {
+            wait_or_give_up(full, parity, ok);
             tc_fence_after_sync();
-            float Lg[32];
-            tmem_ld_32x32b_x32(tq + kColL + 32 * lb, Lg);
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar(kBarLFree + lb));
+            float Lg[18];
+            tmem_ld_32x32b_18(tl, Lg);
+            tc_fence_before_sync();
+            mbar_arrive_lane0(full + 8u * (uint32_t)(kBarLFree - kBarLFull), lane);
+            float l[9], m = -INFINITY;
+#pragma unroll
+            for (int s = 0; s < 9; ++s) { l[s] = (Lg[s] + Lg[9 + s]) * P.scale_log2e + biasl[s]; m = fmaxf(m, l[s]); }
+            float e[9], sum = 0.f;
+#pragma unroll
+            for (int s = 0; s < 9; ++s) { e[s] = fast_exp2(l[s] - m); sum += e[s]; }
+            const float inv = rcp_approx(sum);                     // the weights leave normalised: the value side only sums
+            float hi[9], lo[9];
             uint32_t row[16];
 #pragma unroll
-            for (int i = 0; i < 16; ++i) row[i] = 0u;
-            if (valid) {
-                float l[9], m = -INFINITY;
-#pragma unroll
-                for (int s = 0; s < 9; ++s) { l[s] = (Lg[s] + Lg[9 + s]) * P.scale_log2e + biasl[s]; m = fmaxf(m, l[s]); }
-                float e[9], sum = 0.f;
-#pragma unroll
-                for (int s = 0; s < 9; ++s) { e[s] = fast_exp2(l[s] - m); sum += e[s]; }
-                const float inv = rcp_approx(sum);               // the weights leave normalised: the value side only sums
-                float hi[9], lo[9];
-#pragma unroll
-                for (int s = 0; s < 9; ++s) {
-                    const float a = e[s] * inv;
-                    hi[s] = __bfloat162float(__float2bfloat16_rn(a));
-                    lo[s] = a - hi[s];
-                }
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    row[i] = pack_bf16(hi[2 * i], hi[2 * i + 1]);
-                    row[4 + i] = row[i];
-                    row[8 + i] = pack_bf16(lo[2 * i], lo[2 * i + 1]);
-                }
-                row[12] = pack_bf16(hi[8], hi[8]);
-                row[13] = pack_bf16(lo[8], 0.f);
+            for (int s = 0; s < 9; ++s) {
+                const float a = e[s] * inv;
+                hi[s] = __bfloat162float(__float2bfloat16_rn(a));
+                lo[s] = a - hi[s];
             }
-            if (!warp_wait(bar(kBarEFree + lb), ((sb >> 1) & 1) ^ 1)) return false;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                row[i] = pack_bf16(hi[2 * i], hi[2 * i + 1]);
+                row[4 + i] = row[i];
+                row[8 + i] = pack_bf16(lo[2 * i], lo[2 * i + 1]);
+            }
+            row[12] = pack_bf16(hi[8], hi[8]);
+            row[13] = pack_bf16(lo[8], 0.f);
+            row[14] = row[15] = 0u;
+            wait_or_give_up(bar(kBarEFree), ((uint32_t)blk & 1u) ^ 1u, ok);
             tc_fence_after_sync();
-            tmem_st_32x32b_x16(tq + kColE + 16 * lb, row);
+            tmem_st_32x32b_x16(tq + kColE, row);
             tmem_wait_st();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar(kBarEReady + lb));
-            return true;
-        };
-
-        int done_blocks = 0;                                       // blocks whose P this warp has delivered
-        int next_sm = pm;                                          // next block whose softmax is this warp's
-        // softmax of this warp's blocks below `upto`
-        auto softmax_upto = [&](int upto) -> bool {
-            while (next_sm < upto) {
-                if (!softmax_block(next_sm, 4 * next_sm + q < my_units)) return false;
-                next_sm += 2;
-            }
-            return true;
-        };
-        for (int ti = 0; ok && ti < my_tiles; ++ti) {
-            const int stage = ti % kKStages;
-            if (!warp_wait(bar(kBarKFull + stage), (ti / kKStages) & 1)) { ok = false; break; }
-            const int u0 = ti * U;
-            for (int ul = (q + 4 - u0 % 4) % 4; ul < U; ul += 4) {
-                const int u = u0 + ul, blk = u >> 2;
-                const int ux = ul * 8;
-                const unsigned char* sK = smem + (size_t)stage * L.kstage_bytes;
-                const unsigned char* sQ = sK + L.halo_pad;
-                uint32_t qf[2][4];                                 // pixel rows 2pm, 2pm+1 of column ux + g
-#pragma unroll
-                for (int i = 0; i < 2; ++i) {
-                    const uint4 v = lds_u4(sQ, (uint32_t)((2 * pm + i) * TW + ux + g) * 64u + tig * 16u);
-                    qf[i][0] = v.x; qf[i][1] = v.y; qf[i][2] = v.z; qf[i][3] = v.w;
-                }
-                const uint32_t off0 = (uint32_t)(ux + g) * 64u + tig * 16u;
-#pragma unroll
-                for (int dx = 0; dx < 3; ++dx) {
-                    const int pc = 3 * blk + dx, pb = pc & 3;
-                    uint4 kc[4];                                   // halo rows 2pm .. 2pm+3 of column dx
-#pragma unroll
-                    for (int r = 0; r < 4; ++r) kc[r] = lds_u4(sK, off0 + (uint32_t)((2 * pm + r) * HW2 + dx) * 64u);
-                    if (!warp_wait(bar(kBarPFree + pb), ((pc >> 2) & 1) ^ 1)) { ok = false; break; }
-                    tc_fence_after_sync();
-#pragma unroll
-                    for (int dy = 0; dy < 3; ++dy) {
-                        const uint4 k0 = kc[dy], k1 = kc[dy + 1];
-                        uint32_t r[8];
-                        r[0] = hmul2_bf16(qf[0][0], k0.x); r[1] = hmul2_bf16(qf[0][1], k0.y);
-                        r[2] = hmul2_bf16(qf[1][0], k1.x); r[3] = hmul2_bf16(qf[1][1], k1.y);
-                        r[4] = hmul2_bf16(qf[0][2], k0.z); r[5] = hmul2_bf16(qf[0][3], k0.w);
-                        r[6] = hmul2_bf16(qf[1][2], k1.z); r[7] = hmul2_bf16(qf[1][3], k1.w);
-                        tmem_st_16x256b_x2(tq + ((uint32_t)(16 * pm) << 16) + kColP + 48 * pb + 16 * dy, r);
-                    }
-                    tmem_wait_st();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(bar(kBarPReady + pb));
-                }
-                if (!ok) break;
-                ++done_blocks;
-                // the logits of the blocks before this one are complete by now (or soon)
-                if (!softmax_upto(blk)) { ok = false; break; }
-            }
-            __syncwarp();
-            if (ok && lane == 0) mbar_arrive(bar(kBarKEmpty + stage));
+            tc_fence_before_sync();
+            mbar_arrive_lane0(bar(kBarEReady), lane);
+            full ^= 8u; tl ^= kOtherL;
+            parity ^= (uint32_t)blk & 1u;
         }
-        // a quadrant the last block lacks: deliver its (empty) share so that the counts complete
-        if (ok && done_blocks < my_blocks) {
-            const int blk = my_blocks - 1;
-            for (int dx = 0; ok && dx < 3; ++dx) {
-                const int pc = 3 * blk + dx, pb = pc & 3;
-                if (!warp_wait(bar(kBarPFree + pb), ((pc >> 2) & 1) ^ 1)) { ok = false; break; }
-                if (lane == 0) mbar_arrive(bar(kBarPReady + pb));
-            }
-        }
-        if (ok && !softmax_upto(my_blocks)) ok = false;
-    } else if (warp < kVWarps) {
-        // =====================================================================================
-        // value warps: warp (qd, m) takes pixel rows 2m, 2m+1 of quadrant qd of every block
-        // =====================================================================================
-        const int qd = warp & 3, m = warp >> 2;
-        const uint32_t tq = tmem + ((uint32_t)(32 * qd + 16 * m) << 16);
-
-        TileWalk vw = walk_begin();
-        for (int ti = 0; ok && ti < my_tiles; ++ti, walk_next(vw, SV)) {
-            const int tx = vw.tx, ty = vw.ty, b = vw.b, stage = vw.stage;
-            if (!warp_wait(bar(kBarVFull + stage), vw.round & 1)) { ok = false; break; }
-            const int u0 = ti * U;
-          for (int ul = (qd + 4 - u0 % 4) % 4; ul < U; ul += 4) {
-            const int u = u0 + ul;
-            const int ux = ul * 8;
-            const int blk = u >> 2;
-            const unsigned char* sV = smem + L.v_off + (size_t)stage * L.halo_pad;
-            const uint32_t off0 = (uint32_t)(ux + g) * 64u + tig * 16u;
-
-            float o_acc[2][8];
-#pragma unroll
-            for (int i = 0; i < 2; ++i)
-#pragma unroll
-                for (int c = 0; c < 8; ++c) o_acc[i][c] = 0.f;
-
-#pragma unroll
-            for (int dx = 0; dx < 3; ++dx) {
-                const int cs = 3 * blk + dx, ds = cs & 1;
-                if (!warp_wait(bar(kBarDFull + ds), (cs >> 1) & 1)) { ok = false; break; }
-                tc_fence_after_sync();
-                const uint32_t colbase = kColD + ds * 112;
-                {
-                    uint32_t dr[48];
-                    const uint32_t ta = tq + colbase;
-                    tmem_ld3_16x256b_x4_nowait(ta, ta + 32, ta + 64, dr);
-                    uint4 vp[4];
-#pragma unroll
-                    for (int r = 0; r < 4; ++r) vp[r] = lds_u4(sV, off0 + (uint32_t)((2 * m + r) * HW2 + dx) * 64u);
-                    float vf[4][8];
-#pragma unroll
-                    for (int r = 0; r < 4; ++r) {
-                        const uint4 v = vp[r];
-                        vf[r][0] = bf16_lo(v.x); vf[r][1] = bf16_hi(v.x);
-                        vf[r][2] = bf16_lo(v.y); vf[r][3] = bf16_hi(v.y);
-                        vf[r][4] = bf16_lo(v.z); vf[r][5] = bf16_hi(v.z);
-                        vf[r][6] = bf16_lo(v.w); vf[r][7] = bf16_hi(v.w);
-                    }
-                    tmem_wait_ld48(dr);
-                    float d[48];
-#pragma unroll
-                    for (int i = 0; i < 48; ++i) d[i] = __uint_as_float(dr[i]);
-#pragma unroll
-                    for (int dy = 0; dy < 3; ++dy) {
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            ffma2(o_acc[0][2 * j], o_acc[0][2 * j + 1], d[16 * dy + 4 * j], d[16 * dy + 4 * j + 1],
-                                  vf[dy][2 * j], vf[dy][2 * j + 1]);
-                            ffma2(o_acc[1][2 * j], o_acc[1][2 * j + 1], d[16 * dy + 4 * j + 2], d[16 * dy + 4 * j + 3],
-                                  vf[dy + 1][2 * j], vf[dy + 1][2 * j + 1]);
-                        }
-                    }
-                }
-                __syncwarp();
-                if (lane == 0) mbar_arrive(bar(kBarDFree + ds));
-            }
-            if (!ok) break;
-
-            {
-                const int x = tx * TW + ux + g, y0 = ty * 4 + 2 * m;
-                __nv_bfloat16* op = P.out + ((size_t)(b * P.H + y0) * P.W + x) * C + h * kHeadDim + tig * 8;
-                const size_t row_stride = (size_t)P.W * C;
-#pragma unroll
-                for (int i = 0; i < 2; ++i) {
-                    if (x < P.W && y0 + i < P.H) {
-                        uint4 r;
-                        r.x = pack_bf16(o_acc[i][0], o_acc[i][1]);
-                        r.y = pack_bf16(o_acc[i][2], o_acc[i][3]);
-                        r.z = pack_bf16(o_acc[i][4], o_acc[i][5]);
-                        r.w = pack_bf16(o_acc[i][6], o_acc[i][7]);
-                        *reinterpret_cast<uint4*>(op + i * row_stride) = r;
-                    }
-                }
-            }
-          }
-            __syncwarp();
-            if (ok && lane == 0) mbar_arrive(bar(kBarVEmpty + stage));
-        }
-        // quadrants of the last block that hold no unit: keep the chunk barriers in step
-        if (ok && my_blocks > 0 && (my_units & 3) != 0 && qd >= (my_units & 3)) {
-            for (int dx = 0; ok && dx < 3; ++dx) {
-                const int cs = 3 * (my_blocks - 1) + dx, ds = cs & 1;
-                if (!warp_wait(bar(kBarDFull + ds), (cs >> 1) & 1)) { ok = false; break; }
-                if (lane == 0) mbar_arrive(bar(kBarDFree + ds));
-            }
-        }
-        tc_fence_before_sync();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bar(kBarVDone));
-    } else if (warp == kCtlK || warp == kCtlK2) {
-        // =====================================================================================
-        // key-side control: the key MMAs (18 per block: 9 taps x two K = 16 halves); warp 16 takes
-        // the even blocks, warp 18 the odd ones, in turn.  The tensor pipe executes one small MMA
-        // at a time, so the two threads overlap each other's waits rather than their MMAs.
-        // =====================================================================================
-        uint32_t leader;
-        const bool elected = elect_one(leader);
-        if (elected && ok) {
-            const uint32_t sBk0 = smem_u32(smem + L.bk_off);
-            // This thread has one thing to wait for at a time, so it parks in the waits (bounded).
-            // The two threads take the blocks in turn: a thread starts block b only when the other
-            // one has got past the P-ready wait of the last chunk of block b - 1, so the P-ready
-            // barriers are waited on strictly in chunk order.
-            const int me = warp == kCtlK ? 0 : 1;
-            if (!mbar_wait(bar(kBarWeights), 0)) ok = false;
-            for (int blk = me, n = 0; ok && blk < my_blocks; blk += 2, ++n) {
-                const int lb = blk & 1;
-                const uint32_t dcol = tmem + kColL + 32 * lb;
-                // even blocks wait for the odd block before (none before block 0: parity 1 of a
-                // fresh barrier tests true), odd blocks for the even block before
-                if (!mbar_wait(bar(kBarTurn + me), me == 0 ? (uint32_t)((n - 1) & 1) : (uint32_t)(n & 1))) { ok = false; break; }
-                if (!mbar_wait(bar(kBarLFree + lb), ((blk >> 1) & 1) ^ 1)) { ok = false; break; }
-#pragma unroll
-                for (int dx = 0; dx < 3; ++dx) {
-                    const int pc = 3 * blk + dx, pb = pc & 3;
-                    if (!mbar_wait(bar(kBarPReady + pb), (pc >> 2) & 1)) { ok = false; break; }
-                    if (dx == 2) mbar_arrive(bar(kBarTurn + (me ^ 1)));
-                    tc_fence_after_sync();
-                    const uint32_t acol = tmem + kColP + 48 * pb;
-                    const uint64_t bdesc = umma_smem_desc(sBk0 + (uint32_t)dx * 4u * 512u, 512, 128);
-#pragma unroll
-                    for (int dy = 0; dy < 3; ++dy) {
-#pragma unroll
-                        for (int kh = 0; kh < 2; ++kh)      // 16 bytes of descriptor address = 1 unit
-                            umma_bf16_ts(dcol, acol + 16 * dy + 8 * kh, bdesc + (uint64_t)((dy * 12 + kh * 2) * 32),
-                                         kIdesc32, (dx != 0 || dy != 0 || kh != 0) ? 1u : 0u);
-                    }
-                    umma_commit(bar(kBarPFree + pb));
-                    if (dx == 2) umma_commit(bar(kBarLFull + lb));
-                }
-            }
-        }
-        ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, leader) != 0;
-        if (warp == kCtlK) {
-            if (my_tiles > 0 && !warp_wait(bar(kBarVDone), 0)) ok = false;
-            tc_fence_after_sync();
-            __syncwarp();
-            tmem_dealloc(tmem, kTmemCols);
-        }
-    } else if (warp == kCtlV) {
-        // =====================================================================================
-        // value-side control: the value MMAs (chunk c = 3 blk + dx -> TMEM slot c & 1).  One thing to
-        // wait for at a time, so the thread parks in the (bounded) waits.
-        // =====================================================================================
-        uint32_t leader;
-        const bool elected = elect_one(leader);
-        if (elected && ok) {
-            const uint32_t sB0 = smem_u32(smem + L.b_off);
-            if (!mbar_wait(bar(kBarWeights), 0)) ok = false;
-            for (int blk = 0; ok && blk < my_blocks; ++blk) {
-                const int eb = blk & 1;
-                if (!mbar_wait(bar(kBarEReady + eb), (blk >> 1) & 1)) { ok = false; break; }
-                const uint32_t acol = tmem + kColE + 16 * eb;
-#pragma unroll
-                for (int dx = 0; dx < 3; ++dx) {
-                    const int cs = 3 * blk + dx, ds = cs & 1;
-                    if (!mbar_wait(bar(kBarDFree + ds), ((cs >> 1) & 1) ^ 1)) { ok = false; break; }
-                    tc_fence_after_sync();
-                    const uint32_t sB = sB0 + dx * 12 * 512;
-                    const uint32_t idesc = kIdesc96;
-                    const uint32_t dcol = tmem + kColD + ds * 112;
-                    umma_bf16_ts(dcol, acol, umma_smem_desc(sB, 128, 512), idesc, 0);
-                    umma_bf16_ts(dcol, acol + 8, umma_smem_desc(sB + 256, 128, 512), idesc, 1);
-                    umma_commit(bar(kBarDFull + ds));
-                    if (dx == 2) umma_commit(bar(kBarEFree + eb));
-                }
-            }
-        }
-        ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, leader) != 0;
     } else {
-        // =====================================================================================
-        // TMA thread: refills the K/q ring and the V ring as their stages are released
-        // =====================================================================================
+        reg_give<kControlRegs>();
+        // no copy is on its way when the block leaves, whatever its readers have given up on
+        auto drain = [&](int full, int slots, int issued) {
+#pragma unroll 1
+            for (int s = 0; s < slots && s < issued; ++s)
+                ok = mbar_wait<true>(bar(full + s), (uint32_t)((issued - 1 - s) / slots) & 1u) && ok;
+        };
         uint32_t leader;
-        const bool elected = elect_one(leader);
-        if (elected && ok) {
-            int left = my_tiles - v_issued + my_tiles - k_issued;
-            uint32_t idle = 0;
-            while (left > 0) {
-                const uint32_t tK = mbar_test_u32(bar(kBarKEmpty + kq.stage), (kq.round - 1) & 1);
-                const uint32_t tV = mbar_test_u32(bar(kBarVEmpty + vq.stage), (vq.round - 1) & 1);
-                const int left_before = left;
-                if (tK != 0 && k_issued < my_tiles) { issue_k_tile(kq); walk_next(kq, kKStages); ++k_issued; --left; }
-                if (tV != 0 && v_issued < my_tiles) {
-                    issue_v_tile(vq); walk_next(vq, SV); ++v_issued; --left;
+        if (elect_one(leader) && my_blocks > 0) {
+            if (warp == kCtlK) {
+                // ---- key MMAs: 18 per block (9 taps x two K = 16 halves) --------------------------------
+                const uint64_t desc = umma_smem_desc(smem_u32(smem + kBkOff), 512, 128);
+                uint32_t full = bar(kBarLFull), parity = 0, dcol = tmem + kColL;
+                int set = 0;
+                ok = mbar_wait<true>(bar(kBarWeights), 0);
+#pragma unroll 1
+                for (int blk = 0; ok && blk < my_blocks; ++blk) {
+                    if (!mbar_wait<true>(full + 8u * (uint32_t)(kBarLFree - kBarLFull), parity ^ 1u)) { ok = false; break; }
+#pragma unroll
+                    for (int dx = 0; dx < 3; ++dx) {
+                        if (!mbar_wait<true>(bar(kBarPReady + dx), (uint32_t)blk & 1u)) { ok = false; break; }
+                        tc_fence_after_sync();
+#pragma unroll
+                        for (int dy = 0; dy < 3; ++dy)
+#pragma unroll
+                            for (int kh = 0; kh < 2; ++kh)          // 16 bytes of descriptor address = 1 unit
+                                umma_bf16_ts(dcol, tmem + kColP + 48 * dx + 16 * dy + 8 * kh, desc + (uint64_t)((dx * 4 + dy * 12 + kh * 2) * 32),
+                                             kIdesc32, (dx != 0 || dy != 0 || kh != 0) ? 1u : 0u);
+                        umma_commit(bar(kBarPFree + dx) + 24u * (uint32_t)set);
+                        if (dx == 2) umma_commit(full);
+                    }
+                    if (kPSets == 2) set ^= 1;
+                    full ^= 8u; dcol ^= kOtherL;
+                    parity ^= (uint32_t)blk & 1u;
                 }
-                if (left != left_before) idle = 0;
-                else {
-                    if (++idle > (1u << 22)) { ok = false; break; }
-                    __nanosleep(200);
+            } else if (warp == kCtlV) {
+                // ---- value MMAs -------------------------------------------------------------------------
+                const uint64_t desc = umma_smem_desc(smem_u32(smem + kBOff), 128, 512);
+                uint32_t done = bar(kBarDFull);
+                ok = mbar_wait<true>(bar(kBarWeights), 0);
+#pragma unroll 1
+                for (int blk = 0; ok && blk < my_blocks; ++blk) {
+                    if (!mbar_wait<true>(bar(kBarEReady), (uint32_t)blk & 1u)) { ok = false; break; }
+#pragma unroll
+                    for (int dx = 0; dx < 3; ++dx) {
+                        if (!mbar_wait<true>(bar(kBarDFree + dx), ((uint32_t)blk & 1u) ^ 1u)) { ok = false; break; }
+                        tc_fence_after_sync();
+                        const uint32_t dcol = tmem + kColD + 96u * dx;
+                        umma_bf16_ts(dcol, tmem + kColE, desc + (uint64_t)(dx * 12 * 32), kIdesc96, 0);
+                        umma_bf16_ts(dcol, tmem + kColE + 8, desc + (uint64_t)(dx * 12 * 32 + 16), kIdesc96, 1);
+                        umma_commit(done + 8u * dx);
+                        if (dx == 2) umma_commit(bar(kBarEFree));
+                    }
+                    if (kVSets == 2) done = done == bar(kBarDFull) ? done + 24u : bar(kBarDFull);
                 }
+            } else if (warp == kCtlTK) {
+                // ---- K and q strips -----------------------------------------------------------------------
+                grid_dependency_wait();
+                StripWalk at(P.strips, 4LL * rank, 4LL * nrank);
+                int slot = 0, blk = 0;
+                uint32_t phase = 1;                                // a fresh barrier is free
+#pragma unroll 1
+                for (; blk < my_blocks; ++blk, at.next()) {
+                    const uint32_t dst = smem_u32(smem) + (uint32_t)slot * kKSlot, full = bar(kBarKFull + slot);
+                    if (!mbar_wait<true>(bar(kBarKEmpty + slot), phase)) { ok = false; break; }
+                    mbar_expect_tx(full, kKSlot);
+                    StripWalk s = at;                              // strips past the last one read as zero: their image does not exist
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        tma_load_4d(dst + (uint32_t)(i * kHaloPlane), &map_k, full, h * kHeadDim, s.x0() - 1, s.y0() - 1, s.b);
+                        tma_load_4d(dst + (uint32_t)kSlot + (uint32_t)i * kQStrip, &map_q, full, h * kHeadDim, s.x0(), s.y0(), s.b);
+                        if (++s.x == s.sx) { s.x = 0; if (++s.y == s.bands) { s.y = 0; ++s.b; } }
+                    }
+                    if (++slot == kKSlots) { slot = 0; phase ^= 1u; }
+                }
+                // What follows in the stream may be launched: as blocks leave, it takes their place and sets itself up.
+                grid_launch_dependents();
+                drain(kBarKFull, kKSlots, blk);
+            } else {
+                // ---- the head's weights, then V strips ------------------------------------------------------
+                grid_dependency_wait();
+                if (P.bimg) {
+                    mbar_expect_tx(bar(kBarWeights), kImgBytes);
+                    bulk_load_1d(smem_u32(smem + kBOff), P.bimg + (size_t)h * kImgBytes, kImgBytes, bar(kBarWeights));
+                } else {
+                    constexpr uint32_t bytes = kWeightFloats * 4;
+                    mbar_expect_tx(bar(kBarRaw), 2 * bytes);
+                    bulk_load_1d(smem_u32(smem + kRawOff), P.wk + (size_t)h * kWeightFloats, bytes, bar(kBarRaw));
+                    bulk_load_1d(smem_u32(smem + kRawOff) + bytes, P.wv + (size_t)h * kWeightFloats, bytes, bar(kBarRaw));
+                }
+                StripWalk at(P.strips, 4LL * rank, 4LL * nrank);
+                int slot = 0, blk = 0;
+                uint32_t phase = 1;
+#pragma unroll 1
+                for (; blk < my_blocks; ++blk, at.next()) {
+                    if (blk == kVSlots - kRawSlots && !mbar_wait<true>(bar(kBarWeights), 0)) { ok = false; break; }
+                    if (!mbar_wait<true>(bar(kBarVEmpty + slot), phase)) { ok = false; break; }
+                    team::load_strips(smem_u32(smem) + kVOff + (uint32_t)slot * kSlot, &map_v, bar(kBarVFull + slot), h * kHeadDim, at);
+                    if (++slot == kVSlots) { slot = 0; phase ^= 1u; }
+                }
+                drain(kBarVFull, kVSlots, blk);
+                if (blk <= kVSlots - kRawSlots) ok = mbar_wait<true>(bar(P.bimg ? kBarWeights : kBarRaw), 0) && ok;
             }
         }
-        ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, leader) != 0;
+        __syncwarp();
     }
-    if (!ok && my_tiles > 0 && lane == 0) atomicExch(P.status, 1);
+    if (!ok) atomicExch(P.status, 1);
+    tc_fence_before_sync();
+    __syncthreads();
+    if (warp == kCtlK) {
+        tc_fence_after_sync();
+        tmem_dealloc(tmem, kTmemCols);
+    }
 }
 
 }  // namespace
@@ -632,79 +525,39 @@ bool umma_ts_supports(slide_attn_dtype dtype, int head_dim, int ksize) {
     return dtype == SLIDE_ATTN_BF16 && head_dim == kHeadDim && ksize == 3;
 }
 
-namespace {
-
-template <int TW>
-cudaError_t setup_one() {
-    return cudaFuncSetAttribute(umma_ts_kernel<TW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
-}
-
-// The main kernel is launched with programmatic stream serialisation: it may begin (barrier set-up,
-// tensor-memory allocation, first tile loads) while the prep kernel before it in the stream is still
-// running; the one thread that reads the prep kernel's output waits for that grid inside the kernel.
-template <int TW>
-cudaError_t launch_one(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv, const UmmaParams& P,
-                       int grid, cudaStream_t stream) {
-    static_assert(v_stages_for(TW) >= 2, "tile width does not fit shared memory");
-    return launch_chained(umma_ts_kernel<TW>, dim3((unsigned)grid), kThreads, smem_layout(TW, v_stages_for(TW)).total, stream, mq, mk, mv, P);
-}
-
-}  // namespace
-
 size_t umma_ts_workspace_bytes(int heads) { return (size_t)heads * kImgBytes; }
 
 cudaError_t umma_ts_setup() {
     if (!tensor_map_available()) return cudaErrorNotSupported;
-    cudaError_t e = setup_one<8>();
-    if (e == cudaSuccess) e = setup_one<16>();
-    if (e == cudaSuccess) e = setup_one<24>();
-    if (e == cudaSuccess) e = setup_one<32>();
-    if (e == cudaSuccess) e = setup_one<40>();
-    if (e == cudaSuccess) e = setup_one<48>();
-    if (e == cudaSuccess) e = setup_one<56>();
-    if (e == cudaSuccess) e = setup_one<64>();
-    return e;
+    return cudaFuncSetAttribute(umma_ts_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
 }
 
 cudaError_t launch_umma_ts_prep(const Problem& p, void* workspace, cudaStream_t stream) {
     return launch_chained(umma_ts_prep_kernel, dim3((unsigned)p.heads, 6), 256, 0, stream, p.wk, p.wv, static_cast<unsigned char*>(workspace));
 }
 
+// `workspace`: the images that launch_umma_ts_prep left there, or null.
 cudaError_t launch_umma_ts(const Problem& p, const void* workspace, int* d_status, int num_sms, cudaStream_t stream) {
-    const int txn = (p.W + 63) / 64;
-    const int TW = ((((p.W + txn - 1) / txn) + 7) / 8) * 8;
     UmmaParams P;
-    P.bimg = static_cast<const unsigned char*>(workspace); P.bias = p.bias;
+    P.wk = p.wk; P.wv = p.wv; P.bimg = static_cast<const unsigned char*>(workspace); P.bias = p.bias;
     P.out = static_cast<__nv_bfloat16*>(p.out);
     P.status = d_status;
-    P.B = p.B; P.H = p.H; P.W = p.W; P.heads = p.heads;
-    P.tiles_x = (p.W + TW - 1) / TW;
-    P.tiles_y = (p.H + 3) / 4;
+    P.H = p.H; P.W = p.W; P.heads = p.heads;
+    P.strips.sx = (p.W + 7) / 8; P.strips.bands = (p.H + 3) / 4;
+    P.strips.total = (long long)p.B * P.strips.bands * P.strips.sx;
+    if (P.strips.total > 0x7fffffffLL - 4) return cudaErrorInvalidConfiguration;
     P.scale_log2e = kLog2e / sqrtf((float)kHeadDim);
 
     const int C = p.heads * kHeadDim;
     CUtensorMap map_q, map_k, map_v;
-    if (!make_tile_map(&map_q, p.q, 2, p.B, p.H, p.W, C, kHeadDim, TW, 4) ||
-        !make_tile_map(&map_k, p.k, 2, p.B, p.H, p.W, C, kHeadDim, TW + 2, 6) ||
-        !make_tile_map(&map_v, p.v, 2, p.B, p.H, p.W, C, kHeadDim, TW + 2, 6))
+    if (!make_tile_map(&map_q, p.q, 2, p.B, p.H, p.W, C, kHeadDim, 8, 4) ||
+        !make_tile_map(&map_k, p.k, 2, p.B, p.H, p.W, C, kHeadDim, 10, 6) ||
+        !make_tile_map(&map_v, p.v, 2, p.B, p.H, p.W, C, kHeadDim, 10, 6))
         return cudaErrorInvalidValue;
-
-    const long long tiles = (long long)P.tiles_x * P.tiles_y * p.B * p.heads;
-    if (tiles > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-    int grid = num_sms;
-    if (grid < p.heads) grid = p.heads;
-    if ((long long)grid > tiles) grid = (int)tiles;
-    switch (TW) {
-        case 8: return launch_one<8>(map_q, map_k, map_v, P, grid, stream);
-        case 16: return launch_one<16>(map_q, map_k, map_v, P, grid, stream);
-        case 24: return launch_one<24>(map_q, map_k, map_v, P, grid, stream);
-        case 32: return launch_one<32>(map_q, map_k, map_v, P, grid, stream);
-        case 40: return launch_one<40>(map_q, map_k, map_v, P, grid, stream);
-        case 48: return launch_one<48>(map_q, map_k, map_v, P, grid, stream);
-        case 56: return launch_one<56>(map_q, map_k, map_v, P, grid, stream);
-        case 64: return launch_one<64>(map_q, map_k, map_v, P, grid, stream);
-        default: return cudaErrorInvalidConfiguration;
-    }
+    const long long blocks = (P.strips.total + 3) / 4;
+    long long grid = num_sms > p.heads ? num_sms : p.heads;      // CTA c takes head c mod heads
+    if (grid > blocks * p.heads) grid = blocks * p.heads;
+    return launch_chained(umma_ts_kernel, dim3((unsigned)grid), kThreads, kSmemBytes, stream, map_q, map_k, map_v, P);
 }
 
 }  // namespace slide_attn
