@@ -21,15 +21,16 @@
 // their upper two, the second their lower two; lane (g, tig) works on column g and channels 8 tig .. 8 tig + 7.  Tiles come by
 // TMA with their halo (zero fill = the padding), K then V.  Five more warps: an MMA and a TMA thread per team; one for weights.
 // The weights (2 x 32 k^4 bf16 per head, laid out by a prep kernel in the order they are used) stay in shared memory for
-// k <= 5 (102 KB at k = 5), so the teams run independently and cover each other's hand-offs; for k >= 7 (400 KB, 1 MB) they are
-// streamed from L2 through a ring that both teams read, 256 pixels per pass over them.
+// k = 3; for k >= 7 (400 KB, 1 MB) they are streamed from L2 through a ring that both teams read, 256 pixels per pass over them.
+// k = 5 (102 KB, resident) has a kernel of its own below.
 //
 // Tensor-memory columns of a team (256): logits, later e (chunk of 16 slots: 8 columns e_hi, 8 e_lo, where its logits were), in
 // the last N; below them the product groups, later the A' groups.  A group = up to GK (GV) taps of one tap column.
 //
-// A call: 64 x 56 x 56, 3 heads, k = 5: 273 us with mma.sync (every CUDA-core multiply beside it cost it pipe time, and every
-// fragment was read from shared memory by every warp), 133 here (71 M warp instructions in 52 % of the issue slots at 1.70 GHz, tensor pipe
-// 38 %); 2 x 128 x 128, 3 heads, k = 7: 137 and 60 us (39 and 40 %: three rounds for 2.6 blocks per team).
+// A call: 2 x 128 x 128, 3 heads, k = 7: 137 us with mma.sync, 60 here (issue slots 39 %, tensor pipe 40 %: three rounds for 2.6 blocks
+// per team).
+#include <type_traits>
+
 #include "common.cuh"
 #include "ptx.cuh"
 
@@ -232,6 +233,21 @@ __device__ __forceinline__ float softmax_in_place(uint32_t col, const float* s_b
     return 1.f / z;
 }
 
+// The tables of the one-hot parts (kOnesBytes, then kUnitBytes), by the whole block; what the tensor core reads comes after a block barrier.
+__device__ __forceinline__ void fill_tables(unsigned char* to, int threads) {
+    for (uint32_t i = threadIdx.x; i < (kOnesBytes + kUnitBytes) / 4; i += threads) {
+        uint32_t v = 0;
+        if (i < kOnesBytes / 4) {
+            if (((i * 4) & 511u) >> 4 == 15) v = kOnesBf16x2;
+        } else {
+            const uint32_t b = (i * 4 - kOnesBytes) % 1280u, core = b >> 7, k = (b & 15u) >> 1;      // k, k + 1 of a row
+            if (core >= 1 && core <= 8) v = (core - 1 == k ? 0x3F80u : 0u) | (core - 1 == k + 1 ? 0x3F800000u : 0u);
+        }
+        *reinterpret_cast<uint32_t*>(to + i * 4) = v;
+    }
+    fence_proxy_async_smem();
+}
+
 template <int K>
 __global__ void __launch_bounds__(kThreads, 1)
 mma_wide_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v, const WideParams P)
@@ -265,17 +281,7 @@ mma_wide_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant
         mbar_init_fence();
     }
     for (int i = threadIdx.x; i < Wd::K2; i += kThreads) s_bias[i] = P.bias ? P.bias[h * Wd::K2 + i] * kLog2e : 0.f;
-    for (uint32_t i = threadIdx.x; i < (kOnesBytes + kUnitBytes) / 4; i += kThreads) {
-        uint32_t v = 0;
-        if (i < kOnesBytes / 4) {
-            if (((i * 4) & 511u) >> 4 == 15) v = kOnesBf16x2;
-        } else {
-            const uint32_t b = (i * 4 - kOnesBytes) % 1280u, core = b >> 7, k = (b & 15u) >> 1;      // k, k + 1 of a row
-            if (core >= 1 && core <= 8) v = (core - 1 == k ? 0x3F80u : 0u) | (core - 1 == k + 1 ? 0x3F800000u : 0u);
-        }
-        *reinterpret_cast<uint32_t*>(smem + Wd::ones_off + i * 4) = v;
-    }
-    fence_proxy_async_smem();
+    fill_tables(smem + Wd::ones_off, kThreads);
     if (warp == kMmaWarp) tmem_alloc(smem_u32(smem + Wd::tmem_off), 512);
     tc_fence_before_sync();
     __syncthreads();
@@ -547,6 +553,395 @@ mma_wide_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant
     }
 }
 
+// ---- k = 5: weights resident, one pipeline over the whole CTA -------------------------------------------------------------------
+// The arithmetic above.  As umma_ts_kernel: a warp has a whole quadrant (32 pixels), lane (g, tig) column g and channels 8 tig .. of
+// four rows, so that a halo row is read and widened once for up to four of them; the stages have warps of their own.  20 warps: two
+// sets of four value warps, which take the blocks in turn, four product, four softmax and four control warps.
+// The one-hot part of the value side takes one K step: beside e_hi (K = 25) the softmax leaves, for every tap column, the five e_hi and
+// five e_lo of its taps, which meet one table of ones for all columns.  (By a unit column per tap and part, as above, it took 70
+// instead of 30 MMAs a block.)
+// Tensor memory: a D buffer of 96 columns for the upper three taps of a tap column, two of 64 for the lower two, in turn, two of
+// products of 80 (five taps), two tiles of 64: logits in 32 columns, later e_hi in 16 and 8 for each tap column.
+//
+// Bound by energy when it runs for seconds (1000 W), else by latency: 51.5 M warp instructions at 64 x 56 x 56, 3 heads, in 48 % of the issue
+// slots, tensor pipe 42 %, value warps waiting for 60 % of the time.  In two teams of eight warps with two rows each as above 71 M.  Calls, a few
+// hundred / for seconds: 64 x 56 x 56, 3 heads 123.5 / 134.5 -> 97 / 112.6 us; 2 x 128 x 128, 3 heads 27.0 -> 24.6.  Without the
+// one step for the one-hot part 104.5 / 118.8.
+struct Five {
+    using Wd = Wide<5>;
+    static constexpr int K = 5, VSets = 2, KSlots = 2, VSlots = 4, G0 = 3, G1 = 2;
+    static constexpr int PWarp = 4 * VSets, SWarp = PWarp + 4, Ctl = SWarp + 4, Threads = (Ctl + 4) * 32;
+    static constexpr int ValueRegs = 136, ProductRegs = 104, SoftmaxRegs = 64, ControlRegs = 40;      // 480 over the five warpgroups: 96 each at the launch
+    static constexpr uint32_t ColD = 0, ColD1 = 96, OtherD1 = 96 ^ 160, ColP = 224, OtherP = 224 ^ 304, ColL = 384;       // x ^ Other: the other one of two
+    static constexpr uint32_t TapBytes = 5 * 4 * 256;             // table of ones: [tap][four groups of 8 columns][k / 8][column][8 k]
+    static constexpr uint32_t v_off = KSlots * Wd::slot, w_off = v_off + VSlots * Wd::slot, ones_off = w_off + Wd::weights, unit_off = ones_off + kOnesBytes,
+                              bias_off = unit_off + TapBytes, inv_off = bias_off + 112, bar_off = inv_off + 2 * 128 * 4;
+    // Pairs of barriers are told apart by bit 3 of their address.  DFull: [set][tap column][upper, lower]: each has one set of readers, which
+    // meets all of its phases.
+    enum : int { KFull = 0, KEmpty = KFull + KSlots, VFull = KEmpty + KSlots, VEmpty = VFull + VSlots, PReady = VEmpty + VSlots, PFree = PReady + 2,
+                 LFull = PFree + 2, EReady = LFull + 2, EFree = EReady + 2, DFree1 = EFree + 2, DFree = DFree1 + 2, Weights, DFull, Bars = DFull + VSets * K * 2 };
+    static_assert(PReady % 2 == 0, "pairs");
+    static constexpr uint32_t tmem_off = bar_off + 8 * Bars, total = tmem_off + 16 + 128;
+    static_assert(total <= kMaxSmem && VSlots % VSets == 0, "shared memory; a slot of V has one set of readers");
+};
+
+__global__ void __launch_bounds__(Five::Threads, 1)
+mma_five_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v, const WideParams P)
+{
+    using F = Five;
+    using Wd = F::Wd;
+    constexpr int K = F::K, HP = Wd::HP;
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char* smem = smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u);
+    const uint32_t bars = smem_u32(smem + F::bar_off);
+    auto bar = [&](int i) { return bars + 8u * (uint32_t)i; };
+    float* s_bias = reinterpret_cast<float*>(smem + F::bias_off);
+    float* s_inv = reinterpret_cast<float*>(smem + F::inv_off);          // [block parity][pixel]: 1 / sum of the weights
+
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
+    const int h = blockIdx.x % P.heads, rank = blockIdx.x / P.heads, nrank = (int)gridDim.x / P.heads;
+    const int blocks = (P.tiles + 1) >> 1, my_blocks = rank < blocks ? (blocks - rank + nrank - 1) / nrank : 0;
+
+    if (threadIdx.x == 0) {
+        auto init = [&](int first, int n, uint32_t count) {
+#pragma unroll 1
+            for (int i = first; i < first + n; ++i) mbar_init_only(bar(i), count);
+        };
+        init(F::KFull, F::KSlots, 1); init(F::KEmpty, F::KSlots, 4);
+        init(F::VFull, F::VSlots, 1); init(F::VEmpty, F::VSlots, 4);
+        init(F::PReady, 2, 4); init(F::PFree, 2, 1);
+        init(F::LFull, 2, 1); init(F::EReady, 2, 4); init(F::EFree, 2, 1);
+        init(F::DFree1, 3, 4); init(F::DFull, F::VSets * K * 2, 1);
+        init(F::Weights, 1, 1);
+        mbar_init_fence();
+    }
+    for (int i = threadIdx.x; i < Wd::K2; i += F::Threads) s_bias[i] = P.bias ? P.bias[h * Wd::K2 + i] * kLog2e : 0.f;
+    for (uint32_t i = threadIdx.x; i < (kOnesBytes + F::TapBytes) / 4; i += F::Threads) {
+        uint32_t v = 0;
+        if (i < kOnesBytes / 4) {
+            if (((i * 4) & 511u) >> 4 == 15) v = kOnesBf16x2;
+        } else {                                                  // k = e_hi of tap 0 .. 4, e_lo of tap 0 .. 4; 32 columns a tap
+            const uint32_t b = i * 4 - kOnesBytes, tap = b >> 10, k = (b >> 7 & 1u) * 8u + ((b & 15u) >> 1);
+            v = (k == tap || k == 5 + tap ? 0x3F80u : 0u) | (k + 1 == tap || k + 1 == 5 + tap ? 0x3F800000u : 0u);
+        }
+        *reinterpret_cast<uint32_t*>(smem + F::ones_off + i * 4) = v;
+    }
+    fence_proxy_async_smem();
+    if (warp == F::Ctl) tmem_alloc(smem_u32(smem + F::tmem_off), 512);
+    tc_fence_before_sync();
+    __syncthreads();
+    tc_fence_after_sync();
+    const uint32_t tmem = *reinterpret_cast<const volatile uint32_t*>(smem + F::tmem_off);
+    const int C = P.heads * kHeadDim, g = lane >> 2, tig = lane & 3, q = warp & 3;
+    const size_t row_pitch = (size_t)P.W * C;
+    const uint32_t lane_off = (uint32_t)(q >> 1) * Wd::plane + (uint32_t)(4 * (q & 1) * HP + g) * 64u + (uint32_t)tig * 16u;
+    // the lane's pixel in its first row, and how many of its four rows are inside (tile `i` past the last: none)
+    struct Place { size_t at; int rows; };
+    auto place = [&](const TileWalk& w, int i) {
+        Place p;
+        const int y = 8 * w.y + 4 * (q & 1), x = 8 * w.x + g;
+        p.rows = i < P.tiles && x < P.W ? P.H - y : 0;
+        p.at = (((size_t)w.b * P.H + y) * P.W + x) * C + h * kHeadDim + tig * 8;
+        return p;
+    };
+    bool ok = true;
+
+    if (warp < F::PWarp) {
+        // ---- values -----------------------------------------------------------------------------------------
+        reg_take<F::ValueRegs>();
+        const int set = warp >> 2;
+        const uint32_t tq = tmem + ((uint32_t)(32 * q) << 16);
+        TileWalk walk(P.tiles_x, P.tiles_y, 2 * (rank + set * nrank) + (q >> 1), 2 * F::VSets * nrank);
+        const uint32_t zero = (uint32_t)(P.H >> 31), ready = bar(F::EReady + set);
+        const float* inv = s_inv + 128 * set + 32 * q + g;
+        int slot = set;
+        uint32_t phase = 0, parity = 0;                            // of the slot; of the block
+#pragma unroll 1
+        for (int blk = set; blk < my_blocks; blk += F::VSets) {
+            const unsigned char* src = smem + F::v_off + (uint32_t)slot * Wd::slot + lane_off;
+            wait_or_give_up(bar(F::VFull + slot), phase, ok);
+            wait_or_give_up(ready, parity, ok);
+            float s[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) s[i] = inv[8 * i];
+            float acc[4][8];
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int c = 0; c < 8; ++c) acc[i][c] = 0.f;
+            uint32_t full = bar(F::DFull + 2 * K * set), free1 = bar(F::DFree1 + set), t1 = tq + (set ? 160u : 96u);        // buffer 5 blk + dx mod 2
+#pragma unroll 1
+            for (int dx = 0; dx < K; ++dx, src += 64, full += 16u, free1 ^= 8u, t1 ^= F::OtherD1) {
+                uint4 y[8];
+                float f[8][8];
+                auto load = [&](int r) { y[r] = *reinterpret_cast<const uint4*>(src + r * HP * 64); };
+                auto widen = [&](int r) {
+                    f[r][0] = bf16_lo(y[r].x); f[r][1] = bf16_hi(y[r].x); f[r][2] = bf16_lo(y[r].y); f[r][3] = bf16_hi(y[r].y);
+                    f[r][4] = bf16_lo(y[r].z); f[r][5] = bf16_hi(y[r].z); f[r][6] = bf16_lo(y[r].w); f[r][7] = bf16_hi(y[r].w);
+                };
+                // taps dy0 .. dy0 + G - 1 of the column, pixel rows 2m, 2m + 1: their A' from `t`
+                auto ask = [&](auto G, uint32_t t, uint32_t (&d)[3][16]) {
+#pragma unroll
+                    for (int i = 0; i < decltype(G)::value; ++i) tmem_ld_16x256b_x4_nowait(t + 32 * i, d[i]);
+                };
+                auto sum = [&](auto G, int dy0, int m, uint32_t (&d)[3][16]) {
+#pragma unroll
+                    for (int i = 0; i < decltype(G)::value; ++i) {
+                        tmem_pass(d[i]);
+#pragma unroll
+                        for (int r = 0; r < 2; ++r)
+#pragma unroll
+                            for (int j = 0; j < 4; ++j)
+                                ffma2(acc[2 * m + r][2 * j], acc[2 * m + r][2 * j + 1], __uint_as_float(d[i][4 * j + 2 * r]), __uint_as_float(d[i][4 * j + 2 * r + 1]),
+                                      f[2 * m + r + dy0 + i][2 * j], f[2 * m + r + dy0 + i][2 * j + 1]);
+                    }
+                };
+                using G0 = std::integral_constant<int, F::G0>;
+                using G1 = std::integral_constant<int, F::G1>;
+                uint32_t d[3][16];
+#pragma unroll
+                for (int r = 0; r < 6; ++r) load(r);
+                wait_or_give_up(full, parity, ok);
+                tc_fence_after_sync();
+                ask(G0(), tq, d);
+                widen(0); widen(1); widen(2); widen(3);
+                tmem_wait_ld();
+                sum(G0(), 0, 0, d);
+                ask(G0(), tq + (16u << 16), d);
+                widen(4); widen(5);
+                load(6); load(7);
+                tmem_wait_ld();
+                tc_fence_before_sync();
+                mbar_arrive_lane0(bar(F::DFree), lane);
+                sum(G0(), 0, 1, d);
+                wait_or_give_up(full + 8u, parity, ok);
+                tc_fence_after_sync();
+                ask(G1(), t1, d);
+                widen(6); widen(7);
+                tmem_wait_ld();
+                sum(G1(), 3, 0, d);
+                ask(G1(), t1 + (16u << 16), d);
+                tmem_wait_ld();
+                tc_fence_before_sync();
+                mbar_arrive_lane0(free1, lane);
+                sum(G1(), 3, 1, d);
+            }
+            // row 0 of the accumulators holds what was read last of halo rows 0 - 4, row 3 of 3 - 7
+            mbar_arrive_lane0_after(bar(F::VEmpty + slot), lane, acc[0][0], acc[3][0], zero);
+            if ((slot += F::VSets) >= F::VSlots) { slot = set; phase ^= 1u; }
+            parity ^= 1u;
+            const Place out = place(walk, 2 * (rank + blk * nrank) + (q >> 1));
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (i < out.rows)
+                    *reinterpret_cast<uint4*>(P.out + out.at + i * row_pitch) =
+                        make_uint4(pack_bf16(acc[i][0] * s[i], acc[i][1] * s[i]), pack_bf16(acc[i][2] * s[i], acc[i][3] * s[i]),
+                                   pack_bf16(acc[i][4] * s[i], acc[i][5] * s[i]), pack_bf16(acc[i][6] * s[i], acc[i][7] * s[i]));
+            walk.next();
+        }
+    } else if (warp < F::SWarp) {
+        // ---- products ---------------------------------------------------------------------------------------
+        reg_take<F::ProductRegs>();
+        uint32_t t = tmem + F::ColP + ((uint32_t)(32 * q) << 16), free = bar(F::PFree), ppar = 1, pb = 0;      // chunk 5 blk + dx: buffer, its barrier, phase
+        TileWalk walk(P.tiles_x, P.tiles_y, 2 * rank + (q >> 1), 2 * nrank);
+        uint4 x[4], xn[4];                                         // q of this block and of the next
+        auto load_q = [&](int blk) {
+            const Place p = place(walk, 2 * (rank + blk * nrank) + (q >> 1));
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                xn[i] = make_uint4(0u, 0u, 0u, 0u);
+                if (i < p.rows) xn[i] = __ldg(reinterpret_cast<const uint4*>(P.q + p.at + i * row_pitch));
+            }
+        };
+        int slot = 0;
+        uint32_t phase = 0;
+        if (my_blocks > 0) load_q(0);
+#pragma unroll 1
+        for (int blk = 0; blk < my_blocks; ++blk) {
+            const unsigned char* src = smem + (uint32_t)slot * Wd::slot + lane_off;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) x[i] = xn[i];
+            walk.next();
+            if (blk + 1 < my_blocks) load_q(blk + 1);
+            wait_or_give_up(bar(F::KFull + slot), phase, ok);
+#pragma unroll 1
+            for (int dx = 0; dx < K; ++dx, src += 64) {
+                uint4 y[8];
+#pragma unroll
+                for (int r = 0; r < 8; ++r) y[r] = *reinterpret_cast<const uint4*>(src + r * HP * 64);
+                wait_or_give_up(free, ppar, ok);
+                tc_fence_after_sync();
+#pragma unroll
+                for (int i = 0; i < K; ++i)
+#pragma unroll
+                    for (int m = 0; m < 2; ++m) {
+                        const uint4 x0 = x[2 * m], x1 = x[2 * m + 1], y0 = y[2 * m + i], y1 = y[2 * m + 1 + i];
+                        const uint32_t r[8] = {hmul2_bf16(x0.x, y0.x), hmul2_bf16(x0.y, y0.y), hmul2_bf16(x1.x, y1.x), hmul2_bf16(x1.y, y1.y),
+                                               hmul2_bf16(x0.z, y0.z), hmul2_bf16(x0.w, y0.w), hmul2_bf16(x1.z, y1.z), hmul2_bf16(x1.w, y1.w)};
+                        tmem_st_16x256b_x2(t + ((uint32_t)(16 * m) << 16) + 16 * i, r);
+                    }
+                tmem_wait_st();
+                tc_fence_before_sync();
+                mbar_arrive_lane0(free - 8u * (uint32_t)(F::PFree - F::PReady), lane);
+                t ^= F::OtherP; free ^= 8u; ppar ^= pb; pb ^= 1u;
+            }
+            mbar_arrive_lane0(bar(F::KEmpty + slot), lane);       // the products of what was read are in tensor memory
+            if (++slot == F::KSlots) { slot = 0; phase ^= 1u; }
+        }
+    } else if (warp < F::Ctl) {
+        // ---- softmax: thread = pixel ----------------------------------------------------------------------------
+        reg_give<F::SoftmaxRegs>();
+        const uint32_t tq = tmem + F::ColL + ((uint32_t)(32 * q) << 16);
+#pragma unroll 1
+        for (int blk = 0; blk < my_blocks; ++blk) {
+            const uint32_t tile = (uint32_t)blk & 1u;
+            wait_or_give_up(bar(F::LFull) + 8u * tile, (uint32_t)blk >> 1 & 1u, ok);
+            tc_fence_after_sync();
+            float l[32];
+            tmem_ld_32x32b_x32(tq + 64u * tile, l);
+            // the largest of all slots first: a running one is -inf while all slots so far are masked by a bias of -inf
+            float m = -INFINITY, z = 0.f;
+#pragma unroll
+            for (int i = 0; i < Wd::K2; ++i) { l[i] = fmaf(l[i], P.scale_log2e, s_bias[i]); m = fmaxf(m, l[i]); }
+            uint32_t hi[16], lo[13];
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+                const float e0 = 2 * i < Wd::K2 ? fast_exp2(l[2 * i] - m) : 0.f, e1 = 2 * i + 1 < Wd::K2 ? fast_exp2(l[2 * i + 1] - m) : 0.f;
+                z += e0; z += e1;
+                hi[i] = i < 13 ? pack_bf16(e0, e1) : 0u;
+                if (i < 13) lo[i] = pack_bf16(e0 - bf16_lo(hi[i]), e1 - bf16_hi(hi[i]));
+            }
+            tmem_st_32x32b_x16(tq + 64u * tile, hi);
+            // halves of two words as one
+            auto both = [&](const uint32_t (&a)[16], int i, const uint32_t (&b)[16], int j) {
+                return __byte_perm(a[i >> 1], b[j >> 1], (i & 1 ? 0x32u : 0x10u) | (j & 1 ? 0x7600u : 0x5400u));
+            };
+            uint32_t low[16];
+#pragma unroll
+            for (int i = 0; i < 16; ++i) low[i] = i < 13 ? lo[i] : 0u;
+#pragma unroll
+            for (int dx = 0; dx < K; ++dx) {
+                const uint32_t row[8] = {both(hi, dx, hi, 5 + dx), both(hi, 10 + dx, hi, 15 + dx), both(hi, 20 + dx, low, dx), both(low, 5 + dx, low, 10 + dx),
+                                         both(low, 15 + dx, low, 20 + dx), 0u, 0u, 0u};
+                tmem_st_32x32b_x8(tq + 64u * tile + 16 + 8 * dx, row);
+            }
+            tmem_wait_st();
+            s_inv[128 * tile + 32 * q + lane] = 1.f / z;
+            tc_fence_before_sync();
+            __syncwarp();
+            mbar_arrive_lane0(bar(F::EReady) + 8u * tile, lane);
+        }
+    } else {
+        reg_give<F::ControlRegs>();
+        // no copy is on its way when the block leaves, whatever its readers have given up on
+        auto drain = [&](int full, int slots, int issued) {
+#pragma unroll 1
+            for (int i = 0; i < slots && i < issued; ++i) ok = mbar_wait<true>(bar(full + i), (uint32_t)((issued - 1 - i) / slots) & 1u) && ok;
+        };
+        auto load_tiles = [&](uint32_t dst, const CUtensorMap* map, uint32_t full, const TileWalk& at) {
+            mbar_expect_tx(full, Wd::slot);
+            // the second tile may be past the last: its image does not exist and it reads as zero
+            int x = at.x + 1, y = at.y, b = at.b;
+            if (x == at.tx) { x = 0; if (++y == at.ty) { y = 0; ++b; } }
+            tma_load_4d(dst, map, full, h * kHeadDim, 8 * at.x - Wd::R, 8 * at.y - Wd::R, at.b);
+            tma_load_4d(dst + Wd::plane, map, full, h * kHeadDim, 8 * x - Wd::R, 8 * y - Wd::R, b);
+        };
+        uint32_t leader;
+        if (elect_one(leader) && my_blocks > 0) {
+            const uint32_t w = smem_u32(smem + F::w_off);
+            if (warp == F::Ctl) {
+                // ---- key MMAs -------------------------------------------------------------------------------
+                constexpr uint32_t id_l = umma_idesc_bf16(128, Wd::N), id16 = umma_idesc_bf16(128, 16);
+                // descriptors, lower halves: weights of tap (0, 0); the ones of column 15 in column 15
+                const uint64_t wd = umma_smem_desc(w, Wd::N * 16, 128), od = umma_smem_desc(smem_u32(smem + F::ones_off), 512, 128);
+                const uint32_t w_lo = (uint32_t)wd, w_hi = (uint32_t)(wd >> 32), o_lo = (uint32_t)od + 15u, o_hi = (uint32_t)(od >> 32);
+                uint32_t p = tmem + F::ColP, ready = bar(F::PReady), ppar = 0, pb = 0;
+                ok = mbar_wait<true>(bar(F::Weights), 0);
+#pragma unroll 1
+                for (int blk = 0; ok && blk < my_blocks; ++blk) {
+                    const uint32_t tile = (uint32_t)blk & 1u, l = tmem + F::ColL + 64u * tile;
+                    if (!mbar_wait<true>(bar(F::EFree) + 8u * tile, ((uint32_t)blk >> 1 & 1u) ^ 1u)) { ok = false; break; }
+#pragma unroll 1
+                    for (int dx = 0; dx < K; ++dx) {
+                        if (!mbar_wait<true>(ready, ppar)) { ok = false; break; }
+                        tc_fence_after_sync();
+#pragma unroll
+                        for (int i = 0; i < K; ++i) {
+                            const uint32_t t = (uint32_t)(i * K + dx), a = p + 16 * i;
+                            const uint32_t b = w_lo + (uint32_t)dx * (K * Wd::tap / 16) + i * (Wd::tap / 16), one = o_lo - (t & 15u), lt = l + (t & 16u);
+                            umma_bf16_ts(l, a, b, w_hi, id_l, i != 0 ? 1u : (uint32_t)dx);
+                            umma_bf16_ts(l, a + 8, b + 2 * Wd::N, w_hi, id_l, 1);                     // the other 16 channels
+                            umma_bf16_ts(lt, a, one, o_hi, id16, 1);
+                            umma_bf16_ts(lt, a + 8, one, o_hi, id16, 1);
+                        }
+                        umma_commit(ready + 8u * (uint32_t)(F::PFree - F::PReady));
+                        p ^= F::OtherP; ready ^= 8u; ppar ^= pb; pb ^= 1u;
+                    }
+                    if (ok) umma_commit(bar(F::LFull) + 8u * tile);
+                }
+            } else if (warp == F::Ctl + 1) {
+                // ---- value MMAs -----------------------------------------------------------------------------
+                const uint64_t wd = umma_smem_desc(w + (uint32_t)Wd::K2 * Wd::tap, 128, 2 * Wd::KS * 128), ud = umma_smem_desc(smem_u32(smem + F::unit_off), 128, 256);
+                const uint32_t w_lo = (uint32_t)wd, w_hi = (uint32_t)(wd >> 32), u_lo = (uint32_t)ud, u_hi = (uint32_t)(ud >> 32);
+                uint32_t d1 = tmem + F::ColD1, free1 = bar(F::DFree1), dpar = 1, dpar1 = 1, db = 0;
+                ok = mbar_wait<true>(bar(F::Weights), 0);
+#pragma unroll 1
+                for (int blk = 0; ok && blk < my_blocks; ++blk) {
+                    const uint32_t tile = (uint32_t)blk & 1u, e = tmem + F::ColL + 64u * tile;
+                    if (!mbar_wait<true>(bar(F::EReady) + 8u * tile, (uint32_t)blk >> 1 & 1u)) { ok = false; break; }
+                    uint32_t full = bar(F::DFull) + 16u * K * tile;
+#pragma unroll 1
+                    for (int dx = 0; ok && dx < K; ++dx, full += 16u) {
+#pragma unroll
+                        for (int gi = 0; gi < 2; ++gi) {
+                            const int G = gi ? F::G1 : F::G0;
+                            if (!mbar_wait<true>(gi ? free1 : bar(F::DFree), gi ? dpar1 : dpar)) { ok = false; break; }
+                            tc_fence_after_sync();
+                            const uint32_t d = gi ? d1 : tmem + F::ColD;
+                            const uint32_t b = w_lo + (uint32_t)dx * (K * Wd::tap / 16) + gi * (F::G0 * Wd::tap / 16);
+#pragma unroll
+                            for (int j = 0; j < Wd::KS; ++j) umma_bf16_ts(d, e + 8 * j, b + 16 * j, w_hi, umma_idesc_bf16(128, 32 * G), j != 0 ? 1u : 0u);
+                            umma_bf16_ts(d, e + 16 + 8u * (uint32_t)dx, u_lo + gi * (F::G0 * 64), u_hi, umma_idesc_bf16(128, 32 * G), 1);
+                            umma_commit(full + 8u * gi);
+                        }
+                        d1 ^= F::OtherD1; free1 ^= 8u; dpar ^= 1u; dpar1 ^= db; db ^= 1u;
+                    }
+                    if (ok) umma_commit(bar(F::EFree) + 8u * tile);
+                }
+            } else {
+                // ---- the head's weights and K, or V -------------------------------------------------------------
+                const bool v = warp == F::Ctl + 3;
+                if (!v) {
+                    grid_dependency_wait();
+                    mbar_expect_tx(bar(F::Weights), Wd::weights);
+                    bulk_load_1d(w, P.weights + (size_t)h * Wd::weights, Wd::weights, bar(F::Weights));
+                }
+                const int slots = v ? F::VSlots : F::KSlots, full = v ? F::VFull : F::KFull, empty = v ? F::VEmpty : F::KEmpty;
+                const uint32_t ring = smem_u32(smem) + (v ? F::v_off : 0u);
+                TileWalk at(P.tiles_x, P.tiles_y, 2 * rank, 2 * nrank);
+                int slot = 0, blk = 0;
+                uint32_t phase = 1;
+#pragma unroll 1
+                for (; blk < my_blocks; ++blk, at.next()) {
+                    if (!mbar_wait<true>(bar(empty + slot), phase)) { ok = false; break; }
+                    load_tiles(ring + (uint32_t)slot * Wd::slot, v ? &map_v : &map_k, bar(full + slot), at);
+                    if (++slot == slots) { slot = 0; phase ^= 1u; }
+                }
+                drain(full, slots, blk);
+                if (!v) ok = mbar_wait<true>(bar(F::Weights), 0) && ok;
+            }
+        }
+        __syncwarp();
+    }
+    if (!ok) atomicExch(P.status, 1);
+    tc_fence_before_sync();
+    __syncthreads();
+    if (warp == F::Ctl) {
+        tc_fence_after_sync();
+        tmem_dealloc(tmem, 512);
+    }
+}
+
 template <int K>
 cudaError_t launch_prep_t(const Problem& p, void* workspace, cudaStream_t stream) {
     return launch_chained(mma_wide_prep_kernel<K>, dim3((unsigned)((2 * Wide<K>::K2 * 4 * Wide<K>::N + 255) / 256), (unsigned)p.heads), 256, 0, stream, p.wk, p.wv,
@@ -561,7 +956,8 @@ cudaError_t launch_t(const Problem& p, const void* workspace, int* d_status, int
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev >= 64 || !configured[dev]) {
-        e = cudaFuncSetAttribute(mma_wide_kernel<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Wd::total);
+        if constexpr (K == 5) e = cudaFuncSetAttribute(mma_five_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Five::total);
+        else e = cudaFuncSetAttribute(mma_wide_kernel<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Wd::total);
         if (e != cudaSuccess) return e;
         if (dev < 64) configured[dev] = true;
     }
@@ -583,7 +979,9 @@ cudaError_t launch_t(const Problem& p, const void* workspace, int* d_status, int
     long long per_head = num_sms / p.heads;
     if (per_head > blocks) per_head = blocks;
     if (per_head < 1) per_head = 1;
-    return launch_chained(mma_wide_kernel<K>, dim3((unsigned)(per_head * p.heads)), kThreads, Wd::total, stream, mk, mv, P);
+    const dim3 grid((unsigned)(per_head * p.heads));
+    if constexpr (K == 5) return launch_chained(mma_five_kernel, grid, Five::Threads, Five::total, stream, mk, mv, P);
+    else return launch_chained(mma_wide_kernel<K>, grid, kThreads, Wd::total, stream, mk, mv, P);
 }
 
 }  // namespace

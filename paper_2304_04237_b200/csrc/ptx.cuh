@@ -39,7 +39,7 @@ __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
 // a waiting warp issues next to no instructions.  `Small`: a loop that the compiler may not unroll, in kernels of which many waits
 // would otherwise fill the instruction cache (41 instead of 63 KB of one of them); elsewhere it costs up to 3 %.
 template <bool Small = false>
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
+__device__ __forceinline__ bool mbar_park(uint32_t bar, uint32_t parity) {
     auto probe = [&]() {
         uint32_t done;
         asm volatile(
@@ -49,15 +49,6 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
             : "=r"(done) : "r"(bar), "r"(parity), "r"(100000u) : "memory");
         return done != 0;
     };
-    {   // a phase that is already complete costs about 30 cycles less without the time hint
-        uint32_t done;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(done) : "r"(bar), "r"(parity) : "memory");
-        if (done) return true;
-    }
     if constexpr (Small) {
 #pragma unroll 1
         for (int spin = 0; spin < 20000; ++spin)
@@ -67,6 +58,18 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
             if (probe()) return true;
     }
     return false;
+}
+// The same behind a probe without the time hint: a phase that is already complete then costs about 30 cycles less.
+template <bool Small = false>
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
+    uint32_t done;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(done) : "r"(bar), "r"(parity) : "memory");
+    if (done) return true;
+    return mbar_park<Small>(bar, parity);
 }
 
 // A wait of a whole warp without a vote: a lane whose wait runs out carries on with `ok` cleared and waits no more, so that the
@@ -79,11 +82,12 @@ __device__ __forceinline__ void wait_or_give_up(uint32_t bar, uint32_t parity, b
         "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
         "selp.u32 %0, 1, 0, p;\n\t}"
         : "=r"(done) : "r"(bar), "r"(parity) : "memory");
-    if (!done && ok) ok = mbar_wait<true>(bar, parity);
+    if (!done && ok) ok = mbar_park<true>(bar, parity);
     __syncwarp();
 }
 
-// Moves registers between the warpgroups of a block (all four warps of one execute it).
+// Moves registers between the warpgroups of a block (all four warps of one execute it): to N a thread from fewer (take) or more
+// (give) at the launch; the other way round is an illegal instruction.
 template <int N> __device__ __forceinline__ void reg_take() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
 template <int N> __device__ __forceinline__ void reg_give() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
 
@@ -273,6 +277,16 @@ __device__ __forceinline__ void umma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, u
         "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
         ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
 }
+// The same with the descriptor in halves.  Only its lower one differs from instruction to instruction, and 32-bit arithmetic on that
+// takes the issuing thread half the instructions.
+__device__ __forceinline__ void umma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t b_hi, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b64 b;\n\t"
+        "setp.ne.b32 p, %5, 0;\n\t"
+        "mov.b64 b, {%2, %3};\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], b, %4, p;\n\t}"
+        ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate) : "memory");
+}
 // registers -> 16 TMEM lanes x 16 columns, fragment layout of tcgen05.ld.16x256b
 __device__ __forceinline__ void tmem_st_16x256b_x2(uint32_t taddr, const uint32_t (&r)[8]) {
     // no memory clobber: shared-memory loads of the next chunk may be scheduled across the store
@@ -284,6 +298,10 @@ __device__ __forceinline__ void tmem_st_32x32b_x16(uint32_t taddr, const uint32_
     asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};"
                  ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
                    "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]) : "memory");
+}
+__device__ __forceinline__ void tmem_st_32x32b_x8(uint32_t taddr, const uint32_t (&r)[8]) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
+                 ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]) : "memory");
 }
 __device__ __forceinline__ void tmem_wait_st() {
     asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");

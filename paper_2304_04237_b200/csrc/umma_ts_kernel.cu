@@ -416,6 +416,7 @@ umma_ts_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
             if (warp == kCtlK) {
                 // ---- key MMAs: 18 per block (9 taps x two K = 16 halves) --------------------------------
                 const uint64_t desc = umma_smem_desc(smem_u32(smem + kBkOff), 512, 128);
+                const uint32_t b_lo = (uint32_t)desc, b_hi = (uint32_t)(desc >> 32);
                 uint32_t full = bar(kBarLFull), parity = 0, dcol = tmem + kColL;
                 int set = 0;
                 ok = mbar_wait<true>(bar(kBarWeights), 0);
@@ -430,7 +431,7 @@ umma_ts_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
                         for (int dy = 0; dy < 3; ++dy)
 #pragma unroll
                             for (int kh = 0; kh < 2; ++kh)          // 16 bytes of descriptor address = 1 unit
-                                umma_bf16_ts(dcol, tmem + kColP + 48 * dx + 16 * dy + 8 * kh, desc + (uint64_t)((dx * 4 + dy * 12 + kh * 2) * 32),
+                                umma_bf16_ts(dcol, tmem + kColP + 48 * dx + 16 * dy + 8 * kh, b_lo + (dx * 4 + dy * 12 + kh * 2) * 32, b_hi,
                                              kIdesc32, (dx != 0 || dy != 0 || kh != 0) ? 1u : 0u);
                         umma_commit(bar(kBarPFree + dx) + 24u * (uint32_t)set);
                         if (dx == 2) umma_commit(full);
@@ -442,6 +443,7 @@ umma_ts_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
             } else if (warp == kCtlV) {
                 // ---- value MMAs -------------------------------------------------------------------------
                 const uint64_t desc = umma_smem_desc(smem_u32(smem + kBOff), 128, 512);
+                const uint32_t b_lo = (uint32_t)desc, b_hi = (uint32_t)(desc >> 32);
                 uint32_t done = bar(kBarDFull);
                 ok = mbar_wait<true>(bar(kBarWeights), 0);
 #pragma unroll 1
@@ -452,8 +454,8 @@ umma_ts_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
                         if (!mbar_wait<true>(bar(kBarDFree + dx), ((uint32_t)blk & 1u) ^ 1u)) { ok = false; break; }
                         tc_fence_after_sync();
                         const uint32_t dcol = tmem + kColD + 96u * dx;
-                        umma_bf16_ts(dcol, tmem + kColE, desc + (uint64_t)(dx * 12 * 32), kIdesc96, 0);
-                        umma_bf16_ts(dcol, tmem + kColE + 8, desc + (uint64_t)(dx * 12 * 32 + 16), kIdesc96, 1);
+                        umma_bf16_ts(dcol, tmem + kColE, b_lo + dx * 12 * 32, b_hi, kIdesc96, 0);
+                        umma_bf16_ts(dcol, tmem + kColE + 8, b_lo + dx * 12 * 32 + 16, b_hi, kIdesc96, 1);
                         umma_commit(done + 8u * dx);
                         if (dx == 2) umma_commit(bar(kBarEFree));
                     }

@@ -29,6 +29,15 @@ def test_wide_variant_matches_oracle(shape, k):
     assert np.array_equal(a, b)
 
 
+def test_k5_kernel_with_many_blocks_matches_oracle():
+    """Nine blocks per CTA, more than any of its rings has slots, an odd last tile, edges in both directions."""
+    x = synth.make_inputs(3, 45, 51, 19, 32, 5, "bf16", 0.05, 0.3, False, seed=55)
+    ref = oracle.forward(x["q"], x["k"], x["v"], x["wk"], x["wv"], x["bias"], 5)
+    a, b = (gpu_forward(x, 5, "bf16", sa.VARIANT_MMA_WIDE) for _ in range(2))
+    assert_close(a, ref, "bf16")
+    assert np.array_equal(a, b)
+
+
 def as_documented(x, k):
     """The kernel's arithmetic in 64 bits, rounded where it rounds: products q k, what the weights differ from the one-hot kernels by,
     and on the value side's learned part exp(logit - largest) are bf16; the result is rounded once."""
