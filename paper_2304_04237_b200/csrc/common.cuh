@@ -88,10 +88,11 @@ size_t umma_ts_workspace_bytes(int heads);
 cudaError_t launch_umma_ts_prep(const Problem& p, void* workspace, cudaStream_t stream);
 cudaError_t launch_umma_ts(const Problem& p, const void* workspace, int* d_status, int num_sms, cudaStream_t stream);
 
-// UMMA_SPLIT variant: fp32 arithmetic on tcgen05 through exact splits (k = 3, head_dim 16, 32 or 64, both dtypes); a prep
-// launch writes the weight images of every head to `workspace`.
+// UMMA_SPLIT variant: fp32 arithmetic on tcgen05 through exact splits (k = 3, head_dim 16, 32 or 64, both dtypes).  `workspace` as
+// for UMMA_TS.
 bool umma_split_supports(int head_dim, int ksize);
 size_t umma_split_workspace_bytes(int heads, int head_dim);
+bool umma_split_builds_images(int B, int H, int W, int heads, int num_sms);      // null is the better workspace
 cudaError_t launch_umma_split_prep(const Problem& p, void* workspace, cudaStream_t stream);
 cudaError_t launch_umma_split(const Problem& p, const void* workspace, int* d_status, int num_sms, cudaStream_t stream);
 

@@ -97,6 +97,7 @@ slide_attn_status launch_problem(slide_attn_ctx* c, const Problem& p, cudaStream
         cudaEventRecord(ev[0], stream);
     }
     cudaError_t err;
+    bool prep;
     if (c->fixed_shift) {
         err = launch_shift_check(p, c->d_status, stream);
         if (ev) cudaEventRecord(ev[1], stream);
@@ -131,9 +132,10 @@ slide_attn_status launch_problem(slide_attn_ctx* c, const Problem& p, cudaStream
             if (err == cudaSuccess) err = launch_mma_wide(p, c->wide_ws, c->d_status, c->num_sms, stream);
             break;
         case SLIDE_ATTN_VARIANT_UMMA_SPLIT:
-            err = launch_umma_split_prep(p, c->split_ws, stream);
+            prep = ev || !umma_split_builds_images(p.B, p.H, p.W, p.heads, c->num_sms);
+            err = prep ? launch_umma_split_prep(p, c->split_ws, stream) : cudaSuccess;
             if (ev) cudaEventRecord(ev[1], stream);
-            if (err == cudaSuccess) err = launch_umma_split(p, c->split_ws, c->d_status, c->num_sms, stream);
+            if (err == cudaSuccess) err = launch_umma_split(p, prep ? c->split_ws : nullptr, c->d_status, c->num_sms, stream);
             break;
         case SLIDE_ATTN_VARIANT_TILE:
             err = launch_strip_prep(p, c->strip_ws, stream);
@@ -523,7 +525,8 @@ slide_attn_status slide_attn_launches_per_forward(const slide_attn_ctx* c, int* 
         case SLIDE_ATTN_VARIANT_UMMA_TS: *n = 1; break;  // fused kernel, weight layout included
         case SLIDE_ATTN_VARIANT_TILE: *n = 2; break;     // weight transpose + fused kernel
         case SLIDE_ATTN_VARIANT_MMA_WIDE: *n = 2; break; // weight images + fused kernel
-        case SLIDE_ATTN_VARIANT_UMMA_SPLIT: *n = 2; break; // weight images + fused kernel
+        case SLIDE_ATTN_VARIANT_UMMA_SPLIT: // weight images, unless the fused kernel lays them out, + fused kernel
+            *n = umma_split_builds_images(c->B, c->H, c->W, c->heads, c->num_sms) ? 1 : 2; break;
         default: *n = 1; break;
     }
     return SLIDE_ATTN_OK;

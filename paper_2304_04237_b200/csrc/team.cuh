@@ -145,6 +145,30 @@ __device__ __forceinline__ void build_contract_item(const float (&w)[8], unsigne
         make_uint4(split::pack_upper(v[0], v[1]), split::pack_upper(v[2], v[3]), split::pack_upper(v[4], v[5]), split::pack_upper(v[6], v[7]));
 }
 
+// The same by slot: 8 k of one slot (of 16, nine used) for all three column groups, for few threads with many items.
+__host__ __device__ constexpr int contract_slots(int head_dim) { return head_dim / 8 * kK2 * 16; }
+template <typename T>
+__device__ __forceinline__ void build_contract_slot(const float* w, unsigned char* img, int item, float most) {
+    const int s = item & 15, kg = item >> 4;
+    float x[8], v[3][8];
+    load_contract_item<T>(w, kg * 48 + s, x);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+        if (sizeof(T) == 4 && !wide(most)) {
+            const float r = rounder(most), hi = __fadd_rn(__fadd_rn(x[e], r), -r), rest = x[e] - hi, mid = __bfloat162float(__float2bfloat16_rn(rest));
+            v[0][e] = hi; v[1][e] = mid; v[2][e] = __bfloat162float(__float2bfloat16_rn(rest - mid));
+        } else {
+            v[0][e] = x[e]; v[1][e] = split::rest(x[e]); v[2][e] = split::rest(v[1][e]);
+        }
+    }
+#pragma unroll
+    for (int part = 0; part < 3; ++part) {
+        const float (&p)[8] = v[part];
+        *reinterpret_cast<uint4*>(img + kg * 768 + part * 256 + (s >> 3) * 128 + (s & 7) * 16) =
+            make_uint4(split::pack_upper(p[0], p[1]), split::pack_upper(p[2], p[3]), split::pack_upper(p[4], p[5]), split::pack_upper(p[6], p[7]));
+    }
+}
+
 // ---- the expansion's operands ----------------------------------------------------------------------------------------------
 // Slot values (softmax weights, gradients) and weights have three bf16 parts each, so their magnitude does not matter.  (With
 // two fp16 parts each, scaled to that type's range, a forward took half the MMAs and was not faster (2 x 128 x 128, 3 heads, fp32: 29.1 us,

@@ -14,7 +14,7 @@
 // Bound by latency: the chain products -> MMA -> softmax -> split rows -> MMA -> sum and its hand-offs, with four compute warps per
 // scheduler to cover it.  Issue slots 30 - 36 % busy at 1.8 GHz, tensor pipe 13 - 24 %, DRAM 14 - 18 %.  A call, before (the CUDA-core kernel that
 // took the shape) and here: 2 x 128 x 128, 3 heads, fp32: 45.2 us in tile_kernel, 28.9; 32 x 28 x 28, 3 heads of 64, bf16: 232 us in
-// strip_kernel, 23.7; 1 x 14 x 14, 1 head, fp32: 14.4 and 8.5 us; heads of 16 (an earlier form of this kernel against strip_kernel): 16 x 56 x 56
+// strip_kernel, 23.7; 1 x 14 x 14, 1 head, fp32: 14.4 and 7.5 us; heads of 16 (an earlier form of this kernel against strip_kernel): 16 x 56 x 56
 // x 3, bf16 197 and 16.1, fp32 184 and 22.7 us.
 #include "team.cuh"
 
@@ -29,17 +29,22 @@ struct Fwd {
     static constexpr int planes = D / Cut<T>::channels;
     static constexpr int chunks = 3 * planes;                                    // product chunks, and D chunks, of a block
     static constexpr uint32_t image = contract_bytes(D) + expand_bytes(D);      // of a head, in shared memory and in the workspace
-    static constexpr uint32_t misc = 8u * (kTeams * kTeamBars + 1) + 16;
+    static constexpr uint32_t misc = 8u * (kTeams * kTeamBars + 2) + 16;
     static constexpr int fit = (int)((227u * 1024u - image - misc - 128) / (kTeams * kSlot));
     static constexpr int ring = fit < kMaxRing ? fit : kMaxRing;                 // slots of a team
     static_assert(ring >= 2, "the ring does not fit");
+    // fp32 weights of a head, either side: they wait in the last slots of a team's ring, which the team does not need before
+    static constexpr uint32_t raw = (uint32_t)D * kK2 * kK2 * 4;
+    static constexpr int raw_slots = (int)((raw + kSlot - 1) / kSlot);
+    static_assert(raw_slots < ring, "fp32 weights");
+    static constexpr uint32_t raw_off = (uint32_t)((ring - raw_slots) * kSlot), raw_off_v = raw_off + (uint32_t)(ring * kSlot);
     static constexpr uint32_t w_off = (uint32_t)(kTeams * ring * kSlot);
     static constexpr uint32_t bar_off = w_off + ((image + 15u) & ~15u);
     static constexpr uint32_t total = bar_off + misc + 128;
 };
 
 struct SplitParams {
-    const unsigned char* img;        // [head] contraction image of wk, expansion image of wv
+    const unsigned char* img;        // [head] contraction image of wk, expansion image of wv; null: built here
     const void* q;
     const float* bias;
     void* out;
@@ -47,6 +52,8 @@ struct SplitParams {
     int H, W, heads;
     Strips strips;
     float scale_log2e;
+    const float* wk;
+    const float* wv;
 };
 
 template <typename T, int D>
@@ -60,7 +67,9 @@ umma_split_prep_kernel(const float* __restrict__ wk, const float* __restrict__ w
     build_images<T>(wk + w, dst, wv + w, dst + contract_bytes(D), D, blockIdx.y);
 }
 
-template <typename T, int D>
+// Build: the CTAs lay out their head's weights themselves (see umma_split_builds_images; a kernel of its own, because the code for it costs
+// others 5 % of a call, 2 x 128 x 128, 3 heads, fp32 28.6 us -> 30.0).
+template <typename T, int D, bool Build>
 __global__ void __launch_bounds__(kThreads, 1)
 umma_split_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v, const SplitParams P)
 {
@@ -71,7 +80,9 @@ umma_split_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
     unsigned char* smem = smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u);
     const uint32_t bars = smem_u32(smem + F::bar_off);
     const uint32_t bar_weights = bars + 8u * (kTeams * kTeamBars);
-    unsigned char* tmem_slot = smem + F::bar_off + 8u * (kTeams * kTeamBars + 1);
+    const uint32_t bar_raw = bar_weights + 8u;
+    unsigned char* tmem_slot = smem + F::bar_off + 8u * (kTeams * kTeamBars + 2);
+    uint32_t* s_most = reinterpret_cast<uint32_t*>(tmem_slot + 8);
 
     const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     const int h = blockIdx.x % P.heads, rank = blockIdx.x / P.heads, nrank = (int)gridDim.x / P.heads;
@@ -84,7 +95,9 @@ umma_split_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < kTeams; ++i) init_team_bars(bars + 8u * (uint32_t)(i * kTeamBars));
-        mbar_init_only(bar_weights, 1);
+        mbar_init_only(bar_weights, Build ? kComputeWarps : 1);
+        mbar_init_only(bar_raw, 1);
+        *s_most = 0u;
         mbar_init_fence();
     }
     if (warp == kMmaWarp) tmem_alloc(smem_u32(tmem_slot), 512);
@@ -99,11 +112,13 @@ umma_split_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
         // ---- TMA thread of a team: the K planes, then the V planes of every block -------------------------
         uint32_t leader;
         if (elect_one(leader)) {
-            int slot = 0;
+            int slot = 0, loads = 0;
             uint32_t phase = 1;                                      // a fresh barrier is free
             StripWalk at(P.strips, 4LL * first, 4LL * step);
+            if (Build) grid_dependency_wait();                       // else the prep kernel has waited before it let this one start
             for (int bi = 0; ok && bi < my_blocks; ++bi, at.next()) {
                 for (int v = 0; v < 2 * NPL; ++v) {
+                    if (Build && loads++ == R - F::raw_slots && !mbar_wait(bar_weights, 0)) { ok = false; break; }       // the fp32 weights make room
                     if (!mbar_wait(bar(kEmpty + slot), phase)) { ok = false; break; }
                     const CUtensorMap* map = v < NPL ? &map_k : &map_v;
                     const int c0 = h * D + (v < NPL ? v : v - NPL) * CH;
@@ -111,6 +126,8 @@ umma_split_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
                     if (++slot == R) { slot = 0; phase ^= 1u; }
                 }
             }
+            // What follows in the stream may be launched: as blocks leave, it takes their place and sets itself up.
+            if (Build && team_id == 0) grid_launch_dependents();
             if (!ok) atomicExch(P.status, 1);
         }
         __syncwarp();
@@ -118,10 +135,17 @@ umma_split_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
         // ---- MMA thread of a team -------------------------------------------------------------------
         uint32_t leader;
         if (elect_one(leader)) {
-            if (warp == kMmaWarp) {                                  // the prep kernel's images, once per CTA
+            if (warp == kMmaWarp) {                                  // the head's weights, once per CTA
                 grid_dependency_wait();
-                mbar_expect_tx(bar_weights, F::image);
-                bulk_load_1d(smem_u32(smem + F::w_off), P.img + (size_t)h * F::image, F::image, bar_weights);
+                if constexpr (!Build) {
+                    mbar_expect_tx(bar_weights, F::image);
+                    bulk_load_1d(smem_u32(smem + F::w_off), P.img + (size_t)h * F::image, F::image, bar_weights);
+                } else {
+                    constexpr size_t floats = F::raw / 4;
+                    mbar_expect_tx(bar_raw, 2 * F::raw);
+                    bulk_load_1d(smem_u32(smem + F::raw_off), P.wk + h * floats, F::raw, bar_raw);
+                    bulk_load_1d(smem_u32(smem + F::raw_off_v), P.wv + h * floats, F::raw, bar_raw);
+                }
             }
             if (my_blocks > 0) ok = mbar_wait(bar_weights, 0);
             const uint64_t kdesc = contract_desc(smem_u32(smem + F::w_off));
@@ -156,6 +180,32 @@ umma_split_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
         const int w = warp % kTeamWarps, wq = w & 3, half = w >> 2, g = lane >> 2, tig = lane & 3;
         const uint32_t quad = tmem + ((uint32_t)(32 * wq) << 16), mine = quad + ((uint32_t)(16 * half) << 16);
         const int C = P.heads * D;
+        if constexpr (Build) {                                       // the head's images, by the compute warps of both teams
+            grid_dependency_wait();
+            ok = warp_wait(bar_raw, 0);
+            const float* raw = reinterpret_cast<const float*>(smem + F::raw_off);
+            const float* raw_v = reinterpret_cast<const float*>(smem + F::raw_off_v);
+            float most = 0.f;
+            if constexpr (sizeof(T) == 4) {
+                uint32_t m = 0;
+                for (int i = threadIdx.x; i < (int)F::raw / 16; i += kComputeWarps * 32) {
+                    const uint4 v = reinterpret_cast<const uint4*>(raw)[i];
+                    m = max(max(m, max(v.x & 0x7fffffffu, v.y & 0x7fffffffu)), max(v.z & 0x7fffffffu, v.w & 0x7fffffffu));
+                }
+                m = __reduce_max_sync(0xffffffffu, m);
+                if (lane == 0) atomicMax(s_most, m);
+                asm volatile("bar.sync 1, %0;" ::"n"(kComputeWarps * 32) : "memory");
+                most = __uint_as_float(*reinterpret_cast<volatile uint32_t*>(s_most));
+            }
+            unsigned char* img = smem + F::w_off;
+            for (int i = threadIdx.x; i < contract_slots(D); i += kComputeWarps * 32) build_contract_slot<T>(raw, img, i, most);
+            // from the other end, so that a thread has as few items of both kinds as can be
+            for (int i = kComputeWarps * 32 - 1 - (int)threadIdx.x; i < D * kK2; i += kComputeWarps * 32)
+                build_expand_item<T>(raw_v, img + contract_bytes(D), i);
+            fence_proxy_async_smem();                                // the tensor core reads these bytes through the async proxy
+            __syncwarp();
+            mbar_arrive_lane0(bar_weights, lane);
+        }
         float bias[kK2];
 #pragma unroll
         for (int s = 0; s < kK2; ++s) bias[s] = P.bias ? P.bias[h * kK2 + s] * kLog2e : 0.f;
@@ -299,12 +349,13 @@ cudaError_t launch_t(const Problem& p, const void* workspace, int* d_status, int
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev >= 64 || !configured[dev]) {
-        e = cudaFuncSetAttribute(umma_split_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F::total);
+        e = cudaFuncSetAttribute(umma_split_kernel<T, D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F::total);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(umma_split_kernel<T, D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F::total);
         if (e != cudaSuccess) return e;
         if (dev < 64) configured[dev] = true;
     }
     SplitParams P;
-    P.img = static_cast<const unsigned char*>(workspace); P.q = p.q; P.bias = p.bias; P.out = p.out; P.status = d_status;
+    P.wk = p.wk; P.wv = p.wv; P.img = static_cast<const unsigned char*>(workspace); P.q = p.q; P.bias = p.bias; P.out = p.out; P.status = d_status;
     P.H = p.H; P.W = p.W; P.heads = p.heads;
     P.strips.sx = (p.W + 7) / 8; P.strips.bands = (p.H + 3) / 4;
     P.strips.total = (long long)p.B * P.strips.bands * P.strips.sx;
@@ -319,7 +370,7 @@ cudaError_t launch_t(const Problem& p, const void* workspace, int* d_status, int
     long long per_head = num_sms / p.heads;
     if (per_head > blocks) per_head = blocks;
     if (per_head < 1) per_head = 1;
-    return launch_chained(umma_split_kernel<T, D>, dim3((unsigned)(per_head * p.heads)), kThreads, F::total, stream, mk, mv, P);
+    return launch_chained(P.img ? umma_split_kernel<T, D, false> : umma_split_kernel<T, D, true>, dim3((unsigned)(per_head * p.heads)), kThreads, F::total, stream, mk, mv, P);
 }
 
 template <typename T, int D> struct Heads { using type = T; static constexpr int dim = D; };
@@ -339,6 +390,15 @@ bool umma_split_supports(int head_dim, int ksize) {
 
 size_t umma_split_workspace_bytes(int heads, int head_dim) {
     return (size_t)heads * (contract_bytes(head_dim) + expand_bytes(head_dim));
+}
+
+// Whether the CTAs of the main launch lay out their head's weights themselves: where no team has more than one block.  Beside a prep
+// launch a team starts on its first block 1 us earlier, as its warps are free for that, but the launch itself takes 2 us of a small call
+// (1 x 14 x 14, 1 head, fp32 8.5 us with it, 7.5 without; 4 x 28 x 28, 3 heads of 16, bf16 7.2 and 5.1; 2 x 128 x 128, 3 heads, fp32, three
+// blocks, 28.6 and 29.0; 32 x 28 x 28, 3 heads of 64, bf16, three blocks, 23.6 and 24.2).
+bool umma_split_builds_images(int B, int H, int W, int heads, int num_sms) {
+    const long long blocks = ((long long)B * ((H + 3) / 4) * ((W + 7) / 8) + 3) / 4, per_head = num_sms / heads;
+    return blocks <= kTeams * (per_head < 1 ? 1 : per_head);
 }
 
 // Weights -> images in `workspace`.

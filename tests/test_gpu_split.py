@@ -13,7 +13,7 @@ import oracle
 import paper_2304_04237_b200 as sa
 from paper_2304_04237_b200 import synth
 
-from util import gpu_forward
+from util import gpu_forward, to_device
 
 pytestmark = pytest.mark.gpu
 
@@ -37,6 +37,30 @@ def test_split_variant_matches_oracle(shape, d, dtype):
         got = gpu_forward(x, 3, dtype, sa.VARIANT_UMMA_SPLIT)
         err = np.abs(got - ref) / np.maximum(1.0, np.abs(ref))
         assert np.isfinite(got).all() and err.max() <= TIGHT[dtype], (sigma_w, float(err.max()))
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("d", [16, 32, 64])
+@pytest.mark.parametrize("launches,shape", [(1, (1, 9, 10, 2)), (1, (7, 33, 40, 1)), (2, (18, 31, 40, 3))], ids=["part", "one", "more"])
+def test_split_variant_weights_laid_out_by_either_kernel(launches, shape, d, dtype):
+    """At most one block per team: the fused kernel lays the weights out, whatever else is in their place later; more: a launch in front
+    does, as it does under kernel timing.  Both write the same bytes."""
+    x = inputs(shape, d, dtype, 0.05)
+    dev = to_device(x, dtype)
+    outs = [torch.full_like(dev["q"], float("nan")) for _ in range(2)]
+    ctx = sa.slide_attn_create(*shape, d, 3, dev["q"].dtype, True)
+    try:
+        sa.slide_attn_set_variant(ctx, sa.VARIANT_UMMA_SPLIT)
+        assert sa.slide_attn_launches_per_forward(ctx) == launches
+        for i, out in enumerate(outs):
+            if i:
+                sa.slide_attn_profile_begin(ctx)
+            sa.slide_attn_forward(ctx, dev["q"], dev["k"], dev["v"], dev["wk"], dev["wv"], dev["bias"], out)
+        assert sa.slide_attn_profile_end(ctx)[2] == 1
+        assert sa.slide_attn_query_status(ctx) == sa.OK
+    finally:
+        sa.slide_attn_destroy(ctx)
+    assert torch.equal(*outs) and bool(torch.isfinite(outs[0]).all())
 
 
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
