@@ -571,7 +571,8 @@ struct Five {
     using Wd = Wide<5>;
     static constexpr int K = 5, VSets = 2, KSlots = 2, VSlots = 4, G0 = 3, G1 = 2;
     static constexpr int PWarp = 4 * VSets, SWarp = PWarp + 4, Ctl = SWarp + 4, Threads = (Ctl + 4) * 32;
-    static constexpr int ValueRegs = 136, ProductRegs = 104, SoftmaxRegs = 64, ControlRegs = 40;      // 480 over the five warpgroups: 96 each at the launch
+    static constexpr int LaunchRegs = 96, ValueRegs = 136, ProductRegs = 104, SoftmaxRegs = 64, ControlRegs = 40;      // a thread: at the launch, then
+    static_assert(VSets * ValueRegs + ProductRegs + SoftmaxRegs + ControlRegs <= Threads / 128 * LaunchRegs, "registers");
     static constexpr uint32_t ColD = 0, ColD1 = 96, OtherD1 = 96 ^ 160, ColP = 224, OtherP = 224 ^ 304, ColL = 384;       // x ^ Other: the other one of two
     static constexpr uint32_t TapBytes = 5 * 4 * 256;             // table of ones: [tap][four groups of 8 columns][k / 8][column][8 k]
     static constexpr uint32_t v_off = KSlots * Wd::slot, w_off = v_off + VSlots * Wd::slot, ones_off = w_off + Wd::weights, unit_off = ones_off + kOnesBytes,
@@ -648,7 +649,7 @@ mma_five_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant
 
     if (warp < F::PWarp) {
         // ---- values -----------------------------------------------------------------------------------------
-        reg_take<F::ValueRegs>();
+        reg_share<F::ValueRegs, F::LaunchRegs>();
         const int set = warp >> 2;
         const uint32_t tq = tmem + ((uint32_t)(32 * q) << 16);
         TileWalk walk(P.tiles_x, P.tiles_y, 2 * (rank + set * nrank) + (q >> 1), 2 * F::VSets * nrank);
@@ -741,7 +742,7 @@ mma_five_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant
         }
     } else if (warp < F::SWarp) {
         // ---- products ---------------------------------------------------------------------------------------
-        reg_take<F::ProductRegs>();
+        reg_share<F::ProductRegs, F::LaunchRegs>();
         uint32_t t = tmem + F::ColP + ((uint32_t)(32 * q) << 16), free = bar(F::PFree), ppar = 1, pb = 0;      // chunk 5 blk + dx: buffer, its barrier, phase
         TileWalk walk(P.tiles_x, P.tiles_y, 2 * rank + (q >> 1), 2 * nrank);
         uint4 x[4], xn[4];                                         // q of this block and of the next
@@ -790,7 +791,7 @@ mma_five_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant
         }
     } else if (warp < F::Ctl) {
         // ---- softmax: thread = pixel ----------------------------------------------------------------------------
-        reg_give<F::SoftmaxRegs>();
+        reg_share<F::SoftmaxRegs, F::LaunchRegs>();
         const uint32_t tq = tmem + F::ColL + ((uint32_t)(32 * q) << 16);
 #pragma unroll 1
         for (int blk = 0; blk < my_blocks; ++blk) {
@@ -832,7 +833,7 @@ mma_five_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant
             mbar_arrive_lane0(bar(F::EReady) + 8u * tile, lane);
         }
     } else {
-        reg_give<F::ControlRegs>();
+        reg_share<F::ControlRegs, F::LaunchRegs>();
         // no copy is on its way when the block leaves, whatever its readers have given up on
         auto drain = [&](int full, int slots, int issued) {
 #pragma unroll 1

@@ -86,10 +86,13 @@ __device__ __forceinline__ void wait_or_give_up(uint32_t bar, uint32_t parity, b
     __syncwarp();
 }
 
-// Moves registers between the warpgroups of a block (all four warps of one execute it): to N a thread from fewer (take) or more
-// (give) at the launch; the other way round is an illegal instruction.
-template <int N> __device__ __forceinline__ void reg_take() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
-template <int N> __device__ __forceinline__ void reg_give() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
+// Moves registers between the warpgroups of a block (all four warps of one execute it): to N a thread from Launch.  (An increase to
+// fewer, or a decrease to more, is an illegal instruction; increases wait for the others' decreases, so the sum may not exceed the launch's.)
+template <int N, int Launch> __device__ __forceinline__ void reg_share() {
+    static_assert(N % 8 == 0 && N >= 24 && N <= 256, "registers");
+    if constexpr (N > Launch) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N));
+    else if constexpr (N < Launch) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N));
+}
 
 // One arrival by lane 0 of a converged warp, without a branch.
 __device__ __forceinline__ void mbar_arrive_lane0(uint32_t bar, int lane) {

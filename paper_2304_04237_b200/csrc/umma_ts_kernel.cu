@@ -48,7 +48,8 @@ constexpr int kHeadDim = 32;
 constexpr int kVSets = 2, kPSets = 2;                    // of four value warps, of four product warps: they take the blocks in turn
 constexpr int kPWarp0 = 4 * kVSets, kSWarp0 = kPWarp0 + 4 * kPSets, kCtlK = kSWarp0 + 4, kCtlV = kCtlK + 1, kCtlTK = kCtlK + 2, kCtlTV = kCtlK + 3;
 constexpr int kThreads = (kCtlTV + 1) * 32;
-constexpr int kValueRegs = 128, kProductRegs = 64, kSoftmaxRegs = 56, kControlRegs = 40;      // 480 over the six warpgroups: 80 each at the launch
+constexpr int kLaunchRegs = 80, kValueRegs = 128, kProductRegs = 64, kSoftmaxRegs = 56, kControlRegs = 40;      // a thread: at the launch, then
+static_assert(kVSets * kValueRegs + kPSets * kProductRegs + kSoftmaxRegs + kControlRegs <= kThreads / 128 * kLaunchRegs, "registers");
 constexpr int kKSlots = 4, kVSlots = 6;
 constexpr uint32_t kQStrip = 4 * 8 * 64;                // bytes of a strip of q
 constexpr uint32_t kKSlot = kSlot + 4 * kQStrip;        // K with its halo, then q, of a block
@@ -227,7 +228,7 @@ umma_ts_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
         // =====================================================================================
         // value warps: set s takes blocks s, s + sets, ..; warp q of it strip q of the block
         // =====================================================================================
-        reg_take<kValueRegs>();
+        reg_share<kValueRegs, kLaunchRegs>();
         build_images(warp);
         const int q = warp & 3, set = warp >> 2, g = lane >> 2, tig = lane & 3;
         const uint32_t tq = tmem + kColD + ((uint32_t)(32 * q) << 16);
@@ -307,7 +308,7 @@ umma_ts_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
         // =====================================================================================
         // product warps: as the value warps
         // =====================================================================================
-        reg_give<kProductRegs>();
+        reg_share<kProductRegs, kLaunchRegs>();
         const int q = warp & 3, set = (warp - kPWarp0) >> 2, g = lane >> 2, tig = lane & 3;
         const uint32_t tq = tmem + kColP + ((uint32_t)(32 * q) << 16);
         const unsigned char* ring = smem + (uint32_t)g * 64u + (uint32_t)tig * 16u;
@@ -354,7 +355,7 @@ umma_ts_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
         // =====================================================================================
         // softmax warps: thread = pixel = TMEM lane 32 q + lane, every block
         // =====================================================================================
-        reg_give<kSoftmaxRegs>();
+        reg_share<kSoftmaxRegs, kLaunchRegs>();
         build_images(4 * kVSets + warp - kSWarp0);
         const uint32_t tq = tmem + ((uint32_t)(32 * (warp & 3)) << 16);
         grid_dependency_wait();
@@ -404,7 +405,7 @@ umma_ts_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
             parity ^= (uint32_t)blk & 1u;
         }
     } else {
-        reg_give<kControlRegs>();
+        reg_share<kControlRegs, kLaunchRegs>();
         // no copy is on its way when the block leaves, whatever its readers have given up on
         auto drain = [&](int full, int slots, int issued) {
 #pragma unroll 1
