@@ -218,6 +218,7 @@ proj_kernel(const ProjParams P)
                 if (++xb == XB) { xb = 0; xphase ^= 1u; }
                 load(t0 + j + TD, x[j]);
             }
+        if (warp == 0 && lane == 0) grid_launch_dependents();        // what follows sets itself up as blocks leave
         if (!ok && lane == 0) atomicExch(P.status, 1);
     } else {
         // ---- Y ------------------------------------------------------------------------------------------

@@ -21,7 +21,7 @@
 //   control warps  one thread each for the key MMAs, the value MMAs, the K and q strips, the head's weights and the V strips
 // Registers move from the others to the value warps (setmaxnreg).  Waits of the compute warps have no vote and no way out (see
 // wait_or_give_up).  Every wait is bounded; one that runs out sets the status word, and tensor memory is released on every path.
-// Every CTA lays out its head's weights itself, in the value and softmax warps, while the first products are made: a prep launch in
+// Every CTA lays out its head's weights itself, in all warps but the control warps, while the first strips come: a prep launch in
 // front cost 1 us at 64 x 56 x 56, 2 heads, and 1.7 us at 32 x 28 x 42, 6 heads.
 //
 // Tensor memory: three value chunks of 96 columns (dx), three P chunks of 48 (3 taps x 32 bf16), two logit tiles of 32, A' of 16.
@@ -101,7 +101,7 @@ static_assert(kSmemBytes <= 227 * 1024, "shared memory");
 constexpr int kRawSlots = 2;
 constexpr uint32_t kRawOff = kVOff + (kVSlots - kRawSlots) * (uint32_t)kSlot;
 static_assert(2 * kWeightFloats * 4 <= kRawSlots * kSlot, "fp32 weights");
-constexpr int kBuilders = 4 * kVSets + 4;               // value and softmax warps, which have nothing else to do yet
+constexpr int kBuilders = kCtlK;                        // all warps but the control warps
 
 // Hand-offs of tensor memory between threads: the side that has read or written TMEM issues
 // tcgen05.wait::ld / ::st (the accesses are then complete) and arrives on an mbarrier; the side that
@@ -188,22 +188,11 @@ umma_ts_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
     // share in L2
     const int my_blocks = rank < blocks ? (blocks - rank + nrank - 1) / nrank : 0;
 
-    if (threadIdx.x == 0) {
-#pragma unroll 1
-        for (int i = 0; i < kKSlots; ++i) { mbar_init_only(bar(kBarKFull + i), 1); mbar_init_only(bar(kBarKEmpty + i), 4); }
-#pragma unroll 1
-        for (int i = 0; i < kVSlots; ++i) { mbar_init_only(bar(kBarVFull + i), 1); mbar_init_only(bar(kBarVEmpty + i), 4); }
-        for (int i = 0; i < 2; ++i) { mbar_init_only(bar(kBarLFull + i), 1); mbar_init_only(bar(kBarLFree + i), 4); }
-        mbar_init_only(bar(kBarEReady), 4);
-        mbar_init_only(bar(kBarEFree), 1);
-#pragma unroll 1
-        for (int i = 0; i < 3 * kVSets; ++i) mbar_init_only(bar(kBarDFull + i), 1);
-#pragma unroll 1
-        for (int i = 0; i < 3 * kPSets; ++i) mbar_init_only(bar(kBarPFree + i), 1);
-#pragma unroll 1
-        for (int i = 0; i < 3; ++i) { mbar_init_only(bar(kBarPReady + i), 4); mbar_init_only(bar(kBarDFree + i), 4); }
-        mbar_init_only(bar(kBarWeights), P.bimg ? 1 : kBuilders);
-        mbar_init_only(bar(kBarRaw), 1);
+    if (threadIdx.x < kBars) {                                     // a thread a barrier: one after the other they took 0.2 us
+        const int i = threadIdx.x;
+        auto in = [&](int first, int n) { return i >= first && i < first + n; };
+        const bool warps = in(kBarKEmpty, kKSlots) || in(kBarVEmpty, kVSlots) || in(kBarLFree, 2) || i == kBarEReady || in(kBarDFree, 3) || in(kBarPReady, 3);
+        mbar_init_only(bar(i), i == kBarWeights && !P.bimg ? (uint32_t)kBuilders : warps ? 4u : 1u);
         mbar_init_fence();
     }
     if (warp == kCtlK) tmem_alloc(smem_u32(smem + kTmemOff), kTmemCols);
@@ -213,23 +202,21 @@ umma_ts_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
     const uint32_t tmem = *reinterpret_cast<const volatile uint32_t*>(smem + kTmemOff);
     bool ok = true;
     // the images of the weights, by the warps that wait for them to be used
-    auto build_images = [&](int builder) {
-        if (P.bimg) return;
+    if (!P.bimg && warp < kBuilders) {
         wait_or_give_up(bar(kBarRaw), 0, ok);
         const float* raw = reinterpret_cast<const float*>(smem + kRawOff);
 #pragma unroll 1
-        for (int item = 32 * builder + lane; item < kItems; item += 32 * kBuilders) build_item(raw, raw + kWeightFloats, smem + kBOff, item);
+        for (int item = threadIdx.x; item < kItems; item += 32 * kBuilders) build_item(raw, raw + kWeightFloats, smem + kBOff, item);
         fence_proxy_async_smem();
         __syncwarp();
         mbar_arrive_lane0(bar(kBarWeights), lane);
-    };
+    }
 
     if (warp < kPWarp0) {
         // =====================================================================================
         // value warps: set s takes blocks s, s + sets, ..; warp q of it strip q of the block
         // =====================================================================================
         reg_share<kValueRegs, kLaunchRegs>();
-        build_images(warp);
         const int q = warp & 3, set = warp >> 2, g = lane >> 2, tig = lane & 3;
         const uint32_t tq = tmem + kColD + ((uint32_t)(32 * q) << 16);
         const uint32_t full = bar(kBarDFull + 3 * set);
@@ -356,7 +343,6 @@ umma_ts_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
         // softmax warps: thread = pixel = TMEM lane 32 q + lane, every block
         // =====================================================================================
         reg_share<kSoftmaxRegs, kLaunchRegs>();
-        build_images(4 * kVSets + warp - kSWarp0);
         const uint32_t tq = tmem + ((uint32_t)(32 * (warp & 3)) << 16);
         grid_dependency_wait();
         float biasl[9];
