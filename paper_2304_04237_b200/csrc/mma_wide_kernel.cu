@@ -603,17 +603,11 @@ mma_five_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant
     const int h = blockIdx.x % P.heads, rank = blockIdx.x / P.heads, nrank = (int)gridDim.x / P.heads;
     const int blocks = (P.tiles + 1) >> 1, my_blocks = rank < blocks ? (blocks - rank + nrank - 1) / nrank : 0;
 
-    if (threadIdx.x == 0) {
-        auto init = [&](int first, int n, uint32_t count) {
-#pragma unroll 1
-            for (int i = first; i < first + n; ++i) mbar_init_only(bar(i), count);
-        };
-        init(F::KFull, F::KSlots, 1); init(F::KEmpty, F::KSlots, 4);
-        init(F::VFull, F::VSlots, 1); init(F::VEmpty, F::VSlots, 4);
-        init(F::PReady, 2, 4); init(F::PFree, 2, 1);
-        init(F::LFull, 2, 1); init(F::EReady, 2, 4); init(F::EFree, 2, 1);
-        init(F::DFree1, 3, 4); init(F::DFull, F::VSets * K * 2, 1);
-        init(F::Weights, 1, 1);
+    if (threadIdx.x < F::Bars) {                                   // a thread a barrier: one after the other they take 0.2 us
+        const int i = threadIdx.x;
+        auto in = [&](int first, int n) { return i >= first && i < first + n; };
+        const bool warps = in(F::KEmpty, F::KSlots) || in(F::VEmpty, F::VSlots) || in(F::PReady, 2) || in(F::EReady, 2) || in(F::DFree1, 3);
+        mbar_init_only(bar(i), warps ? 4u : 1u);
         mbar_init_fence();
     }
     for (int i = threadIdx.x; i < Wd::K2; i += F::Threads) s_bias[i] = P.bias ? P.bias[h * Wd::K2 + i] * kLog2e : 0.f;
