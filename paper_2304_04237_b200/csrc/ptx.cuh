@@ -36,40 +36,48 @@ __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
 
 // Bounded wait: false if the phase did not complete within the limit (about two seconds).  Each
 // probe may park the thread for up to 100 us (the hardware wakes it when the phase completes), so
-// a waiting warp issues next to no instructions.  `Small`: a loop that the compiler may not unroll, in kernels of which many waits
-// would otherwise fill the instruction cache (41 instead of 63 KB of one of them); elsewhere it costs up to 3 %.
-template <bool Small = false>
+// a waiting warp issues next to no instructions.
 __device__ __forceinline__ bool mbar_park(uint32_t bar, uint32_t parity) {
-    auto probe = [&]() {
+#pragma unroll 1
+    for (int spin = 0; spin < 20000; ++spin) {
         uint32_t done;
         asm volatile(
             "{\n\t.reg .pred p;\n\t"
             "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
             "selp.u32 %0, 1, 0, p;\n\t}"
             : "=r"(done) : "r"(bar), "r"(parity), "r"(100000u) : "memory");
-        return done != 0;
-    };
-    if constexpr (Small) {
-#pragma unroll 1
-        for (int spin = 0; spin < 20000; ++spin)
-            if (probe()) return true;
-    } else {
-        for (int spin = 0; spin < 20000; ++spin)
-            if (probe()) return true;
+        if (done) return true;
     }
     return false;
 }
-// The same behind a probe without the time hint: a phase that is already complete then costs about 30 cycles less.
+// The same behind a probe without the time hint: a phase that is already complete then costs about 30 cycles less.  `Small`: the loop
+// may not be unrolled, in kernels of which many waits would otherwise fill the instruction cache (41 instead of 63 KB of one of
+// them); elsewhere that costs up to 3 %.
 template <bool Small = false>
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
-    uint32_t done;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(done) : "r"(bar), "r"(parity) : "memory");
-    if (done) return true;
-    return mbar_park<Small>(bar, parity);
+    {
+        uint32_t done;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(done) : "r"(bar), "r"(parity) : "memory");
+        if (done) return true;
+    }
+    if constexpr (Small) {
+        return mbar_park(bar, parity);
+    } else {
+        for (int spin = 0; spin < 20000; ++spin) {
+            uint32_t done;
+            asm volatile(
+                "{\n\t.reg .pred p;\n\t"
+                "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
+                "selp.u32 %0, 1, 0, p;\n\t}"
+                : "=r"(done) : "r"(bar), "r"(parity), "r"(100000u) : "memory");
+            if (done) return true;
+        }
+        return false;
+    }
 }
 
 // A wait of a whole warp without a vote: a lane whose wait runs out carries on with `ok` cleared and waits no more, so that the
@@ -82,7 +90,7 @@ __device__ __forceinline__ void wait_or_give_up(uint32_t bar, uint32_t parity, b
         "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
         "selp.u32 %0, 1, 0, p;\n\t}"
         : "=r"(done) : "r"(bar), "r"(parity) : "memory");
-    if (!done && ok) ok = mbar_park<true>(bar, parity);
+    if (!done && ok) ok = mbar_park(bar, parity);
     __syncwarp();
 }
 

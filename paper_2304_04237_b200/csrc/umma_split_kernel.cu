@@ -29,7 +29,7 @@ struct Fwd {
     static constexpr int planes = D / Cut<T>::channels;
     static constexpr int chunks = 3 * planes;                                    // product chunks, and D chunks, of a block
     static constexpr uint32_t image = contract_bytes(D) + expand_bytes(D);      // of a head, in shared memory and in the workspace
-    static constexpr uint32_t misc = 8u * (kTeams * kTeamBars + 2) + 16;
+    static constexpr uint32_t misc = 8u * (kTeams * kTeamBars + 1) + 16 + 16;       // barriers, tensor-memory slot; largest weight, another barrier
     static constexpr int fit = (int)((227u * 1024u - image - misc - 128) / (kTeams * kSlot));
     static constexpr int ring = fit < kMaxRing ? fit : kMaxRing;                 // slots of a team
     static_assert(ring >= 2, "the ring does not fit");
@@ -80,9 +80,9 @@ umma_split_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
     unsigned char* smem = smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u);
     const uint32_t bars = smem_u32(smem + F::bar_off);
     const uint32_t bar_weights = bars + 8u * (kTeams * kTeamBars);
-    const uint32_t bar_raw = bar_weights + 8u;
-    unsigned char* tmem_slot = smem + F::bar_off + 8u * (kTeams * kTeamBars + 2);
-    uint32_t* s_most = reinterpret_cast<uint32_t*>(tmem_slot + 8);
+    unsigned char* tmem_slot = smem + F::bar_off + 8u * (kTeams * kTeamBars + 1);
+    const uint32_t bar_raw = smem_u32(tmem_slot) + 16u;
+    uint32_t* s_most = reinterpret_cast<uint32_t*>(tmem_slot + 24);
 
     const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     const int h = blockIdx.x % P.heads, rank = blockIdx.x / P.heads, nrank = (int)gridDim.x / P.heads;
@@ -96,8 +96,7 @@ umma_split_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_consta
     if (threadIdx.x == 0) {
         for (int i = 0; i < kTeams; ++i) init_team_bars(bars + 8u * (uint32_t)(i * kTeamBars));
         mbar_init_only(bar_weights, Build ? kComputeWarps : 1);
-        mbar_init_only(bar_raw, 1);
-        *s_most = 0u;
+        if (Build) { mbar_init_only(bar_raw, 1); *s_most = 0u; }
         mbar_init_fence();
     }
     if (warp == kMmaWarp) tmem_alloc(smem_u32(tmem_slot), 512);
