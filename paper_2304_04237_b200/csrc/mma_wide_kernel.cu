@@ -563,7 +563,7 @@ mma_wide_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant
 // Tensor memory: a D buffer of 96 columns for the upper three taps of a tap column, two of 64 for the lower two, in turn, two of
 // products of 80 (five taps), two tiles of 64: logits in 32 columns, later e_hi in 16 and 8 for each tap column.
 //
-// Bound by energy when it runs for seconds (1000 W), else by latency: 51.5 M warp instructions at 64 x 56 x 56, 3 heads, in 48 % of the issue
+// Bound by energy when it runs for seconds (1000 W), else by latency: 50.4 M warp instructions at 64 x 56 x 56, 3 heads, in 48 % of the issue
 // slots, tensor pipe 42 %, value warps waiting for 60 % of the time.  In two teams of eight warps with two rows each as above 71 M.  Calls, a few
 // hundred / for seconds: 64 x 56 x 56, 3 heads 123.5 / 134.5 -> 97 / 112.6 us; 2 x 128 x 128, 3 heads 27.0 -> 24.6.  Without the
 // one step for the one-hot part 104.5 / 118.8.

@@ -26,11 +26,12 @@
 //
 // Tensor memory: three value chunks of 96 columns (dx), three P chunks of 48 (3 taps x 32 bf16), two logit tiles of 32, A' of 16.
 //
-// What bounds it: instruction issue and latency on the CUDA cores.  14.5 M warp instructions at 64 x 56 x 56, 2 heads, in 53 % of the
-// slots; the value warps wait for 40 % of the time, the product warps for 50 %, so that no stage alone is the bound.  With value
-// and product warps of two rows each on tiles of 4 rows x up to 64 columns it was 18.3 M (every halo row widened for two output rows
-// instead of three, twice the hand-offs).  Calls, a few hundred / for seconds, when the power limit takes clocks down to 1.69 GHz here
-// and 1.84 before: 64 x 56 x 56, 2 heads 32.3 / 33.2 -> 27.6 / 31.4 us, 32 x 28 x 42, 6 heads 23.5 / 23.4 -> 19.7 / 20.9.
+// What bounds it: instruction issue and latency on the CUDA cores, and power in runs of seconds.  15.3 M warp instructions at 64 x 56 x 56,
+// 2 heads, in 47 % of the slots (57 % while an SM has work); the value warps wait for 40 % of the time, the product warps for 50 %, so that no
+// stage alone is the bound.  With value and product warps of two rows each on tiles of 4 rows x up to 64 columns it was 18.3 M (every
+// halo row widened for two output rows instead of three, twice the hand-offs).  Calls, a few hundred / for seconds, when the power limit
+// takes clocks down to 1.69 GHz here and 1.84 before: 64 x 56 x 56, 2 heads 32.3 / 34.0 -> 26.1 / 30.8 us, 32 x 28 x 42, 6 heads 23.5 / 23.4 ->
+// 19.4 / 20.5, 2 x 56 x 56, 2 heads 7.9 -> 5.6.
 // The code has to stay small: the instruction cache holds 32 KB, and a build of 112 KB (waits' spin loops and tile loops unrolled by
 // the compiler) took 47 us.  Loops over tap columns not unrolled: 37 us.  fma.rn.f32x2 as two FMAs each: 3 % slower.  One set of
 // product warps: 28.8; all of a chunk's accumulators read at once (160 registers): 29.6; two value chunks instead of three: the same.
