@@ -471,7 +471,7 @@ def main():
                  "proj_qkv_ms": qkv_ms, "proj_qkv_gbs": 4 * tok_bytes / (qkv_ms * 1e-3) / 1e9,
                  "proj_o_ms": o_ms, "proj_o_gbs": 2 * tok_bytes / (o_ms * 1e-3) / 1e9,
                  "bytes_min_three_stages": 10 * tok_bytes, "bytes_min_fused": 2 * tok_bytes,
-                 "kernels": "projection GEMM (Eq. 1, three outputs), attention (prep + main), projection GEMM (Eq. 3)"}
+                 "kernels": "projection GEMM (Eq. 1, three outputs), attention, projection GEMM (Eq. 3)"}
 
     # end to end through the host-buffer entry point: pinned host inputs in, pinned result out
     e2e = None
