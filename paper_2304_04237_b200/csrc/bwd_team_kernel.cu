@@ -240,6 +240,7 @@ bwd_point_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constan
                     umma_commit(bar(kDFull + db));
                 }
             }
+            if (ok) ok = wait_last_phases(bar(kPFree), 2, pn);      // no commit on its way when the block leaves
             if (!ok) atomicExch(P.status, 1);
         }
         __syncwarp();

@@ -176,6 +176,8 @@ bwd_weight_umma_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                 }
                 if (ok) umma_commit(bar(kEmpty + st));               // its rows have been read
             }
+            // no commit on its way when the block leaves
+            if (ok) { ok = wait_last_phases(bar(kAFree), 2, n); ok = wait_last_phases(bar(kEmpty), 2, it) && ok; }
             if (!ok) atomicExch(P.status, 1);
         }
         __syncwarp();

@@ -317,6 +317,8 @@ mma_wide_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant
                                 if (++ws == 3) { ws = 0; phase ^= 1u; }
                             }
                 }
+                // the last commits, here and in the MMA threads, are not on their way any more when the block leaves
+                if (ok) ok = wait_last_phases(wbar(kWEmpty), 3, rounds * K * (NGK + NGV));
             }
             if (!ok) atomicExch(P.status, 1);
         }
@@ -424,6 +426,7 @@ mma_wide_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant
                     }
                 }
             }
+            if (ok) ok = wait_last_phases(bar(kPFree), PB, my_blocks * K * NGK);
             if (!ok) atomicExch(P.status, 1);
         }
         __syncwarp();
@@ -828,11 +831,8 @@ mma_five_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant
         }
     } else {
         reg_share<F::ControlRegs, F::LaunchRegs>();
-        // no copy is on its way when the block leaves, whatever its readers have given up on
-        auto drain = [&](int full, int slots, int issued) {
-#pragma unroll 1
-            for (int i = 0; i < slots && i < issued; ++i) ok = mbar_wait<true>(bar(full + i), (uint32_t)((issued - 1 - i) / slots) & 1u) && ok;
-        };
+        // no copy or commit is on its way when the block leaves, whatever its readers have given up on
+        auto drain = [&](int first, int slots, int uses) { ok = wait_last_phases(bar(first), slots, uses) && ok; };
         auto load_tiles = [&](uint32_t dst, const CUtensorMap* map, uint32_t full, const TileWalk& at) {
             mbar_expect_tx(full, Wd::slot);
             // the second tile may be past the last: its image does not exist and it reads as zero
@@ -874,6 +874,7 @@ mma_five_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant
                     }
                     if (ok) umma_commit(bar(F::LFull) + 8u * tile);
                 }
+                if (ok) drain(F::PFree, 2, K * my_blocks);
             } else if (warp == F::Ctl + 1) {
                 // ---- value MMAs -----------------------------------------------------------------------------
                 const uint64_t wd = umma_smem_desc(w + (uint32_t)Wd::K2 * Wd::tap, 128, 2 * Wd::KS * 128), ud = umma_smem_desc(smem_u32(smem + F::unit_off), 128, 256);
@@ -903,6 +904,7 @@ mma_five_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant
                     }
                     if (ok) umma_commit(bar(F::EFree) + 8u * tile);
                 }
+                if (ok) drain(F::EFree, 2, my_blocks);
             } else {
                 // ---- the head's weights and K, or V -------------------------------------------------------------
                 const bool v = warp == F::Ctl + 3;

@@ -177,6 +177,7 @@ proj_kernel(const ProjParams P)
                 if (ok) umma_commit(bar(kXFree + xb));
                 if (++xb == XB) { xb = 0; xphase ^= 1u; }
             }
+            if (ok) ok = wait_last_phases(bar(kXFree), XB, my_tiles);       // no commit on its way when the block leaves
             if (!ok) atomicExch(P.status, 1);
         }
         __syncwarp();

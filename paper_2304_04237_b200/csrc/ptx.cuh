@@ -80,6 +80,16 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
     }
 }
 
+// Waits until the last arrivals on `slots` barriers from `first` on, used in turn `uses` times in all, have come: with them nothing that
+// arrives by itself, a copy or a commit of the tensor core, is still on its way to shared memory that the block is about to leave, where
+// the next block sets up barriers of its own.  For a thread by itself, and barriers of which one use begins after the one before was waited for.
+__device__ __forceinline__ bool wait_last_phases(uint32_t first, int slots, int uses) {
+    bool ok = true;
+#pragma unroll 1
+    for (int i = 0; i < slots && i < uses; ++i) ok = mbar_wait<true>(first + 8u * (uint32_t)i, (uint32_t)((uses - 1 - i) / slots) & 1u) && ok;
+    return ok;
+}
+
 // A wait of a whole warp without a vote: a lane whose wait runs out carries on with `ok` cleared and waits no more, so that the
 // warp stays together whatever happens, and says so at its end.  (With a vote and a way out behind every wait, a wait on a phase that
 // is already complete took 124 cycles, without 76.)

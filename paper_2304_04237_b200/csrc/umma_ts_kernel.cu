@@ -393,12 +393,9 @@ umma_ts_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
         }
     } else {
         reg_share<kControlRegs, kLaunchRegs>();
-        // no copy is on its way when the block leaves, whatever its readers have given up on
-        auto drain = [&](int full, int slots, int issued) {
-#pragma unroll 1
-            for (int s = 0; s < slots && s < issued; ++s)
-                ok = mbar_wait<true>(bar(full + s), (uint32_t)((issued - 1 - s) / slots) & 1u) && ok;
-        };
+        // no copy or commit is on its way when the block leaves, whatever its readers have given up on; the barriers that are not
+        // waited for here have readers that waited for their last phase
+        auto drain = [&](int first, int slots, int uses) { ok = wait_last_phases(bar(first), slots, uses) && ok; };
         uint32_t leader;
         if (elect_one(leader) && my_blocks > 0) {
             if (warp == kCtlK) {
@@ -428,6 +425,7 @@ umma_ts_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
                     full ^= 8u; dcol ^= kOtherL;
                     parity ^= (uint32_t)blk & 1u;
                 }
+                if (ok) drain(kBarPFree, 3 * kPSets, 3 * my_blocks);
             } else if (warp == kCtlV) {
                 // ---- value MMAs -------------------------------------------------------------------------
                 const uint64_t desc = umma_smem_desc(smem_u32(smem + kBOff), 128, 512);
@@ -449,6 +447,7 @@ umma_ts_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
                     }
                     if (kVSets == 2) done = done == bar(kBarDFull) ? done + 24u : bar(kBarDFull);
                 }
+                if (ok) drain(kBarEFree, 1, my_blocks);
             } else if (warp == kCtlTK) {
                 // ---- K and q strips -----------------------------------------------------------------------
                 grid_dependency_wait();
