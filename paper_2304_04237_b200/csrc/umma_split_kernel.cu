@@ -405,7 +405,7 @@ bool umma_split_builds_images(int B, int H, int W, int heads, int num_sms) {
 cudaError_t launch_umma_split_prep(const Problem& p, void* workspace, cudaStream_t stream) {
     return of_heads(p, [&](auto heads) {
         using H = decltype(heads);
-        return launch_chained(umma_split_prep_kernel<typename H::type, H::dim>, dim3((unsigned)p.heads, prep_parts(H::dim)), 256, 0, stream, p.wk, p.wv,
+        return launch_spread<umma_split_prep_kernel<typename H::type, H::dim>>(dim3((unsigned)p.heads, prep_parts(H::dim)), 256, stream, p.wk, p.wv,
                               static_cast<unsigned char*>(workspace));
     });
 }

@@ -1,0 +1,61 @@
+"""Kernels that start early must not hold up the ones behind them: calls of a chain one after the other take no longer than the same calls
+each repeated by itself (small blocks of a prep kernel, launched while most of the chip was still busy, piled up on a few SMs: 1.11 - 1.20
+times, now 1.01 - 1.03).  Times are the least of several, taken in turn in one process, so that clocks and load are the same for both."""
+import pytest
+import torch
+
+import paper_2304_04237_b200 as sa
+
+pytestmark = pytest.mark.gpu
+
+
+class Calls:
+    def __init__(self, B, H, W, heads, d, k=3):
+        gen = torch.Generator(device="cuda").manual_seed(1)
+        C, k2 = heads * d, k * k
+        self.ctx = sa.slide_attn_create(B, H, W, heads, d, k, torch.bfloat16, False)
+        self.maps = [torch.randn(B, H, W, heads, d, device="cuda", generator=gen).to(torch.bfloat16) for _ in range(8)]
+        self.w = [torch.eye(k2, device="cuda") + 0.05 * torch.randn(C, k2, k2, device="cuda", generator=gen) for _ in range(2)]
+        self.dw = [torch.empty_like(w) for w in self.w]
+
+    def forward(self):
+        sa.slide_attn_forward(self.ctx, *self.maps[:3], *self.w, None, self.maps[3])
+
+    def backward(self):
+        sa.slide_attn_backward(self.ctx, *self.maps[:3], *self.w, None, self.maps[4], *self.maps[5:], *self.dw, None)
+
+    def close(self):
+        assert sa.slide_attn_query_status(self.ctx) == sa.OK
+        sa.slide_attn_destroy(self.ctx)
+
+
+def times_of(fns, calls=40, repeats=9):
+    best = [float("inf")] * len(fns)
+    for _ in range(repeats):
+        for i, fn in enumerate(fns):
+            fn()
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            for _ in range(calls):
+                fn()
+            b.record()
+            torch.cuda.synchronize()
+            best[i] = min(best[i], a.elapsed_time(b) / calls * 1e3)
+    return best
+
+
+@pytest.mark.parametrize("shape", [(3, 54, 54, 8, 32), (8, 56, 56, 3, 32)], ids=lambda s: "x".join(map(str, s)))
+def test_training_step_takes_no_longer_than_its_calls(shape):
+    c = Calls(*shape)
+    forward, backward, step = times_of([c.forward, c.backward, lambda: (c.forward(), c.backward())])
+    c.close()
+    assert step <= 1.06 * (forward + backward), (forward, backward, step)
+
+
+def test_forwards_of_two_kinds_take_no_longer_than_each():
+    """UMMA_TS, then UMMA_SPLIT with a prep launch."""
+    a, b = Calls(8, 56, 56, 3, 32), Calls(8, 56, 56, 3, 64)
+    one, other, both = times_of([a.forward, b.forward, lambda: (a.forward(), b.forward())])
+    a.close()
+    b.close()
+    assert both <= 1.06 * (one + other), (one, other, both)
