@@ -42,8 +42,9 @@ bool make_tile_map(CUtensorMap* map, const void* base, int elem_bytes, int B, in
 // has to execute griddepcontrol.wait before it touches anything that one may write or read, and in any case before it completes:
 // whoever waits for it takes all that was launched earlier as complete.  The prep kernels wait first of all and only then let the
 // main kernel behind them start, so a main kernel never runs beside what was ahead of its prep kernel.  Chained so, back-to-back forwards have no launch gap between them.
-// Kernels that lay their weights out themselves, and projections, let the next one start when their last loads are sent for: 2 x 56 x 56,
-// 2 heads, bf16, k = 3 7.3 us -> 6.2, block 4 x 28 x 28, 6 heads 17.6 -> 16.9.  They wait for all that was launched earlier in the threads that load.
+// Kernels that lay their weights out themselves, and projections that no prep or check kernel follows, let the next one start when their
+// last loads are sent for: 2 x 56 x 56, 2 heads, bf16, k = 3 7.3 us -> 6.2, block 4 x 28 x 28, 6 heads 17.6 -> 16.9.  They wait for all that
+// was launched earlier in the threads that load.
 // (The others do not let theirs start early: waiting beside them, the next prep kernel's blocks made a 2 x 128 x 128 x 3 heads
 // call with k = 7 take 70 us instead of 59, others up to 6 % longer.)
 template <typename... Params, typename... Args>
@@ -163,7 +164,8 @@ bool proj_supports(int c_in, int c_out);
 bool proj_wants_image(long long rows, int c_in, int c_out, int nmat, int num_sms);
 size_t proj_image_bytes(int c_in, int c_out, int nmat);
 cudaError_t launch_proj_prep(const float* wa, int nmat_a, void* image_a, const float* wb, int nmat_b, void* image_b, int c_in, int c_out, cudaStream_t stream);
+// `early`: the kernel behind may start before this one is complete.
 cudaError_t launch_proj(const void* x, long long rows, int c_in, const float* w, const void* image, int c_out, int nmat,
-                        void* const* y, int* d_status, int num_sms, cudaStream_t stream);
+                        void* const* y, bool early, int* d_status, int num_sms, cudaStream_t stream);
 
 }  // namespace slide_attn

@@ -53,6 +53,7 @@ struct ProjParams {
     int rows, K;
     int groups, units, per_group; // units of U columns: in all, of a group (the last one may have fewer)
     int* status;
+    bool early;                   // let the kernel behind this one start before this one is complete
 };
 
 // channel of K index / column n within a unit: the order in which tcgen05.st lays X out, and in which tcgen05.ld hands Y out
@@ -164,6 +165,9 @@ proj_kernel(const ProjParams P)
             uint32_t xphase = 0, dphase = 1;
             for (int t = 0; ok && t < my_tiles; ++t) {
                 if (!mbar_wait(bar(kXFull + xb), xphase)) { ok = false; break; }
+                // The last tile is here: what follows sets itself up as blocks leave.  (In a load warp the line cost a register too many at
+                // C = 256, 48 bytes of spills instead of 4.)
+                if (P.early && t == my_tiles - 1) grid_launch_dependents();
                 for (int ch = 0; ch < nchunks; ++ch, ++it) {
                     if (!mbar_wait(bar(kDFree + db), dphase)) { ok = false; break; }
                     tc_fence_after_sync();
@@ -219,7 +223,6 @@ proj_kernel(const ProjParams P)
                 if (++xb == XB) { xb = 0; xphase ^= 1u; }
                 load(t0 + j + TD, x[j]);
             }
-        if (warp == 0 && lane == 0) grid_launch_dependents();        // what follows sets itself up as blocks leave
         if (!ok && lane == 0) atomicExch(P.status, 1);
     } else {
         // ---- Y ------------------------------------------------------------------------------------------
@@ -348,14 +351,14 @@ cudaError_t launch_proj_prep(const float* wa, int nmat_a, void* image_a, const f
 }
 
 cudaError_t launch_proj(const void* x, long long rows, int c_in, const float* w, const void* image, int c_out, int nmat,
-                        void* const* y, int* d_status, int num_sms, cudaStream_t stream)
+                        void* const* y, bool early, int* d_status, int num_sms, cudaStream_t stream)
 {
     if (!proj_supports(c_in, c_out) || nmat < 1 || nmat > 3 || rows < 1 || rows > 0x7fffff00LL) return cudaErrorInvalidValue;
     const int U = unit_of(c_in, c_out);
     ProjParams P;
     P.x = static_cast<const __nv_bfloat16*>(x); P.w = w; P.image = static_cast<const unsigned char*>(image);
     for (int i = 0; i < 3; ++i) P.y[i] = static_cast<__nv_bfloat16*>(i < nmat ? y[i] : nullptr);
-    P.ycols = c_out; P.rows = (int)rows; P.K = c_in; P.units = c_out * nmat / U; P.status = d_status;
+    P.ycols = c_out; P.rows = (int)rows; P.K = c_in; P.units = c_out * nmat / U; P.status = d_status; P.early = early;
     const Split split = split_columns(rows, c_in, P.units, U, image ? 2 : 4, num_sms);
     P.per_group = split.per_group; P.groups = split.groups;
     const Kernel kernel = U == 32 ? kernel_for<32>(c_in) : kernel_for<16>(c_in);
