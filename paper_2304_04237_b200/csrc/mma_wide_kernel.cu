@@ -103,45 +103,63 @@ struct WideParams {
     float scale_log2e;
 };
 
-// Prep: fp32 [C][slot][tap] -> bf16, taps in the order o = dx K + dy (tap t = dy K + dx), first the key side, then the value side,
-// one 16-byte item per thread.
+constexpr int kPrepThreads = 512;
+
+// Prep: fp32 [C][slot][tap] -> bf16, taps in the order o = dx K + dy (tap t = dy K + dx), first the key side, then the value side; of a
+// tap, items of 16 bytes:
 //   key tap, item (j, n): k 8j .. 8j + 7 (channels in the order tcgen05.st lays the products out), column n = slot
 //   value tap, item (n, j): column n (channel in the order tcgen05.ld hands them out), k 8j .. 8j + 7 = slots
+// A block takes eight channels (four of its side) x 16 slots, whose weights are runs of memory, through shared memory to all of their taps.
+// Bound by latency: one or two rounds of loads, one of items.  (Before, a thread gathered its eight weights, 4 k^2 bytes apart, from memory: a
+// sector for each, which depended on neighbours on the same SM for the rest of it, and when a kernel in front let this one start early its blocks lay on a few
+// SMs: forwards of 8 x 56 x 56, 3 heads, k = 3 and then k = 7 58.6 us, here 51.8; 54.7 where nothing starts early.  By themselves, 1 x 14 x 14,
+// 8 heads, k = 7 21.5 and 18.3, k = 9 43.2 and 32.4; 4 x 28 x 28, 4 heads, k = 5 9.7 and 9.3; 1 x 14 x 14, 1 head, k = 7 17.4 and 17.7.)
 template <int K>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kPrepThreads)
 mma_wide_prep_kernel(const float* __restrict__ wk, const float* __restrict__ wv, unsigned char* __restrict__ img)
 {
     using Wd = Wide<K>;
-    constexpr int K2 = Wd::K2, N = Wd::N, per_tap = 4 * N;
+    constexpr int K2 = Wd::K2, Pitch = 16 * K2 + 1;      // odd, so that neither slots nor channels meet in a bank
+    __shared__ float s_w[8][Pitch];
     grid_dependency_wait();
     grid_launch_dependents();
-    const int h = blockIdx.y;
-    const float* wkh = wk + (size_t)h * kHeadDim * K2 * K2;
-    const float* wvh = wv + (size_t)h * kHeadDim * K2 * K2;
-    for (int i = blockIdx.x * 256 + threadIdx.x; i < 2 * K2 * per_tap; i += gridDim.x * 256) {
-        const int side = i >= K2 * per_tap, r = side ? i - K2 * per_tap : i;
-        const int o = r / per_tap, item = r % per_tap, t = (o % K) * K + o / K;
-        unsigned char* tap = img + (size_t)h * Wd::weights + (size_t)(side * K2 + o) * Wd::tap;
+    const int side = (int)blockIdx.x / (4 * Wd::KS), four = (int)blockIdx.x % (4 * Wd::KS) / Wd::KS, s0 = 16 * ((int)blockIdx.x % Wd::KS), h = blockIdx.y;
+    const int slots = K2 - s0 < 16 ? K2 - s0 : 16;
+    {                                                    // two warps a channel
+        const int e = threadIdx.x >> 6, i8 = 8 * four + e;
+        const int c = side ? 8 * ((i8 & 7) >> 1) + 2 * (i8 >> 3) + (i8 & 1) : 8 * ((i8 & 15) >> 2) + (i8 & 3) + (i8 >= 16 ? 4 : 0);
+        const float* src = (side ? wv : wk) + ((size_t)(h * kHeadDim + c) * K2 + s0) * K2;
+        constexpr int Deep = 13;                         // loads in flight: one round of them for k <= 7, two for k = 9
+        for (int i0 = threadIdx.x & 63; i0 < slots * K2; i0 += 64 * Deep) {
+            float x[Deep];
+#pragma unroll
+            for (int j = 0; j < Deep; ++j) x[j] = i0 + 64 * j < slots * K2 ? __ldg(src + i0 + 64 * j) : 0.f;
+#pragma unroll
+            for (int j = 0; j < Deep; ++j)
+                if (i0 + 64 * j < slots * K2) s_w[e][i0 + 64 * j] = x[j];
+        }
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < 16 * K2; i += kPrepThreads) {
+        const int o = i >> 4, item = i & 15, t = (o % K) * K + o / K;
         float v[8];
         uint32_t at;
         if (side == 0) {
-            const int n = item % N, j = item / N;
+            const int n = s0 + item;
 #pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const int kap = 8 * j + e, c = 8 * ((kap & 15) >> 2) + (kap & 3) + (kap >= 16 ? 4 : 0);
-                v[e] = n < K2 ? wkh[((size_t)c * K2 + n) * K2 + t] - (n == t ? 1.f : 0.f) : 0.f;
-            }
-            at = (uint32_t)(j * N * 16 + n * 16);
+            for (int e = 0; e < 8; ++e) v[e] = n < K2 ? s_w[e][item * K2 + t] - (n == t ? 1.f : 0.f) : 0.f;
+            at = (uint32_t)(four * Wd::N * 16 + n * 16);
         } else {
-            const int n = item & 31, j = item >> 5, c = 8 * ((n & 7) >> 1) + 2 * (n >> 3) + (n & 1);
+            const int n = item & 7, first = item & 8;
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
-                const int s = 8 * j + e;
-                v[e] = s < K2 ? wvh[((size_t)c * K2 + s) * K2 + t] - (s == t ? 1.f : 0.f) : 0.f;
+                const int s = s0 + first + e;
+                v[e] = s < K2 ? s_w[n][(first + e) * K2 + t] - (s == t ? 1.f : 0.f) : 0.f;
             }
-            at = (uint32_t)((n >> 3) * (2 * Wd::KS * 128) + j * 128 + (n & 7) * 16);
+            at = (uint32_t)(four * (2 * Wd::KS * 128) + (s0 + first) * 16 + n * 16);
         }
-        *reinterpret_cast<uint4*>(tap + at) = make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
+        *reinterpret_cast<uint4*>(img + (size_t)h * Wd::weights + (size_t)(side * K2 + o) * Wd::tap + at) =
+            make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
     }
 }
 
@@ -941,7 +959,7 @@ mma_five_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant
 
 template <int K>
 cudaError_t launch_prep_t(const Problem& p, void* workspace, cudaStream_t stream) {
-    return launch_chained(mma_wide_prep_kernel<K>, dim3((unsigned)((2 * Wide<K>::K2 * 4 * Wide<K>::N + 255) / 256), (unsigned)p.heads), 256, 0, stream, p.wk, p.wv,
+    return launch_chained(mma_wide_prep_kernel<K>, dim3((unsigned)(8 * Wide<K>::KS), (unsigned)p.heads), kPrepThreads, 0, stream, p.wk, p.wv,
                           static_cast<unsigned char*>(workspace));
 }
 

