@@ -183,7 +183,8 @@ slide_attn_status slide_attn_set_fixed_shift(slide_attn_ctx* ctx, int enable);
 slide_attn_status slide_attn_detect_fixed_shift(slide_attn_ctx* ctx, const float* wk, const float* wv,
                                                 int* is_fixed, void* cuda_stream);
 
-/* Number of kernels one slide_attn_forward launches with the current variant.  *n [out, host]. */
+/* Number of kernels one slide_attn_forward launches with the current variant (kernel timing off: see
+ * slide_attn_profile_begin).  *n [out, host]. */
 slide_attn_status slide_attn_launches_per_forward(const slide_attn_ctx* ctx, int* n);
 
 /*
@@ -298,6 +299,10 @@ slide_attn_status slide_attn_forward_noalloc(const void* q, const void* k, const
  * of Eq. 2 / Eq. 12).  After slide_attn_profile_begin every slide_attn_forward on this context
  * records CUDA events on its stream around (a) all kernels of the call and (b) the main fused
  * kernel alone; up to 1024 forwards are kept (later ones overwrite the oldest).
+ * (b) is without the layout of the weights.  Variants whose main kernel lays them out itself (UMMA_TS, and
+ * UMMA_SPLIT where slide_attn_launches_per_forward says 1) therefore launch the layout as a kernel of its own, and a
+ * main kernel that reads what it left, while timing is on: the same result bits, but neither (a) nor (b) is then the
+ * time of an ordinary forward; for that, time back-to-back forwards with timing off.
  * slide_attn_profile_end waits for the recorded events and reports the mean durations in
  * milliseconds and the number of forwards averaged, then stops recording.
  *   forward_ms, main_ms, n  [out, host]; any may be NULL.
