@@ -54,20 +54,27 @@ enum : int { kWFull = kTeams * kTeamBars, kWEmpty = kWFull + 3, kBars = kWEmpty 
 
 constexpr int least(int a, int b) { return a < b ? a : b; }
 
+// What the window makes of a head's weights and of a tile, in every kernel here.
 template <int K>
-struct Wide {
+struct Window {
     static constexpr int K2 = K * K, R = K / 2;
     static constexpr int KS = (K2 + 15) / 16;            // K steps of the value side
     static constexpr int N = 16 * KS;                    // columns of the logits
-    static constexpr bool resident = K <= 5;
-    static constexpr int GK = K == 5 ? 5 : K == 7 ? 4 : 3, GV = K == 9 ? 2 : 3;
-    static constexpr int NGK = (K + GK - 1) / GK, NGV = (K + GV - 1) / GV;
-    static constexpr int PB = least(3, (256 - N) / (16 * GK)), DB = 2;
-    static_assert(DB * 32 * GV <= 256 - N && PB >= 2, "tensor memory");
     static constexpr int HP = 8 + 2 * R;                 // edge of a tile with its halo
     static constexpr uint32_t plane = (uint32_t)(HP * HP * 64), slot = 2 * plane;
     static constexpr uint32_t tap = (uint32_t)(N * 64);  // weights of a tap, either side
     static constexpr uint32_t weights = 2u * K2 * tap;   // of a head
+};
+
+// mma_wide_kernel: k = 3, 7, 9.
+template <int K>
+struct Wide : Window<K> {
+    using Window<K>::N; using Window<K>::tap; using Window<K>::weights; using Window<K>::slot;
+    static constexpr bool resident = K == 3;
+    static constexpr int GK = K == 7 ? 4 : 3, GV = K == 9 ? 2 : 3;
+    static constexpr int NGK = (K + GK - 1) / GK, NGV = (K + GV - 1) / GV;
+    static constexpr int PB = least(3, (256 - N) / (16 * GK)), DB = 2;
+    static_assert(DB * 32 * GV <= 256 - N && PB >= 2, "tensor memory");
     static constexpr uint32_t chunk = (uint32_t)(GK > GV ? GK : GV) * tap;
     static constexpr uint32_t w_bytes = resident ? weights : 3 * chunk;
     static constexpr uint32_t misc = kOnesBytes + kUnitBytes + 336 + kInvBytes + 8u * kBars + 16;
@@ -93,7 +100,7 @@ struct TileWalk {
 };
 
 struct WideParams {
-    const unsigned char* weights;    // [head][Wide::weights]
+    const unsigned char* weights;    // [head][Window::weights]
     const __nv_bfloat16* q;
     const float* bias;
     __nv_bfloat16* out;
@@ -118,7 +125,7 @@ template <int K>
 __global__ void __launch_bounds__(kPrepThreads)
 mma_wide_prep_kernel(const float* __restrict__ wk, const float* __restrict__ wv, unsigned char* __restrict__ img)
 {
-    using Wd = Wide<K>;
+    using Wd = Window<K>;
     constexpr int K2 = Wd::K2, Pitch = 16 * K2 + 1;      // odd, so that neither slots nor channels meet in a bank
     __shared__ float s_w[8][Pitch];
     grid_dependency_wait();
@@ -211,7 +218,7 @@ __device__ __forceinline__ void sum_group(uint32_t t, const unsigned char* src, 
 // Softmax of the lane's pixel, whose N logits start at tensor-memory column `col`; leaves e_hi, e_lo in their place, returns 1 / sum.
 template <int K>
 __device__ __forceinline__ float softmax_in_place(uint32_t col, const float* s_bias, float scale_log2e) {
-    using Wd = Wide<K>;
+    using Wd = Window<K>;
     constexpr int K2 = Wd::K2, KS = Wd::KS;
     constexpr bool keep = KS <= 2;                       // the logits stay in registers between the passes
     float l[keep ? KS : 1][16];
@@ -251,21 +258,6 @@ __device__ __forceinline__ float softmax_in_place(uint32_t col, const float* s_b
     return 1.f / z;
 }
 
-// The tables of the one-hot parts (kOnesBytes, then kUnitBytes), by the whole block; what the tensor core reads comes after a block barrier.
-__device__ __forceinline__ void fill_tables(unsigned char* to, int threads) {
-    for (uint32_t i = threadIdx.x; i < (kOnesBytes + kUnitBytes) / 4; i += threads) {
-        uint32_t v = 0;
-        if (i < kOnesBytes / 4) {
-            if (((i * 4) & 511u) >> 4 == 15) v = kOnesBf16x2;
-        } else {
-            const uint32_t b = (i * 4 - kOnesBytes) % 1280u, core = b >> 7, k = (b & 15u) >> 1;      // k, k + 1 of a row
-            if (core >= 1 && core <= 8) v = (core - 1 == k ? 0x3F80u : 0u) | (core - 1 == k + 1 ? 0x3F800000u : 0u);
-        }
-        *reinterpret_cast<uint32_t*>(to + i * 4) = v;
-    }
-    fence_proxy_async_smem();
-}
-
 template <int K>
 __global__ void __launch_bounds__(kThreads, 1)
 mma_wide_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v, const WideParams P)
@@ -299,7 +291,17 @@ mma_wide_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant
         mbar_init_fence();
     }
     for (int i = threadIdx.x; i < Wd::K2; i += kThreads) s_bias[i] = P.bias ? P.bias[h * Wd::K2 + i] * kLog2e : 0.f;
-    fill_tables(smem + Wd::ones_off, kThreads);
+    for (uint32_t i = threadIdx.x; i < (kOnesBytes + kUnitBytes) / 4; i += kThreads) {
+        uint32_t v = 0;
+        if (i < kOnesBytes / 4) {
+            if (((i * 4) & 511u) >> 4 == 15) v = kOnesBf16x2;
+        } else {
+            const uint32_t b = (i * 4 - kOnesBytes) % 1280u, core = b >> 7, k = (b & 15u) >> 1;      // k, k + 1 of a row
+            if (core >= 1 && core <= 8) v = (core - 1 == k ? 0x3F80u : 0u) | (core - 1 == k + 1 ? 0x3F800000u : 0u);
+        }
+        *reinterpret_cast<uint32_t*>(smem + Wd::ones_off + i * 4) = v;
+    }
+    fence_proxy_async_smem();
     if (warp == kMmaWarp) tmem_alloc(smem_u32(smem + Wd::tmem_off), 512);
     tc_fence_before_sync();
     __syncthreads();
@@ -589,7 +591,7 @@ mma_wide_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant
 // hundred / for seconds: 64 x 56 x 56, 3 heads 123.5 / 134.5 -> 97 / 112.6 us; 2 x 128 x 128, 3 heads 27.0 -> 24.6.  Without the
 // one step for the one-hot part 104.5 / 118.8.
 struct Five {
-    using Wd = Wide<5>;
+    using Wd = Window<5>;
     static constexpr int K = 5, VSets = 2, KSlots = 2, VSlots = 4, G0 = 3, G1 = 2;
     static constexpr int PWarp = 4 * VSets, SWarp = PWarp + 4, Ctl = SWarp + 4, Threads = (Ctl + 4) * 32;
     static constexpr int LaunchRegs = 96, ValueRegs = 136, ProductRegs = 104, SoftmaxRegs = 64, ControlRegs = 40;      // a thread: at the launch, then
@@ -959,20 +961,20 @@ mma_five_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant
 
 template <int K>
 cudaError_t launch_prep_t(const Problem& p, void* workspace, cudaStream_t stream) {
-    return launch_chained(mma_wide_prep_kernel<K>, dim3((unsigned)(8 * Wide<K>::KS), (unsigned)p.heads), kPrepThreads, 0, stream, p.wk, p.wv,
+    return launch_chained(mma_wide_prep_kernel<K>, dim3((unsigned)(8 * Window<K>::KS), (unsigned)p.heads), kPrepThreads, 0, stream, p.wk, p.wv,
                           static_cast<unsigned char*>(workspace));
 }
 
 template <int K>
 cudaError_t launch_t(const Problem& p, const void* workspace, int* d_status, int num_sms, cudaStream_t stream) {
-    using Wd = Wide<K>;
+    using Wd = Window<K>;
     static bool configured[64] = {};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev >= 64 || !configured[dev]) {
         if constexpr (K == 5) e = cudaFuncSetAttribute(mma_five_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Five::total);
-        else e = cudaFuncSetAttribute(mma_wide_kernel<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Wd::total);
+        else e = cudaFuncSetAttribute(mma_wide_kernel<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Wide<K>::total);
         if (e != cudaSuccess) return e;
         if (dev < 64) configured[dev] = true;
     }
@@ -996,7 +998,7 @@ cudaError_t launch_t(const Problem& p, const void* workspace, int* d_status, int
     if (per_head < 1) per_head = 1;
     const dim3 grid((unsigned)(per_head * p.heads));
     if constexpr (K == 5) return launch_chained(mma_five_kernel, grid, Five::Threads, Five::total, stream, mk, mv, P);
-    else return launch_chained(mma_wide_kernel<K>, grid, kThreads, Wd::total, stream, mk, mv, P);
+    else return launch_chained(mma_wide_kernel<K>, grid, kThreads, Wide<K>::total, stream, mk, mv, P);
 }
 
 }  // namespace
@@ -1008,10 +1010,10 @@ bool mma_wide_supports(slide_attn_dtype dtype, int head_dim, int ksize) {
 
 size_t mma_wide_workspace_bytes(int heads, int ksize) {
     switch (ksize) {
-        case 3: return (size_t)heads * Wide<3>::weights;
-        case 5: return (size_t)heads * Wide<5>::weights;
-        case 7: return (size_t)heads * Wide<7>::weights;
-        case 9: return (size_t)heads * Wide<9>::weights;
+        case 3: return (size_t)heads * Window<3>::weights;
+        case 5: return (size_t)heads * Window<5>::weights;
+        case 7: return (size_t)heads * Window<7>::weights;
+        case 9: return (size_t)heads * Window<9>::weights;
         default: return 0;
     }
 }

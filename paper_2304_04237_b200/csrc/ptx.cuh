@@ -212,18 +212,6 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
-// One non-blocking probe of a phase.
-// Same test as a 0/1 word, without a branch: several can be in flight before the first is used.
-__device__ __forceinline__ uint32_t mbar_test_u32(uint32_t bar, uint32_t parity) {
-    uint32_t done;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(done) : "r"(bar), "r"(parity) : "memory");
-    return done;
-}
-
 // Elects one lane of a fully converged warp; `leader` receives its lane id in every lane.  Code that
 // issues tcgen05.mma or TMA copies from ONE thread should be guarded by this and not by a test of
 // the lane id: behind elect.sync the compiler keeps the operands of those instructions in the

@@ -187,7 +187,7 @@ umma_ts_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
     const int blocks = (int)((P.strips.total + 3) >> 2);
     // blocks are dealt round-robin: neighbouring CTAs work on neighbouring blocks at the same time, which keeps the halos they
     // share in L2
-    const int my_blocks = rank < blocks ? (blocks - rank + nrank - 1) / nrank : 0;
+    const int my_blocks = (blocks - rank + nrank - 1) / nrank;       // at least one: no head has more CTAs than blocks
 
     if (threadIdx.x < kBars) {                                     // a thread a barrier: one after the other they took 0.2 us
         const int i = threadIdx.x;
@@ -397,7 +397,7 @@ umma_ts_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
         // waited for here have readers that waited for their last phase
         auto drain = [&](int first, int slots, int uses) { ok = wait_last_phases(bar(first), slots, uses) && ok; };
         uint32_t leader;
-        if (elect_one(leader) && my_blocks > 0) {
+        if (elect_one(leader)) {
             if (warp == kCtlK) {
                 // ---- key MMAs: 18 per block (9 taps x two K = 16 halves) --------------------------------
                 const uint64_t desc = umma_smem_desc(smem_u32(smem + kBkOff), 512, 128);
