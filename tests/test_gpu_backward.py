@@ -76,6 +76,16 @@ def test_backward_matches_oracle(shape, dtype):
 
 
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("heads", [17, 140])
+def test_backward_with_many_heads(heads, dtype):
+    """Nine blocks of the prep kernel a head: two an SM, which the shared memory they ask for leaves room for, and more than eight, for which
+    they ask for none."""
+    x, dout = inputs((1, 5, 9, heads, 3), dtype)
+    ref = ob.backward(x["q"], x["k"], x["v"], x["wk"], x["wv"], x["bias"], 3, dout)
+    check(gpu_backward(x, dout, 3, dtype)[0], ref, dtype, f"{heads} {dtype}")
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
 def test_backward_no_bias_dense_weights_and_repeat(dtype):
     """Weights far from one-hot, no bias; a second call on the same context overwrites (does not
     accumulate into) every gradient."""
