@@ -101,10 +101,10 @@ int launches_of(const slide_attn_ctx* c) {
     }
 }
 
-// Whether the first kernel of a forward is the attention itself.  It may then be launched beside a projection ahead of it and set itself up.  Small
-// blocks of a prep or check kernel would wait, piled up on the SMs that come free first: blocks of 4 x 56 x 56, 4 heads of 64 take 31.7 us
-// so and 39.1 with an early start; 16 x 56 x 56, 2 heads, k = 7 70.8 and 74.7; fixed shift, 8 x 56 x 56, 8 heads 37.0 and 37.7.  64 x 56 x 56,
-// 2 heads, where the attention does start early, 54.0, without 56.5.
+// Whether the first kernel of a forward is the attention itself.  It may then be launched beside a projection ahead of it and set itself up
+// (blocks of 64 x 56 x 56, 2 heads 54.0 us so, 56.5 without).  Small blocks of a prep or check kernel would wait, piled up on the SMs that come
+// free first: 4 x 28 x 28, 4 heads, k = 9 44.6 with an early start and 41.8 without, k = 7 28.8 and 27.9; 16 x 56 x 56, 2 heads, k = 7 71.0 and
+// 69.8; 4 x 56 x 56, 4 heads of 64 39.1 and 31.4, were the prep kernel not spread (launch_spread).
 bool starts_at_once(const slide_attn_ctx* c) { return launches_of(c) == 1; }
 
 // Launches the context's variant on problem `p` (the context's shape, or a batch slice of it).

@@ -14,7 +14,7 @@
 // Bound by latency: the chain products -> MMA -> softmax -> split rows -> MMA -> sum and its hand-offs, with four compute warps per
 // scheduler to cover it.  Issue slots 30 - 36 % busy at 1.8 GHz, tensor pipe 13 - 24 %, DRAM 14 - 18 %.  A call, before (the CUDA-core kernel that
 // took the shape) and here: 2 x 128 x 128, 3 heads, fp32: 45.2 us in tile_kernel, 28.9; 32 x 28 x 28, 3 heads of 64, bf16: 232 us in
-// strip_kernel, 23.7; 1 x 14 x 14, 1 head, fp32: 14.4 and 7.5 us; heads of 16 (an earlier form of this kernel against strip_kernel): 16 x 56 x 56
+// strip_kernel, 23.7; 1 x 14 x 14, 1 head, fp32: 14.4 and 7.5 - 8.1 us; heads of 16 (an earlier form of this kernel against strip_kernel): 16 x 56 x 56
 // x 3, bf16 197 and 16.1, fp32 184 and 22.7 us.
 #include "team.cuh"
 
@@ -393,9 +393,10 @@ size_t umma_split_workspace_bytes(int heads, int head_dim) {
 }
 
 // Whether the CTAs of the main launch lay out their head's weights themselves: where no team has more than one block.  Beside a prep
-// launch a team starts on its first block 1 us earlier, as its warps are free for that, but the launch itself takes 2 us of a small call
-// (1 x 14 x 14, 1 head, fp32 8.5 us with it, 7.5 without; 4 x 28 x 28, 3 heads of 16, bf16 7.2 and 5.1; 2 x 128 x 128, 3 heads, fp32, three
-// blocks, 28.6 and 29.0; 32 x 28 x 28, 3 heads of 64, bf16, three blocks, 23.6 and 24.2).
+// launch a team starts on its first block 1 us earlier, as its warps are free for that, but the launch itself takes 2 us of a small call.
+// With it / without, us: 1 x 14 x 14, 1 head, fp32 8.5 - 8.9 / 7.5 - 8.1; 4 x 28 x 28, 3 heads of 16, bf16 7.2 / 5.1; heads of 64, bf16, a block for
+// every other SM 8.9 / 9.1, for every team 11.6 / 11.0.  Two blocks a team: 98 x 16 x 16, 3 heads, fp32 20.3 / 18.7, of 64, bf16 18.5 / 17.4, so the
+// line could lie there; three: 2 x 128 x 128, 3 heads, fp32 28.6 / 29.0, 32 x 28 x 28, 3 heads of 64, bf16 23.6 / 24.2.
 bool umma_split_builds_images(int B, int H, int W, int heads, int num_sms) {
     const long long blocks = ((long long)B * ((H + 3) / 4) * ((W + 7) / 8) + 3) / 4, per_head = num_sms / heads;
     return blocks <= kTeams * (per_head < 1 ? 1 : per_head);
