@@ -68,6 +68,8 @@ struct TeamParams {
 // Images of a head (blockIdx.x) and, spread over all blocks, zeros for what later kernels add to.  Comes right behind the forward of a
 // training step, which lets it start early: spread over the SMs (launch_spread) a step of 8 x 56 x 56, 3 heads, bf16 takes 70.7 us,
 // piled up 77.8; 3 x 54 x 54, 8 heads 75.0 and 84.0; 23 x 27 x 10, 3 heads, fp32 62.4 and 66.4.
+// (One block an SM, for fp32, whose blocks take longer, two: 6 x 42 x 10, 4 heads, fp32 50.0 and 48.9, 4 x 28 x 28, 8 heads 63.2 and 62.8; 3 x 54 x 54,
+// 8 heads, bf16 78.5 and 79.2.)
 template <typename T>
 __global__ void __launch_bounds__(256)
 bwd_prep_kernel(const float* __restrict__ wk, const float* __restrict__ wv, unsigned char* __restrict__ images, float* dwk, float* dwv, float* dbias)
@@ -605,7 +607,7 @@ cudaError_t launch_t(BwdPass what, const Problem& p, const BackwardArgs& ga, con
     if (what == BwdPass::point) {
         CUtensorMap mk, mv;
         if (!make_tile_map(&mk, p.k, es, p.B, p.H, p.W, C, ch, 10, 6) || !make_tile_map(&mv, p.v, es, p.B, p.H, p.W, C, ch, 10, 6)) return cudaErrorInvalidValue;
-        e = launch_spread<bwd_prep_kernel<T>>(dim3((unsigned)p.heads, 9), 256, stream, p.wk, p.wv, ws.images, ga.dwk, ga.dwv, ga.dbias);
+        e = launch_spread<bwd_prep_kernel<T>, sizeof(T) == 4 ? 2 : 1>(dim3((unsigned)p.heads, 9), 256, stream, p.wk, p.wv, ws.images, ga.dwk, ga.dwv, ga.dbias);
         if (e != cudaSuccess) return e;
         return launch_chained(bwd_point_kernel<T>, grid, kThreads, Plan<kPointImages>::total, stream, mk, mv, P);
     }

@@ -63,10 +63,10 @@ inline cudaError_t launch_chained(void (*kernel)(Params...), dim3 grid, int thre
 }
 
 // The same for a prep kernel of few small blocks that may follow a kernel which lets it start early: with so much shared memory that an
-// SM takes no more than its share of the blocks.  (They come while most SMs are still busy; without it they pile up, eight and more on
+// SM takes no more than its share of the blocks, or `Least` of them.  (They come while most SMs are still busy; without it they pile up, eight and more on
 // the first few SMs that come free, and wait and work there: a forward of 8 x 56 x 56, 3 heads, bf16 and one with heads of 64 in turn 28.3 us
 // spread, 34.3 piled up, 31.2 without early starts.  By themselves forwards with a prep launch take the same either way.)
-template <auto Kernel, typename... Args>
+template <auto Kernel, unsigned Least = 1, typename... Args>
 inline cudaError_t launch_spread(dim3 grid, int threads, cudaStream_t stream, Args... args) {
     constexpr int kMost = 224 * 1024, kOwn = 2048;         // of 228 KB; a block's own and the system's beside it
     static int sms[64] = {};                               // of each device, once the kernel is set up there
@@ -80,7 +80,9 @@ inline cudaError_t launch_spread(dim3 grid, int threads, cudaStream_t stream, Ar
         if (e != cudaSuccess) return e;
         if (dev < 64) sms[dev] = n;
     }
-    const unsigned blocks = grid.x * grid.y, share = (blocks + (unsigned)n - 1) / (unsigned)n;
+    const unsigned blocks = grid.x * grid.y;
+    unsigned share = (blocks + (unsigned)n - 1) / (unsigned)n;
+    if (share < Least) share = Least;
     return launch_chained(Kernel, grid, threads, share > 8 ? 0 : kMost / share - kOwn, stream, args...);
 }
 

@@ -86,7 +86,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
 __device__ __forceinline__ bool wait_last_phases(uint32_t first, int slots, int uses) {
     bool ok = true;
 #pragma unroll 1
-    for (int i = 0; i < slots && i < uses; ++i) ok = mbar_wait<true>(first + 8u * (uint32_t)i, (uint32_t)((uses - 1 - i) / slots) & 1u) && ok;
+    for (int i = 0; i < slots && i < uses; ++i) ok = mbar_park(first + 8u * (uint32_t)i, (uint32_t)((uses - 1 - i) / slots) & 1u) && ok;
     return ok;
 }
 

@@ -406,8 +406,11 @@ bool umma_split_builds_images(int B, int H, int W, int heads, int num_sms) {
 cudaError_t launch_umma_split_prep(const Problem& p, void* workspace, cudaStream_t stream) {
     return of_heads(p, [&](auto heads) {
         using H = decltype(heads);
-        return launch_spread<umma_split_prep_kernel<typename H::type, H::dim>>(dim3((unsigned)p.heads, prep_parts(H::dim)), 256, stream, p.wk, p.wv,
-                              static_cast<unsigned char*>(workspace));
+        const dim3 grid((unsigned)p.heads, prep_parts(H::dim));
+        unsigned char* img = static_cast<unsigned char*>(workspace);
+        // Heads of 16 have little to lay out: spread, 17 x 48 x 51, 7 heads, bf16 takes 29.5 us instead of 29.2, and what follows UMMA_TS gains 2 % at most.
+        if constexpr (H::dim > 16) return launch_spread<umma_split_prep_kernel<typename H::type, H::dim>>(grid, 256, stream, p.wk, p.wv, img);
+        else return launch_chained(umma_split_prep_kernel<typename H::type, H::dim>, grid, 256, 0, stream, p.wk, p.wv, img);
     });
 }
 
